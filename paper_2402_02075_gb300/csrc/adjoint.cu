@@ -294,7 +294,7 @@ cgks_status cgks_linearize(cgks_ctx* ctx) {
     k_recon_jac<<<grid_for(F.nc, 128), 128, 0, ctx->stream>>>(ra, ctx->Jr);
   }
   PointArgs pa{F.ngp, F.nf, F.nc, F.gp_face, F.fL, F.fR, F.ftag, F.gp_x, F.gp_A, F.fshift, F.ctr, ctx->rc,
-               ctx->dt, ctx->gpr, ph, ctx->derr};
+               ctx->dt, ctx->gpr, ph, ctx->derr, ctx->tab};
   k_point_jac<<<grid_for(F.ngp, 128), 128, 0, ctx->stream>>>(pa, ctx->Jp);
   CK(cudaMemcpyAsync(ctx->adt, ctx->dt, sizeof(double) * F.nc, cudaMemcpyDeviceToDevice, ctx->stream));
   CK(cudaGetLastError());

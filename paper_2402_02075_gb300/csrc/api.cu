@@ -6,6 +6,7 @@
 #include <new>
 #include <string>
 
+#include "fastmath.cuh"
 #include "internal.cuh"
 
 static thread_local std::string g_create_error;
@@ -273,6 +274,17 @@ static cgks_status check_params(cgks_ctx* ctx, const cgks_params* p) {
   return CGKS_OK;
 }
 
+static cgks_status upload_tables(cgks_ctx* ctx) {
+  struct Table {  // the same for every context
+    double t[HALF_TABLE];
+    Table() { half_table_fill(t); }
+  };
+  static const Table table;
+  CKS(dalloc(ctx, ctx->ctx_allocs, &ctx->tab, HALF_TABLE));
+  CK(cudaMemcpyAsync(ctx->tab, table.t, sizeof(table.t), cudaMemcpyHostToDevice, ctx->stream));
+  return CGKS_OK;
+}
+
 cgks_status cgks_create(const cgks_params* params, void* cuda_stream, cgks_ctx** out) {
   if (!out) return cgks_fail(nullptr, CGKS_EINVAL, "out is NULL");
   *out = nullptr;
@@ -299,7 +311,8 @@ cgks_status cgks_create(const cgks_params* params, void* cuda_stream, cgks_ctx**
       (s = dalloc(ctx, ctx->ctx_allocs, &ctx->d_count, 1)) != CGKS_OK ||
       (s = dalloc(ctx, ctx->ctx_allocs, &ctx->d_skipped, 1)) != CGKS_OK ||
       (s = dalloc(ctx, ctx->ctx_allocs, &ctx->nrm_part, 1024)) != CGKS_OK ||
-      (s = dalloc(ctx, ctx->ctx_allocs, &ctx->nrm, 1)) != CGKS_OK) {
+      (s = dalloc(ctx, ctx->ctx_allocs, &ctx->nrm, 1)) != CGKS_OK ||
+      (s = upload_tables(ctx)) != CGKS_OK) {
     g_create_error = ctx->err;
     cgks_destroy(ctx);
     return s;

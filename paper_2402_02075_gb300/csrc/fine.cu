@@ -144,7 +144,7 @@ cgks_status fine_fluxes(cgks_ctx* ctx, const double* W, const double* G, const d
   }
   if (ctx->P.dt_mode == 1) CKS(global_min_dt(ctx, ctx->dt, F.nc));
   PointArgs pa{F.ngp, F.nf, F.nc, F.gp_face, F.fL, F.fR, F.ftag, F.gp_x, F.gp_A, F.fshift, F.ctr, ctx->rc,
-               ctx->dt, ctx->gpr, ph, ctx->derr};
+               ctx->dt, ctx->gpr, ph, ctx->derr, ctx->tab};
   {
     ProfScope ps(ctx, state ? PK_POINTS : PK_POINTS_FLUX, (double)F.ngp,
                  F.ngp * (52.0 + (state ? 8.0 * CGKS_GPR : 40.0)) + F.nf * 36.0 + F.nc * 432.0);

@@ -17,6 +17,7 @@
 #pragma once
 #include <cstring>
 
+#include "flux.cuh"
 #include "internal.cuh"
 #include "kinetic.cuh"
 
@@ -547,6 +548,7 @@ struct PointArgs {
   double* gpr;  // [ngp][CGKS_GPR] records: flux x weight / dt (5), interface state (5), area vector (3), alpha
   Phys ph;
   DevErr* err;
+  const double* tab;  // table of half_gauss (device)
 };
 
 // inputs of one Gauss point: unit normal n, 1/|weight x area|, face, cells, the left and right
@@ -732,16 +734,55 @@ HD void point_flux(const double nd[3], double iw, bool bnd, int tag, const T WLg
   if (STATE) rotate_out<T>(Wacc, n, t1, t2, Wg);
 }
 
+// value and gradient (global frame) of a reconstruction polynomial at offset X from its centroid: with
+// t_d = c_d + (H X)_d / 2 (H the Hessian) the gradient is 2 t - c and the value c_0 + X.t
+HD void eval_both(const double* rcp, const double X[3], double Wv[5], double Gq[15]) {
+  const double hx = 0.5 * X[0], hy = 0.5 * X[1], hz = 0.5 * X[2];
+#pragma unroll
+  for (int q = 0; q < 5; ++q) {
+    const double2* c2 = reinterpret_cast<const double2*>(rcp + 10 * q);
+    const double2 A = c2[0], B = c2[1], C = c2[2], D = c2[3], E = c2[4];
+    // (A.x A.y) (B.x B.y) ...: 1 X Y Z X^2 Y^2 Z^2 XY YZ XZ
+    const double tx = A.y + C.x * X[0] + D.y * hy + E.y * hz;
+    const double ty = B.x + C.y * X[1] + D.y * hx + E.x * hz;
+    const double tz = B.y + D.x * X[2] + E.x * hy + E.y * hx;
+    Wv[q] = A.x + X[0] * tx + X[1] * ty + X[2] * tz;
+    Gq[3 * q + 0] = 2.0 * tx - A.y;
+    Gq[3 * q + 1] = 2.0 * ty - B.x;
+    Gq[3 * q + 2] = 2.0 * tz - B.y;
+  }
+}
+
 // one contiguous record per point, so that the gather reads a face's points as one segment; STATE
 // false (the defect of the V-cycle): the flux alone, in the record's first five entries
 template <bool STATE = true>
 HD void gks_point_body(int64_t g, const PointArgs& a) {
-  PointIn p;
-  point_inputs(g, a, p);
+  const int64_t ngp = a.ngp, nf = a.nf, nc = a.nc;
+  const int64_t f = a.gp_face[g];
+  const int64_t L = a.fL[f], R = a.fR[f];
+  const int tag = a.ftag[f];
+  const double x[3] = {a.gp_x[g], a.gp_x[ngp + g], a.gp_x[2 * ngp + g]};
+  const double Av[3] = {a.gp_A[g], a.gp_A[ngp + g], a.gp_A[2 * ngp + g]};
+  const double a2 = Av[0] * Av[0] + Av[1] * Av[1] + Av[2] * Av[2], iw = fast_rsqrt(a2);
+  const double n[3] = {Av[0] * iw, Av[1] * iw, Av[2] * iw};
+  double WL[5], GL[15], WR[5], GR[15], X[3], dtf = a.dt[L];
+#pragma unroll
+  for (int d = 0; d < 3; ++d) X[d] = x[d] - a.ctr[d * nc + L];
+  eval_both(a.rc + (int64_t)CGKS_RC * L, X, WL, GL);
+  if (R >= 0) {
+#pragma unroll
+    for (int d = 0; d < 3; ++d) X[d] = x[d] - a.ctr[d * nc + R];
+    if (tag >= 0)  // a periodic face
+#pragma unroll
+      for (int d = 0; d < 3; ++d) X[d] -= a.fshift[d * nf + f];
+    eval_both(a.rc + (int64_t)CGKS_RC * R, X, WR, GR);
+    dtf = fmin(dtf, a.dt[R]);
+  } else if (!bc_ghost<double>(tag, n, WL, GL, WR, GR, a.ph.gamma, a.ph.Winf)) {
+    set_err(a.err, CGKS_ENAN, (int)f, 3);
+  }
   double Fg[5], Wg[5], alpha;
-  point_flux<double, STATE>(p.n, p.iw, p.R < 0, a.ftag[p.f], p.WL, p.GL, p.WR, p.GR, p.dtf, a.ph, Fg, Wg, alpha, a.err,
-                            p.f);
-  const int64_t ngp = a.ngp;
+  const int bad = gks_flux<STATE>(n, a2 * iw, R < 0, WL, GL, WR, GR, dtf, a.ph, a.tab, Fg, Wg, alpha);
+  if (bad) set_err(a.err, CGKS_ENAN, (int)f, bad);
   double2* dst = reinterpret_cast<double2*>(a.gpr + (int64_t)CGKS_GPR * g);
   dst[0] = make_double2(Fg[0], Fg[1]);
   dst[1] = make_double2(Fg[2], Fg[3]);
@@ -752,8 +793,8 @@ HD void gks_point_body(int64_t g, const PointArgs& a) {
   dst[2] = make_double2(Fg[4], Wg[0]);
   dst[3] = make_double2(Wg[1], Wg[2]);
   dst[4] = make_double2(Wg[3], Wg[4]);
-  dst[5] = make_double2(a.gp_A[g], a.gp_A[ngp + g]);
-  dst[6] = make_double2(a.gp_A[2 * ngp + g], alpha);
+  dst[5] = make_double2(Av[0], Av[1]);
+  dst[6] = make_double2(Av[2], alpha);
 }
 
 // forward-mode linearisation of one Gauss point: Jp[(10 k + o) ngp + g] = d out_o / d in_k with

@@ -127,6 +127,7 @@ struct cgks_ctx {
   double *ffl = nullptr;            // first-order face fluxes of level 0
   float* ffl32 = nullptr;           // their FP32 directional derivatives
   double *nrm_part = nullptr, *nrm = nullptr, *h_nrm = nullptr;
+  double* tab = nullptr;            // table of half_gauss (fastmath.cuh), built with the context
   DevErr* derr = nullptr;
   DevErr* h_err = nullptr;
   int64_t* d_count = nullptr;
