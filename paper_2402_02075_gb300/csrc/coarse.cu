@@ -8,7 +8,8 @@
 // KFVS face fluxes x area (FP64)
 __global__ void k_kfvs_faces(int64_t nf, const int32_t* __restrict__ fL, const int32_t* __restrict__ fR,
                              const int32_t* __restrict__ ftag, const double* __restrict__ nS, int64_t nc,
-                             const double* __restrict__ W, double* __restrict__ ff, Phys ph, DevErr* err) {
+                             const double* __restrict__ W, double* __restrict__ ff, Phys ph, DevErr* err,
+                             const double* __restrict__ tab) {
   const int64_t f = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (f >= nf) return;
   const double s = nS[3 * nf + f];
@@ -28,7 +29,7 @@ __global__ void k_kfvs_faces(int64_t nf, const int32_t* __restrict__ fL, const i
   } else if (!bc_ghost<double>(ftag[f], n, WL, nullptr, WR, nullptr, ph.gamma, ph.Winf)) {
     set_err(err, CGKS_ENAN, (int)L, 20);
   }
-  if (!kfvs_flux<double>(WL, WR, n, ph.K, ph.gamma - 1.0, F)) set_err(err, CGKS_ENAN, (int)L, 21);
+  if (!kfvs_flux<double>(WL, WR, n, ph.K, ph.gamma - 1.0, F, tab)) set_err(err, CGKS_ENAN, (int)L, 21);
 #pragma unroll
   for (int q = 0; q < 5; ++q) ff[q * nf + f] = s * F[q];
 }
@@ -288,7 +289,8 @@ cgks_status kfvs_residual(cgks_ctx* ctx, int lev, const double* W, double* res) 
   {
     ProfScope ps(ctx, PK_KFVS_FACES, (double)L.nf, L.nf * 84.0 + L.nc * 40.0);
     const int b = spread_block(L.nf, 256, ctx->n_sm);
-    k_kfvs_faces<<<grid_for(L.nf, b), b, 0, ctx->stream>>>(L.nf, L.fL, L.fR, L.ftag, L.nS, L.nc, W, ff, ph, ctx->derr);
+    k_kfvs_faces<<<grid_for(L.nf, b), b, 0, ctx->stream>>>(L.nf, L.fL, L.fR, L.ftag, L.nS, L.nc, W, ff, ph, ctx->derr,
+                                                     ctx->tab);
   }
   {
     ProfScope ps(ctx, PK_KFVS_GATHER, (double)L.nc, L.nc * 44.0 + entries * 4.0 + L.nf * 48.0);

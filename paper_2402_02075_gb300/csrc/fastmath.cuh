@@ -103,7 +103,7 @@ __device__ __forceinline__ double exp_scaled(double r, int n, const double* __re
 // exp(-x), x >= 0 (10 FP64 operations; 0 above 700, where the flux's weights vanish; NaN stays NaN)
 HD double exp_neg(double x, const double* __restrict__ tab) {
 #ifdef __CUDA_ARCH__
-  if (!(__double2hiint(x) < 0x4085e000)) return x != x ? x : 0.0;  // 700
+  if (__double2hiint(x) >= 0x4085e000) return x != x ? x : 0.0;  // 700, or not a number
   const int n = __float2int_rn(half_to_float(x) * 92.332482616893658f);  // 64 / ln 2
   const double nd = int_to_double(n);
   return exp_scaled(fma(-nd, HALF_L2, fma(-nd, HALF_L1, x)), n, tab);
@@ -113,11 +113,29 @@ HD double exp_neg(double x, const double* __restrict__ tab) {
 #endif
 }
 
+// x > 0 (false for NaN, zero and below 2^-1042) by an integer comparison of the high word
+HD bool positive(double x) {
+#ifdef __CUDA_ARCH__
+  return (unsigned)(__double2hiint(x) - 1) < 0x7ff00000u;
+#else
+  return x > 0.0;
+#endif
+}
+
+// the smaller of two positive numbers, by an integer comparison (a NaN loses, as with fmin)
+HD double min_positive(double a, double b) {
+#ifdef __CUDA_ARCH__
+  return __double_as_longlong(b) < __double_as_longlong(a) ? b : a;
+#else
+  return fmin(a, b);
+#endif
+}
+
 // m0 = erfc(y)/2, e = exp(-y^2)
 HD void half_gauss(double y, const double* __restrict__ tab, double& m0, double& e) {
 #ifdef __CUDA_ARCH__
   const double a = fabs(y);
-  if (!(a < (double)HALF_MAX)) {
+  if (__double2hiint(a) >= 0x40180000) {  // 6, or not a number
     half_gauss_general(y, m0, e);
     return;
   }
@@ -138,7 +156,7 @@ HD void half_gauss(double y, const double* __restrict__ tab, double& m0, double&
   q = fma(d, q, c23.x);
   q = fma(d, q, c01.y);
   m0 = e * q;
-  if (y < 0.0) m0 = 1.0 - m0;
+  if (__double2hiint(y) < 0) m0 = 1.0 - m0;
 #else
   (void)tab;
   m0 = 0.5 * erfc(y);

@@ -776,7 +776,7 @@ HD void gks_point_body(int64_t g, const PointArgs& a) {
 #pragma unroll
       for (int d = 0; d < 3; ++d) X[d] -= a.fshift[d * nf + f];
     eval_both(a.rc + (int64_t)CGKS_RC * R, X, WR, GR);
-    dtf = fmin(dtf, a.dt[R]);
+    dtf = min_positive(dtf, a.dt[R]);
   } else if (!bc_ghost<double>(tag, n, WL, GL, WR, GR, a.ph.gamma, a.ph.Winf)) {
     set_err(a.err, CGKS_ENAN, (int)f, 3);
   }

@@ -47,7 +47,7 @@ HD bool gks_side(const double w[5], const double n[3], double s, double gm1, con
   double e;
   half_gauss(-s * (g.sl * g.U), tab, g.m0, e);
   g.beta = (s * 0.56418958354775628695) * (e * g.sl);
-  return w[0] > 0.0 && g.p > 0.0;
+  return positive(w[0]) && positive(g.p);
 }
 
 // time coefficients of Eq. 2nd-flux integrated over [0, dt] that multiply the two sides' moments
@@ -288,7 +288,7 @@ HD int gks_flux(const double n[3], double weight, bool bnd, const double WL[5], 
   const double er = 0.5 * (gr.U * ar1 + gr.h * gr.m0) + (k2 * gr.h + 0.5 * jm2) * gr.m0;
   const double E = gl.rho * el + gr.rho * er;
   const double p = gm1 * (E - 0.5 * Mn * U), h = p * r;
-  if (!(rho > 0.0 && p > 0.0) && !bad) bad = 5;
+  if (!(positive(rho) && positive(p)) && !bad) bad = 5;
   // collision times (Sec. 2.3)
   const double jump = fabs((gl.p - gr.p) * fast_rcp(gl.p + gr.p));
   double tau, tn;
@@ -301,7 +301,7 @@ HD int gks_flux(const double n[3], double weight, bool bnd, const double WL[5], 
   }
   // exact integrals over [0, dt] of the time coefficients
   // (tn vanishes where the viscosity and the pressure jump do)
-  const double edt = tn > 0.0 ? exp_neg(dt * fast_rcp(tn), tab) : 0.0, om = 1.0 - edt;
+  const double edt = positive(tn) ? exp_neg(dt * fast_rcp(tn), tab) : 0.0, om = 1.0 - edt;
   const double q4 = tn * om, tte = tn * dt * edt;
   const double q1 = dt - q4, q5 = (tau + tn) * q4 - tte;
   const double q2 = q5 - tau * dt;

@@ -4,6 +4,7 @@
 #pragma once
 #include <cuda_runtime.h>
 
+#include "fastmath.cuh"
 #include "internal.cuh"
 
 
@@ -321,21 +322,43 @@ HD bool bc_ghost(int tag, const T n[3], const T W[5], const T* G, T Wg[5], T* Gg
 // right), added into F in the global frame.  With U = u . n, h = p / rho = 1/(2 lambda) and the
 // half-space moments m_k = <u_n^k> / rho: mass rho m1; momentum rho (m1 u + (m2 - U m1) n), since the
 // tangential velocity is carried with the normal flux; energy rho (m3 + m1 (|u|^2 - U^2 + (K+2) h))/2.
-// One division (1/rho) and one reciprocal square root (sqrt(lambda) = 1/sqrt(2 h)) per side.
+// One reciprocal (1/rho) and one reciprocal square root (sqrt(lambda) = 1/sqrt(2 h)) per side.  In FP64
+// the FP64 pipe bounds the face kernel: reciprocals and the half-space pair are those of fastmath.cuh
+// (tab its table).
 template <typename T>
-HD bool kfvs_side(const T w[5], const T n[3], T K, T gm1, T s, T F[5]) {
-  const T r = T(1) / w[0];
+HD T kfvs_rcp(T x) { return T(1) / x; }
+template <>
+HD double kfvs_rcp<double>(double x) { return fast_rcp(x); }
+template <typename T>
+HD T kfvs_rsqrt(T x) { return trsqrt(x); }
+template <>
+HD double kfvs_rsqrt<double>(double x) { return fast_rsqrt(x); }
+template <typename T>
+HD void kfvs_half(T y, const double*, T& m0, T& e) {
+  m0 = T(0.5) * terfc(y);
+  e = texp(-y * y);
+}
+template <>
+HD void kfvs_half<double>(double y, const double* tab, double& m0, double& e) { half_gauss(y, tab, m0, e); }
+template <typename T>
+HD bool kfvs_positive(T x) { return x > T(0); }
+template <>
+HD bool kfvs_positive<double>(double x) { return positive(x); }
+
+template <typename T>
+HD bool kfvs_side(const T w[5], const T n[3], T K, T gm1, T s, T F[5], const double* tab) {
+  const T r = kfvs_rcp(w[0]);
   const T u[3] = {w[1] * r, w[2] * r, w[3] * r};
   const T u2 = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
   const T p = gm1 * (w[4] - T(0.5) * (w[1] * u[0] + w[2] * u[1] + w[3] * u[2]));
   const T h = p * r;
-  const T sl = trsqrt(T(2) * h);  // sqrt(lambda)
+  const T sl = kfvs_rsqrt(T(2) * h);  // sqrt(lambda)
   const T U = u[0] * n[0] + u[1] * n[1] + u[2] * n[2];
   const T x = sl * U;
-  T m[4];
-  m[0] = T(0.5) * terfc(-s * x);
+  T m[4], e;
+  kfvs_half(-s * x, tab, m[0], e);
   // U m0 + s exp(-lambda U^2) / (2 sqrt(pi lambda)), 1/sqrt(lambda) = 2 h sqrt(lambda)
-  m[1] = U * m[0] + s * T(0.56418958354775628695) * texp(-x * x) * (h * sl);
+  m[1] = U * m[0] + s * T(0.56418958354775628695) * e * (h * sl);
   m[2] = U * m[1] + h * m[0];
   m[3] = U * m[2] + T(2) * h * m[1];
   const T rho = w[0];
@@ -344,16 +367,17 @@ HD bool kfvs_side(const T w[5], const T n[3], T K, T gm1, T s, T F[5]) {
 #pragma unroll
   for (int d = 0; d < 3; ++d) F[1 + d] += rm1 * u[d] + rn * n[d];
   F[4] += T(0.5) * rho * (m[3] + m[1] * (u2 - U * U + (T(2) + K) * h));
-  return w[0] > T(0) && p > T(0);
+  return kfvs_positive(w[0]) && kfvs_positive(p);
 }
 
 // KFVS flux (int_{u_n > 0} u_n psi g^l + int_{u_n < 0} u_n psi g^r) in the global frame through a
 // face with unit normal n
 template <typename T>
-HD bool kfvs_flux(const T WL[5], const T WR[5], const T n[3], T K, T gm1, T F[5]) {
+HD bool kfvs_flux(const T WL[5], const T WR[5], const T n[3], T K, T gm1, T F[5],
+                  const double* tab = nullptr) {
 #pragma unroll
   for (int q = 0; q < 5; ++q) F[q] = T(0);
-  const bool okl = kfvs_side<T>(WL, n, K, gm1, T(1), F);
-  const bool okr = kfvs_side<T>(WR, n, K, gm1, T(-1), F);
+  const bool okl = kfvs_side<T>(WL, n, K, gm1, T(1), F, tab);
+  const bool okr = kfvs_side<T>(WR, n, K, gm1, T(-1), F, tab);
   return okl && okr;
 }
