@@ -207,6 +207,13 @@ HD void rotate_out(const T f[5], const T n[3], const T t1[3], const T t2[3], T F
 }
 
 
+// x^(1/(gamma - 1)); the exponent of a diatomic gas is 5/2 (a power costs about 150 FP64 instructions)
+template <typename T>
+HD T tpow_igm1(T x, T igm1) {
+  if (igm1 > T(2.5 - 1e-14) && igm1 < T(2.5 + 1e-14)) return x * x * tsqrt(x);
+  return tpow(x, igm1);
+}
+
 // ghost state (and gradient when G != nullptr) of a boundary face with outward unit normal n.
 // tag 1 slip wall (mirror), 2 no-slip adiabatic wall (mirror, velocity reversed), 3 farfield by 1D
 // Riemann invariants, 4 supersonic inflow (free stream), 5 supersonic outflow (copy).
@@ -268,15 +275,16 @@ HD bool bc_ghost(int tag, const T n[3], const T W[5], const T* G, T Wg[5], T* Gg
     return true;
   }
   if (tag == 3) {
-    const T gm1 = gamma - T(1);
-    const T rho = W[0];
-    const T u[3] = {W[1] / rho, W[2] / rho, W[3] / rho};
+    // the state beyond has the entropy of the side the flow comes from, so that its density is that
+    // side's times (c_b/c)^(2/(gamma - 1))
+    const T gm1 = gamma - T(1), igm1 = T(1) / gm1;
+    const T rho = W[0], r = T(1) / rho, ri = T(Winf[0]), rri = T(1) / ri;
+    const T u[3] = {W[1] * r, W[2] * r, W[3] * r};
     const T p = gm1 * (W[4] - T(0.5) * rho * (u[0] * u[0] + u[1] * u[1] + u[2] * u[2]));
-    const T ri = T(Winf[0]);
-    const T ui[3] = {T(Winf[1]) / ri, T(Winf[2]) / ri, T(Winf[3]) / ri};
+    const T ui[3] = {T(Winf[1]) * rri, T(Winf[2]) * rri, T(Winf[3]) * rri};
     const T pi = gm1 * (T(Winf[4]) - T(0.5) * ri * (ui[0] * ui[0] + ui[1] * ui[1] + ui[2] * ui[2]));
     if (!(rho > T(0)) || !(p > T(0))) return false;
-    const T c = tsqrt(gamma * p / rho), ci = tsqrt(gamma * pi / ri);
+    const T c = tsqrt(gamma * p * r), ci = tsqrt(gamma * pi * rri);
     const T un = u[0] * n[0] + u[1] * n[1] + u[2] * n[2];
     const T uni = ui[0] * n[0] + ui[1] * n[1] + ui[2] * n[2];
     if (un >= c) {
@@ -289,20 +297,14 @@ HD bool bc_ghost(int tag, const T n[3], const T W[5], const T* G, T Wg[5], T* Gg
       for (int q = 0; q < 5; ++q) Wg[q] = T(Winf[q]);
       return true;
     }
-    const T Rp = un + T(2) * c / gm1, Rm = uni - T(2) * ci / gm1;
+    const T Rp = un + T(2) * c * igm1, Rm = uni - T(2) * ci * igm1;
     const T unb = T(0.5) * (Rp + Rm), cb = T(0.25) * gm1 * (Rp - Rm);
-    T s, ut[3];
-    if (unb > T(0)) {
-      s = p / tpow(rho, gamma);
+    const bool out = unb > T(0);
+    T ut[3];
 #pragma unroll
-      for (int d = 0; d < 3; ++d) ut[d] = u[d] - un * n[d];
-    } else {
-      s = pi / tpow(ri, gamma);
-#pragma unroll
-      for (int d = 0; d < 3; ++d) ut[d] = ui[d] - uni * n[d];
-    }
-    const T rb = tpow(cb * cb / (gamma * s), T(1) / gm1);
-    const T pb = rb * cb * cb / gamma;
+    for (int d = 0; d < 3; ++d) ut[d] = out ? u[d] - un * n[d] : ui[d] - uni * n[d];
+    const T m = cb / (out ? c : ci);
+    const T rb = (out ? rho : ri) * tpow_igm1<T>(m * m, igm1);
     T ub[3], u2 = T(0);
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
@@ -312,7 +314,7 @@ HD bool bc_ghost(int tag, const T n[3], const T W[5], const T* G, T Wg[5], T* Gg
     Wg[0] = rb;
 #pragma unroll
     for (int d = 0; d < 3; ++d) Wg[1 + d] = rb * ub[d];
-    Wg[4] = pb / gm1 + T(0.5) * rb * u2;
+    Wg[4] = rb * cb * cb * (igm1 / gamma) + T(0.5) * rb * u2;
     return true;
   }
   return false;
@@ -325,14 +327,15 @@ HD bool bc_ghost(int tag, const T n[3], const T W[5], const T* G, T Wg[5], T* Gg
 // One reciprocal (1/rho) and one reciprocal square root (sqrt(lambda) = 1/sqrt(2 h)) per side.  In FP64
 // the FP64 pipe bounds the face kernel: reciprocals and the half-space pair are those of fastmath.cuh
 // (tab its table).
+// reciprocal and reciprocal square root: fastmath.cuh in FP64
 template <typename T>
-HD T kfvs_rcp(T x) { return T(1) / x; }
+HD T trcp(T x) { return T(1) / x; }
 template <>
-HD double kfvs_rcp<double>(double x) { return fast_rcp(x); }
+HD double trcp<double>(double x) { return fast_rcp(x); }
 template <typename T>
-HD T kfvs_rsqrt(T x) { return trsqrt(x); }
+HD T trsqrt_fast(T x) { return trsqrt(x); }
 template <>
-HD double kfvs_rsqrt<double>(double x) { return fast_rsqrt(x); }
+HD double trsqrt_fast<double>(double x) { return fast_rsqrt(x); }
 template <typename T>
 HD void kfvs_half(T y, const double*, T& m0, T& e) {
   m0 = T(0.5) * terfc(y);
@@ -347,12 +350,12 @@ HD bool kfvs_positive<double>(double x) { return positive(x); }
 
 template <typename T>
 HD bool kfvs_side(const T w[5], const T n[3], T K, T gm1, T s, T F[5], const double* tab) {
-  const T r = kfvs_rcp(w[0]);
+  const T r = trcp(w[0]);
   const T u[3] = {w[1] * r, w[2] * r, w[3] * r};
   const T u2 = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
   const T p = gm1 * (w[4] - T(0.5) * (w[1] * u[0] + w[2] * u[1] + w[3] * u[2]));
   const T h = p * r;
-  const T sl = kfvs_rsqrt(T(2) * h);  // sqrt(lambda)
+  const T sl = trsqrt_fast(T(2) * h);  // sqrt(lambda)
   const T U = u[0] * n[0] + u[1] * n[1] + u[2] * n[2];
   const T x = sl * U;
   T m[4], e;
