@@ -62,6 +62,7 @@ struct ReconArgs {
   double *rc, *dt;
   Phys ph;
   DevErr* err;
+  const int32_t* nbr;  // [6][nc] cell across each local face, -1 on the boundary (null: from the faces)
 };
 
 // value of stencil input c of slot s as T: with T = DualD the one seeded input carries derivative 1
@@ -208,16 +209,134 @@ HD T time_step(int64_t i, const ReconArgs& a, const T Q0[5]) {
   return ph.cfl_fine * V / s;
 }
 
-HD void reconstruct_body(int64_t i, const ReconArgs& a) {
-  {
-    __align__(16) double out[CGKS_RC];
-    reconstruct_cell<double>(i, a, -1, out);
-    double2* dst = reinterpret_cast<double2*>(a.rc + (int64_t)CGKS_RC * i);
+// the non-linear combination of one variable (Sec. 3.4): b the p^2 coefficients of X,Y,Z,X^2,Y^2,Z^2,XY,
+// YZ,XZ, p1 the compressed Green-Gauss gradient, gl the least-squares gradient -> its 10 coefficients.
+// The indicator's first part, sum_d <(d_d p2)^2> = |b_0..2|^2 + tr(M H^2), takes the squared Hessian once
+HD void weno_variable(double Q0, const double b[9], const double p1[3], const double gl[3], double V23, double V43,
+                      const double M2[6], double eps, double out[10]) {
+  const double a0 = Q0 - (b[3] * M2[0] + b[4] * M2[1] + b[5] * M2[2] + b[6] * M2[3] + b[7] * M2[4] + b[8] * M2[5]);
+  const double bGG = V23 * (p1[0] * p1[0] + p1[1] * p1[1] + p1[2] * p1[2]);
+  const double bLS = V23 * (gl[0] * gl[0] + gl[1] * gl[1] + gl[2] * gl[2]);
+  const double beta1 = min_positive(bGG, bLS);
+  const double s6 = b[6] * b[6], s7 = b[7] * b[7], s8 = b[8] * b[8];
+  const double c6 = s6 + s8, c7 = s6 + s7, c8 = s7 + s8;
+  const double hxx = 4.0 * b[3] * b[3] + c6, hyy = 4.0 * b[4] * b[4] + c7, hzz = 4.0 * b[5] * b[5] + c8;
+  // twice the off-diagonal entries of the squared Hessian, half of each
+  const double hxy = 2.0 * b[6] * (b[3] + b[4]) + b[8] * b[7];
+  const double hyz = 2.0 * b[7] * (b[4] + b[5]) + b[6] * b[8];
+  const double hxz = 2.0 * b[8] * (b[3] + b[5]) + b[6] * b[7];
+  double off = M2[3] * hxy;
+  off += M2[4] * hyz;
+  off += M2[5] * hxz;
+  double first = b[0] * b[0] + b[1] * b[1] + b[2] * b[2];
+  first += M2[0] * hxx;
+  first += M2[1] * hyy;
+  first += M2[2] * hzz;
+  first += 2.0 * off;
+  // 4 (b_3^2 + b_4^2 + b_5^2) + b_6^2 + b_7^2 + b_8^2
+  const double second = (hxx + hyy + hzz) - (c6 + s7);
+  const double beta2 = V23 * first + V43 * second;
+  const double rden = fast_rcp(Q0 * Q0 + beta1 + 1e-40);
+  const double bt1 = beta1 * rden, bt2 = beta2 * rden;
+  const double sig = bt2 - bt1;
+  // w_m = g_m (1 + (sig/d_m)^2) with d_m = eps + beta~_m and g_1 = g_2 = 1/2, normalised with one
+  // reciprocal: w_1 : w_2 = (d_1^2 + sig^2) d_2^2 : (d_2^2 + sig^2) d_1^2
+  const double d1 = eps + bt1, d2 = eps + bt2;
+  const double s2 = sig * sig, d11 = d1 * d1, d22 = d2 * d2;
+  const double A1 = (d11 + s2) * d22, A2 = (d22 + s2) * d11;
+  const double inv = fast_rcp(A1 + A2);
+  const double w1 = A1 * inv, w2 = A2 * inv;
+  const double c2 = 2.0 * w2, c1 = w1 - w2;
+  out[0] = c2 * a0 + c1 * Q0;
 #pragma unroll
-    for (int k = 0; k < CGKS_RC / 2; ++k) dst[k] = make_double2(out[2 * k], out[2 * k + 1]);
+  for (int d = 0; d < 3; ++d) out[1 + d] = c2 * b[d] + c1 * p1[d];
+#pragma unroll
+  for (int j = 3; j < 9; ++j) out[1 + j] = c2 * b[j];
+}
+
+// ghost average and gradient (W 5, grad W 15) of boundary slot m of cell i
+HD void recon_ghost(int64_t i, int m, const ReconArgs& a, double Wg[5], double Gg[15]) {
+  const int64_t nc = a.nc, nf = a.nf, f = a.cf[(int64_t)m * nc + i];
+  double Q0[5], G0[15];
+#pragma unroll
+  for (int q = 0; q < 5; ++q) Q0[q] = a.W[q * nc + i];
+#pragma unroll
+  for (int j = 0; j < 15; ++j) G0[j] = a.G[j * nc + i];
+  const double n[3] = {a.fnrm[f], a.fnrm[nf + f], a.fnrm[2 * nf + f]};
+  if (!bc_ghost<double>(a.ftag[f], n, Q0, G0, Wg, Gg, a.ph.gamma, a.ph.Winf)) set_err(a.err, CGKS_ENAN, (int)i, 1);
+}
+
+// cell across local face m of cell i, -1 on the boundary
+HD int32_t recon_neighbour(int64_t i, int m, const ReconArgs& a) {
+  const int64_t k = (int64_t)m * a.nc + i;
+  if (a.nbr) return a.nbr[k];
+  const int64_t f = a.cf[k];
+  return a.fR[f] < 0 ? -1 : (a.cside[k] ? a.fL[f] : a.fR[f]);
+}
+
+// reconstruction of variable q of cell i.  ghost(m, v) gives the boundary slot's (W_q, gradient of W_q).
+// Each neighbour's difference and gradient are added into a coefficient on their own (one fused
+// multiply-add per operator entry).  Green-Gauss from the differences: the outward S n / |Omega| of a
+// closed cell sum to zero, so sum (Q_m + Q_0) w_m = sum (Q_m - Q_0) w_m, without the cancellation
+template <typename Ghost>
+HD void reconstruct_variable(int64_t i, int q, const ReconArgs& a, const Ghost& ghost, double out[10]) {
+  const int64_t nc = a.nc;
+  const int nt = a.ctype[i] == 7 ? 5 : a.ctype[i];  // faces: pyramids (type 7) have 5
+  const double Q0 = a.W[q * nc + i];
+  double b[9], gg[3] = {0.0, 0.0, 0.0}, gl[3] = {0.0, 0.0, 0.0};
+#pragma unroll
+  for (int j = 0; j < 9; ++j) b[j] = 0.0;
+  int32_t nb[6];
+#pragma unroll
+  for (int m = 0; m < 6; ++m) nb[m] = m < nt ? recon_neighbour(i, m, a) : 0;
+  double v[6][4];
+#pragma unroll
+  for (int m = 0; m < 6; ++m) {
+    if (m >= nt) continue;
+    if (nb[m] >= 0) {
+      v[m][0] = a.W[q * nc + nb[m]];
+#pragma unroll
+      for (int d = 0; d < 3; ++d) v[m][1 + d] = a.G[(3 * q + d) * nc + nb[m]];
+    } else {
+      ghost(m, v[m]);
+    }
   }
-  double Q0[5];
 #pragma unroll
+  for (int m = 0; m < 6; ++m) {
+    if (m >= nt) continue;
+    const double dQ = v[m][0] - Q0;
+#pragma unroll
+    for (int j = 0; j < 9; ++j) {
+      b[j] += a.Kop[(j * 24 + m) * nc + i] * dQ;
+      b[j] += a.Kop[(j * 24 + 6 + 3 * m) * nc + i] * v[m][1];
+      b[j] += a.Kop[(j * 24 + 7 + 3 * m) * nc + i] * v[m][2];
+      b[j] += a.Kop[(j * 24 + 8 + 3 * m) * nc + i] * v[m][3];
+    }
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      gg[d] += a.ggw[(3 * m + d) * nc + i] * dQ;
+      gl[d] += a.lsw[(3 * m + d) * nc + i] * dQ;
+    }
+  }
+  double M2[6];
+#pragma unroll
+  for (int j = 0; j < 6; ++j) M2[j] = a.aux[(2 + j) * nc + i];
+  const double al = a.alpha[i];
+  const double p1[3] = {al * gg[0], al * gg[1], al * gg[2]};
+  weno_variable(Q0, b, p1, gl, a.aux[i], a.aux[nc + i], M2, a.ph.weno_eps, out);
+}
+
+HD void reconstruct_body(int64_t i, const ReconArgs& a) {
+  const auto ghost_of = [&](int q) {
+    return [&a, i, q](int m, double v[4]) {
+      double Wg[5], Gg[15];
+      recon_ghost(i, m, a, Wg, Gg);
+      v[0] = Wg[q];
+      for (int d = 0; d < 3; ++d) v[1 + d] = Gg[3 * q + d];
+    };
+  };
+  for (int q = 0; q < 5; ++q) reconstruct_variable(i, q, a, ghost_of(q), a.rc + (int64_t)CGKS_RC * i + 10 * q);
+  double Q0[5];
   for (int q = 0; q < 5; ++q) Q0[q] = a.W[q * a.nc + i];
   a.dt[i] = time_step<double>(i, a, Q0);
 }

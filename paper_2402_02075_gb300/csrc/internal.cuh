@@ -66,6 +66,7 @@ struct Fine {
   double *fshift = nullptr, *fnrm = nullptr, *fctr = nullptr;    // [3][nf] each
   int32_t *cf = nullptr;                                         // [6][nc] face of each local face
   int8_t* cside = nullptr;                                       // [6][nc] 0: cell is L, 1: R
+  int32_t* nbr = nullptr;                                        // [6][nc] cell across each local face, -1 none
   int32_t *c2f_ptr = nullptr, *c2f = nullptr;                    // cell -> faces (ascending)
   double *Kop = nullptr;                                         // [216][nc] p^2 operator
   double *ggw = nullptr;                                         // [18][nc] outward S n / (2|Omega|)

@@ -514,6 +514,18 @@ __global__ void k_cell_geom(int64_t nc, const int8_t* ctype, const int64_t* cptr
   for (int j = 0; j < 6; ++j) m2[j * nc + c] = M2[j] / V;
 }
 
+// cell across each local face (-1 on the boundary and for absent faces), for the reconstruction
+__global__ void k_neighbours(int64_t nc, const int8_t* ctype, const int32_t* cf, const int8_t* cside, const int32_t* fL,
+                             const int32_t* fR, int32_t* nbr) {
+  const int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (c >= nc) return;
+  for (int m = 0; m < 6; ++m) {
+    const int64_t k = (int64_t)m * nc + c;
+    const int32_t f = cf[k];
+    nbr[k] = m >= cell_nfaces(ctype[c]) || fR[f] < 0 ? -1 : (cside[k] ? fL[f] : fR[f]);
+  }
+}
+
 // cell -> faces CSR with ascending face ids (the deterministic gather order)
 __global__ void k_fill_c2f(int64_t nc, const int8_t* ctype, const int32_t* cf, const int32_t* ptr, int32_t* c2f) {
   int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -635,6 +647,8 @@ cgks_status build_fine_mesh(cgks_ctx* ctx, int64_t n_nodes, const double* xyz, i
   if (nb)
     k_write_boundary<<<grid_for(nb, B), B, 0, st>>>(nb, n_int + np, nonper, brank, bowner, d_btag, nc, F.fL, F.fR,
                                                     F.ftag, F.ftagR, F.flf, F.cf, F.cside);
+  CKS(dalloc(ctx, M, &F.nbr, 6 * nc));
+  k_neighbours<<<grid_for(nc, B), B, 0, st>>>(nc, F.ctype, F.cf, F.cside, F.fL, F.fR, F.nbr);
   // Gauss points
   int32_t* gcnt;
   CKS(dalloc(ctx, tmp, &gcnt, nf));
