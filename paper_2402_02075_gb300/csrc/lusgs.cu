@@ -14,6 +14,7 @@
 #include <algorithm>
 #include <vector>
 
+#include "fastmath.cuh"
 #include "internal.cuh"
 
 namespace {
@@ -74,7 +75,7 @@ __global__ void k_jpl_assign(int64_t nc, const int32_t* __restrict__ ptr, const 
 }
 
 __device__ __forceinline__ void euler_flux_n(const double W[5], const double n[3], double g, double F[5]) {
-  const double rho = W[0], r = 1.0 / rho;
+  const double rho = W[0], r = fast_rcp(rho);
   const double u[3] = {W[1] * r, W[2] * r, W[3] * r};
   const double p = (g - 1.0) * (W[4] - 0.5 * rho * (u[0] * u[0] + u[1] * u[1] + u[2] * u[2]));
   const double un = u[0] * n[0] + u[1] * n[1] + u[2] * n[2];
@@ -85,75 +86,89 @@ __device__ __forceinline__ void euler_flux_n(const double W[5], const double n[3
 }
 
 __device__ __forceinline__ double wave_speed(const double* W, int64_t nc, int64_t i, const double n[3], double g) {
-  const double rho = W[i], r = 1.0 / rho;
+  const double rho = W[i], r = fast_rcp(rho);
   const double u[3] = {W[nc + i] * r, W[2 * nc + i] * r, W[3 * nc + i] * r};
   const double p = (g - 1.0) * (W[4 * nc + i] - 0.5 * rho * (u[0] * u[0] + u[1] * u[1] + u[2] * u[2]));
   return fabs(u[0] * n[0] + u[1] * n[1] + u[2] * n[2]) + sqrt(g * p * r);
 }
 
-// lambda of every face: max over its cells of |U.n| + c (the cell's own on boundary faces)
+// lambda of every face: max over its cells of |U.n| + c (the cell's own on boundary faces); nS: unit
+// normal and length of the face's summed area vector
 __global__ void k_lusgs_lambda(int64_t nf, const int32_t* __restrict__ fL, const int32_t* __restrict__ fR,
-                               const double* __restrict__ Sn, int64_t nc, const double* __restrict__ W, double g,
+                               const double* __restrict__ nS, int64_t nc, const double* __restrict__ W, double g,
                                double* __restrict__ lam) {
   const int64_t f = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (f >= nf) return;
-  const double S[3] = {Sn[f], Sn[nf + f], Sn[2 * nf + f]};
-  const double s = sqrt(S[0] * S[0] + S[1] * S[1] + S[2] * S[2]);
-  if (s == 0.0) {
+  if (nS[3 * nf + f] == 0.0) {
     lam[f] = 0.0;
     return;
   }
-  const double n[3] = {S[0] / s, S[1] / s, S[2] / s};
+  const double n[3] = {nS[f], nS[nf + f], nS[2 * nf + f]};
   const int32_t a = fL[f], b = fR[f];
   const double la = wave_speed(W, nc, a, n, g);
   lam[f] = b >= 0 ? fmax(la, wave_speed(W, nc, b, n, g)) : la;
 }
 
-// D_i = |Omega_i| / dt_i + 1/2 sum_p lambda_p S_p, in ascending face order
+// Threads per cell of the kernels below.  A colour of a level holds a few hundred to a few thousand
+// cells of 10 to 40 faces, and each sweep waits for the one before it, so the time of a sweep is that
+// of one cell: a thread that walks the faces alone takes 100 us (a warp's FP64 instruction takes 64
+// clocks of its sub-partition, about 100 of them per face, and the loads are dependent).  LANES threads
+// share the faces and add their parts in a fixed tree: a quarter warp, or a whole warp where the
+// colour has so few cells that every sub-partition still gets at most two.  V-cycle of the 64x32x8 ramp
+// (8.4 k and 4 k coarse cells, 38 sweeps per step and level): 2.3 ms against 9.7.
+template <int LANES>
+__device__ __forceinline__ double lane_sum(double v) {
+#pragma unroll
+  for (int d = LANES / 2; d > 0; d >>= 1) v += __shfl_xor_sync(0xffffffffu, v, d);
+  return v;
+}
+
+// D_i = |Omega_i| / dt_i + 1/2 sum_p lambda_p S_p
+template <int LANES>
 __global__ void k_lusgs_diag(int64_t nc, int64_t nf, const int32_t* __restrict__ ptr, const int32_t* __restrict__ c2f,
                              const int32_t* __restrict__ fL, const int32_t* __restrict__ fR,
-                             const double* __restrict__ Sn, const double* __restrict__ lam,
+                             const double* __restrict__ nS, const double* __restrict__ lam,
                              const double* __restrict__ vol, const double* __restrict__ dt, double* __restrict__ D) {
-  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (i >= nc) return;
+  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, i = t / LANES;
+  const bool live = i < nc;
   double s = 0.0;
-  for (int32_t k = ptr[i]; k < ptr[i + 1]; ++k) {
+  const int32_t e = live ? ptr[i + 1] : 0;
+  for (int32_t k = live ? ptr[i] + (int)(t % LANES) : 0; k < e; k += LANES) {
     const int64_t f = c2f[k];
     if (fL[f] == fR[f]) continue;
-    const double S[3] = {Sn[f], Sn[nf + f], Sn[2 * nf + f]};
-    s += lam[f] * sqrt(S[0] * S[0] + S[1] * S[1] + S[2] * S[2]);
+    s += lam[f] * nS[3 * nf + f];
   }
-  D[i] = vol[i] / dt[i] + 0.5 * s;
+  s = lane_sum<LANES>(s);
+  if (live && t % LANES == 0) D[i] = vol[i] / dt[i] + 0.5 * s;
 }
 
 struct SweepArgs {
   int64_t nc, nf;
   const int32_t *ptr, *c2f, *fL, *fR, *color, *cells;
-  const double *Sn, *lam, *W, *R, *F, *D;
+  const double *nS, *lam, *W, *R, *F, *D;
   double* dU;
   double gamma;
 };
 
 // forward (FWD) or backward sweep over the cells of colour k: neighbours of a lower (forward) or
 // higher (backward) colour contribute 1/2 [F_n(U_j + dU_j) - F_n(U_j) - lambda dU_j] S
-template <bool FWD>
+template <bool FWD, int LANES>
 __global__ void k_lusgs_sweep(SweepArgs a, int64_t count, int32_t k) {
-  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (t >= count) return;
-  const int64_t nc = a.nc, nf = a.nf, i = a.cells[t];
-  double acc[5];
-#pragma unroll
-  for (int q = 0; q < 5; ++q) acc[q] = FWD ? a.R[q * nc + i] + a.F[q * nc + i] : 0.0;
-  for (int32_t e = a.ptr[i]; e < a.ptr[i + 1]; ++e) {
+  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, pos = t / LANES;
+  const int64_t nc = a.nc, nf = a.nf;
+  const bool live = pos < count;
+  const int64_t i = live ? a.cells[pos] : 0;
+  double acc[5] = {0, 0, 0, 0, 0};
+  const int32_t end = live ? a.ptr[i + 1] : 0;
+  for (int32_t e = live ? a.ptr[i] + (int)(t % LANES) : 0; e < end; e += LANES) {
     const int64_t f = a.c2f[e];
     const int64_t j = other_cell(a.fL, a.fR, f, i);
     if (j < 0) continue;
     if (FWD ? a.color[j] >= k : a.color[j] <= k) continue;
-    const double S[3] = {a.Sn[f], a.Sn[nf + f], a.Sn[2 * nf + f]};
-    const double s = sqrt(S[0] * S[0] + S[1] * S[1] + S[2] * S[2]);
+    const double s = a.nS[3 * nf + f];
     if (s == 0.0) continue;
     const double sg = a.fL[f] == i ? 1.0 : -1.0;
-    const double n[3] = {sg * (S[0] / s), sg * (S[1] / s), sg * (S[2] / s)};
+    const double n[3] = {sg * a.nS[f], sg * a.nS[nf + f], sg * a.nS[2 * nf + f]};
     double Wj[5], Wp[5], dUj[5], Fp[5], F0[5];
 #pragma unroll
     for (int q = 0; q < 5; ++q) {
@@ -163,16 +178,25 @@ __global__ void k_lusgs_sweep(SweepArgs a, int64_t count, int32_t k) {
     }
     euler_flux_n(Wp, n, a.gamma, Fp);
     euler_flux_n(Wj, n, a.gamma, F0);
-    const double lam = a.lam[f];
+    const double lam = a.lam[f], hs = 0.5 * s;
 #pragma unroll
-    for (int q = 0; q < 5; ++q) {
-      const double o = 0.5 * ((Fp[q] - F0[q]) - lam * dUj[q]) * s;
-      acc[q] = FWD ? acc[q] - o : acc[q] + o;
-    }
+    for (int q = 0; q < 5; ++q) acc[q] += ((Fp[q] - F0[q]) - lam * dUj[q]) * hs;
   }
+#pragma unroll
+  for (int q = 0; q < 5; ++q) acc[q] = lane_sum<LANES>(acc[q]);
+  if (!live || t % LANES != 0) return;
   const double Di = a.D[i];
 #pragma unroll
-  for (int q = 0; q < 5; ++q) a.dU[q * nc + i] = FWD ? acc[q] / Di : a.dU[q * nc + i] - acc[q] / Di;
+  for (int q = 0; q < 5; ++q)
+    a.dU[q * nc + i] = FWD ? (a.R[q * nc + i] + a.F[q * nc + i] - acc[q]) / Di : a.dU[q * nc + i] - acc[q] / Di;
+}
+
+template <bool FWD>
+void sweep(const SweepArgs& a, int64_t cnt, int32_t k, int n_sm, cudaStream_t st) {
+  if (cnt <= (int64_t)n_sm * 4 * 2)
+    k_lusgs_sweep<FWD, 32><<<grid_for(32 * cnt, 32), 32, 0, st>>>(a, cnt, k);
+  else
+    k_lusgs_sweep<FWD, 8><<<grid_for(8 * cnt, 64), 64, 0, st>>>(a, cnt, k);
 }
 
 // W += dU, skipping (and counting) cells whose rho or p would not stay positive
@@ -261,22 +285,18 @@ cgks_status lusgs_step(cgks_ctx* ctx, int l) {
   CoarseBuf& B = ctx->C[l];
   cudaStream_t st = ctx->stream;
   const double g = ctx->P.gamma;
-  k_lusgs_lambda<<<grid_for(L.nf, 256), 256, 0, st>>>(L.nf, L.fL, L.fR, L.Sn, L.nc, B.W, g, B.lam);
-  k_lusgs_diag<<<grid_for(L.nc, 256), 256, 0, st>>>(L.nc, L.nf, L.c2f_ptr, L.c2f, L.fL, L.fR, L.Sn, B.lam, L.vol,
-                                                     B.dt, B.Dg);
-  SweepArgs a{L.nc, L.nf, L.c2f_ptr, L.c2f, L.fL, L.fR, B.color, B.order, L.Sn, B.lam, B.W, B.R, B.F, B.Dg, B.dU, g};
+  k_lusgs_lambda<<<grid_for(L.nf, 128), 128, 0, st>>>(L.nf, L.fL, L.fR, L.nS, L.nc, B.W, g, B.lam);
+  k_lusgs_diag<8><<<grid_for(8 * L.nc, 128), 128, 0, st>>>(L.nc, L.nf, L.c2f_ptr, L.c2f, L.fL, L.fR, L.nS, B.lam, L.vol,
+                                                           B.dt, B.Dg);
+  SweepArgs a{L.nc, L.nf, L.c2f_ptr, L.c2f, L.fL, L.fR, B.color, B.order, L.nS, B.lam, B.W, B.R, B.F, B.Dg, B.dU, g};
   const int32_t ncol = (int32_t)B.coff.size() - 1;
   for (int32_t k = 0; k < ncol; ++k) {
-    const int64_t cnt = B.coff[k + 1] - B.coff[k];
-    SweepArgs ak = a;
-    ak.cells = B.order + B.coff[k];
-    k_lusgs_sweep<true><<<grid_for(cnt, 128), 128, 0, st>>>(ak, cnt, k);
+    a.cells = B.order + B.coff[k];
+    sweep<true>(a, B.coff[k + 1] - B.coff[k], k, ctx->n_sm, st);
   }
   for (int32_t k = ncol - 1; k >= 0; --k) {
-    const int64_t cnt = B.coff[k + 1] - B.coff[k];
-    SweepArgs ak = a;
-    ak.cells = B.order + B.coff[k];
-    k_lusgs_sweep<false><<<grid_for(cnt, 128), 128, 0, st>>>(ak, cnt, k);
+    a.cells = B.order + B.coff[k];
+    sweep<false>(a, B.coff[k + 1] - B.coff[k], k, ctx->n_sm, st);
   }
   k_lusgs_apply<<<grid_for(L.nc, 256), 256, 0, st>>>(L.nc, B.dU, B.W, g, (unsigned long long*)ctx->d_skipped,
                                                       ctx->derr);
