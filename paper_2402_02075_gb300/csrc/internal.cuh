@@ -236,7 +236,7 @@ cgks_status kfvs_residual(cgks_ctx* ctx, int lev, const double* W, double* res);
 cgks_status kfvs_jvp(cgks_ctx* ctx, int lev, const double* W0, const double* X, int x_is_state, double* res);
 cgks_status coarse_dt(cgks_ctx* ctx, int lev, const double* W, double* dt);
 cgks_status vcycle_once(cgks_ctx* ctx, double* norm_dev);
-// LU-SGS step on coarse level l for the defect C[l].R + C[l].F with the time steps in C[l].dt
-cgks_status lusgs_step(cgks_ctx* ctx, int l);
+// LU-SGS step on coarse level l for the defect C[l].R + F with the time steps in C[l].dt
+cgks_status lusgs_step(cgks_ctx* ctx, int l, const double* F);
 cgks_status lusgs_color_count(cgks_ctx* ctx, int l, int32_t* colors, int32_t* n_colors);
 cgks_status step_once(cgks_ctx* ctx, double* norm_dev);

@@ -278,8 +278,8 @@ cgks_status lusgs_colors(cgks_ctx* ctx, int l) {
   return CGKS_OK;
 }
 
-// one LU-SGS step on level l for the defect B.R + B.F with the time steps in B.dt
-cgks_status lusgs_step(cgks_ctx* ctx, int l) {
+// one LU-SGS step on level l for the defect B.R + F with the time steps in B.dt
+cgks_status lusgs_step(cgks_ctx* ctx, int l, const double* F) {
   CKS(lusgs_colors(ctx, l));
   const Level& L = ctx->L[l];
   CoarseBuf& B = ctx->C[l];
@@ -288,7 +288,7 @@ cgks_status lusgs_step(cgks_ctx* ctx, int l) {
   k_lusgs_lambda<<<grid_for(L.nf, 128), 128, 0, st>>>(L.nf, L.fL, L.fR, L.nS, L.nc, B.W, g, B.lam);
   k_lusgs_diag<8><<<grid_for(8 * L.nc, 128), 128, 0, st>>>(L.nc, L.nf, L.c2f_ptr, L.c2f, L.fL, L.fR, L.nS, B.lam, L.vol,
                                                            B.dt, B.Dg);
-  SweepArgs a{L.nc, L.nf, L.c2f_ptr, L.c2f, L.fL, L.fR, B.color, B.order, L.nS, B.lam, B.W, B.R, B.F, B.Dg, B.dU, g};
+  SweepArgs a{L.nc, L.nf, L.c2f_ptr, L.c2f, L.fL, L.fR, B.color, B.order, L.nS, B.lam, B.W, B.R, F, B.Dg, B.dU, g};
   const int32_t ncol = (int32_t)B.coff.size() - 1;
   for (int32_t k = 0; k < ncol; ++k) {
     a.cells = B.order + B.coff[k];
