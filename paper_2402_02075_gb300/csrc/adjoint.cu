@@ -35,9 +35,10 @@ __global__ void __launch_bounds__(128) k_point_jac(PointArgs a, double* Jp) {
   if (g < a.ngp) point_jacobian_body(g, a, Jp);
 }
 
-__global__ void __launch_bounds__(128) k_recon_jac(ReconArgs a, double* Jr) {
-  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (i < a.nc) recon_jacobian_body(i, a, Jr);
+// 32 cells x (5 variables and the time step) per block, as the reconstruction
+__global__ void __launch_bounds__(192, 2) k_recon_jac(ReconArgs a, double* Jr) {
+  const int64_t i = blockIdx.x * (int64_t)32 + (threadIdx.x & 31);
+  if (i < a.nc) recon_jacobian_variable(i, threadIdx.x >> 5, a, Jr);
 }
 
 // ---- transposed product ------------------------------------------------------------------------
@@ -60,9 +61,11 @@ __global__ void __launch_bounds__(512) k_vjp_slots(VjpArgs a) {
   const int tx = threadIdx.x, ty = threadIdx.y;
   const int64_t i = blockIdx.x * (int64_t)32 + tx;
   for (int o = ty; o < CGKS_RJ_OUT; o += 16) cbs[o][tx] = i < a.nc ? a.cbuf[(int64_t)o * a.nc + i] : 0.0;
+  __shared__ bool dense[32];
+  if (ty == 0 && i < a.nc) dense[tx] = vjp_boundary_cell(i, a);
   __syncthreads();
   if (i >= a.nc) return;
-  for (int g = ty; g < 20 + 6 * 5; g += 16) vjp_slot_body(i, g, a, &cbs[0][tx], 32);
+  for (int g = ty; g < 20 + 6 * 5; g += 16) vjp_slot_body(i, g, a, &cbs[0][tx], 32, dense[tx]);
 }
 
 // the reconstruction's transposed product recomputed per cell (adjoint_recompute 1), in place of
@@ -244,7 +247,8 @@ static ReconArgs lin_recon_args(cgks_ctx* ctx) {
   const Fine& F = ctx->F;
   const int64_t nc = F.nc;
   return ReconArgs{F.nc, F.nf, F.ctype, F.cf, F.fL, F.fR, F.ftag, F.cside, F.fnrm, F.Kop, F.ggw, F.lsw, F.aux, F.dtw,
-                   F.vol, ctx->aWG, ctx->aWG + 5 * nc, ctx->aWG + 20 * nc, nullptr, nullptr, make_phys(ctx->P), ctx->derr};
+                   F.vol, ctx->aWG, ctx->aWG + 5 * nc, ctx->aWG + 20 * nc, nullptr, nullptr, make_phys(ctx->P), ctx->derr,
+                   F.nbr};
 }
 
 static cgks_status run_vjp(cgks_ctx* ctx, const double* rbar, const double* gbar, double* out) {
@@ -281,7 +285,7 @@ cgks_status cgks_linearize(cgks_ctx* ctx) {
   const Phys ph = make_phys(ctx->P);
   CKS(fine_fluxes(ctx, ctx->W, ctx->G, ctx->alpha));  // coefficients and time steps at the state
   ReconArgs ra{F.nc, F.nf, F.ctype, F.cf, F.fL, F.fR, F.ftag, F.cside, F.fnrm, F.Kop, F.ggw, F.lsw, F.aux, F.dtw,
-               F.vol, ctx->W, ctx->G, ctx->alpha, ctx->rc, ctx->dt, ph, ctx->derr};
+               F.vol, ctx->W, ctx->G, ctx->alpha, ctx->rc, ctx->dt, ph, ctx->derr, F.nbr};
   ctx->lin_recompute = ctx->P.adjoint_recompute != 0;
   if (ctx->lin_recompute) {
     // keep the state; the reconstruction's transposed product is recomputed from it in every product
@@ -291,7 +295,7 @@ cgks_status cgks_linearize(cgks_ctx* ctx) {
     CK(cudaMemcpyAsync(ctx->aWG + 20 * F.nc, ctx->alpha, sizeof(double) * F.nc, cudaMemcpyDeviceToDevice, ctx->stream));
   } else {
     if (!ctx->Jr) CKS(dalloc(ctx, ctx->mesh_allocs, &ctx->Jr, (size_t)CGKS_RJ_ROWS * F.nc));
-    k_recon_jac<<<grid_for(F.nc, 128), 128, 0, ctx->stream>>>(ra, ctx->Jr);
+    k_recon_jac<<<grid_for(F.nc, 32), 192, 0, ctx->stream>>>(ra, ctx->Jr);
   }
   PointArgs pa{F.ngp, F.nf, F.nc, F.gp_face, F.fL, F.fR, F.ftag, F.gp_x, F.gp_A, F.fshift, F.ctr, ctx->rc,
                ctx->dt, ctx->gpr, ph, ctx->derr, ctx->tab};

@@ -19,6 +19,14 @@ struct VjpArgs {
   double *out;                // [20][nc]: cotangents of (W, G)
 };
 
+// whether cell i has a boundary face (its ghosts then tie its own inputs to every variable)
+HD bool vjp_boundary_cell(int64_t i, const VjpArgs& a) {
+  const int nt = a.ctype[i] == 7 ? 5 : a.ctype[i];
+  for (int m = 0; m < nt; ++m)
+    if (a.fR[a.cf[(int64_t)m * a.nc + i]] < 0) return true;
+  return false;
+}
+
 // per Gauss point: cotangents of (flux, interface state) from those of (Res, Gnew) of its two cells,
 // times Jp^T -> cotangents of the point inputs
 HD void vjp_point_body(int64_t g, const VjpArgs& a) {
@@ -78,18 +86,23 @@ HD void vjp_coef_body(int64_t i, const VjpArgs& a) {
 #pragma unroll
       for (int q = 0; q < 5; ++q) {
         const double w = pb[q], gx = pb[5 + 3 * q], gy = pb[6 + 3 * q], gz = pb[7 + 3 * q];
-        // basis 1, X, Y, Z, X^2, Y^2, Z^2, XY, YZ, XZ and its gradient
+        // basis 1, X, Y, Z, X^2, Y^2, Z^2, XY, YZ, XZ and its gradient, through w X + g (the FP64 pipe
+        // bounds this kernel: 19 operations per variable instead of 31)
         double* c = cb + 10 * q;
+        const double ax = w * X[0] + gx, ay = w * X[1] + gy, az = w * X[2] + gz;
         c[0] += w;
-        c[1] += w * X[0] + gx;
-        c[2] += w * X[1] + gy;
-        c[3] += w * X[2] + gz;
-        c[4] += w * X[0] * X[0] + 2.0 * X[0] * gx;
-        c[5] += w * X[1] * X[1] + 2.0 * X[1] * gy;
-        c[6] += w * X[2] * X[2] + 2.0 * X[2] * gz;
-        c[7] += w * X[0] * X[1] + X[1] * gx + X[0] * gy;
-        c[8] += w * X[1] * X[2] + X[2] * gy + X[1] * gz;
-        c[9] += w * X[0] * X[2] + X[2] * gx + X[0] * gz;
+        c[1] += ax;
+        c[2] += ay;
+        c[3] += az;
+        c[4] += X[0] * (ax + gx);
+        c[5] += X[1] * (ay + gy);
+        c[6] += X[2] * (az + gz);
+        c[7] += X[1] * ax;
+        c[7] += X[0] * gy;
+        c[8] += X[2] * ay;
+        c[8] += X[1] * gz;
+        c[9] += X[2] * ax;
+        c[9] += X[0] * gz;
       }
       cb[CGKS_RC] += w_dt * a.pbar[(int64_t)g * CGKS_PB + 40];
     }
@@ -99,17 +112,25 @@ HD void vjp_coef_body(int64_t i, const VjpArgs& a) {
 }
 
 // phase 2, per cell and row group g with the cell's 51 cotangents cb[o * cs]:
-//   g < 20   own-slot input c = g: self[c][i] = sum_o Jr[51 c + o][i] cb[o]
+//   g < 20   own-slot input c = g: self[c][i] = sum_o Jr[51 c + o][i] cb[o]; on a cell without boundary
+//            faces (dense false) over the rows that can differ from zero, its variable's 10 coefficients
+//            and the time step
 //   g >= 20  neighbour slot s = 1 + (g - 20) / 5, variable q = (g - 20) % 5: its 4 inputs (W_q and the
 //            gradient of W_q) into the record of the slot's face for the cell across it (absent
 //            slots and boundary faces write nothing)
-HD void vjp_slot_body(int64_t i, int g, const VjpArgs& a, const double* cb, int cs) {
+HD void vjp_slot_body(int64_t i, int g, const VjpArgs& a, const double* cb, int cs, bool dense) {
   const int64_t nc = a.nc;
   if (g < 20) {
     const double* J = a.Jr + (int64_t)(CGKS_RJ_OUT * g) * nc + i;
-    double v = 0.0;
+    double v = g < 5 ? J[(int64_t)CGKS_RC * nc] * cb[CGKS_RC * cs] : 0.0;
+    if (dense) {
+#pragma unroll 10
+      for (int o = 0; o < CGKS_RC; ++o) v += J[(int64_t)o * nc] * cb[o * cs];
+    } else {
+      const int o0 = 10 * (g < 5 ? g : (g - 5) / 3);
 #pragma unroll
-    for (int o = 0; o < CGKS_RJ_OUT; ++o) v += J[(int64_t)o * nc] * cb[o * cs];
+      for (int o = 0; o < 10; ++o) v += J[(int64_t)(o0 + o) * nc] * cb[(o0 + o) * cs];
+    }
     a.self[(int64_t)g * nc + i] = v;
     return;
   }
@@ -130,16 +151,18 @@ HD void vjp_slot_body(int64_t i, int g, const VjpArgs& a, const double* cb, int 
   }
 }
 
+HD void vjp_slot_body(int64_t i, int g, const VjpArgs& a, const double* cb, int cs) {
+  vjp_slot_body(i, g, a, cb, cs, vjp_boundary_cell(i, a));
+}
 
 // per cell, the reconstruction's part of the transposed product recomputed from the state instead of
 // read from the stored linearisation (adjoint_recompute 1).  cb (stride cs) holds the cotangents of
 // the cell's 50 coefficients and of its time step; out: the cotangents of its own (W, grad W) ->
-// self, and those of each interior neighbour's (W_q, grad W_q) -> the record of that face side.  The
-// reverse mode of reconstruct_cell written out step by step: per variable the WENO combination of
-// Sec. 3.4 (weights, smoothness indicators, the minimum in beta_1 taking the smaller branch and half
-// of each at a tie, as the forward-mode linearisation does), then the linear maps of p^2 (Sec. 3.1),
-// Green-Gauss and least squares; then the ghost states of boundary faces (a function of the cell's own
-// W and grad W: their transposed Jacobian from forward-mode duals) and the local time step.
+// self, and those of each interior neighbour's (W_q, grad W_q) -> the record of that face side.  Per
+// variable the transposed linearisation of the WENO combination of Sec. 3.4 (weno_linear, at the same
+// stencil sums as the stored one), then the linear maps of p^2 (Sec. 3.1), Green-Gauss and least squares;
+// then the ghost states of boundary faces (a function of the cell's own W and grad W: their transposed
+// Jacobian from forward-mode duals) and the local time step.
 HD void vjp_recon_body(int64_t i, const ReconArgs& a, const VjpArgs& v, const double* cb, int64_t cs) {
   const int64_t nc = a.nc, nf = a.nf;
   const int nt = a.ctype[i] == 7 ? 5 : a.ctype[i];
@@ -165,113 +188,31 @@ HD void vjp_recon_body(int64_t i, const ReconArgs& a, const VjpArgs& v, const do
   double M2[6];
 #pragma unroll
   for (int j = 0; j < 6; ++j) M2[j] = a.aux[(2 + j) * nc + i];
-  const double g1 = 0.5, g2 = 0.5;
   for (int q = 0; q < 5; ++q) {
-    // stencil of variable q and the forward quantities
-    double Qn[6], Gn[6][3], b[9], gg[3] = {0, 0, 0}, gl[3] = {0, 0, 0};
-    for (int j = 0; j < 9; ++j) b[j] = 0.0;
+    // stencil of variable q, its sums and the linearised combination
+    double v4[6][4], b[9], gg[3], gl[3];
     for (int m = 0; m < nt; ++m) {
-      const int64_t f = a.cf[(int64_t)m * nc + i];
-      if (a.fR[f] >= 0) {
-        const int64_t nb = a.cside[(int64_t)m * nc + i] ? a.fL[f] : a.fR[f];
-        Qn[m] = a.W[q * nc + nb];
-        for (int e = 0; e < 3; ++e) Gn[m][e] = a.G[(3 * q + e) * nc + nb];
-      } else {
-        Qn[m] = gval[m][q];
-        for (int e = 0; e < 3; ++e) Gn[m][e] = gval[m][5 + 3 * q + e];
-      }
-      const double dQ = Qn[m] - Q0[q];
-      for (int j = 0; j < 9; ++j) {  // in the forward reconstruction's order
-        b[j] += a.Kop[(j * 24 + m) * nc + i] * dQ;
-        b[j] += a.Kop[(j * 24 + 6 + 3 * m) * nc + i] * Gn[m][0];
-        b[j] += a.Kop[(j * 24 + 7 + 3 * m) * nc + i] * Gn[m][1];
-        b[j] += a.Kop[(j * 24 + 8 + 3 * m) * nc + i] * Gn[m][2];
-      }
-      for (int d = 0; d < 3; ++d) {
-        gg[d] += a.ggw[(3 * m + d) * nc + i] * (Qn[m] + Q0[q]);
-        gl[d] += a.lsw[(3 * m + d) * nc + i] * dQ;
-      }
+      const int32_t nb = recon_neighbour(i, m, a);
+      v4[m][0] = nb >= 0 ? a.W[q * nc + nb] : gval[m][q];
+      for (int e = 0; e < 3; ++e) v4[m][1 + e] = nb >= 0 ? a.G[(3 * q + e) * nc + nb] : gval[m][5 + 3 * q + e];
     }
-    const double a0 = Q0[q] - (b[3] * M2[0] + b[4] * M2[1] + b[5] * M2[2] + b[6] * M2[3] + b[7] * M2[4] + b[8] * M2[5]);
-    const double p1[3] = {al * gg[0], al * gg[1], al * gg[2]};
-    const double bGG = V23 * (p1[0] * p1[0] + p1[1] * p1[1] + p1[2] * p1[2]);
-    const double bLS = V23 * (gl[0] * gl[0] + gl[1] * gl[1] + gl[2] * gl[2]);
-    const double beta1 = fmin(bGG, bLS);
-    const double vv[3][3] = {{2.0 * b[3], b[6], b[8]}, {b[6], 2.0 * b[4], b[7]}, {b[8], b[7], 2.0 * b[5]}};
-    double first = 0.0;
-    for (int d = 0; d < 3; ++d) {
-      const double* x = vv[d];
-      first += b[d] * b[d] + M2[0] * x[0] * x[0] + M2[1] * x[1] * x[1] + M2[2] * x[2] * x[2] +
-               2.0 * (M2[3] * x[0] * x[1] + M2[4] * x[1] * x[2] + M2[5] * x[0] * x[2]);
-    }
-    const double second = 4.0 * (b[3] * b[3] + b[4] * b[4] + b[5] * b[5]) + b[6] * b[6] + b[7] * b[7] + b[8] * b[8];
-    const double beta2 = V23 * first + V43 * second;
-    const double rden = 1.0 / (Q0[q] * Q0[q] + beta1 + 1e-40);
-    const double bt1 = beta1 * rden, bt2 = beta2 * rden, dif = bt2 - bt1;
-    const double d1 = ph.weno_eps + bt1, d2 = ph.weno_eps + bt2;
-    const double s2 = dif * dif, d11 = d1 * d1, d22 = d2 * d2;
-    const double A1 = g1 * (d11 + s2) * d22, A2 = g2 * (d22 + s2) * d11;
-    const double inv = 1.0 / (A1 + A2);
-    const double w1 = A1 * inv, w2 = A2 * inv;
-    const double c2 = w2 * (1.0 / g2), c1 = w1 - w2 * (g1 / g2);
-    // reverse: out[0] = c2 a0 + c1 Q0, out[1+d] = c2 b[d] + c1 p1[d] (d < 3), out[1+j] = c2 b[j] (j >= 3)
+    recon_sums(i, nt, Q0[q], a, v4, b, gg, gl);
+    WenoLin w;
+    weno_linear(Q0[q], b, gg, gl, al, V23, V43, M2, ph.weno_eps, w);
+    // out[0] = c2 a0 + c1 Q0, out[1+d] = c2 b[d] + c1 p1[d] (d < 3), out[1+j] = c2 b[j] (j >= 3), c1 = 1 - c2
     double ob[10];
     for (int k = 0; k < 10; ++k) ob[k] = cb[(10 * q + k) * cs];
-    double c2b = ob[0] * a0, c1b = ob[0] * Q0[q];
-    for (int d = 0; d < 3; ++d) {
-      c2b += ob[1 + d] * b[d];
-      c1b += ob[1 + d] * p1[d];
-    }
+    double c2b = ob[0] * (w.a0 - Q0[q]);
+    for (int d = 0; d < 3; ++d) c2b += ob[1 + d] * (b[d] - w.p1[d]);
     for (int j = 3; j < 9; ++j) c2b += ob[1 + j] * b[j];
-    const double a0b = c2 * ob[0];
-    double q0b = c1 * ob[0];
-    double bb[9], p1b[3];
-    for (int d = 0; d < 3; ++d) {
-      bb[d] = c2 * ob[1 + d];
-      p1b[d] = c1 * ob[1 + d];
-    }
-    for (int j = 3; j < 9; ++j) bb[j] = c2 * ob[1 + j];
-    // weights
-    const double w1b = c1b, w2b = c2b * (1.0 / g2) - c1b * (g1 / g2);
-    const double t = w1b * w1 + w2b * w2;
-    const double A1b = inv * (w1b - t), A2b = inv * (w2b - t);
-    const double d11b = A1b * g1 * d22 + A2b * g2 * (d22 + s2);
-    const double d22b = A1b * g1 * (d11 + s2) + A2b * g2 * d11;
-    const double s2b = A1b * g1 * d22 + A2b * g2 * d11;
-    const double bt1b = 2.0 * d1 * d11b - 2.0 * dif * s2b, bt2b = 2.0 * d2 * d22b + 2.0 * dif * s2b;
-    double beta1b = bt1b * rden;
-    const double beta2b = bt2b * rden;
-    const double rdenb = bt1b * beta1 + bt2b * beta2;
-    q0b += -rden * rden * 2.0 * Q0[q] * rdenb;
-    beta1b += -rden * rden * rdenb;
-    // smoothness indicator of p^2
-    const double firstb = V23 * beta2b, secondb = V43 * beta2b;
-    double vb[3][3];
-    for (int d = 0; d < 3; ++d) {
-      const double* x = vv[d];
-      bb[d] += 2.0 * b[d] * firstb;
-      vb[d][0] = firstb * (2.0 * M2[0] * x[0] + 2.0 * M2[3] * x[1] + 2.0 * M2[5] * x[2]);
-      vb[d][1] = firstb * (2.0 * M2[1] * x[1] + 2.0 * M2[3] * x[0] + 2.0 * M2[4] * x[2]);
-      vb[d][2] = firstb * (2.0 * M2[2] * x[2] + 2.0 * M2[4] * x[1] + 2.0 * M2[5] * x[0]);
-    }
-    bb[3] += 2.0 * vb[0][0] + 8.0 * b[3] * secondb;
-    bb[4] += 2.0 * vb[1][1] + 8.0 * b[4] * secondb;
-    bb[5] += 2.0 * vb[2][2] + 8.0 * b[5] * secondb;
-    bb[6] += vb[0][1] + vb[1][0] + 2.0 * b[6] * secondb;
-    bb[7] += vb[1][2] + vb[2][1] + 2.0 * b[7] * secondb;
-    bb[8] += vb[0][2] + vb[2][0] + 2.0 * b[8] * secondb;
-    // beta_1 = min(beta_GG, beta_LS)
-    const double bGGb = bGG < bLS ? beta1b : (bGG > bLS ? 0.0 : 0.5 * beta1b);
-    const double bLSb = bGG < bLS ? 0.0 : (bGG > bLS ? beta1b : 0.5 * beta1b);
-    double glb[3], ggb[3];
-    for (int d = 0; d < 3; ++d) {
-      p1b[d] += 2.0 * V23 * p1[d] * bGGb;
-      glb[d] = 2.0 * V23 * gl[d] * bLSb;
-      ggb[d] = al * p1b[d];
-    }
-    // a0 = Q0 - sum_j b_j M2_j
-    q0b += a0b;
+    const double a0b = w.c2 * ob[0];
+    double q0b = w.c1 * ob[0] + w.gQ * c2b + a0b, bb[9], glb[3], ggb[3];
+    for (int j = 0; j < 9; ++j) bb[j] = w.c2 * ob[1 + j] + w.gb[j] * c2b;
     for (int j = 3; j < 9; ++j) bb[j] -= a0b * M2[j - 3];
+    for (int d = 0; d < 3; ++d) {
+      glb[d] = w.gl[d] * c2b;
+      ggb[d] = al * (w.c1 * ob[1 + d] + w.gp[d] * c2b);
+    }
     // the linear maps, slot by slot
     for (int m = 0; m < nt; ++m) {
       const int64_t f = a.cf[(int64_t)m * nc + i];
@@ -286,7 +227,7 @@ HD void vjp_recon_body(int64_t i, const ReconArgs& a, const VjpArgs& v, const do
         ggsum += a.ggw[(3 * m + d) * nc + i] * ggb[d];
       }
       const double Qnb = dQb + ggsum;
-      q0b += ggsum - dQb;
+      q0b -= Qnb;
       if (a.fR[f] >= 0) {
         double* rec = v.rec + (2 * f + a.cside[(int64_t)m * nc + i]) * 20;
         rec[q] = Qnb;

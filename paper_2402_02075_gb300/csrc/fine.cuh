@@ -65,127 +65,6 @@ struct ReconArgs {
   const int32_t* nbr;  // [6][nc] cell across each local face, -1 on the boundary (null: from the faces)
 };
 
-// value of stencil input c of slot s as T: with T = DualD the one seeded input carries derivative 1
-template <typename T>
-struct Seed {
-  HD static T at(double v, bool) { return v; }
-};
-template <>
-struct Seed<DualD> {
-  HD static DualD at(double v, bool on) { return DualD(v, on ? 1.0 : 0.0); }
-};
-
-// reconstruction of cell i: 10 coefficients per variable.  Seeds of the
-// forward-mode linearisation: 20 s + c is component c of (W 5, grad W 15) of stencil slot s (slot 0
-// the cell, slot 1 + m its neighbour through local face m); seed < 0 for none
-template <typename T>
-HD void reconstruct_cell(int64_t i, const ReconArgs& a, int seed, T out[CGKS_RC]) {
-  const int64_t nc = a.nc, nf = a.nf;
-  const int nt = a.ctype[i] == 7 ? 5 : a.ctype[i];  // faces: pyramids (type 7) have 5
-  const Phys& ph = a.ph;
-  T Q0[5];
-#pragma unroll
-  for (int q = 0; q < 5; ++q) Q0[q] = Seed<T>::at(a.W[q * nc + i], seed == q);
-  // p^2 coefficients b[q][j] of X,Y,Z,X^2,Y^2,Z^2,XY,YZ,XZ; Green-Gauss and least-squares gradients
-  T b[5][9], gg[5][3], gl[5][3];
-#pragma unroll
-  for (int q = 0; q < 5; ++q) {
-#pragma unroll
-    for (int j = 0; j < 9; ++j) b[q][j] = 0.0;
-#pragma unroll
-    for (int d = 0; d < 3; ++d) gg[q][d] = gl[q][d] = 0.0;
-  }
-  for (int m = 0; m < nt; ++m) {
-    const int64_t f = a.cf[(int64_t)m * nc + i];
-    T Qn[5], Gn[15];
-    if (a.fR[f] >= 0) {
-      const int64_t nb = a.cside[(int64_t)m * nc + i] ? a.fL[f] : a.fR[f];
-      const int s0 = 20 * (m + 1);
-#pragma unroll
-      for (int q = 0; q < 5; ++q) Qn[q] = Seed<T>::at(a.W[q * nc + nb], seed == s0 + q);
-#pragma unroll
-      for (int j = 0; j < 15; ++j) Gn[j] = Seed<T>::at(a.G[j * nc + nb], seed == s0 + 5 + j);
-    } else {
-      T G0[15];
-#pragma unroll
-      for (int j = 0; j < 15; ++j) G0[j] = Seed<T>::at(a.G[j * nc + i], seed == 5 + j);
-      const T n[3] = {a.fnrm[f], a.fnrm[nf + f], a.fnrm[2 * nf + f]};
-      if (!bc_ghost<T>(a.ftag[f], n, Q0, G0, Qn, Gn, T(ph.gamma), ph.Winf)) set_err(a.err, CGKS_ENAN, (int)i, 1);
-    }
-    T dQ[5];
-#pragma unroll
-    for (int q = 0; q < 5; ++q) dQ[q] = Qn[q] - Q0[q];
-    // the difference column and the three gradient columns of this neighbour, each added into the
-    // coefficient on its own (one fused multiply-add per operator entry)
-#pragma unroll
-    for (int j = 0; j < 9; ++j) {
-      const double k0 = a.Kop[(j * 24 + m) * nc + i];
-      const double kx = a.Kop[(j * 24 + 6 + 3 * m) * nc + i];
-      const double ky = a.Kop[(j * 24 + 7 + 3 * m) * nc + i];
-      const double kz = a.Kop[(j * 24 + 8 + 3 * m) * nc + i];
-#pragma unroll
-      for (int q = 0; q < 5; ++q) {
-        b[q][j] += k0 * dQ[q];
-        b[q][j] += kx * Gn[3 * q];
-        b[q][j] += ky * Gn[3 * q + 1];
-        b[q][j] += kz * Gn[3 * q + 2];
-      }
-    }
-#pragma unroll
-    for (int d = 0; d < 3; ++d) {
-      const double wg = a.ggw[(3 * m + d) * nc + i], wl = a.lsw[(3 * m + d) * nc + i];
-#pragma unroll
-      for (int q = 0; q < 5; ++q) {
-        gg[q][d] += wg * (Qn[q] + Q0[q]);
-        gl[q][d] += wl * dQ[q];
-      }
-    }
-  }
-  const double V23 = a.aux[i], V43 = a.aux[nc + i];
-  double M2[6];
-#pragma unroll
-  for (int j = 0; j < 6; ++j) M2[j] = a.aux[(2 + j) * nc + i];
-  const double al = a.alpha[i];
-  const double g1 = 0.5, g2 = 0.5;
-#pragma unroll
-  for (int q = 0; q < 5; ++q) {
-    const T* bq = b[q];
-    const T a0 = Q0[q] - (bq[3] * M2[0] + bq[4] * M2[1] + bq[5] * M2[2] + bq[6] * M2[3] + bq[7] * M2[4] + bq[8] * M2[5]);
-    const T p1[3] = {al * gg[q][0], al * gg[q][1], al * gg[q][2]};
-    const T bGG = V23 * (p1[0] * p1[0] + p1[1] * p1[1] + p1[2] * p1[2]);
-    const T bLS = V23 * (gl[q][0] * gl[q][0] + gl[q][1] * gl[q][1] + gl[q][2] * gl[q][2]);
-    const T beta1 = fmin(bGG, bLS);
-    // |Omega|^(2/3) sum_d (avg of (d_d p2)^2) + |Omega|^(4/3) sum_{|a|=2} (D^a p2)^2
-    const T v[3][3] = {{2.0 * bq[3], bq[6], bq[8]}, {bq[6], 2.0 * bq[4], bq[7]}, {bq[8], bq[7], 2.0 * bq[5]}};
-    T first = 0.0;
-#pragma unroll
-    for (int d = 0; d < 3; ++d) {
-      const T* x = v[d];
-      const T vMv = M2[0] * x[0] * x[0] + M2[1] * x[1] * x[1] + M2[2] * x[2] * x[2] +
-                    2.0 * (M2[3] * x[0] * x[1] + M2[4] * x[1] * x[2] + M2[5] * x[0] * x[2]);
-      first += bq[d] * bq[d] + vMv;
-    }
-    const T second = 4.0 * (bq[3] * bq[3] + bq[4] * bq[4] + bq[5] * bq[5]) + bq[6] * bq[6] + bq[7] * bq[7] + bq[8] * bq[8];
-    const T beta2 = V23 * first + V43 * second;
-    const T rden = 1.0 / (Q0[q] * Q0[q] + beta1 + 1e-40);
-    const T bt1 = beta1 * rden, bt2 = beta2 * rden;
-    const T sig = fabs(bt2 - bt1);
-    // w_m = g_m (1 + (sig/d_m)^2) with d_m = eps + beta~_m, normalised with one division:
-    // w_1 : w_2 = g_1 (d_1^2 + sig^2) d_2^2 : g_2 (d_2^2 + sig^2) d_1^2
-    const T d1 = ph.weno_eps + bt1, d2 = ph.weno_eps + bt2;
-    const T s2 = sig * sig, d11 = d1 * d1, d22 = d2 * d2;
-    const T A1 = g1 * (d11 + s2) * d22, A2 = g2 * (d22 + s2) * d11;
-    const T inv = 1.0 / (A1 + A2);
-    const T w1 = A1 * inv, w2 = A2 * inv;
-    const T c2 = w2 * (1.0 / g2), c1 = w1 - w2 * (g1 / g2);
-    out[10 * q + 0] = c2 * a0 + c1 * Q0[q];
-#pragma unroll
-    for (int d = 0; d < 3; ++d) out[10 * q + 1 + d] = c2 * bq[d] + c1 * p1[d];
-#pragma unroll
-    for (int j = 3; j < 9; ++j) out[10 * q + 1 + j] = c2 * bq[j];
-  }
-}
-
 // local time step of cell i from its average Q0: CFL |Omega| / sum_p S_p (|U.n_p| + c + 2 nu S_p / |Omega|)
 template <typename T>
 HD T time_step(int64_t i, const ReconArgs& a, const T Q0[5]) {
@@ -207,6 +86,37 @@ HD T time_step(int64_t i, const ReconArgs& a, const T Q0[5]) {
   }
   if (!(Q0[0] > 0.0) || !(p > 0.0) || !isfinite(Q0[4])) set_err(a.err, CGKS_ENAN, (int)i, 2);
   return ph.cfl_fine * V / s;
+}
+
+// stencil sums of one variable of cell i: the p^2 coefficients b, Green-Gauss and least-squares gradients;
+// v[m] = (W_q, gradient of W_q) of slot m.  Each neighbour's difference and gradient are added into a
+// coefficient on their own (one fused multiply-add per operator entry).  Green-Gauss from the differences:
+// the outward S n / |Omega| of a closed cell sum to zero, so sum (Q_m + Q_0) w_m = sum (Q_m - Q_0) w_m,
+// without the cancellation
+HD void recon_sums(int64_t i, int nt, double Q0, const ReconArgs& a, const double v[6][4], double b[9], double gg[3],
+                   double gl[3]) {
+  const int64_t nc = a.nc;
+#pragma unroll
+  for (int j = 0; j < 9; ++j) b[j] = 0.0;
+#pragma unroll
+  for (int d = 0; d < 3; ++d) gg[d] = gl[d] = 0.0;
+#pragma unroll
+  for (int m = 0; m < 6; ++m) {
+    if (m >= nt) continue;
+    const double dQ = v[m][0] - Q0;
+#pragma unroll
+    for (int j = 0; j < 9; ++j) {
+      b[j] += a.Kop[(j * 24 + m) * nc + i] * dQ;
+      b[j] += a.Kop[(j * 24 + 6 + 3 * m) * nc + i] * v[m][1];
+      b[j] += a.Kop[(j * 24 + 7 + 3 * m) * nc + i] * v[m][2];
+      b[j] += a.Kop[(j * 24 + 8 + 3 * m) * nc + i] * v[m][3];
+    }
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      gg[d] += a.ggw[(3 * m + d) * nc + i] * dQ;
+      gl[d] += a.lsw[(3 * m + d) * nc + i] * dQ;
+    }
+  }
 }
 
 // the non-linear combination of one variable (Sec. 3.4): b the p^2 coefficients of X,Y,Z,X^2,Y^2,Z^2,XY,
@@ -274,18 +184,12 @@ HD int32_t recon_neighbour(int64_t i, int m, const ReconArgs& a) {
   return a.fR[f] < 0 ? -1 : (a.cside[k] ? a.fL[f] : a.fR[f]);
 }
 
-// reconstruction of variable q of cell i.  ghost(m, v) gives the boundary slot's (W_q, gradient of W_q).
-// Each neighbour's difference and gradient are added into a coefficient on their own (one fused
-// multiply-add per operator entry).  Green-Gauss from the differences: the outward S n / |Omega| of a
-// closed cell sum to zero, so sum (Q_m + Q_0) w_m = sum (Q_m - Q_0) w_m, without the cancellation
+// reconstruction of variable q of cell i.  ghost(m, v) gives the boundary slot's (W_q, gradient of W_q)
 template <typename Ghost>
 HD void reconstruct_variable(int64_t i, int q, const ReconArgs& a, const Ghost& ghost, double out[10]) {
   const int64_t nc = a.nc;
   const int nt = a.ctype[i] == 7 ? 5 : a.ctype[i];  // faces: pyramids (type 7) have 5
   const double Q0 = a.W[q * nc + i];
-  double b[9], gg[3] = {0.0, 0.0, 0.0}, gl[3] = {0.0, 0.0, 0.0};
-#pragma unroll
-  for (int j = 0; j < 9; ++j) b[j] = 0.0;
   int32_t nb[6];
 #pragma unroll
   for (int m = 0; m < 6; ++m) nb[m] = m < nt ? recon_neighbour(i, m, a) : 0;
@@ -301,23 +205,8 @@ HD void reconstruct_variable(int64_t i, int q, const ReconArgs& a, const Ghost& 
       ghost(m, v[m]);
     }
   }
-#pragma unroll
-  for (int m = 0; m < 6; ++m) {
-    if (m >= nt) continue;
-    const double dQ = v[m][0] - Q0;
-#pragma unroll
-    for (int j = 0; j < 9; ++j) {
-      b[j] += a.Kop[(j * 24 + m) * nc + i] * dQ;
-      b[j] += a.Kop[(j * 24 + 6 + 3 * m) * nc + i] * v[m][1];
-      b[j] += a.Kop[(j * 24 + 7 + 3 * m) * nc + i] * v[m][2];
-      b[j] += a.Kop[(j * 24 + 8 + 3 * m) * nc + i] * v[m][3];
-    }
-#pragma unroll
-    for (int d = 0; d < 3; ++d) {
-      gg[d] += a.ggw[(3 * m + d) * nc + i] * dQ;
-      gl[d] += a.lsw[(3 * m + d) * nc + i] * dQ;
-    }
-  }
+  double b[9], gg[3], gl[3];
+  recon_sums(i, nt, Q0, a, v, b, gg, gl);
   double M2[6];
 #pragma unroll
   for (int j = 0; j < 6; ++j) M2[j] = a.aux[(2 + j) * nc + i];
@@ -341,36 +230,211 @@ HD void reconstruct_body(int64_t i, const ReconArgs& a) {
   a.dt[i] = time_step<double>(i, a, Q0);
 }
 
-// forward-mode linearisation of the reconstruction of cell i into Jr [CGKS_RJ_ROWS][nc]: rows
+// the non-linear combination of one variable at its stencil sums, and its linearisation.  The outputs are
+// (c2 a0 + c1 Q0, c2 b_d + c1 p1_d, c2 b_j) with c1 = 1 - c2 (the weights add up to one), so all of the
+// nonlinearity is the derivative of c2 = 2 w_2: gb, gp, gl, gQ with respect to b, p1, the least-squares
+// gradient and Q0, by reverse mode (the minimum in beta_1 takes the smaller branch, half of each at a tie)
+struct WenoLin {
+  double c2, c1, a0, p1[3], gb[9], gp[3], gl[3], gQ;
+};
+
+HD void weno_linear(double Q0, const double b[9], const double gg[3], const double gl[3], double al, double V23, double V43,
+                    const double M2[6], double eps, WenoLin& w) {
+  w.a0 = Q0 - (b[3] * M2[0] + b[4] * M2[1] + b[5] * M2[2] + b[6] * M2[3] + b[7] * M2[4] + b[8] * M2[5]);
+  for (int d = 0; d < 3; ++d) w.p1[d] = al * gg[d];
+  const double bGG = V23 * (w.p1[0] * w.p1[0] + w.p1[1] * w.p1[1] + w.p1[2] * w.p1[2]);
+  const double bLS = V23 * (gl[0] * gl[0] + gl[1] * gl[1] + gl[2] * gl[2]);
+  const double beta1 = fmin(bGG, bLS);
+  const double vv[3][3] = {{2.0 * b[3], b[6], b[8]}, {b[6], 2.0 * b[4], b[7]}, {b[8], b[7], 2.0 * b[5]}};
+  double first = 0.0, vb[3][3];
+  for (int d = 0; d < 3; ++d) {
+    const double* x = vv[d];
+    const double Mx[3] = {M2[0] * x[0] + M2[3] * x[1] + M2[5] * x[2], M2[3] * x[0] + M2[1] * x[1] + M2[4] * x[2],
+                          M2[5] * x[0] + M2[4] * x[1] + M2[2] * x[2]};
+    first += b[d] * b[d] + x[0] * Mx[0] + x[1] * Mx[1] + x[2] * Mx[2];
+    for (int e = 0; e < 3; ++e) vb[d][e] = 2.0 * Mx[e];
+  }
+  const double second = 4.0 * (b[3] * b[3] + b[4] * b[4] + b[5] * b[5]) + b[6] * b[6] + b[7] * b[7] + b[8] * b[8];
+  const double beta2 = V23 * first + V43 * second;
+  const double rden = 1.0 / (Q0 * Q0 + beta1 + 1e-40);
+  const double bt1 = beta1 * rden, bt2 = beta2 * rden, dif = bt2 - bt1;
+  const double d1 = eps + bt1, d2 = eps + bt2;
+  const double s2 = dif * dif, d11 = d1 * d1, d22 = d2 * d2;
+  const double A1 = (d11 + s2) * d22, A2 = (d22 + s2) * d11;
+  const double inv = 1.0 / (A1 + A2);
+  const double w1 = A1 * inv, w2 = A2 * inv;
+  w.c2 = 2.0 * w2;
+  w.c1 = w1 - w2;
+  // d c2 = 2 d w2 = 2 inv (w1 dA2 - w2 dA1)
+  const double A1b = -2.0 * inv * w2, A2b = 2.0 * inv * w1;
+  const double d11b = A1b * d22 + A2b * (d22 + s2), d22b = A1b * (d11 + s2) + A2b * d11;
+  const double s2b = A1b * d22 + A2b * d11;
+  const double bt1b = 2.0 * d1 * d11b - 2.0 * dif * s2b, bt2b = 2.0 * d2 * d22b + 2.0 * dif * s2b;
+  const double rdenb = bt1b * beta1 + bt2b * beta2, dr = -rden * rden * rdenb;
+  w.gQ = 2.0 * Q0 * dr;
+  const double beta1b = bt1b * rden + dr, beta2b = bt2b * rden;
+  const double f1 = V23 * beta2b, f2 = V43 * beta2b;
+  for (int d = 0; d < 3; ++d) w.gb[d] = 2.0 * b[d] * f1;
+  for (int d = 0; d < 3; ++d) w.gb[3 + d] = 2.0 * vb[d][d] * f1 + 8.0 * b[3 + d] * f2;
+  w.gb[6] = (vb[0][1] + vb[1][0]) * f1 + 2.0 * b[6] * f2;
+  w.gb[7] = (vb[1][2] + vb[2][1]) * f1 + 2.0 * b[7] * f2;
+  w.gb[8] = (vb[0][2] + vb[2][0]) * f1 + 2.0 * b[8] * f2;
+  const double share = bGG < bLS ? 1.0 : (bGG > bLS ? 0.0 : 0.5);
+  for (int d = 0; d < 3; ++d) {
+    w.gp[d] = 2.0 * V23 * w.p1[d] * (share * beta1b);
+    w.gl[d] = 2.0 * V23 * gl[d] * ((1.0 - share) * beta1b);
+  }
+}
+
+// derivatives of a variable's 10 coefficients along a change (db, dgg, dgl, dQ0) of its sums
+HD void weno_column(const WenoLin& w, const double b[9], double Q0, double al, const double M2[6], const double db[9],
+                    const double dgg[3], const double dgl[3], double dQ0, double out[10]) {
+  double dc = w.gQ * dQ0, da0 = dQ0;
+#pragma unroll
+  for (int j = 0; j < 9; ++j) dc += w.gb[j] * db[j];
+#pragma unroll
+  for (int j = 0; j < 6; ++j) da0 -= db[3 + j] * M2[j];
+  double dp[3];
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    dp[d] = al * dgg[d];
+    dc += w.gp[d] * dp[d];
+    dc += w.gl[d] * dgl[d];
+  }
+  out[0] = w.c2 * da0 + w.c1 * dQ0 + dc * (w.a0 - Q0);
+#pragma unroll
+  for (int d = 0; d < 3; ++d) out[1 + d] = w.c2 * db[d] + w.c1 * dp[d] + dc * (b[d] - w.p1[d]);
+#pragma unroll
+  for (int j = 3; j < 9; ++j) out[1 + j] = w.c2 * db[j] + dc * b[j];
+}
+
+// linearisation of variable q (0..4) of cell i, or of its time step (5), into Jr [CGKS_RJ_ROWS][nc]: rows
 // 51 c + o of the own slot (input c of (W, grad W), output o of (50 coefficients, time step)), then
 // for neighbour slot s = 1..6 the rows CGKS_RJ_SELF + ((s - 1) 5 + q) 40 + 10 c4 + j: input c4 of
-// (W_q, d/dx, d/dy, d/dz of W_q), output coefficient j of variable q; absent slots (boundary faces,
-// fewer faces) are zero
-HD void recon_jacobian_body(int64_t i, const ReconArgs& a, double* Jr) {
-  const int64_t nc = a.nc;
+// (W_q, d/dx, d/dy, d/dz of W_q), output coefficient j of variable q.  Only the rows that can differ
+// from zero are written (the array starts at zero and which these are is the mesh's): absent slots and
+// boundary faces have no neighbour rows, and of the own slot a cell without boundary faces has the rows
+// of its variable's own input alone; on a boundary cell the ghosts are functions of all 20 own inputs.
+// Each stencil input is a column of the cell's linear maps (weno_column), so the whole takes about 4,500
+// FP64 operations per cell; evaluating the reconstruction on dual numbers once per input took 140 times
+// the reconstruction
+HD void recon_jacobian_variable(int64_t i, int q, const ReconArgs& a, double* Jr) {
+  const int64_t nc = a.nc, nf = a.nf;
   const int nt = a.ctype[i] == 7 ? 5 : a.ctype[i];
-  for (int k = 0; k < 20; ++k) {
-    DualD out[CGKS_RC];
-    reconstruct_cell<DualD>(i, a, k, out);
-    for (int o = 0; o < CGKS_RC; ++o) Jr[(int64_t)(CGKS_RJ_OUT * k + o) * nc + i] = out[o].d;
-    double ddt = 0.0;
-    if (k < 5) {
-      DualD Q0[5];
-      for (int q = 0; q < 5; ++q) Q0[q] = DualD(a.W[q * nc + i], q == k ? 1.0 : 0.0);
-      ddt = time_step<DualD>(i, a, Q0).d;
+  if (q == 5) {
+    for (int k = 0; k < 5; ++k) {
+      DualD Q[5];
+      for (int c = 0; c < 5; ++c) Q[c] = DualD(a.W[c * nc + i], c == k ? 1.0 : 0.0);
+      Jr[(int64_t)(CGKS_RJ_OUT * k + CGKS_RC) * nc + i] = time_step<DualD>(i, a, Q).d;
     }
-    Jr[(int64_t)(CGKS_RJ_OUT * k + CGKS_RC) * nc + i] = ddt;
+    return;
   }
-  for (int s = 1; s <= 6; ++s) {
-    const bool live = s <= nt && a.fR[a.cf[(int64_t)(s - 1) * nc + i]] >= 0;
-    for (int c = 0; c < 20; ++c) {
-      const int q = c < 5 ? c : (c - 5) / 3, c4 = c < 5 ? 0 : 1 + (c - 5) % 3;
-      DualD out[CGKS_RC];
-      if (live) reconstruct_cell<DualD>(i, a, 20 * s + c, out);
-      const int64_t row = CGKS_RJ_SELF + ((s - 1) * 5 + q) * 40 + 10 * c4;
-      for (int j = 0; j < 10; ++j) Jr[(row + j) * nc + i] = live ? out[10 * q + j].d : 0.0;
+  const double Q0 = a.W[q * nc + i];
+  double v[6][4];
+  unsigned bnd = 0;
+#pragma unroll
+  for (int m = 0; m < 6; ++m) {
+    if (m >= nt) continue;
+    const int32_t nb = recon_neighbour(i, m, a);
+    if (nb >= 0) {
+      v[m][0] = a.W[q * nc + nb];
+#pragma unroll
+      for (int d = 0; d < 3; ++d) v[m][1 + d] = a.G[(3 * q + d) * nc + nb];
+    } else {
+      bnd |= 1u << m;
+      double Wg[5], Gg[15];
+      recon_ghost(i, m, a, Wg, Gg);
+#pragma unroll
+      for (int c = 0; c < 5; ++c)
+        if (c == q) {
+          v[m][0] = Wg[c];
+#pragma unroll
+          for (int d = 0; d < 3; ++d) v[m][1 + d] = Gg[3 * c + d];
+        }
     }
   }
+  double b[9], gg[3], gl[3], M2[6];
+  recon_sums(i, nt, Q0, a, v, b, gg, gl);
+#pragma unroll
+  for (int j = 0; j < 6; ++j) M2[j] = a.aux[(2 + j) * nc + i];
+  const double al = a.alpha[i];
+  WenoLin w;
+  weno_linear(Q0, b, gg, gl, al, a.aux[i], a.aux[nc + i], M2, a.ph.weno_eps, w);
+  const double zero[3] = {0.0, 0.0, 0.0};
+  double sb[9], sg[3], sl[3];  // minus the sums of the value columns: the change with Q0
+#pragma unroll
+  for (int j = 0; j < 9; ++j) sb[j] = 0.0;
+#pragma unroll
+  for (int d = 0; d < 3; ++d) sg[d] = sl[d] = 0.0;
+  for (int m = 0; m < nt; ++m) {
+    double db[9], dg[3], dl[3], out[10];
+#pragma unroll
+    for (int j = 0; j < 9; ++j) sb[j] -= db[j] = a.Kop[(j * 24 + m) * nc + i];
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      sg[d] -= dg[d] = a.ggw[(3 * m + d) * nc + i];
+      sl[d] -= dl[d] = a.lsw[(3 * m + d) * nc + i];
+    }
+    if (bnd >> m & 1) continue;
+    const int64_t row = CGKS_RJ_SELF + (m * 5 + q) * 40;
+    weno_column(w, b, Q0, al, M2, db, dg, dl, 0.0, out);
+#pragma unroll
+    for (int j = 0; j < 10; ++j) Jr[(row + j) * nc + i] = out[j];
+    for (int e = 0; e < 3; ++e) {
+#pragma unroll
+      for (int j = 0; j < 9; ++j) db[j] = a.Kop[(j * 24 + 6 + 3 * m + e) * nc + i];
+      weno_column(w, b, Q0, al, M2, db, zero, zero, 0.0, out);
+#pragma unroll
+      for (int j = 0; j < 10; ++j) Jr[(row + 10 * (1 + e) + j) * nc + i] = out[j];
+    }
+  }
+  for (int c = 0; c < 20; ++c) {
+    if (!bnd && c != q) continue;
+    double db[9], dg[3], dl[3], out[10];
+    const double own = c == q ? 1.0 : 0.0;
+#pragma unroll
+    for (int j = 0; j < 9; ++j) db[j] = own * sb[j];
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      dg[d] = own * sg[d];
+      dl[d] = own * sl[d];
+    }
+    for (int m = 0; m < nt; ++m) {
+      if (!(bnd >> m & 1)) continue;
+      const int64_t f = a.cf[(int64_t)m * nc + i];
+      const DualD n[3] = {DualD(a.fnrm[f]), DualD(a.fnrm[nf + f]), DualD(a.fnrm[2 * nf + f])};
+      DualD Wd[5], Gd[15], Wg[5], Gg[15];
+      for (int k = 0; k < 5; ++k) Wd[k] = DualD(a.W[k * nc + i], c == k ? 1.0 : 0.0);
+      for (int k = 0; k < 15; ++k) Gd[k] = DualD(a.G[k * nc + i], c == 5 + k ? 1.0 : 0.0);
+      bc_ghost<DualD>(a.ftag[f], n, Wd, Gd, Wg, Gg, DualD(a.ph.gamma), a.ph.Winf);
+      double x = 0.0, y[3] = {0.0, 0.0, 0.0};
+#pragma unroll
+      for (int k = 0; k < 5; ++k)
+        if (k == q) {
+          x = Wg[k].d;
+#pragma unroll
+          for (int d = 0; d < 3; ++d) y[d] = Gg[3 * k + d].d;
+        }
+#pragma unroll
+      for (int j = 0; j < 9; ++j) {
+        db[j] += a.Kop[(j * 24 + m) * nc + i] * x;
+#pragma unroll
+        for (int d = 0; d < 3; ++d) db[j] += a.Kop[(j * 24 + 6 + 3 * m + d) * nc + i] * y[d];
+      }
+#pragma unroll
+      for (int d = 0; d < 3; ++d) {
+        dg[d] += a.ggw[(3 * m + d) * nc + i] * x;
+        dl[d] += a.lsw[(3 * m + d) * nc + i] * x;
+      }
+    }
+    weno_column(w, b, Q0, al, M2, db, dg, dl, own, out);
+#pragma unroll
+    for (int j = 0; j < 10; ++j) Jr[(int64_t)(CGKS_RJ_OUT * c + 10 * q + j) * nc + i] = out[j];
+  }
+}
+
+HD void recon_jacobian_body(int64_t i, const ReconArgs& a, double* Jr) {
+  for (int q = 0; q < 6; ++q) recon_jacobian_variable(i, q, a, Jr);
 }
 
 // ---- gas-kinetic point flux -------------------------------------------------------------------
