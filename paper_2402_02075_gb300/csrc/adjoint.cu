@@ -61,11 +61,11 @@ __global__ void __launch_bounds__(512) k_vjp_slots(VjpArgs a) {
   const int tx = threadIdx.x, ty = threadIdx.y;
   const int64_t i = blockIdx.x * (int64_t)32 + tx;
   for (int o = ty; o < CGKS_RJ_OUT; o += 16) cbs[o][tx] = i < a.nc ? a.cbuf[(int64_t)o * a.nc + i] : 0.0;
-  __shared__ bool dense[32];
-  if (ty == 0 && i < a.nc) dense[tx] = vjp_boundary_cell(i, a);
+  __shared__ int kind[32];
+  if (ty == 0 && i < a.nc) kind[tx] = vjp_cell_kind(i, a);
   __syncthreads();
   if (i >= a.nc) return;
-  for (int g = ty; g < 20 + 6 * 5; g += 16) vjp_slot_body(i, g, a, &cbs[0][tx], 32, dense[tx]);
+  for (int g = ty; g < 20 + 6 * 5; g += 16) vjp_slot_body(i, g, a, &cbs[0][tx], 32, kind[tx]);
 }
 
 // the reconstruction's transposed product recomputed per cell (adjoint_recompute 1), in place of
@@ -254,7 +254,7 @@ static ReconArgs lin_recon_args(cgks_ctx* ctx) {
 static cgks_status run_vjp(cgks_ctx* ctx, const double* rbar, const double* gbar, double* out) {
   const Fine& F = ctx->F;
   VjpArgs va{F.nc, F.nf, F.ngp, F.ctype, F.cside, F.cf, F.fL, F.fR, F.gp_face, F.gp_ptr, F.gp_x, F.gp_A, F.fshift,
-             F.ctr, F.vol, ctx->adt, ctx->Jp, ctx->Jr, rbar, gbar, ctx->pbar, ctx->aself, ctx->arec, ctx->acb, out};
+             F.ctr, F.vol, ctx->adt, ctx->Jp, ctx->Jr, rbar, gbar, ctx->pbar, ctx->aself, ctx->arec, ctx->acb, out, F.ftag};
   k_vjp_points<<<grid_for(F.ngp, 128), 128, 0, ctx->stream>>>(va);
   k_vjp_coef<<<grid_for(F.nc, 128), 128, 0, ctx->stream>>>(va);
   if (ctx->lin_recompute)

@@ -17,14 +17,21 @@ struct VjpArgs {
   double *pbar, *self, *rec;  // [ngp][42] (41 used), [20][nc], [2 nf][20]
   double* cbuf;               // [51][nc]: cotangents of each cell's coefficients and time step
   double *out;                // [20][nc]: cotangents of (W, G)
+  const int32_t* ftag;        // face tags (null: every boundary face counts as mixing)
 };
 
-// whether cell i has a boundary face (its ghosts then tie its own inputs to every variable)
-HD bool vjp_boundary_cell(int64_t i, const VjpArgs& a) {
+// what the own inputs of cell i reach besides their own average's coefficients: 0 nothing (no boundary
+// face), 1 their own variable's (ghosts are functions of the gradient too), 2 every variable's (a ghost
+// that mixes them)
+HD int vjp_cell_kind(int64_t i, const VjpArgs& a) {
   const int nt = a.ctype[i] == 7 ? 5 : a.ctype[i];
-  for (int m = 0; m < nt; ++m)
-    if (a.fR[a.cf[(int64_t)m * a.nc + i]] < 0) return true;
-  return false;
+  int kind = 0;
+  for (int m = 0; m < nt; ++m) {
+    const int64_t f = a.cf[(int64_t)m * a.nc + i];
+    if (a.fR[f] < 0) kind = !a.ftag || ghost_mixes(a.ftag[f]) ? 2 : (kind > 1 ? kind : 1);
+    if (kind == 2) break;
+  }
+  return kind;
 }
 
 // per Gauss point: cotangents of (flux, interface state) from those of (Res, Gnew) of its two cells,
@@ -112,21 +119,21 @@ HD void vjp_coef_body(int64_t i, const VjpArgs& a) {
 }
 
 // phase 2, per cell and row group g with the cell's 51 cotangents cb[o * cs]:
-//   g < 20   own-slot input c = g: self[c][i] = sum_o Jr[51 c + o][i] cb[o]; on a cell without boundary
-//            faces (dense false) over the rows that can differ from zero, its variable's 10 coefficients
-//            and the time step
+//   g < 20   own-slot input c = g: self[c][i] = sum_o Jr[51 c + o][i] cb[o]; over the rows that
+//            can differ from zero (kind, vjp_cell_kind): all, its variable's 10 coefficients and the time
+//            step, or for a gradient none
 //   g >= 20  neighbour slot s = 1 + (g - 20) / 5, variable q = (g - 20) % 5: its 4 inputs (W_q and the
 //            gradient of W_q) into the record of the slot's face for the cell across it (absent
 //            slots and boundary faces write nothing)
-HD void vjp_slot_body(int64_t i, int g, const VjpArgs& a, const double* cb, int cs, bool dense) {
+HD void vjp_slot_body(int64_t i, int g, const VjpArgs& a, const double* cb, int cs, int kind) {
   const int64_t nc = a.nc;
   if (g < 20) {
     const double* J = a.Jr + (int64_t)(CGKS_RJ_OUT * g) * nc + i;
     double v = g < 5 ? J[(int64_t)CGKS_RC * nc] * cb[CGKS_RC * cs] : 0.0;
-    if (dense) {
+    if (kind == 2) {
 #pragma unroll 10
       for (int o = 0; o < CGKS_RC; ++o) v += J[(int64_t)o * nc] * cb[o * cs];
-    } else {
+    } else if (kind == 1 || g < 5) {
       const int o0 = 10 * (g < 5 ? g : (g - 5) / 3);
 #pragma unroll
       for (int o = 0; o < 10; ++o) v += J[(int64_t)(o0 + o) * nc] * cb[(o0 + o) * cs];
@@ -152,7 +159,7 @@ HD void vjp_slot_body(int64_t i, int g, const VjpArgs& a, const double* cb, int 
 }
 
 HD void vjp_slot_body(int64_t i, int g, const VjpArgs& a, const double* cb, int cs) {
-  vjp_slot_body(i, g, a, cb, cs, vjp_boundary_cell(i, a));
+  vjp_slot_body(i, g, a, cb, cs, vjp_cell_kind(i, a));
 }
 
 // per cell, the reconstruction's part of the transposed product recomputed from the state instead of

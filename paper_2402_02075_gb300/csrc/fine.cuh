@@ -308,13 +308,16 @@ HD void weno_column(const WenoLin& w, const double b[9], double Q0, double al, c
   for (int j = 3; j < 9; ++j) out[1 + j] = w.c2 * db[j] + dc * b[j];
 }
 
+HD bool ghost_mixes(int tag) { return tag <= 3; }  // boundary kinds 1 and 2 (walls), 3 (farfield)
+
 // linearisation of variable q (0..4) of cell i, or of its time step (5), into Jr [CGKS_RJ_ROWS][nc]: rows
 // 51 c + o of the own slot (input c of (W, grad W), output o of (50 coefficients, time step)), then
 // for neighbour slot s = 1..6 the rows CGKS_RJ_SELF + ((s - 1) 5 + q) 40 + 10 c4 + j: input c4 of
 // (W_q, d/dx, d/dy, d/dz of W_q), output coefficient j of variable q.  Only the rows that can differ
 // from zero are written (the array starts at zero and which these are is the mesh's): absent slots and
-// boundary faces have no neighbour rows, and of the own slot a cell without boundary faces has the rows
-// of its variable's own input alone; on a boundary cell the ghosts are functions of all 20 own inputs.
+// boundary faces have no neighbour rows; of the own slot a variable has the rows of its own average, of
+// its own gradient next to a boundary face, and of all 20 inputs where the ghost mixes the variables
+// (walls and farfield).
 // Each stencil input is a column of the cell's linear maps (weno_column), so the whole takes about 4,500
 // FP64 operations per cell; evaluating the reconstruction on dual numbers once per input took 140 times
 // the reconstruction
@@ -332,6 +335,7 @@ HD void recon_jacobian_variable(int64_t i, int q, const ReconArgs& a, double* Jr
   const double Q0 = a.W[q * nc + i];
   double v[6][4];
   unsigned bnd = 0;
+  bool mixed = false;
 #pragma unroll
   for (int m = 0; m < 6; ++m) {
     if (m >= nt) continue;
@@ -342,6 +346,7 @@ HD void recon_jacobian_variable(int64_t i, int q, const ReconArgs& a, double* Jr
       for (int d = 0; d < 3; ++d) v[m][1 + d] = a.G[(3 * q + d) * nc + nb];
     } else {
       bnd |= 1u << m;
+      mixed = mixed || ghost_mixes(a.ftag[a.cf[(int64_t)m * nc + i]]);
       double Wg[5], Gg[15];
       recon_ghost(i, m, a, Wg, Gg);
 #pragma unroll
@@ -389,7 +394,7 @@ HD void recon_jacobian_variable(int64_t i, int q, const ReconArgs& a, double* Jr
     }
   }
   for (int c = 0; c < 20; ++c) {
-    if (!bnd && c != q) continue;
+    if (c != q && !mixed && !(bnd && c >= 5 && (c - 5) / 3 == q)) continue;
     double db[9], dg[3], dl[3], out[10];
     const double own = c == q ? 1.0 : 0.0;
 #pragma unroll
@@ -980,43 +985,122 @@ HD void gks_point_body(int64_t g, const PointArgs& a) {
   dst[6] = make_double2(Av[2], alpha);
 }
 
-// forward-mode linearisation of one Gauss point: Jp[(10 k + o) ngp + g] = d out_o / d in_k with
-// inputs k = (W_L 5, grad W_L 15, W_R 5, grad W_R 15, dt_f) at the point and outputs o = (flux 5,
-// interface state 5) as gks_point_body stores them; the right-side columns of a boundary point
-// are zero (its ghost is a function of the left side)
+// linearisation of one Gauss point: Jp[(10 k + o) ngp + g] = d out_o / d in_k with inputs k = (W_L 5,
+// grad W_L 15, W_R 5, grad W_R 15, dt_f) at the point and outputs o = (flux 5, interface state 5) as
+// gks_point_body stores them; the right-side columns of a boundary point are zero (its ghost is a function
+// of the left side).
+// The flux is linear in the gradients, so their 30 columns are responses to gradients of rank one
+// (gks_gradient_column, about 250 FP64 operations each); the ten columns of the states are dual evaluations
+// of one side (a right column is a left one seen from the other side: F_n(L, R) = -F_-n(R, L)), about 3,000
+// each; the time step's is a dual evaluation with passive states.  Evaluating all 41 on dual numbers took
+// 246,000 FP64 operations per point
 HD void point_jacobian_body(int64_t g, const PointArgs& a, double* Jp) {
   PointIn p;
   point_inputs(g, a, p);
   const bool bnd = p.R < 0;
   const int tag = a.ftag[p.f];
   const int64_t ngp = a.ngp;
-  for (int k = 0; k < CGKS_PJ_IN; ++k) {
+  const Phys& ph = a.ph;
+  const double weight = 1.0 / p.iw, sdt = weight * fast_rcp(p.dtf);
+  const auto store = [&](int k, const double col[10], double sf, double sw) {
+#pragma unroll
+    for (int o = 0; o < 10; ++o) Jp[(int64_t)(10 * k + o) * ngp + g] = (o < 5 ? sf : sw) * col[o];
+  };
+  if (bnd && !bc_ghost<double>(tag, p.n, p.WL, p.GL, p.WR, p.GR, ph.gamma, ph.Winf)) set_err(a.err, CGKS_ENAN, (int)p.f, 3);
+  const double nm[3] = {-p.n[0], -p.n[1], -p.n[2]};
+  // states
+  for (int k = 0; k < 10; ++k) {
+    const bool right = k >= 5;
+    const int q = right ? k - 5 : k;
     double col[10];
-    if (bnd && k >= 20 && k < 40) {
+    DualD F[5], Wg[5], al, W[5];
+#pragma unroll
+    for (int c = 0; c < 5; ++c) W[c] = DualD(right ? p.WR[c] : p.WL[c], c == q ? 1.0 : 0.0);
+    if (right && bnd) {
 #pragma unroll
       for (int o = 0; o < 10; ++o) col[o] = 0.0;
+      store(20 + q, col, 1.0, 1.0);
+      continue;
+    }
+    if (bnd) {
+      DualD G[15], Wr[5], Gr[15];
+      const DualD nd[3] = {DualD(p.n[0]), DualD(p.n[1]), DualD(p.n[2])};
+#pragma unroll
+      for (int j = 0; j < 15; ++j) G[j] = DualD(p.GL[j]);
+      bc_ghost<DualD>(tag, nd, W, G, Wr, Gr, DualD(ph.gamma), ph.Winf);  // the ghost gradient is linear in G alone
+      const int bad = gks_flux_t<true, DualD, DualD, DualD, DualD>(p.n, weight, true, W, p.GL, Wr, p.GR, DualD(p.dtf), ph,
+                                                                   a.tab, F, Wg, al);
+      if (bad) set_err(a.err, CGKS_ENAN, (int)p.f, bad);
     } else {
-      DualD WL[5], GL[15], WR[5], GR[15], Fg[5], Wg[5], al;
-#pragma unroll
-      for (int q = 0; q < 5; ++q) {
-        WL[q] = DualD(p.WL[q], k == q ? 1.0 : 0.0);
-        WR[q] = DualD(bnd ? 0.0 : p.WR[q], k == 20 + q ? 1.0 : 0.0);
-      }
-#pragma unroll
-      for (int j = 0; j < 15; ++j) {
-        GL[j] = DualD(p.GL[j], k == 5 + j ? 1.0 : 0.0);
-        GR[j] = DualD(bnd ? 0.0 : p.GR[j], k == 25 + j ? 1.0 : 0.0);
-      }
-      const DualD dtf(p.dtf, k == 40 ? 1.0 : 0.0);
-      point_flux<DualD>(p.n, p.iw, bnd, tag, WL, GL, WR, GR, dtf, a.ph, Fg, Wg, al, a.err, p.f);
-#pragma unroll
-      for (int q = 0; q < 5; ++q) {
-        col[q] = Fg[q].d;
-        col[5 + q] = Wg[q].d;
-      }
+      const int bad = gks_flux_t<true, DualD, double, DualD, double>(right ? nm : p.n, weight, false, W, right ? p.GR : p.GL,
+                                                                     right ? p.WL : p.WR, right ? p.GL : p.GR, p.dtf, ph,
+                                                                     a.tab, F, Wg, al);
+      if (bad) set_err(a.err, CGKS_ENAN, (int)p.f, bad);
     }
 #pragma unroll
-    for (int o = 0; o < 10; ++o) Jp[(int64_t)(10 * k + o) * ngp + g] = col[o];
+    for (int o = 0; o < 5; ++o) {
+      col[o] = F[o].d;
+      col[5 + o] = Wg[o].d;
+    }
+    store(right ? 20 + q : q, col, right ? -1.0 : 1.0, 1.0);
+  }
+  // time step
+  {
+    DualD WL[5], WR[5], F[5], Wg[5], al;
+#pragma unroll
+    for (int q = 0; q < 5; ++q) {
+      WL[q] = DualD(p.WL[q]);
+      WR[q] = DualD(p.WR[q]);
+    }
+    gks_flux_t<true, DualD, DualD, DualD, DualD>(p.n, weight, bnd, WL, p.GL, WR, p.GR, DualD(p.dtf, 1.0), ph, a.tab, F, Wg,
+                                                 al);
+    double col[10];
+#pragma unroll
+    for (int o = 0; o < 5; ++o) {
+      col[o] = F[o].d;
+      col[5 + o] = Wg[o].d;
+    }
+    store(40, col, 1.0, 1.0);
+  }
+  // gradients: unit e_q along the axis d; on a boundary the ghost's gradient is another of rank one
+  GksSide<double> gl, gr;
+  GksCentre<double> c;
+  const double gm1 = ph.gamma - 1.0;
+  gks_side<double>(p.WL, p.n, 1.0, gm1, a.tab, gl);
+  gks_side<double>(p.WR, p.n, -1.0, gm1, a.tab, gr);
+  gks_centre<double, double, double, double>(gl, gr, p.dtf, ph, a.tab, c);
+  for (int j = 0; j < 15; ++j) {
+    const int q = j / 3;
+    double A[5], B[5], d[3], r[3], col[10], add[10];
+#pragma unroll
+    for (int k = 0; k < 5; ++k) A[k] = B[k] = k == q ? 1.0 : 0.0;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) r[k] = d[k] = k == j % 3 ? 1.0 : 0.0;
+    gks_gradient_column(gl, c, A, d, p.n, sdt, ph, col);
+    if (!bnd) {
+      store(5 + j, col, 1.0, 1.0);
+      gks_gradient_column(gr, c, A, d, p.n, sdt, ph, col);
+      store(25 + j, col, 1.0, 1.0);
+      continue;
+    }
+    if (tag == 1 || tag == 2 || tag == 5) {
+      if (tag != 5) {
+        const double dn = d[0] * p.n[0] + d[1] * p.n[1] + d[2] * p.n[2];
+        const double an = A[1] * p.n[0] + A[2] * p.n[1] + A[3] * p.n[2];
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+          r[k] = d[k] - 2.0 * dn * p.n[k];
+          B[1 + k] = tag == 1 ? A[1 + k] - 2.0 * an * p.n[k] : -A[1 + k];
+        }
+      }
+      gks_gradient_column(gr, c, B, r, p.n, sdt, ph, add);
+#pragma unroll
+      for (int o = 0; o < 10; ++o) col[o] += add[o];
+    }
+    store(5 + j, col, 1.0, 1.0);
+#pragma unroll
+    for (int o = 0; o < 10; ++o) col[o] = 0.0;
+    store(25 + j, col, 1.0, 1.0);
   }
 }
 

@@ -24,15 +24,20 @@
 #include "fastmath.cuh"
 #include "kinetic.cuh"
 
+// The state dependence can be differentiated by dual numbers: S is the scalar of a side's state, T of
+// what both sides and the time step enter (double for the flux itself; one of the sides or both DualD
+// for a column of the linearisation); gradients stay double.
 // one side of the interface: state, half-space seeds
+template <typename S>
 struct GksSide {
-  double rho, r, u[3], U, ut[3];  // density, 1/rho, velocity, its normal and tangential parts
-  double p, h, l2, sl;            // pressure, p/rho, rho/p, 1/sqrt(2 h)
-  double m0, beta;                // half-space mass fraction, s g(0)/rho (s the side: u_n > 0 or < 0)
+  S rho, r, u[3], U, ut[3];  // density, 1/rho, velocity, its normal and tangential parts
+  S p, h, l2, sl;            // pressure, p/rho, rho/p, 1/sqrt(2 h)
+  S m0, beta;                // half-space mass fraction, s g(0)/rho (s the side: u_n > 0 or < 0)
 };
 
 // s = +1 left, -1 right; false where the state is not physical
-HD bool gks_side(const double w[5], const double n[3], double s, double gm1, const double* tab, GksSide& g) {
+template <typename S>
+HD bool gks_side(const S w[5], const double n[3], double s, double gm1, const double* tab, GksSide<S>& g) {
   g.rho = w[0];
   g.r = fast_rcp(w[0]);
 #pragma unroll
@@ -44,44 +49,46 @@ HD bool gks_side(const double w[5], const double n[3], double s, double gm1, con
   for (int d = 0; d < 3; ++d) g.ut[d] = g.u[d] - g.U * n[d];
   g.sl = fast_rsqrt(2.0 * g.h);
   g.l2 = 2.0 * g.sl * g.sl;
-  double e;
+  S e;
   half_gauss(-s * (g.sl * g.U), tab, g.m0, e);
   g.beta = (s * 0.56418958354775628695) * (e * g.sl);
   return positive(w[0]) && positive(g.p);
 }
 
 // time coefficients of Eq. 2nd-flux integrated over [0, dt] that multiply the two sides' moments
+template <typename T>
 struct GksTime {
-  double q4, q5, tq4;     // of g, of -(a.u) g and of -A g in the flux
-  double edt, etd, etau;  // the same in the interface state at dt
+  T q4, q5, tq4;     // of g, of -(a.u) g and of -A g in the flux
+  T edt, etd, etau;  // the same in the interface state at dt
 };
 
 // sums over both sides in the frame moving with the interface's tangential velocity: gradients of the
 // interface equilibrium (mass, normal momentum, tangential momentum and energy, per direction) and the
 // moments of the time-integrated flux (F), of the state at dt (W) and of the time-integrated state (I)
+template <typename T>
 struct GksAcc {
-  double rho[3], mn[3], T[3][3], e[3];
-  double F0, F1, F4, FT[3], W0, W1, W4, WT[3], I0, I4;
+  T rho[3], mn[3], Tm[3][3], e[3];
+  T F0, F1, F4, FT[3], W0, W1, W4, WT[3], I0, I4;
 };
 
 // adds one side: G the conservative gradients (15), ut_c the interface's tangential velocity.  STATE: the
 // state at dt as well; heat: the time-integrated state's rows that the Prandtl correction uses.  FIRST:
 // the sums start with this side
-template <bool STATE, bool FIRST>
-HD void gks_add_side(const GksSide& g, const double G[15], const double n[3], const double utc[3], double gm1, double gamma,
-                     double k2, const GksTime& t, bool heat, GksAcc& a) {
-  double del[3];
+template <bool STATE, bool FIRST, typename S, typename T>
+HD void gks_add_side(const GksSide<S>& g, const double G[15], const double n[3], const T utc[3], double gm1, double gamma,
+                     double k2, const GksTime<T>& t, bool heat, GksAcc<T>& a) {
+  T del[3];
 #pragma unroll
   for (int d = 0; d < 3; ++d) del[d] = g.ut[d] - utc[d];
-  const double hd2 = 0.5 * (del[0] * del[0] + del[1] * del[1] + del[2] * del[2]);
-  const double hu2 = 0.5 * (g.u[0] * g.u[0] + g.u[1] * g.u[1] + g.u[2] * g.u[2]);
+  const T hd2 = 0.5 * (del[0] * del[0] + del[1] * del[1] + del[2] * del[2]);
+  const S hu2 = 0.5 * (g.u[0] * g.u[0] + g.u[1] * g.u[1] + g.u[2] * g.u[2]);
   // primitive gradients
-  double R[3][3], gp[3], th[3], Rn[3];
+  S R[3][3], gp[3], th[3], Rn[3];
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
 #pragma unroll
     for (int i = 0; i < 3; ++i) R[i][k] = G[3 * (1 + i) + k] - g.u[i] * G[k];
-    double x = G[12 + k] - hu2 * G[k];
+    S x = G[12 + k] - hu2 * G[k];
     x -= g.u[0] * R[0][k];
     x -= g.u[1] * R[1][k];
     x -= g.u[2] * R[2][k];
@@ -90,144 +97,145 @@ HD void gks_add_side(const GksSide& g, const double G[15], const double n[3], co
     Rn[k] = n[0] * R[0][k] + n[1] * R[1][k] + n[2] * R[2][k];
   }
   // moments and the coefficients X_k, Y_k
-  const double U = g.U, h = g.h, m0 = g.m0, beta = g.beta;
-  const double m1 = U * m0 + h * beta;
-  const double hm0 = h * m0, m2 = U * m1 + hm0;
-  const double hm1 = h * m1, m3 = U * m2 + 2.0 * hm1;
-  const double m4 = U * m3 + 3.0 * (h * m2);
-  const double X2 = 2.0 * m1, X3 = 3.0 * m2, X4 = 4.0 * m3;
-  const double Y0 = -0.5 * U * (beta * g.l2), Y1 = 0.5 * beta, Y3 = 3.0 * m1, Y4 = 2.0 * X3;
-  const double kap = k2 * h, k2m0 = k2 * m0, k2m1 = k2 * m1, kd = kap + hd2;
-  double dm0[3];
+  const S U = g.U, h = g.h, m0 = g.m0, beta = g.beta;
+  const S m1 = U * m0 + h * beta;
+  const S hm0 = h * m0, m2 = U * m1 + hm0;
+  const S hm1 = h * m1, m3 = U * m2 + 2.0 * hm1;
+  const S m4 = U * m3 + 3.0 * (h * m2);
+  const S X2 = 2.0 * m1, X3 = 3.0 * m2, X4 = 4.0 * m3;
+  const S Y0 = -0.5 * U * (beta * g.l2), Y1 = 0.5 * beta, Y3 = 3.0 * m1, Y4 = 2.0 * X3;
+  const S kap = k2 * h, k2m0 = k2 * m0, k2m1 = k2 * m1;
+  const T kd = hd2 + kap;
+  T dm0[3];
 #pragma unroll
   for (int d = 0; d < 3; ++d) dm0[d] = del[d] * m0;
   // gradients of the interface equilibrium; the D_0, D_1 of each direction serve below
-  double D0[3], D1[3];
+  S D0[3], D1[3];
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
     D0[k] = m0 * G[k] + beta * Rn[k] + Y0 * th[k];
     D1[k] = m1 * G[k] + m0 * Rn[k] + Y1 * th[k];
-    const double D2 = m2 * G[k] + X2 * Rn[k] + m0 * th[k];
-    double e = FIRST ? 0.5 * D2 : a.e[k] + 0.5 * D2;
+    const S D2 = m2 * G[k] + X2 * Rn[k] + m0 * th[k];
+    T e = FIRST ? T(0.5 * D2) : a.e[k] + 0.5 * D2;
     e += kd * D0[k];
     e += k2m0 * th[k];
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
       e += dm0[i] * R[i][k];
-      double T = FIRST ? m0 * R[i][k] : a.T[i][k] + m0 * R[i][k];
-      a.T[i][k] = T + del[i] * D0[k];
+      const T v = FIRST ? T(m0 * R[i][k]) : a.Tm[i][k] + m0 * R[i][k];
+      a.Tm[i][k] = v + del[i] * D0[k];
     }
     a.e[k] = e;
-    a.rho[k] = FIRST ? D0[k] : a.rho[k] + D0[k];
-    a.mn[k] = FIRST ? D1[k] : a.mn[k] + D1[k];
+    a.rho[k] = FIRST ? T(D0[k]) : a.rho[k] + D0[k];
+    a.mn[k] = FIRST ? T(D1[k]) : a.mn[k] + D1[k];
   }
   // derivatives along n and along the tangential velocity
   const double rn = n[0] * G[0] + n[1] * G[1] + n[2] * G[2];
-  const double pn = n[0] * gp[0] + n[1] * gp[1] + n[2] * gp[2];
-  const double rS = g.ut[0] * G[0] + g.ut[1] * G[1] + g.ut[2] * G[2];
-  const double pS = g.ut[0] * gp[0] + g.ut[1] * gp[1] + g.ut[2] * gp[2];
-  double Rv[3], RS[3], Rt[3];
+  const S pn = n[0] * gp[0] + n[1] * gp[1] + n[2] * gp[2];
+  const S rS = g.ut[0] * G[0] + g.ut[1] * G[1] + g.ut[2] * G[2];
+  const S pS = g.ut[0] * gp[0] + g.ut[1] * gp[1] + g.ut[2] * gp[2];
+  S Rv[3], RS[3], Rt[3];
 #pragma unroll
   for (int i = 0; i < 3; ++i) {
     Rv[i] = n[0] * R[i][0] + n[1] * R[i][1] + n[2] * R[i][2];
     RS[i] = g.ut[0] * R[i][0] + g.ut[1] * R[i][1] + g.ut[2] * R[i][2];
     Rt[i] = U * Rv[i] + (RS[i] + gp[i]);
   }
-  const double Rnn = n[0] * Rv[0] + n[1] * Rv[1] + n[2] * Rv[2];
-  const double RnS = n[0] * RS[0] + n[1] * RS[1] + n[2] * RS[2];
-  const double Rnt = n[0] * Rt[0] + n[1] * Rt[1] + n[2] * Rt[2];
-  const double thn = pn - h * rn, thS = pS - h * rS;
-  const double tr = R[0][0] + R[1][1] + R[2][2], Dv = tr - Rnn;
+  const S Rnn = n[0] * Rv[0] + n[1] * Rv[1] + n[2] * Rv[2];
+  const S RnS = n[0] * RS[0] + n[1] * RS[1] + n[2] * RS[2];
+  const S Rnt = n[0] * Rt[0] + n[1] * Rt[1] + n[2] * Rt[2];
+  const S thn = pn - h * rn, thS = pS - h * rS;
+  const S tr = R[0][0] + R[1][1] + R[2][2], Dv = tr - Rnn;
   // minus the time derivatives (Euler)
-  const double rt = U * rn + (rS + tr);
-  const double tht = U * pn + pS + (gamma * h) * tr - h * rt;
+  const S rt = U * rn + (rS + tr);
+  const S tht = U * pn + pS + (gamma * h) * tr - h * rt;
   // rows of <u_n^k (a.u) psi> (al) and of -<u_n^k A psi> (At), k = 0..3 for the powers of u_n and e0, e1
   // for the energy rows of k = 0, 1
-  const double rSD = rS + Dv;
-  double al0 = m1 * rn + m0 * Rnn + Y1 * thn;
+  const S rSD = rS + Dv;
+  S al0 = m1 * rn + m0 * Rnn + Y1 * thn;
   al0 += m0 * rSD;
   al0 += beta * RnS;
   al0 += Y0 * thS;
-  double al1 = m2 * rn + X2 * Rnn + m0 * thn;
+  S al1 = m2 * rn + X2 * Rnn + m0 * thn;
   al1 += m1 * rSD;
   al1 += m0 * RnS;
   al1 += Y1 * thS;
-  double al2 = m3 * rn + X3 * Rnn + Y3 * thn;
+  S al2 = m3 * rn + X3 * Rnn + Y3 * thn;
   al2 += m2 * rSD;
   al2 += X2 * RnS;
   al2 += m0 * thS;
-  double al3 = m4 * rn + X4 * Rnn + Y4 * thn;
+  S al3 = m4 * rn + X4 * Rnn + Y4 * thn;
   al3 += m3 * rSD;
   al3 += X3 * RnS;
   al3 += Y3 * thS;
-  const double At0 = m0 * rt + beta * Rnt + Y0 * tht;
-  const double At1 = m1 * rt + m0 * Rnt + Y1 * tht;
-  const double At2 = m2 * rt + X2 * Rnt + m0 * tht;
-  const double At3 = m3 * rt + X3 * Rnt + Y3 * tht;
+  const S At0 = m0 * rt + beta * Rnt + Y0 * tht;
+  const S At1 = m1 * rt + m0 * Rnt + Y1 * tht;
+  const S At2 = m2 * rt + X2 * Rnt + m0 * tht;
+  const S At3 = m3 * rt + X3 * Rnt + Y3 * tht;
   // tangential rows of a.u, k = 0, 1
-  double Ta0[3], Ta1[3];
+  S Ta0[3], Ta1[3];
 #pragma unroll
   for (int i = 0; i < 3; ++i) {
-    const double b = RS[i] + th[i];
+    const S b = RS[i] + th[i];
     Ta0[i] = m1 * Rv[i] + m0 * b + h * D0[i];
     Ta1[i] = m2 * Rv[i] + m1 * b + h * D1[i];
   }
-  const double v4 = 0.5 * m2 + kap * m0, f4 = 0.5 * m3 + kap * m1;  // energy rows of psi and u psi
+  const S v4 = 0.5 * m2 + kap * m0, f4 = 0.5 * m3 + kap * m1;  // energy rows of psi and u psi
   {
     // flux: q4 <u psi> - q5 <u (a.u) psi> - tau q4 <u A psi>
-    const double qr = t.q4 * g.rho, z1 = t.q5 * al1 - t.tq4 * At1, z2 = t.q5 * al2 - t.tq4 * At2,
+    const T qr = t.q4 * g.rho, z1 = t.q5 * al1 - t.tq4 * At1, z2 = t.q5 * al2 - t.tq4 * At2,
                  z3 = t.q5 * al3 - t.tq4 * At3;
-    const double hn = t.q5 * thn, hb = t.q5 * thS - t.tq4 * tht, dv = t.q5 * Dv;
-    const double F0 = qr * m1 - z1, F1 = qr * m2 - z2;
-    double F4 = qr * f4 - 0.5 * z3;
+    const T hn = t.q5 * thn, hb = t.q5 * thS - t.tq4 * tht, dv = t.q5 * Dv;
+    const T F0 = qr * m1 - z1, F1 = qr * m2 - z2;
+    T F4 = qr * f4 - 0.5 * z3;
     F4 -= kap * z1;
     F4 -= (k2 * m2) * hn;
     F4 -= k2m1 * hb;
     F4 -= hm1 * dv;
     F4 += hd2 * F0;
-    const double c = t.tq4 * m1;
+    const T c = t.tq4 * m1;
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
-      const double T = t.q5 * Ta1[i] - c * Rt[i];
-      F4 -= del[i] * T;
-      const double x = del[i] * F0 - T;
+      const T v = t.q5 * Ta1[i] - c * Rt[i];
+      F4 -= del[i] * v;
+      const T x = del[i] * F0 - v;
       a.FT[i] = FIRST ? x : a.FT[i] + x;
     }
     a.F0 = FIRST ? F0 : a.F0 + F0;
     a.F1 = FIRST ? F1 : a.F1 + F1;
     a.F4 = FIRST ? F4 : a.F4 + F4;
     if (heat) {
-      const double z0 = t.q5 * al0 - t.tq4 * At0, I0 = qr * m0 - z0;
-      double I4 = qr * v4 - 0.5 * z2;
+      const T z0 = t.q5 * al0 - t.tq4 * At0, I0 = qr * m0 - z0;
+      T I4 = qr * v4 - 0.5 * z2;
       I4 -= kap * z0;
       I4 -= k2m1 * hn;
       I4 -= k2m0 * hb;
       I4 -= hm0 * dv;
       I4 += hd2 * I0;
-      const double qT = t.q5 * (del[0] * Ta0[0] + del[1] * Ta0[1] + del[2] * Ta0[2]);
-      const double qA = (t.tq4 * m0) * (del[0] * Rt[0] + del[1] * Rt[1] + del[2] * Rt[2]);
+      const T qT = t.q5 * (del[0] * Ta0[0] + del[1] * Ta0[1] + del[2] * Ta0[2]);
+      const T qA = (t.tq4 * m0) * (del[0] * Rt[0] + del[1] * Rt[1] + del[2] * Rt[2]);
       I4 -= qT - qA;
       a.I0 = FIRST ? I0 : a.I0 + I0;
       a.I4 = FIRST ? I4 : a.I4 + I4;
     }
   }
   if (STATE) {
-    const double qr = t.edt * g.rho, z0 = t.etd * al0 - t.etau * At0, z1 = t.etd * al1 - t.etau * At1,
+    const T qr = t.edt * g.rho, z0 = t.etd * al0 - t.etau * At0, z1 = t.etd * al1 - t.etau * At1,
                  z2 = t.etd * al2 - t.etau * At2;
-    const double hn = t.etd * thn, hb = t.etd * thS - t.etau * tht, dv = t.etd * Dv;
-    const double W0 = qr * m0 - z0, W1 = qr * m1 - z1;
-    double W4 = qr * v4 - 0.5 * z2;
+    const T hn = t.etd * thn, hb = t.etd * thS - t.etau * tht, dv = t.etd * Dv;
+    const T W0 = qr * m0 - z0, W1 = qr * m1 - z1;
+    T W4 = qr * v4 - 0.5 * z2;
     W4 -= kap * z0;
     W4 -= k2m1 * hn;
     W4 -= k2m0 * hb;
     W4 -= hm0 * dv;
     W4 += hd2 * W0;
-    const double c = t.etau * m0;
+    const T c = t.etau * m0;
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
-      const double T = t.etd * Ta0[i] - c * Rt[i];
-      W4 -= del[i] * T;
-      const double x = del[i] * W0 - T;
+      const T v = t.etd * Ta0[i] - c * Rt[i];
+      W4 -= del[i] * v;
+      const T x = del[i] * W0 - v;
       a.WT[i] = FIRST ? x : a.WT[i] + x;
     }
     a.W0 = FIRST ? W0 : a.W0 + W0;
@@ -236,17 +244,17 @@ HD void gks_add_side(const GksSide& g, const double G[15], const double n[3], co
   }
 }
 
-// moments (mass F0, normal momentum F1, tangential momentum T, energy F4) of the frame moving with the
+// moments (mass F0, normal momentum F1, tangential momentum Ft, energy F4) of the frame moving with the
 // tangential velocity ut -> conservative vector of the global frame, times c
-HD void gks_to_global(double F0, double F1, double F4, const double T[3], const double n[3], const double ut[3], double hut2,
-                      double c, double out[5]) {
+template <typename T, typename C>
+HD void gks_to_global(T F0, T F1, T F4, const T Ft[3], const double n[3], const T ut[3], T hut2, C c, T out[5]) {
   out[0] = c * F0;
-  const double x = F1 - (n[0] * T[0] + n[1] * T[1] + n[2] * T[2]);
-  double e = F4 + hut2 * F0;
+  const T x = F1 - (n[0] * Ft[0] + n[1] * Ft[1] + n[2] * Ft[2]);
+  T e = F4 + hut2 * F0;
 #pragma unroll
   for (int i = 0; i < 3; ++i) {
-    e += ut[i] * T[i];
-    double v = T[i] + ut[i] * F0;
+    e += ut[i] * Ft[i];
+    T v = Ft[i] + ut[i] * F0;
     v += x * n[i];
     out[1 + i] = c * v;
   }
@@ -261,39 +269,45 @@ HD T viscosity(const Phys& ph, T t);
 // states and gradients of both sides (global frame; on a boundary face the ghost's), dt the face's time
 // step.  F: flux x weight averaged over dt; Wg (STATE): the interface state at dt; alpha (STATE): the
 // compression factor (1 on boundary faces and with the factor off).  Returns 0, or the number of the
-// check that failed (4 a side, 5 the interface state)
-template <bool STATE>
-HD int gks_flux(const double n[3], double weight, bool bnd, const double WL[5], const double GL[15], const double WR[5],
-                const double GR[15], double dt, const Phys& ph, const double* tab, double F[5], double Wg[5],
-                double& alpha) {
+// check that failed (4 a side, 5 the interface state).  gks_flux is the flux itself, gks_flux_t its dual form
+// what the equilibrium part of a flux and of a column of its linearisation share
+template <typename T>
+struct GksCentre {
+  T rho, Mn, U, p, h, E, ut[3];            // density, momentum, velocity, ..., energy in the moving frame
+  T om, q1, q2, q3, dt;                    // time coefficients of its terms, the time step
+  GksTime<T> t;
+};
+
+// interface equilibrium W^c = int_{u>0} psi g^l + int_{u<0} psi g^r (Eq. compatibility2), the collision
+// times and the integrals over [0, dt] of the time coefficients; false where the state is not physical
+template <typename SL, typename SR, typename T, typename D>
+HD bool gks_centre(const GksSide<SL>& gl, const GksSide<SR>& gr, D dt, const Phys& ph, const double* tab, GksCentre<T>& c) {
   const double gm1 = ph.gamma - 1.0, k2 = 0.5 * (ph.K + 2.0);
-  GksSide gl, gr;
-  const bool okl = gks_side(WL, n, 1.0, gm1, tab, gl), okr = gks_side(WR, n, -1.0, gm1, tab, gr);
-  int bad = okl && okr ? 0 : 4;
-  // interface equilibrium W^c = int_{u>0} psi g^l + int_{u<0} psi g^r (Eq. compatibility2)
-  const double a0 = gl.rho * gl.m0, b0 = gr.rho * gr.m0;
-  const double al1 = gl.U * gl.m0 + gl.h * gl.beta, ar1 = gr.U * gr.m0 + gr.h * gr.beta;
-  const double rho = a0 + b0, Mn = gl.rho * al1 + gr.rho * ar1;
-  const double r = fast_rcp(rho), U = Mn * r;
-  double ut[3], jm2 = 0.0, jl2 = 0.0;
+  const SL a0 = gl.rho * gl.m0, al1 = gl.U * gl.m0 + gl.h * gl.beta;
+  const SR b0 = gr.rho * gr.m0, ar1 = gr.U * gr.m0 + gr.h * gr.beta;
+  c.rho = a0 + b0;
+  c.Mn = gl.rho * al1 + gr.rho * ar1;
+  const T r = fast_rcp(c.rho);
+  c.U = c.Mn * r;
+  T jl2 = 0.0, jr2 = 0.0;
 #pragma unroll
   for (int d = 0; d < 3; ++d) {
-    ut[d] = (a0 * gl.ut[d] + b0 * gr.ut[d]) * r;
-    const double x = gl.ut[d] - ut[d], y = gr.ut[d] - ut[d];
+    c.ut[d] = (a0 * gl.ut[d] + b0 * gr.ut[d]) * r;
+    const T x = gl.ut[d] - c.ut[d], y = gr.ut[d] - c.ut[d];
     jl2 += x * x;
-    jm2 += y * y;
+    jr2 += y * y;
   }
   // energy in the frame moving with the tangential velocity of the interface
-  const double el = 0.5 * (gl.U * al1 + gl.h * gl.m0) + (k2 * gl.h + 0.5 * jl2) * gl.m0;
-  const double er = 0.5 * (gr.U * ar1 + gr.h * gr.m0) + (k2 * gr.h + 0.5 * jm2) * gr.m0;
-  const double E = gl.rho * el + gr.rho * er;
-  const double p = gm1 * (E - 0.5 * Mn * U), h = p * r;
-  if (!(positive(rho) && positive(p)) && !bad) bad = 5;
+  const T el = 0.5 * (gl.U * al1 + gl.h * gl.m0) + (0.5 * jl2 + k2 * gl.h) * gl.m0;
+  const T er = 0.5 * (gr.U * ar1 + gr.h * gr.m0) + (0.5 * jr2 + k2 * gr.h) * gr.m0;
+  c.E = gl.rho * el + gr.rho * er;
+  c.p = gm1 * (c.E - 0.5 * c.Mn * c.U);
+  c.h = c.p * r;
   // collision times (Sec. 2.3)
-  const double jump = fabs((gl.p - gr.p) * fast_rcp(gl.p + gr.p));
-  double tau, tn;
+  const T jump = fabs((gl.p - gr.p) * fast_rcp(gl.p + gr.p));
+  T tau, tn;
   if (ph.viscous) {
-    tau = viscosity<double>(ph, ph.gamma * h) * fast_rcp(p);
+    tau = viscosity<T>(ph, ph.gamma * c.h) * fast_rcp(c.p);
     tn = tau + ph.c_press * jump * dt;
   } else {
     tn = (ph.eps_inviscid + ph.c_press * jump) * dt;
@@ -301,74 +315,99 @@ HD int gks_flux(const double n[3], double weight, bool bnd, const double WL[5], 
   }
   // exact integrals over [0, dt] of the time coefficients
   // (tn vanishes where the viscosity and the pressure jump do)
-  const double edt = positive(tn) ? exp_neg(dt * fast_rcp(tn), tab) : 0.0, om = 1.0 - edt;
-  const double q4 = tn * om, tte = tn * dt * edt;
-  const double q1 = dt - q4, q5 = (tau + tn) * q4 - tte;
-  const double q2 = q5 - tau * dt;
-  const double q3 = 0.5 * dt * dt - tau * dt + tau * q4;
-  const GksTime t{q4, q5, tau * q4, edt, edt * (tau + dt), edt * tau};
+  T edt = 0.0;
+  if (positive(tn)) edt = exp_neg(dt * fast_rcp(tn), tab);
+  c.om = 1.0 - edt;
+  c.dt = dt;
+  const T q4 = tn * c.om, tte = tn * dt * edt;
+  c.q1 = dt - q4;
+  c.t.q4 = q4;
+  c.t.q5 = (tau + tn) * q4 - tte;
+  c.t.tq4 = tau * q4;
+  c.t.edt = edt;
+  c.t.etd = edt * (tau + dt);
+  c.t.etau = edt * tau;
+  c.q2 = c.t.q5 - tau * dt;
+  c.q3 = 0.5 * dt * dt - tau * dt + tau * q4;
+  return positive(c.rho) && positive(c.p);
+}
+
+// T: the wider of the scalars of the sides and the time step.  n, weight and the gradients are double
+template <bool STATE, typename SL, typename SR, typename T, typename D>
+HD int gks_flux_t(const double n[3], double weight, bool bnd, const SL WL[5], const double GL[15], const SR WR[5],
+                  const double GR[15], D dt, const Phys& ph, const double* tab, T F[5], T Wg[5], T& alpha) {
+  const double gm1 = ph.gamma - 1.0, k2 = 0.5 * (ph.K + 2.0);
+  GksSide<SL> gl;
+  GksSide<SR> gr;
+  const bool okl = gks_side(WL, n, 1.0, gm1, tab, gl), okr = gks_side(WR, n, -1.0, gm1, tab, gr);
+  GksCentre<T> c;
+  const bool okc = gks_centre<SL, SR, T, D>(gl, gr, dt, ph, tab, c);
+  const int bad = !(okl && okr) ? 4 : (okc ? 0 : 5);
+  const T rho = c.rho, Mn = c.Mn, U = c.U, p = c.p, h = c.h, E = c.E, om = c.om, q1 = c.q1, q2 = c.q2, q3 = c.q3;
+  const T(&ut)[3] = c.ut;
+  const GksTime<T>& t = c.t;
   const bool heat = ph.viscous && ph.prandtl != 1.0;
   alpha = 1.0;
   if (STATE && !bnd && ph.cf) {  // compression factor (interior faces), 1/sqrt(gamma h) = sl sqrt(2/gamma)
-    const double dp = fabs(gl.p - gr.p);
-    double dm = 0.0;
+    const T dp = fabs(gl.p - gr.p);
+    T dm = 0.0;
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
-      const double x = gl.u[d] * gl.sl - gr.u[d] * gr.sl;
+      const T x = gl.u[d] * gl.sl - gr.u[d] * gr.sl;
       dm += x * x;
     }
-    const double A = dp * (gl.r * gl.l2 + gr.r * gr.l2) + (2.0 / ph.gamma) * dm;
+    const T A = dp * (gl.r * gl.l2 + gr.r * gr.l2) + (2.0 / ph.gamma) * dm;
     alpha = fast_rcp(1.0 + A * A);
   }
-  GksAcc a;
-  gks_add_side<STATE, true>(gl, GL, n, ut, gm1, ph.gamma, k2, t, heat, a);
-  gks_add_side<STATE, false>(gr, GR, n, ut, gm1, ph.gamma, k2, t, heat, a);
+  GksAcc<T> a;
+  gks_add_side<STATE, true, SL, T>(gl, GL, n, ut, gm1, ph.gamma, k2, t, heat, a);
+  gks_add_side<STATE, false, SR, T>(gr, GR, n, ut, gm1, ph.gamma, k2, t, heat, a);
   // equilibrium part, full space: X = (0, 1, 2 m1, 3 m2, 4 m3), Y = (0, 0, 1, 3 m1, 6 m2)
   {
-    double Rn[3], gp[3], th[3], Tn[3], TS[3];
+    T Rn[3], gp[3], th[3], Tn[3], TS[3];
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
       Rn[k] = a.mn[k] - U * a.rho[k];
-      double x = a.e[k] - U * a.mn[k];
+      T x = a.e[k] - U * a.mn[k];
       x += (0.5 * U * U) * a.rho[k];
       gp[k] = gm1 * x;
       th[k] = gp[k] - h * a.rho[k];
     }
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
-      Tn[i] = n[0] * a.T[i][0] + n[1] * a.T[i][1] + n[2] * a.T[i][2];
-      TS[i] = ut[0] * a.T[i][0] + ut[1] * a.T[i][1] + ut[2] * a.T[i][2];
+      Tn[i] = n[0] * a.Tm[i][0] + n[1] * a.Tm[i][1] + n[2] * a.Tm[i][2];
+      TS[i] = ut[0] * a.Tm[i][0] + ut[1] * a.Tm[i][1] + ut[2] * a.Tm[i][2];
     }
-    const double rn = n[0] * a.rho[0] + n[1] * a.rho[1] + n[2] * a.rho[2];
-    const double Rnn = n[0] * Rn[0] + n[1] * Rn[1] + n[2] * Rn[2];
-    const double thn = n[0] * th[0] + n[1] * th[1] + n[2] * th[2];
-    const double rS = ut[0] * a.rho[0] + ut[1] * a.rho[1] + ut[2] * a.rho[2];
-    const double RnS = ut[0] * Rn[0] + ut[1] * Rn[1] + ut[2] * Rn[2];
-    const double thS = ut[0] * th[0] + ut[1] * th[1] + ut[2] * th[2];
-    const double Dv = (a.T[0][0] + a.T[1][1] + a.T[2][2]) - (n[0] * Tn[0] + n[1] * Tn[1] + n[2] * Tn[2]);
-    const double m2 = U * U + h, m3 = U * m2 + 2.0 * h * U, m4 = U * m3 + 3.0 * h * m2;
-    const double X2 = 2.0 * U, X3 = 3.0 * m2, X4 = 4.0 * m3, Y3 = 3.0 * U, Y4 = 2.0 * X3, kap = k2 * h;
-    const double rSD = rS + Dv;
-    const double c0 = U * rn + Rnn + rSD;  // <u^k (a.u)>: minus the time derivatives of mass, momentum, ...
-    double c1 = m2 * rn + X2 * Rnn + thn;
+    const T rn = n[0] * a.rho[0] + n[1] * a.rho[1] + n[2] * a.rho[2];
+    const T Rnn = n[0] * Rn[0] + n[1] * Rn[1] + n[2] * Rn[2];
+    const T thn = n[0] * th[0] + n[1] * th[1] + n[2] * th[2];
+    const T rS = ut[0] * a.rho[0] + ut[1] * a.rho[1] + ut[2] * a.rho[2];
+    const T RnS = ut[0] * Rn[0] + ut[1] * Rn[1] + ut[2] * Rn[2];
+    const T thS = ut[0] * th[0] + ut[1] * th[1] + ut[2] * th[2];
+    const T Dv = (a.Tm[0][0] + a.Tm[1][1] + a.Tm[2][2]) - (n[0] * Tn[0] + n[1] * Tn[1] + n[2] * Tn[2]);
+    const T m2 = U * U + h, m3 = U * m2 + 2.0 * h * U, m4 = U * m3 + 3.0 * h * m2;
+    const T X2 = 2.0 * U, X3 = 3.0 * m2, X4 = 4.0 * m3, Y3 = 3.0 * U, Y4 = 2.0 * X3, kap = k2 * h;
+    const T rSD = rS + Dv;
+    const T c0 = U * rn + Rnn + rSD;  // <u^k (a.u)>: minus the time derivatives of mass, momentum, ...
+    T c1 = m2 * rn + X2 * Rnn + thn;
     c1 += U * rSD;
     c1 += RnS;
-    double c2 = m3 * rn + X3 * Rnn + Y3 * thn;
+    T c2 = m3 * rn + X3 * Rnn + Y3 * thn;
     c2 += m2 * rSD;
     c2 += X2 * RnS;
     c2 += thS;
-    double c3 = m4 * rn + X4 * Rnn + Y4 * thn;
+    T c3 = m4 * rn + X4 * Rnn + Y4 * thn;
     c3 += m3 * rSD;
     c3 += X3 * RnS;
     c3 += Y3 * thS;
-    double e0 = 0.5 * c2 + kap * c0;
+    T e0 = 0.5 * c2 + kap * c0;
     e0 += k2 * (U * thn + thS);
     e0 += h * Dv;
-    double e1 = 0.5 * c3 + kap * c1;
+    T e1 = 0.5 * c3 + kap * c1;
     e1 += (k2 * m2) * thn;
     e1 += (k2 * U) * thS;
     e1 += (h * U) * Dv;
-    double T0[3], T1[3];
+    T T0[3], T1[3];
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
       T0[i] = U * Tn[i] + (TS[i] + gp[i]);
@@ -376,15 +415,15 @@ HD int gks_flux(const double n[3], double weight, bool bnd, const double WL[5], 
       T1[i] += U * (TS[i] + th[i]);
     }
     // minus the time slope's rows in u psi
-    const double Rt = c1 - U * c0;
-    double pt = e0 - U * c1;
+    const T Rt = c1 - U * c0;
+    T pt = e0 - U * c1;
     pt += (0.5 * U * U) * c0;
-    const double tht = gm1 * pt - h * c0;
-    const double A2 = m2 * c0 + X2 * Rt + tht;
-    const double A3 = m3 * c0 + X3 * Rt + Y3 * tht;
-    double eA = 0.5 * A3 + kap * c1;
+    const T tht = gm1 * pt - h * c0;
+    const T A2 = m2 * c0 + X2 * Rt + tht;
+    const T A3 = m3 * c0 + X3 * Rt + Y3 * tht;
+    T eA = 0.5 * A3 + kap * c1;
     eA += (k2 * U) * tht;
-    const double q23 = q2 - q3;
+    const T q23 = q2 - q3;
     a.F0 += q1 * Mn;
     a.F0 += q23 * c1;
     a.F1 += q1 * (Mn * U + p);
@@ -393,14 +432,14 @@ HD int gks_flux(const double n[3], double weight, bool bnd, const double WL[5], 
     a.F4 += (q1 * U) * (E + p);
     a.F4 += q2 * e1;
     a.F4 -= q3 * eA;
-    const double q3U = q3 * U;
+    const T q3U = q3 * U;
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
       a.FT[i] += q2 * T1[i];
       a.FT[i] -= q3U * T0[i];
     }
     if (STATE) {
-      const double od = om * dt;
+      const T od = om * dt;
       a.W0 += om * rho;
       a.W0 -= od * c0;
       a.W1 += om * Mn;
@@ -413,18 +452,143 @@ HD int gks_flux(const double n[3], double weight, bool bnd, const double WL[5], 
     if (heat) {
       // heat flux about U^c of the time-integrated distribution, scaled by (1/Pr - 1); its normal
       // momentum is the mass flux F0
-      const double I0 = a.I0 + q1 * rho + q23 * c0, I4 = a.I4 + q1 * E + q23 * e0;
-      const double U2 = U * U;
-      double qn = a.F4 - U * (a.F1 + I4);
+      const T I0 = a.I0 + q1 * rho + q23 * c0, I4 = a.I4 + q1 * E + q23 * e0;
+      const T U2 = U * U;
+      T qn = a.F4 - U * (a.F1 + I4);
       qn += (1.5 * U2) * a.F0;
       qn -= (0.5 * U2 * U) * I0;
       a.F4 += (1.0 / ph.prandtl - 1.0) * qn;
     }
   }
-  const double hut2 = 0.5 * (ut[0] * ut[0] + ut[1] * ut[1] + ut[2] * ut[2]);
+  const T hut2 = 0.5 * (ut[0] * ut[0] + ut[1] * ut[1] + ut[2] * ut[2]);
   gks_to_global(a.F0, a.F1, a.F4, a.FT, n, ut, hut2, weight * fast_rcp(dt), F);
   if (STATE) {
     gks_to_global(a.W0, a.W1, a.W4, a.WT, n, ut, hut2, 1.0, Wg);
   }
   return bad;
+}
+
+// the flux itself
+template <bool STATE>
+HD int gks_flux(const double n[3], double weight, bool bnd, const double WL[5], const double GL[15], const double WR[5],
+                const double GR[15], double dt, const Phys& ph, const double* tab, double F[5], double Wg[5],
+                double& alpha) {
+  return gks_flux_t<STATE, double, double, double, double>(n, weight, bnd, WL, GL, WR, GR, dt, ph, tab, F, Wg, alpha);
+}
+
+// response of a point's time-averaged flux x weight / dt (out 0..4) and interface state (out 5..9), both
+// linear in the gradients, to a unit of the gradient dW = A along the direction d (d W_q/dx_k = A_q d_k) of
+// one side: gks_flux with a gradient of rank one, where every derivative is that amplitude times n.d, u_t.d
+// or d itself
+HD void gks_gradient_column(const GksSide<double>& g, const GksCentre<double>& c, const double A[5], const double d[3],
+                            const double n[3], double sdt, const Phys& ph, double out[10]) {
+  const double gm1 = ph.gamma - 1.0, k2 = 0.5 * (ph.K + 2.0);
+  const double U = g.U, h = g.h, m0 = g.m0, beta = g.beta;
+  double del[3], R[3];
+  const double hu2 = 0.5 * (g.u[0] * g.u[0] + g.u[1] * g.u[1] + g.u[2] * g.u[2]);
+  double x = A[4] - hu2 * A[0];
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    del[i] = g.ut[i] - c.ut[i];
+    R[i] = A[1 + i] - g.u[i] * A[0];
+    x -= g.u[i] * R[i];
+  }
+  const double hd2 = 0.5 * (del[0] * del[0] + del[1] * del[1] + del[2] * del[2]);
+  const double gr = A[0], gp = gm1 * x, th = gp - h * gr, Rn = n[0] * R[0] + n[1] * R[1] + n[2] * R[2];
+  const double dn = n[0] * d[0] + n[1] * d[1] + n[2] * d[2];
+  const double ds = g.ut[0] * d[0] + g.ut[1] * d[1] + g.ut[2] * d[2], ud = U * dn + ds;
+  const double m1 = U * m0 + h * beta, hm0 = h * m0, m2 = U * m1 + hm0, hm1 = h * m1, m3 = U * m2 + 2.0 * hm1,
+               m4 = U * m3 + 3.0 * (h * m2);
+  const double X2 = 2.0 * m1, X3 = 3.0 * m2, X4 = 4.0 * m3, Y0 = -0.5 * U * (beta * g.l2), Y1 = 0.5 * beta, Y3 = 3.0 * m1,
+               Y4 = 2.0 * X3;
+  const double kap = k2 * h, k2m0 = k2 * m0, k2m1 = k2 * m1;
+  const double D0 = m0 * gr + beta * Rn + Y0 * th, D1 = m1 * gr + m0 * Rn + Y1 * th, D2 = m2 * gr + X2 * Rn + m0 * th,
+               D3 = m3 * gr + X3 * Rn + Y3 * th, D4 = m4 * gr + X4 * Rn + Y4 * th;
+  const double tr = R[0] * d[0] + R[1] * d[1] + R[2] * d[2], Dv = tr - dn * Rn;
+  const double rt = ud * gr + tr, Rnt = ud * Rn + gp * dn, tht = ud * gp + (ph.gamma * h) * tr - h * rt;
+  const double thn = dn * th, thS = ds * th;
+  const double al0 = dn * D1 + ds * D0 + m0 * Dv, al1 = dn * D2 + ds * D1 + m1 * Dv, al2 = dn * D3 + ds * D2 + m2 * Dv,
+               al3 = dn * D4 + ds * D3 + m3 * Dv;
+  const double At0 = m0 * rt + beta * Rnt + Y0 * tht, At1 = m1 * rt + m0 * Rnt + Y1 * tht,
+               At2 = m2 * rt + X2 * Rnt + m0 * tht, At3 = m3 * rt + X3 * Rnt + Y3 * tht;
+  double F0, F1, F4, FT[3], W0, W1, W4, WT[3], I0 = 0.0, I4 = 0.0;
+  const bool heat = ph.viscous && ph.prandtl != 1.0;
+  {
+    const GksTime<double>& t = c.t;
+    const double z0 = t.q5 * al0 - t.tq4 * At0, z1 = t.q5 * al1 - t.tq4 * At1, z2 = t.q5 * al2 - t.tq4 * At2,
+                 z3 = t.q5 * al3 - t.tq4 * At3;
+    const double hn = t.q5 * thn, hb = t.q5 * thS - t.tq4 * tht, dv = t.q5 * Dv;
+    const double y0 = t.etd * al0 - t.etau * At0, y1 = t.etd * al1 - t.etau * At1, y2 = t.etd * al2 - t.etau * At2;
+    const double wn = t.etd * thn, wb = t.etd * thS - t.etau * tht, wv = t.etd * Dv;
+    F0 = -z1;
+    F1 = -z2;
+    F4 = hd2 * F0 - (0.5 * z3 + kap * z1 + (k2 * m2) * hn + k2m1 * hb + hm1 * dv);
+    W0 = -y0;
+    W1 = -y1;
+    W4 = hd2 * W0 - (0.5 * y2 + kap * y0 + k2m1 * wn + k2m0 * wb + hm0 * wv);
+    if (heat) {
+      I0 = -z0;
+      I4 = hd2 * I0 - (0.5 * z2 + kap * z0 + k2m1 * hn + k2m0 * hb + hm0 * dv);
+    }
+    const double a0 = m1 * dn + m0 * ds, a1 = m2 * dn + m1 * ds, b0 = m0 * th + h * D0, b1 = m1 * th + h * D1;
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      const double Ta0 = a0 * R[i] + b0 * d[i], Ta1 = a1 * R[i] + b1 * d[i], Rt = ud * R[i] + gp * d[i];
+      const double v = t.q5 * Ta1 - (t.tq4 * m1) * Rt, y = t.etd * Ta0 - (t.etau * m0) * Rt;
+      F4 -= del[i] * v;
+      FT[i] = del[i] * F0 - v;
+      W4 -= del[i] * y;
+      WT[i] = del[i] * W0 - y;
+      if (heat) I4 -= del[i] * (t.q5 * Ta0 - (t.tq4 * m0) * Rt);
+    }
+  }
+  // the interface equilibrium's gradient (amplitudes along d) and its terms
+  {
+    const double Uc = c.U, hc = c.h, kc = k2 * hc;
+    double T[3];
+    double e = 0.5 * D2 + (kap + hd2) * D0 + k2m0 * th;
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      T[i] = m0 * R[i] + del[i] * D0;
+      e += (del[i] * m0) * R[i];
+    }
+    const double Rc = D1 - Uc * D0, pc = gm1 * (e - Uc * D1 + (0.5 * Uc * Uc) * D0), tc = pc - hc * D0;
+    const double dc = c.ut[0] * d[0] + c.ut[1] * d[1] + c.ut[2] * d[2];
+    const double nT = n[0] * T[0] + n[1] * T[1] + n[2] * T[2];
+    const double Dc = (T[0] * d[0] + T[1] * d[1] + T[2] * d[2]) - dn * nT;
+    const double n2 = Uc * Uc + hc, n3 = Uc * n2 + 2.0 * hc * Uc, n4 = Uc * n3 + 3.0 * hc * n2;
+    const double E2 = n2 * D0 + 2.0 * Uc * Rc + tc, E3 = n3 * D0 + 3.0 * n2 * Rc + 3.0 * Uc * tc,
+                 E4 = n4 * D0 + 4.0 * n3 * Rc + 6.0 * n2 * tc;
+    const double c0 = dn * D1 + dc * D0 + Dc, c1 = dn * E2 + dc * D1 + Uc * Dc, c2 = dn * E3 + dc * E2 + n2 * Dc,
+                 c3 = dn * E4 + dc * E3 + n3 * Dc;
+    const double tn = dn * tc, tS = dc * tc;
+    const double e0 = 0.5 * c2 + kc * c0 + k2 * (Uc * tn + tS) + hc * Dc;
+    const double e1 = 0.5 * c3 + kc * c1 + (k2 * n2) * tn + (k2 * Uc) * tS + (hc * Uc) * Dc;
+    const double Rt = c1 - Uc * c0, tt = gm1 * (e0 - Uc * c1 + (0.5 * Uc * Uc) * c0) - hc * c0;
+    const double A2 = n2 * c0 + 2.0 * Uc * Rt + tt, A3 = n3 * c0 + 3.0 * n2 * Rt + 3.0 * Uc * tt;
+    const double eA = 0.5 * A3 + kc * c1 + (k2 * Uc) * tt;
+    const double q23 = c.q2 - c.q3, od = c.om * c.dt;
+    F0 += q23 * c1;
+    F1 += c.q2 * c2 - c.q3 * A2;
+    F4 += c.q2 * e1 - c.q3 * eA;
+    W0 -= od * c0;
+    W1 -= od * c1;
+    W4 -= od * e0;
+    const double s0 = Uc * dn + dc, s1 = n2 * dn + Uc * dc, v1 = hc * D1 + Uc * tc;
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      const double T0 = s0 * T[i] + pc * d[i], T1 = s1 * T[i] + v1 * d[i];
+      FT[i] += c.q2 * T1 - (c.q3 * Uc) * T0;
+      WT[i] -= od * T0;
+    }
+    if (heat) {
+      I0 += q23 * c0;
+      I4 += q23 * e0;
+      const double qn = F4 - Uc * (F1 + I4) + (1.5 * Uc * Uc) * F0 - (0.5 * Uc * Uc * Uc) * I0;
+      F4 += (1.0 / ph.prandtl - 1.0) * qn;
+    }
+  }
+  const double hut2 = 0.5 * (c.ut[0] * c.ut[0] + c.ut[1] * c.ut[1] + c.ut[2] * c.ut[2]);
+  gks_to_global(F0, F1, F4, FT, n, c.ut, hut2, sdt, out);
+  gks_to_global(W0, W1, W4, WT, n, c.ut, hut2, 1.0, out + 5);
 }

@@ -158,6 +158,25 @@ HD DualD pow(DualD x, double y) {
   return {p, y * p / x.v * x.d};
 }
 HD bool isfinite(DualD x) { return isfinite(x.v); }
+// the functions of fastmath.cuh; (erfc(y)/2)' = -exp(-y^2)/sqrt(pi)
+HD DualD fast_rcp(DualD x) {
+  const double r = fast_rcp(x.v);
+  return {r, -(r * r) * x.d};
+}
+HD DualD fast_rsqrt(DualD x) {
+  const double r = fast_rsqrt(x.v);
+  return {r, -0.5 * (r * r * r) * x.d};
+}
+HD bool positive(DualD x) { return positive(x.v); }
+HD DualD exp_neg(DualD x, const double* tab) {
+  const double e = exp_neg(x.v, tab);
+  return {e, -e * x.d};
+}
+HD void half_gauss(DualD y, const double* tab, DualD& m0, DualD& e) {
+  half_gauss(y.v, tab, m0.v, e.v);
+  m0.d = -0.56418958354775628695 * e.v * y.d;
+  e.d = -2.0 * y.v * e.v * y.d;
+}
 template <>
 HD DualD tsqrt<DualD>(DualD x) { return sqrt(x); }
 template <>
