@@ -46,7 +46,17 @@ __global__ void k_bucket_min(int64_t nf, const int32_t* fL, const int32_t* fR, c
   atomicMin(&bucket[face_hash(fL, fR, f, seed, nfc)], (int32_t)f);
 }
 
-__device__ bool skew_confirmed(const Level& P, int32_t a, int32_t b, double kmin2) {
+// area-weighted centres of the faces, once per pass (one division per face and axis; the skewness test
+// would take it again for every candidate a face is near)
+__global__ void k_face_centres(int64_t nf, const double* __restrict__ amom, const double* __restrict__ area,
+                               double* __restrict__ fx) {
+  const int64_t f = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (f >= nf) return;
+#pragma unroll
+  for (int e = 0; e < 3; ++e) fx[e * nf + f] = __ddiv_rn(amom[e * nf + f], area[f]);
+}
+
+__device__ bool skew_confirmed(const Level& P, const double* __restrict__ fx, int32_t a, int32_t b, double kmin2) {
   const int64_t nc = P.nc, nf = P.nf;
   const double Va = P.vol[a], Vb = P.vol[b];
   const double Vs = __dadd_rn(Va, Vb);
@@ -66,7 +76,7 @@ __device__ bool skew_confirmed(const Level& P, int32_t a, int32_t b, double kmin
       double d[3], S[3];
 #pragma unroll
       for (int e = 0; e < 3; ++e) {
-        double xg = __ddiv_rn(P.amom[e * nf + g], P.area[g]);
+        double xg = fx[e * nf + g];
         if (asR) xg = __dsub_rn(xg, P.shift[e * nf + g]);
         d[e] = __dsub_rn(xg, Cc[e]);
         S[e] = P.Sn[e * nf + g];
@@ -82,40 +92,65 @@ __device__ bool skew_confirmed(const Level& P, int32_t a, int32_t b, double kmin
   return true;
 }
 
-__global__ void k_select_confirm(Level P, uint64_t seed, uint64_t nfc, const int32_t* bucket, double kmin2,
-                                 int8_t* conf) {
+// confirmed faces into `list` (in any order; *n counts them): the winners of their hash buckets that pass the
+// skewness test
+__global__ void k_select_confirm(Level P, uint64_t seed, uint64_t nfc, const int32_t* bucket, const double* fx,
+                                 double kmin2, int32_t* list, int32_t* n) {
   const int64_t f = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (f >= P.nf) return;
-  int8_t ok = 0;
-  if (is_candidate(P.fR, P.ftag, f) && bucket[face_hash(P.fL, P.fR, f, seed, nfc)] == (int32_t)f)
-    ok = skew_confirmed(P, P.fL[f], P.fR[f], kmin2) ? 1 : 0;
-  conf[f] = ok;
+  if (is_candidate(P.fR, P.ftag, f) && bucket[face_hash(P.fL, P.fR, f, seed, nfc)] == (int32_t)f &&
+      skew_confirmed(P, fx, P.fL[f], P.fR[f], kmin2))
+    list[atomicAdd(n, 1)] = (int32_t)f;
 }
 
-// smallest confirmed face of each unmatched cell whose other cell is unmatched
-__global__ void k_best_face(Level P, const int8_t* conf, const int32_t* partner, int32_t* best) {
-  const int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (c >= P.nc) return;
-  int32_t b = INT32_MAX;
-  if (partner[c] < 0)
-    for (int32_t k = P.c2f_ptr[c]; k < P.c2f_ptr[c + 1]; ++k) {
-      const int32_t g = P.c2f[k];
-      if (!conf[g]) continue;
-      const int32_t o = P.fL[g] == c ? P.fR[g] : P.fL[g];
-      if (partner[o] < 0 && g < b) b = g;
-    }
-  best[c] = b;
+// Rounds of the greedy matching: in each, a live face (confirmed, both cells unmatched) that is the smallest
+// live face of both its cells merges them.  best[c] holds (rounds to go, face), so that a later round's
+// entries undercut an earlier one's and nothing is reset.  A round is two passes over the live faces,
+// propose and match; match drops the dead ones into the next round's list.  On meshes numbered along grid
+// lines a face waits for a chain of smaller ones, 20 to 150 rounds for a pass, so a round has to be cheap
+// and the host reads the count of live faces once for MATCH_ROUNDS of them.  (Per round 10 us against 15
+// over all cells and faces with a host read each, 64,000-cell box; finishing the long tail in one block
+// took 50 us per round.)
+#define MATCH_ROUNDS 16
+
+__device__ __forceinline__ unsigned long long match_key(int32_t round, int32_t f) {
+  return ((unsigned long long)(unsigned)(INT32_MAX - round) << 32) | (unsigned)f;
 }
 
-__global__ void k_match_round(Level P, const int8_t* conf, const int32_t* best, int32_t* partner,
-                              unsigned long long* matched) {
-  const int64_t f = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (f >= P.nf || !conf[f]) return;
+__device__ __forceinline__ void match_propose(const Level& P, int32_t f, int32_t round, const int32_t* partner,
+                                              unsigned long long* best) {
   const int32_t a = P.fL[f], b = P.fR[f];
-  if (best[a] == (int32_t)f && best[b] == (int32_t)f) {
+  if (partner[a] >= 0 || partner[b] >= 0) return;
+  const unsigned long long key = match_key(round, f);
+  atomicMin(&best[a], key);
+  atomicMin(&best[b], key);
+}
+
+// whether the face stays live
+__device__ __forceinline__ bool match_merge(const Level& P, int32_t f, int32_t round, int32_t* partner,
+                                            const unsigned long long* best) {
+  const int32_t a = P.fL[f], b = P.fR[f];
+  const unsigned long long key = match_key(round, f), ba = best[a], bb = best[b];
+  if (ba == key && bb == key) {
     partner[a] = b;
     partner[b] = a;
-    atomicAdd(matched, 1ULL);
+    return false;
+  }
+  // dead: a cell was matched before this round's proposals (its entry is not of this round)
+  return (ba >> 32) == (key >> 32) && (bb >> 32) == (key >> 32);
+}
+
+__global__ void k_match_propose(Level P, const int32_t* list, const int32_t* n, int32_t round, const int32_t* partner,
+                                unsigned long long* best) {
+  for (int32_t k = blockIdx.x * blockDim.x + threadIdx.x; k < *n; k += gridDim.x * blockDim.x)
+    match_propose(P, list[k], round, partner, best);
+}
+
+__global__ void k_match_merge(Level P, const int32_t* list, const int32_t* n, int32_t round, int32_t* partner,
+                              const unsigned long long* best, int32_t* next, int32_t* nnext) {
+  for (int32_t k = blockIdx.x * blockDim.x + threadIdx.x; k < *n; k += gridDim.x * blockDim.x) {
+    const int32_t f = list[k];
+    if (match_merge(P, f, round, partner, best)) next[atomicAdd(nnext, 1)] = f;
   }
 }
 
@@ -359,31 +394,46 @@ static cgks_status coarsen_pass(cgks_ctx* ctx, const Level& P, Level& Q, int32_t
   k_count_candidates<<<grid_for(P.nf, B), B, 0, st>>>(P.nf, P.fR, P.ftag, (unsigned long long*)ctx->d_count);
   int64_t nfc = 0;
   CKS(read_count(ctx, &nfc));
-  int8_t* conf;
-  int32_t *partner, *best, *rep, *cid;
-  CKS(dalloc(ctx, tmp, &conf, P.nf));
+  int32_t *partner, *rep, *cid;
   CKS(dalloc(ctx, tmp, &partner, P.nc));
-  CKS(dalloc(ctx, tmp, &best, P.nc));
   CKS(dalloc(ctx, tmp, &rep, P.nc));
   CKS(dalloc(ctx, tmp, &cid, P.nc));
   CK(cudaMemsetAsync(partner, 0xFF, sizeof(int32_t) * P.nc, st));
   if (nfc > 0) {
-    int32_t* bucket;
+    int32_t *bucket, *list[2], *n;
+    unsigned long long* best;
+    double* fx;
     CKS(dalloc(ctx, tmp, &bucket, nfc));
+    CKS(dalloc(ctx, tmp, &list[0], nfc));
+    CKS(dalloc(ctx, tmp, &list[1], nfc));
+    CKS(dalloc(ctx, tmp, &n, MATCH_ROUNDS + 1));
+    CKS(dalloc(ctx, tmp, &best, P.nc));
+    CKS(dalloc(ctx, tmp, &fx, 3 * P.nf));
     CK(cudaMemsetAsync(bucket, 0x7F, sizeof(int32_t) * nfc, st));
+    CK(cudaMemsetAsync(best, 0xFF, sizeof(unsigned long long) * P.nc, st));
     k_bucket_min<<<grid_for(P.nf, B), B, 0, st>>>(P.nf, P.fL, P.fR, P.ftag, seed, (uint64_t)nfc, bucket);
+    k_face_centres<<<grid_for(P.nf, B), B, 0, st>>>(P.nf, P.amom, P.area, fx);
     const double kmin2 = ctx->P.skew_min * ctx->P.skew_min;
-    k_select_confirm<<<grid_for(P.nf, B), B, 0, st>>>(P, seed, (uint64_t)nfc, bucket, kmin2, conf);
-    for (int64_t round = 0; round <= P.nf; ++round) {
-      k_best_face<<<grid_for(P.nc, B), B, 0, st>>>(P, conf, partner, best);
-      CK(cudaMemsetAsync(ctx->d_count, 0, sizeof(int64_t), st));
-      k_match_round<<<grid_for(P.nf, B), B, 0, st>>>(P, conf, best, partner, (unsigned long long*)ctx->d_count);
-      int64_t matched = 0;
-      CKS(read_count(ctx, &matched));
-      if (matched == 0) break;
+    k_select_confirm<<<grid_for(P.nf, 128), 128, 0, st>>>(P, seed, (uint64_t)nfc, bucket, fx, kmin2, list[0], n);
+    const unsigned gb = grid_for(nfc, B) < 2u * ctx->n_sm ? grid_for(nfc, B) : 2u * ctx->n_sm;
+    // every round with a live face merges at least the smallest one, so nfc rounds bound the loop
+    for (int64_t round = 0; round <= nfc; round += MATCH_ROUNDS) {
+      if (round > 0) {
+        int32_t live = 0;
+        CK(cudaMemcpyAsync(ctx->h_count, n + MATCH_ROUNDS, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
+        CK(cudaStreamSynchronize(st));
+        live = *reinterpret_cast<int32_t*>(ctx->h_count);
+        if (live == 0) break;
+        CK(cudaMemcpyAsync(n, n + MATCH_ROUNDS, sizeof(int32_t), cudaMemcpyDeviceToDevice, st));
+        CK(cudaMemsetAsync(n + 1, 0, sizeof(int32_t) * MATCH_ROUNDS, st));
+      }
+      for (int r = 0; r < MATCH_ROUNDS; ++r) {
+        const int32_t k = (int32_t)round + r;
+        k_match_propose<<<gb, B, 0, st>>>(P, list[r & 1], n + r, k, partner, best);
+        k_match_merge<<<gb, B, 0, st>>>(P, list[r & 1], n + r, k, partner, best, list[1 - (r & 1)], n + r + 1);
+      }
     }
-  } else {
-    CK(cudaMemsetAsync(conf, 0, P.nf, st));
+    CK(cudaGetLastError());
   }
   k_rep_flag<<<grid_for(P.nc, B), B, 0, st>>>(P.nc, partner, rep);
   int64_t ncc = 0;
