@@ -359,8 +359,8 @@ static cgks_status csr_from_counts(cgks_ctx* ctx, std::vector<void*>& M, int32_t
   CKS(dalloc(ctx, M, ptr, n + 1));
   CKS(scan_exclusive(ctx, cnt, *ptr, n, total));
   const int32_t t32 = (int32_t)*total;
+  // (pageable: copied out of t32 before the call returns)
   CK(cudaMemcpyAsync(*ptr + n, &t32, sizeof(int32_t), cudaMemcpyHostToDevice, ctx->stream));
-  CK(cudaStreamSynchronize(ctx->stream));
   return CGKS_OK;
 }
 
@@ -383,9 +383,10 @@ static cgks_status build_c2f(cgks_ctx* ctx, std::vector<void*>& M, std::vector<v
 static cgks_status coarsen_pass(cgks_ctx* ctx, const Level& P, Level& Q, int32_t* map) {
   std::vector<void*> tmp;
   struct Guard {
+    cgks_ctx* ctx;
     std::vector<void*>& t;
-    ~Guard() { free_list(t); }
-  } guard{tmp};
+    ~Guard() { free_list(ctx, t); }
+  } guard{ctx, tmp};
   auto& M = ctx->mesh_allocs;
   cudaStream_t st = ctx->stream;
   const int B = 256;
@@ -465,7 +466,6 @@ static cgks_status coarsen_pass(cgks_ctx* ctx, const Level& P, Level& Q, int32_t
   CKS(dalloc(ctx, M, &Q.shift, 3 * Q.nf));
   k_coarse_face_write<<<grid_for(P.nc, 64), 64, 0, st>>>(P, partner, rep, cid, map, oint, obnd, ti, Q);
   CKS(build_c2f(ctx, M, tmp, Q));
-  CK(cudaStreamSynchronize(st));
   CKS(check_device_error(ctx, "coarsening pass"));
   return CGKS_OK;
 }
@@ -515,8 +515,7 @@ cgks_status build_levels(cgks_ctx* ctx) {
     CKS(dalloc(ctx, M, &cur.agg, tot));
     k_member_fill<<<grid_for(prev.nc, 256), 256, 0, st>>>(prev.nc, comp, cur.agg_ptr, cursor, cur.agg);
     k_sort_segments<<<grid_for(cur.nc, 128), 128, 0, st>>>(cur.nc, cur.agg_ptr, cur.agg);
-    CK(cudaStreamSynchronize(st));
-    free_list(tmp);
+    free_list(ctx, tmp);
     ctx->L.push_back(cur);
   }
   for (Level& L : ctx->L) {

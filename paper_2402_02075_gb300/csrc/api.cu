@@ -1,5 +1,6 @@
 // C ABI of libcgks (include/cgks.h): context, mesh upload, state, residual, explicit steps,
 // V-cycles, steady solve; plus the allocation, scan and error plumbing shared by the kernels.
+#include <algorithm>
 #include <chrono>
 #include <cmath>
 #include <cstring>
@@ -19,22 +20,60 @@ cgks_status cgks_fail(cgks_ctx* c, cgks_status s, const std::string& msg) {
   return s;
 }
 
+// Device memory of a context.  Freed blocks stay with the context and serve its later allocations: a mesh
+// upload takes about 150 arrays, most of them temporary, and cudaMalloc and cudaFree (which waits for the
+// device) cost more than its kernels on small meshes; a step with a norm history took two of them.
+// Every use is on the context's stream, so a block is reused in stream order.  An upload gives back what
+// is above kPoolKeep at its end, and an allocation that fails gives back everything and tries again.
+static constexpr size_t kPoolKeep = (size_t)256 << 20;
+
+static void pool_trim(cgks_ctx* ctx, size_t keep) {
+  auto& pool = ctx->pool;
+  size_t total = 0;
+  for (const PoolBlock& b : pool) total += b.bytes;
+  std::sort(pool.begin(), pool.end(), [](const PoolBlock& x, const PoolBlock& y) { return x.bytes < y.bytes; });
+  while (!pool.empty() && total > keep) {
+    total -= pool.back().bytes;
+    ctx->block_bytes.erase(pool.back().p);
+    cudaFree(pool.back().p);
+    pool.pop_back();
+  }
+}
+
 cgks_status dev_alloc(cgks_ctx* ctx, std::vector<void*>& list, void** p, size_t bytes) {
   *p = nullptr;
-  cudaError_t e = cudaMalloc(p, bytes);
-  if (e != cudaSuccess) {
-    cudaGetLastError();
-    return cgks_fail(ctx, CGKS_ENOMEM, std::string("cudaMalloc of ") + std::to_string(bytes) + " bytes: " +
-                                           cudaGetErrorString(e));
+  const size_t want = (bytes + 511) / 512 * 512;
+  auto& pool = ctx->pool;
+  size_t best = pool.size();
+  for (size_t k = 0; k < pool.size(); ++k)  // the smallest block that fits without wasting more than half of it
+    if (pool[k].bytes >= want && pool[k].bytes <= 2 * want && (best == pool.size() || pool[k].bytes < pool[best].bytes)) best = k;
+  if (best < pool.size()) {
+    *p = pool[best].p;
+    pool[best] = pool.back();
+    pool.pop_back();
+  } else {
+    cudaError_t e = cudaMalloc(p, want);
+    if (e != cudaSuccess) {
+      cudaGetLastError();
+      pool_trim(ctx, 0);
+      e = cudaMalloc(p, want);
+    }
+    if (e != cudaSuccess) {
+      cudaGetLastError();
+      *p = nullptr;
+      return cgks_fail(ctx, CGKS_ENOMEM, std::string("cudaMalloc of ") + std::to_string(bytes) + " bytes: " +
+                                             cudaGetErrorString(e));
+    }
+    ctx->block_bytes[*p] = want;
   }
   list.push_back(*p);
-  e = cudaMemsetAsync(*p, 0, bytes, ctx->stream);
+  const cudaError_t e = cudaMemsetAsync(*p, 0, bytes, ctx->stream);
   if (e != cudaSuccess) return cgks_fail(ctx, CGKS_ECUDA, cudaGetErrorString(e));
   return CGKS_OK;
 }
 
-void free_list(std::vector<void*>& list) {
-  for (void* p : list) cudaFree(p);
+void free_list(cgks_ctx* ctx, std::vector<void*>& list) {
+  for (void* p : list) ctx->pool.push_back({p, ctx->block_bytes[p]});
   list.clear();
 }
 
@@ -156,8 +195,7 @@ cgks_status scan_exclusive(cgks_ctx* ctx, const int32_t* in, int32_t* out, int64
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     *total = *ctx->h_count;
   }
-  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-  free_list(tmp);
+  free_list(ctx, tmp);
   if (e != cudaSuccess) return cgks_fail(ctx, CGKS_ECUDA, std::string("scan: ") + cudaGetErrorString(e));
   return CGKS_OK;
 }
@@ -332,8 +370,9 @@ cgks_status cgks_destroy(cgks_ctx* ctx) {
   }
   for (cudaEvent_t e : ctx->gev)
     if (e) cudaEventDestroy(e);
-  free_list(ctx->mesh_allocs);
-  free_list(ctx->ctx_allocs);
+  free_list(ctx, ctx->mesh_allocs);
+  free_list(ctx, ctx->ctx_allocs);
+  pool_trim(ctx, 0);
   if (ctx->h_err) cudaFreeHost(ctx->h_err);
   if (ctx->h_count) cudaFreeHost(ctx->h_count);
   if (ctx->h_nrm) cudaFreeHost(ctx->h_nrm);
@@ -366,7 +405,7 @@ cgks_status cgks_mesh_upload(cgks_ctx* ctx, int64_t n_nodes, const double* xyz, 
       if (bface_ptr[b + 1] < bface_ptr[b]) return cgks_fail(ctx, CGKS_EMESH, "bface_ptr not monotone");
   }
   CK(cudaStreamSynchronize(ctx->stream));
-  free_list(ctx->mesh_allocs);
+  free_list(ctx, ctx->mesh_allocs);
   // the adjoint's arrays were in mesh_allocs
   ctx->Jp = ctx->Jr = ctx->adt = ctx->pbar = ctx->aself = ctx->arec = ctx->avec = ctx->apart = ctx->akry = nullptr;
   ctx->ajc = ctx->acb = ctx->aWG = nullptr;
@@ -408,6 +447,7 @@ cgks_status cgks_mesh_upload(cgks_ctx* ctx, int64_t n_nodes, const double* xyz, 
   CKS(dalloc(ctx, M, &ctx->ffl, 5 * F.nf));
   CKS(dalloc(ctx, M, &ctx->ffl32, 5 * F.nf));
   CK(cudaStreamSynchronize(ctx->stream));
+  pool_trim(ctx, kPoolKeep);
   ctx->has_mesh = true;
   return CGKS_OK;
 }
@@ -555,7 +595,7 @@ static cgks_status run_iterations(cgks_ctx* ctx, int n, double* norm_hist, bool 
   for (int k = 0; k < n && s == CGKS_OK; ++k) s = multigrid ? vcycle_once(ctx, hist ? hist + k : nullptr)
                                                             : step_once(ctx, hist ? hist + k : nullptr);
   if (s == CGKS_OK && hist) s = read_norm(ctx, hist, norm_hist, n);
-  free_list(tmp);
+  free_list(ctx, tmp);
   CKS(s);
   ctx->iters += n;
   return check_device_error(ctx, name);
@@ -662,7 +702,7 @@ cgks_status cgks_steady_solve(cgks_ctx* ctx, int multigrid, double drop, int64_t
   }
   if (exec) cudaGraphExecDestroy(exec);
   const double sec = std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();
-  free_list(tmp);
+  free_list(ctx, tmp);
   CKS(s);
   ctx->iters += it;
   if (iters_done) *iters_done = it;

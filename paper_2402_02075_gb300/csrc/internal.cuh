@@ -5,6 +5,7 @@
 
 #include <cstdint>
 #include <string>
+#include <unordered_map>
 #include <vector>
 
 #include "cgks.h"
@@ -109,6 +110,12 @@ struct ProfRec {
   double units, bytes;
 };
 
+// a freed device block that the context keeps
+struct PoolBlock {
+  void* p;
+  size_t bytes;
+};
+
 struct cgks_ctx {
   cgks_params P{};
   cudaStream_t stream = nullptr;
@@ -152,6 +159,8 @@ struct cgks_ctx {
   std::vector<int32_t> h_cnodes, h_bnodes, h_btag, h_pairs;
   std::vector<void*> mesh_allocs;   // freed on re-upload / destroy
   std::vector<void*> ctx_allocs;    // freed on destroy
+  std::vector<PoolBlock> pool;      // freed blocks, and the size of every block the context holds
+  std::unordered_map<void*, size_t> block_bytes;
   // kernel timing (cgks_profile): event pairs per kernel kind, with the units and the algorithmic
   // bytes of each recorded launch
   bool prof = false;
@@ -192,7 +201,8 @@ template <typename T>
 cgks_status dalloc(cgks_ctx* ctx, std::vector<void*>& list, T** p, size_t count) {
   return dev_alloc(ctx, list, reinterpret_cast<void**>(p), sizeof(T) * (count ? count : 1));
 }
-void free_list(std::vector<void*>& list);
+// the blocks of `list` back to the context
+void free_list(cgks_ctx* ctx, std::vector<void*>& list);
 
 inline unsigned grid_for(int64_t n, int block) { return (unsigned)((n + block - 1) / block); }
 

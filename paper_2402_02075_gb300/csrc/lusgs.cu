@@ -242,7 +242,7 @@ cgks_status lusgs_colors(cgks_ctx* ctx, int l) {
   std::vector<void*> tmp;
   cgks_status s = dalloc(ctx, tmp, &sel, L.nc);
   if (s != CGKS_OK) {
-    free_list(tmp);
+    free_list(ctx, tmp);
     return s;
   }
   std::vector<int32_t> minus1(L.nc, -1);
@@ -259,7 +259,7 @@ cgks_status lusgs_colors(cgks_ctx* ctx, int l) {
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e == cudaSuccess) left = *ctx->h_count;
   }
-  free_list(tmp);
+  free_list(ctx, tmp);
   CK(e);
   if (left > 0) return cgks_fail(ctx, CGKS_EINVAL, "LU-SGS colouring did not finish");
   // colour-major order, ascending cell id within a colour (counting sort on the host)

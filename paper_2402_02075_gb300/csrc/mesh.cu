@@ -568,9 +568,10 @@ cgks_status build_fine_mesh(cgks_ctx* ctx, int64_t n_nodes, const double* xyz, i
                             const int32_t* periodic_pairs, int64_t n_periodic) {
   std::vector<void*> tmp;
   struct Guard {
+    cgks_ctx* ctx;
     std::vector<void*>& t;
-    ~Guard() { free_list(t); }
-  } guard{tmp};
+    ~Guard() { free_list(ctx, t); }
+  } guard{ctx, tmp};
   cudaStream_t st = ctx->stream;
   Fine& F = ctx->F;
   auto& M = ctx->mesh_allocs;
