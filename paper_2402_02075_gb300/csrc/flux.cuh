@@ -10,9 +10,13 @@
 //  - with m_k = <u_n^k> over the half space divided by rho, and beta = +-g(0)/rho, integration by parts
 //    in u_n gives the normal moments of a slope (d, R_n, th) without any division or coefficient:
 //      D_k = <u_n^k a> = m_k d + X_k R_n + Y_k th,
-//      X = (beta, m_0, 2 m_1, 3 m_2, 4 m_3),  Y = (-beta U/(2 h), beta/2, m_0, 3 m_1, 6 m_2);
-//    the tangential momentum row is m_k R, the energy row D_{k+2}/2 + (K+2)/2 (h D_k + m_k th), and the
-//    moments of c a (c the tangential peculiar velocity) reuse the D_k of the tangential directions;
+//      X = (beta, m_0, 2 m_1, 3 m_2),  Y = (-beta U/(2 h), beta/2, m_0, 3 m_1);
+//    the tangential momentum row is m_k R, the energy row D_{k+2}/2 + (K+2)/2 (h D_k + m_k th);
+//  - with A the time slope, -A = u.d + ... as a slope (rt, Rt, tht), the rows of a.u are those of -A plus the
+//    non-equilibrium part alone, which the recurrences of X and Y in k reduce to
+//      a_k d_n th + h Y_k sig,  a_k = Y_{k+1} - U Y_k - X_k,  sig = 2 d_n R_n - (gamma - 1) tr R
+//    (heat flux and normal stress) in the normal rows and h X_k (d_n R_i + d_i R_n) + h Y_k d_i th (shear) in
+//    the tangential ones;
 //  - no face frame: a vector is kept in the global frame, its normal component taken with n where it is
 //    needed, so nothing is rotated in or out.  Tangential vectors may carry a normal component that
 //    the final projection removes;
@@ -58,8 +62,8 @@ HD bool gks_side(const S w[5], const double n[3], double s, double gm1, const do
 // time coefficients of Eq. 2nd-flux integrated over [0, dt] that multiply the two sides' moments
 template <typename T>
 struct GksTime {
-  T q4, q5, tq4;     // of g, of -(a.u) g and of -A g in the flux
-  T edt, etd, etau;  // the same in the interface state at dt
+  T q4, q5, q54;    // in the flux: of g, of -(a.u) g, and that less the one of -A g
+  T edt, etd, edd;  // the same in the interface state at dt
 };
 
 // sums over both sides in the frame moving with the interface's tangential velocity: gradients of the
@@ -98,105 +102,88 @@ HD void gks_add_side(const GksSide<S>& g, const double G[15], const double n[3],
   }
   // moments and the coefficients X_k, Y_k
   const S U = g.U, h = g.h, m0 = g.m0, beta = g.beta;
-  const S m1 = U * m0 + h * beta;
+  const S hb = h * beta, m1 = U * m0 + hb;
   const S hm0 = h * m0, m2 = U * m1 + hm0;
   const S hm1 = h * m1, m3 = U * m2 + 2.0 * hm1;
-  const S m4 = U * m3 + 3.0 * (h * m2);
-  const S X2 = 2.0 * m1, X3 = 3.0 * m2, X4 = 4.0 * m3;
-  const S Y0 = -0.5 * U * (beta * g.l2), Y1 = 0.5 * beta, Y3 = 3.0 * m1, Y4 = 2.0 * X3;
+  const S X2 = 2.0 * m1, X3 = 3.0 * m2;
+  const S Y0 = -0.5 * U * (beta * g.l2), Y1 = 0.5 * beta, Y3 = 3.0 * m1;
   const S kap = k2 * h, k2m0 = k2 * m0, k2m1 = k2 * m1;
   const T kd = hd2 + kap;
   T dm0[3];
 #pragma unroll
   for (int d = 0; d < 3; ++d) dm0[d] = del[d] * m0;
-  // gradients of the interface equilibrium; the D_0, D_1 of each direction serve below
-  S D0[3], D1[3];
+  // gradients of the interface equilibrium
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
-    D0[k] = m0 * G[k] + beta * Rn[k] + Y0 * th[k];
-    D1[k] = m1 * G[k] + m0 * Rn[k] + Y1 * th[k];
+    const S D0 = m0 * G[k] + beta * Rn[k] + Y0 * th[k];
+    const S D1 = m1 * G[k] + m0 * Rn[k] + Y1 * th[k];
     const S D2 = m2 * G[k] + X2 * Rn[k] + m0 * th[k];
     T e = FIRST ? T(0.5 * D2) : a.e[k] + 0.5 * D2;
-    e += kd * D0[k];
+    e += kd * D0;
     e += k2m0 * th[k];
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
       e += dm0[i] * R[i][k];
       const T v = FIRST ? T(m0 * R[i][k]) : a.Tm[i][k] + m0 * R[i][k];
-      a.Tm[i][k] = v + del[i] * D0[k];
+      a.Tm[i][k] = v + del[i] * D0;
     }
     a.e[k] = e;
-    a.rho[k] = FIRST ? T(D0[k]) : a.rho[k] + D0[k];
-    a.mn[k] = FIRST ? T(D1[k]) : a.mn[k] + D1[k];
+    a.rho[k] = FIRST ? T(D0) : a.rho[k] + D0;
+    a.mn[k] = FIRST ? T(D1) : a.mn[k] + D1;
   }
   // derivatives along n and along the tangential velocity
-  const double rn = n[0] * G[0] + n[1] * G[1] + n[2] * G[2];
-  const S pn = n[0] * gp[0] + n[1] * gp[1] + n[2] * gp[2];
+  const S rn = n[0] * G[0] + n[1] * G[1] + n[2] * G[2];
+  const S thn = n[0] * th[0] + n[1] * th[1] + n[2] * th[2];
   const S rS = g.ut[0] * G[0] + g.ut[1] * G[1] + g.ut[2] * G[2];
-  const S pS = g.ut[0] * gp[0] + g.ut[1] * gp[1] + g.ut[2] * gp[2];
-  S Rv[3], RS[3], Rt[3];
+  const S thS = g.ut[0] * th[0] + g.ut[1] * th[1] + g.ut[2] * th[2];
+  S Rv[3], Rt[3];
 #pragma unroll
   for (int i = 0; i < 3; ++i) {
     Rv[i] = n[0] * R[i][0] + n[1] * R[i][1] + n[2] * R[i][2];
-    RS[i] = g.ut[0] * R[i][0] + g.ut[1] * R[i][1] + g.ut[2] * R[i][2];
-    Rt[i] = U * Rv[i] + (RS[i] + gp[i]);
+    S x = gp[i] + U * Rv[i];
+    x += g.ut[0] * R[i][0];
+    x += g.ut[1] * R[i][1];
+    x += g.ut[2] * R[i][2];
+    Rt[i] = x;
   }
   const S Rnn = n[0] * Rv[0] + n[1] * Rv[1] + n[2] * Rv[2];
-  const S RnS = n[0] * RS[0] + n[1] * RS[1] + n[2] * RS[2];
   const S Rnt = n[0] * Rt[0] + n[1] * Rt[1] + n[2] * Rt[2];
-  const S thn = pn - h * rn, thS = pS - h * rS;
-  const S tr = R[0][0] + R[1][1] + R[2][2], Dv = tr - Rnn;
+  const S tr = R[0][0] + R[1][1] + R[2][2];
   // minus the time derivatives (Euler)
   const S rt = U * rn + (rS + tr);
-  const S tht = U * pn + pS + (gamma * h) * tr - h * rt;
-  // rows of <u_n^k (a.u) psi> (al) and of -<u_n^k A psi> (At), k = 0..3 for the powers of u_n and e0, e1
-  // for the energy rows of k = 0, 1
-  const S rSD = rS + Dv;
-  S al0 = m1 * rn + m0 * Rnn + Y1 * thn;
-  al0 += m0 * rSD;
-  al0 += beta * RnS;
-  al0 += Y0 * thS;
-  S al1 = m2 * rn + X2 * Rnn + m0 * thn;
-  al1 += m1 * rSD;
-  al1 += m0 * RnS;
-  al1 += Y1 * thS;
-  S al2 = m3 * rn + X3 * Rnn + Y3 * thn;
-  al2 += m2 * rSD;
-  al2 += X2 * RnS;
-  al2 += m0 * thS;
-  S al3 = m4 * rn + X4 * Rnn + Y4 * thn;
-  al3 += m3 * rSD;
-  al3 += X3 * RnS;
-  al3 += Y3 * thS;
+  const S tht = U * thn + thS + (gm1 * h) * tr;
+  // rows of -<u_n^k A psi>, k = 0..3, and the coefficients a_k, h Y_k of the non-equilibrium part
   const S At0 = m0 * rt + beta * Rnt + Y0 * tht;
   const S At1 = m1 * rt + m0 * Rnt + Y1 * tht;
   const S At2 = m2 * rt + X2 * Rnt + m0 * tht;
   const S At3 = m3 * rt + X3 * Rnt + Y3 * tht;
-  // tangential rows of a.u, k = 0, 1
-  S Ta0[3], Ta1[3];
+  const S a0 = U * Y0 + Y1, a1 = U * Y1, a3 = 3.0 * hm0;  // minus a_0, minus a_1; a_2 = h beta
+  const S b0 = h * Y0, b1 = 0.5 * hb, b3 = 3.0 * hm1;     // b_2 = h m_0
+  const S sig = 2.0 * Rnn - gm1 * tr, dvs = (1.0 - gm1 * k2) * tr - Rnn;
 #pragma unroll
-  for (int i = 0; i < 3; ++i) {
-    const S b = RS[i] + th[i];
-    Ta0[i] = m1 * Rv[i] + m0 * b + h * D0[i];
-    Ta1[i] = m2 * Rv[i] + m1 * b + h * D1[i];
-  }
+  for (int i = 0; i < 3; ++i) Rv[i] = Rv[i] + Rn[i];  // the shear d_n R_i + d_i R_n from here on
   const S v4 = 0.5 * m2 + kap * m0, f4 = 0.5 * m3 + kap * m1;  // energy rows of psi and u psi
   {
     // flux: q4 <u psi> - q5 <u (a.u) psi> - tau q4 <u A psi>
-    const T qr = t.q4 * g.rho, z1 = t.q5 * al1 - t.tq4 * At1, z2 = t.q5 * al2 - t.tq4 * At2,
-                 z3 = t.q5 * al3 - t.tq4 * At3;
-    const T hn = t.q5 * thn, hb = t.q5 * thS - t.tq4 * tht, dv = t.q5 * Dv;
+    const T qr = t.q4 * g.rho, hn = t.q5 * thn, hs = t.q5 * sig, hd = t.q5 * dvs, ht = t.q54 * tht;
+    T z1 = t.q54 * At1 - a1 * hn;
+    z1 += b1 * hs;
+    T z2 = t.q54 * At2 + hb * hn;
+    z2 += hm0 * hs;
+    T z3 = t.q54 * At3 + a3 * hn;
+    z3 += b3 * hs;
     const T F0 = qr * m1 - z1, F1 = qr * m2 - z2;
     T F4 = qr * f4 - 0.5 * z3;
     F4 -= kap * z1;
-    F4 -= (k2 * m2) * hn;
-    F4 -= k2m1 * hb;
-    F4 -= hm1 * dv;
+    F4 -= k2m1 * ht;
+    F4 -= (kap * m0) * hn;
+    F4 -= hm1 * hd;
     F4 += hd2 * F0;
-    const T c = t.tq4 * m1;
+    const T cA = t.q54 * m1, cS = t.q5 * hm0, ch = t.q5 * b1;
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
-      const T v = t.q5 * Ta1[i] - c * Rt[i];
+      T v = cA * Rt[i] + cS * Rv[i];
+      v += ch * th[i];
       F4 -= del[i] * v;
       const T x = del[i] * F0 - v;
       a.FT[i] = FIRST ? x : a.FT[i] + x;
@@ -205,35 +192,46 @@ HD void gks_add_side(const GksSide<S>& g, const double G[15], const double n[3],
     a.F1 = FIRST ? F1 : a.F1 + F1;
     a.F4 = FIRST ? F4 : a.F4 + F4;
     if (heat) {
-      const T z0 = t.q5 * al0 - t.tq4 * At0, I0 = qr * m0 - z0;
+      T z0 = t.q54 * At0 - a0 * hn;
+      z0 += b0 * hs;
+      const T I0 = qr * m0 - z0;
       T I4 = qr * v4 - 0.5 * z2;
       I4 -= kap * z0;
-      I4 -= k2m1 * hn;
-      I4 -= k2m0 * hb;
-      I4 -= hm0 * dv;
+      I4 -= k2m0 * ht;
+      I4 -= (k2 * hb) * hn;
+      I4 -= hm0 * hd;
       I4 += hd2 * I0;
-      const T qT = t.q5 * (del[0] * Ta0[0] + del[1] * Ta0[1] + del[2] * Ta0[2]);
-      const T qA = (t.tq4 * m0) * (del[0] * Rt[0] + del[1] * Rt[1] + del[2] * Rt[2]);
-      I4 -= qT - qA;
+      const T dA = t.q54 * m0, dS = t.q5 * hb, dh = t.q5 * b0;
+#pragma unroll
+      for (int i = 0; i < 3; ++i) {
+        T v = dA * Rt[i] + dS * Rv[i];
+        v += dh * th[i];
+        I4 -= del[i] * v;
+      }
       a.I0 = FIRST ? I0 : a.I0 + I0;
       a.I4 = FIRST ? I4 : a.I4 + I4;
     }
   }
   if (STATE) {
-    const T qr = t.edt * g.rho, z0 = t.etd * al0 - t.etau * At0, z1 = t.etd * al1 - t.etau * At1,
-                 z2 = t.etd * al2 - t.etau * At2;
-    const T hn = t.etd * thn, hb = t.etd * thS - t.etau * tht, dv = t.etd * Dv;
+    const T qr = t.edt * g.rho, hn = t.etd * thn, hs = t.etd * sig, hd = t.etd * dvs, ht = t.edd * tht;
+    T z0 = t.edd * At0 - a0 * hn;
+    z0 += b0 * hs;
+    T z1 = t.edd * At1 - a1 * hn;
+    z1 += b1 * hs;
+    T z2 = t.edd * At2 + hb * hn;
+    z2 += hm0 * hs;
     const T W0 = qr * m0 - z0, W1 = qr * m1 - z1;
     T W4 = qr * v4 - 0.5 * z2;
     W4 -= kap * z0;
-    W4 -= k2m1 * hn;
-    W4 -= k2m0 * hb;
-    W4 -= hm0 * dv;
+    W4 -= k2m0 * ht;
+    W4 -= (k2 * hb) * hn;
+    W4 -= hm0 * hd;
     W4 += hd2 * W0;
-    const T c = t.etau * m0;
+    const T dA = t.edd * m0, dS = t.etd * hb, dh = t.etd * b0;
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
-      const T v = t.etd * Ta0[i] - c * Rt[i];
+      T v = dA * Rt[i] + dS * Rv[i];
+      v += dh * th[i];
       W4 -= del[i] * v;
       const T x = del[i] * W0 - v;
       a.WT[i] = FIRST ? x : a.WT[i] + x;
@@ -322,11 +320,11 @@ HD bool gks_centre(const GksSide<SL>& gl, const GksSide<SR>& gr, D dt, const Phy
   const T q4 = tn * c.om, tte = tn * dt * edt;
   c.q1 = dt - q4;
   c.t.q4 = q4;
-  c.t.q5 = (tau + tn) * q4 - tte;
-  c.t.tq4 = tau * q4;
+  c.t.q54 = tn * q4 - tte;
+  c.t.q5 = c.t.q54 + tau * q4;
   c.t.edt = edt;
-  c.t.etd = edt * (tau + dt);
-  c.t.etau = edt * tau;
+  c.t.edd = edt * dt;
+  c.t.etd = c.t.edd + edt * tau;
   c.q2 = c.t.q5 - tau * dt;
   c.q3 = 0.5 * dt * dt - tau * dt + tau * q4;
   return positive(c.rho) && positive(c.p);
@@ -362,21 +360,25 @@ HD int gks_flux_t(const double n[3], double weight, bool bnd, const SL WL[5], co
   GksAcc<T> a;
   gks_add_side<STATE, true, SL, T>(gl, GL, n, ut, gm1, ph.gamma, k2, t, heat, a);
   gks_add_side<STATE, false, SR, T>(gr, GR, n, ut, gm1, ph.gamma, k2, t, heat, a);
-  // equilibrium part, full space: X = (0, 1, 2 m1, 3 m2, 4 m3), Y = (0, 0, 1, 3 m1, 6 m2)
+  // equilibrium part, full space: X = (0, 1, 2 m1, 3 m2), Y = (0, 0, 1, 3 m1)
   {
-    T Rn[3], gp[3], th[3], Tn[3], TS[3];
+    T Rn[3], th[3], Tn[3], T0[3];
+    const T hU2 = 0.5 * U * U;
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
       Rn[k] = a.mn[k] - U * a.rho[k];
       T x = a.e[k] - U * a.mn[k];
-      x += (0.5 * U * U) * a.rho[k];
-      gp[k] = gm1 * x;
-      th[k] = gp[k] - h * a.rho[k];
+      x += hU2 * a.rho[k];
+      T0[k] = gm1 * x;  // pressure gradient, then minus the tangential momentum's time derivative
+      th[k] = T0[k] - h * a.rho[k];
     }
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
       Tn[i] = n[0] * a.Tm[i][0] + n[1] * a.Tm[i][1] + n[2] * a.Tm[i][2];
-      TS[i] = ut[0] * a.Tm[i][0] + ut[1] * a.Tm[i][1] + ut[2] * a.Tm[i][2];
+      T0[i] += U * Tn[i];
+      T0[i] += ut[0] * a.Tm[i][0];
+      T0[i] += ut[1] * a.Tm[i][1];
+      T0[i] += ut[2] * a.Tm[i][2];
     }
     const T rn = n[0] * a.rho[0] + n[1] * a.rho[1] + n[2] * a.rho[2];
     const T Rnn = n[0] * Rn[0] + n[1] * Rn[1] + n[2] * Rn[2];
@@ -385,61 +387,43 @@ HD int gks_flux_t(const double n[3], double weight, bool bnd, const SL WL[5], co
     const T RnS = ut[0] * Rn[0] + ut[1] * Rn[1] + ut[2] * Rn[2];
     const T thS = ut[0] * th[0] + ut[1] * th[1] + ut[2] * th[2];
     const T Dv = (a.Tm[0][0] + a.Tm[1][1] + a.Tm[2][2]) - (n[0] * Tn[0] + n[1] * Tn[1] + n[2] * Tn[2]);
-    const T m2 = U * U + h, m3 = U * m2 + 2.0 * h * U, m4 = U * m3 + 3.0 * h * m2;
-    const T X2 = 2.0 * U, X3 = 3.0 * m2, X4 = 4.0 * m3, Y3 = 3.0 * U, Y4 = 2.0 * X3, kap = k2 * h;
-    const T rSD = rS + Dv;
-    const T c0 = U * rn + Rnn + rSD;  // <u^k (a.u)>: minus the time derivatives of mass, momentum, ...
-    T c1 = m2 * rn + X2 * Rnn + thn;
-    c1 += U * rSD;
-    c1 += RnS;
-    T c2 = m3 * rn + X3 * Rnn + Y3 * thn;
-    c2 += m2 * rSD;
-    c2 += X2 * RnS;
-    c2 += thS;
-    T c3 = m4 * rn + X4 * Rnn + Y4 * thn;
-    c3 += m3 * rSD;
-    c3 += X3 * RnS;
-    c3 += Y3 * thS;
-    T e0 = 0.5 * c2 + kap * c0;
-    e0 += k2 * (U * thn + thS);
-    e0 += h * Dv;
-    T e1 = 0.5 * c3 + kap * c1;
-    e1 += (k2 * m2) * thn;
-    e1 += (k2 * U) * thS;
-    e1 += (h * U) * Dv;
-    T T0[3], T1[3];
-#pragma unroll
-    for (int i = 0; i < 3; ++i) {
-      T0[i] = U * Tn[i] + (TS[i] + gp[i]);
-      T1[i] = m2 * Tn[i] + h * a.mn[i];
-      T1[i] += U * (TS[i] + th[i]);
-    }
-    // minus the time slope's rows in u psi
-    const T Rt = c1 - U * c0;
-    T pt = e0 - U * c1;
-    pt += (0.5 * U * U) * c0;
-    const T tht = gm1 * pt - h * c0;
-    const T A2 = m2 * c0 + X2 * Rt + tht;
-    const T A3 = m3 * c0 + X3 * Rt + Y3 * tht;
+    const T tr = Dv + Rnn;
+    const T m2 = U * U + h, m3 = U * m2 + 2.0 * h * U, kap = k2 * h;
+    // minus the time derivatives: mass, normal momentum (Rt, c1 with the mass's), th
+    const T c0 = U * rn + (rS + tr);
+    T Rt = U * Rnn + (RnS + thn);
+    Rt += h * rn;
+    const T c1 = U * c0 + Rt;
+    const T tht = U * thn + thS + (gm1 * h) * tr;
+    const T sig = 2.0 * Rnn - gm1 * tr, dvs = (1.0 - gm1 * k2) * tr - Rnn;
+    T A2 = m2 * c0 + tht;
+    A2 += (2.0 * U) * Rt;
+    T A3 = m3 * c0 + (3.0 * m2) * Rt;
+    A3 += (3.0 * U) * tht;
     T eA = 0.5 * A3 + kap * c1;
     eA += (k2 * U) * tht;
-    const T q23 = q2 - q3;
+    T e1 = (k2 + 1.5) * thn + (1.5 * U) * sig;  // non-equilibrium energy flux over h
+    e1 += U * dvs;
+    const T q23 = q2 - q3, q2h = q2 * h;
     a.F0 += q1 * Mn;
     a.F0 += q23 * c1;
     a.F1 += q1 * (Mn * U + p);
-    a.F1 += q2 * c2;
-    a.F1 -= q3 * A2;
+    a.F1 += q23 * A2;
+    a.F1 += q2h * sig;
     a.F4 += (q1 * U) * (E + p);
-    a.F4 += q2 * e1;
-    a.F4 -= q3 * eA;
-    const T q3U = q3 * U;
+    a.F4 += q23 * eA;
+    a.F4 += q2h * e1;
+    const T qU = q23 * U;
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
-      a.FT[i] += q2 * T1[i];
-      a.FT[i] -= q3U * T0[i];
+      a.FT[i] += qU * T0[i];
+      a.FT[i] += q2h * (Tn[i] + Rn[i]);
     }
+    T e0 = 0.5 * A2 + kap * c0;  // energy's time derivative (minus)
+    e0 += k2 * tht;
+    e0 += h * (dvs + 0.5 * sig);
     if (STATE) {
-      const T od = om * dt;
+      const T od = om * c.dt;
       a.W0 += om * rho;
       a.W0 -= od * c0;
       a.W1 += om * Mn;
@@ -497,49 +481,46 @@ HD void gks_gradient_column(const GksSide<double>& g, const GksCentre<double>& c
   const double gr = A[0], gp = gm1 * x, th = gp - h * gr, Rn = n[0] * R[0] + n[1] * R[1] + n[2] * R[2];
   const double dn = n[0] * d[0] + n[1] * d[1] + n[2] * d[2];
   const double ds = g.ut[0] * d[0] + g.ut[1] * d[1] + g.ut[2] * d[2], ud = U * dn + ds;
-  const double m1 = U * m0 + h * beta, hm0 = h * m0, m2 = U * m1 + hm0, hm1 = h * m1, m3 = U * m2 + 2.0 * hm1,
-               m4 = U * m3 + 3.0 * (h * m2);
-  const double X2 = 2.0 * m1, X3 = 3.0 * m2, X4 = 4.0 * m3, Y0 = -0.5 * U * (beta * g.l2), Y1 = 0.5 * beta, Y3 = 3.0 * m1,
-               Y4 = 2.0 * X3;
+  const double hb = h * beta, m1 = U * m0 + hb, hm0 = h * m0, m2 = U * m1 + hm0, hm1 = h * m1, m3 = U * m2 + 2.0 * hm1;
+  const double X2 = 2.0 * m1, X3 = 3.0 * m2, Y0 = -0.5 * U * (beta * g.l2), Y1 = 0.5 * beta, Y3 = 3.0 * m1;
   const double kap = k2 * h, k2m0 = k2 * m0, k2m1 = k2 * m1;
-  const double D0 = m0 * gr + beta * Rn + Y0 * th, D1 = m1 * gr + m0 * Rn + Y1 * th, D2 = m2 * gr + X2 * Rn + m0 * th,
-               D3 = m3 * gr + X3 * Rn + Y3 * th, D4 = m4 * gr + X4 * Rn + Y4 * th;
-  const double tr = R[0] * d[0] + R[1] * d[1] + R[2] * d[2], Dv = tr - dn * Rn;
-  const double rt = ud * gr + tr, Rnt = ud * Rn + gp * dn, tht = ud * gp + (ph.gamma * h) * tr - h * rt;
-  const double thn = dn * th, thS = ds * th;
-  const double al0 = dn * D1 + ds * D0 + m0 * Dv, al1 = dn * D2 + ds * D1 + m1 * Dv, al2 = dn * D3 + ds * D2 + m2 * Dv,
-               al3 = dn * D4 + ds * D3 + m3 * Dv;
+  const double D0 = m0 * gr + beta * Rn + Y0 * th, D1 = m1 * gr + m0 * Rn + Y1 * th, D2 = m2 * gr + X2 * Rn + m0 * th;
+  const double tr = R[0] * d[0] + R[1] * d[1] + R[2] * d[2], Rnn = dn * Rn;
+  const double rt = ud * gr + tr, Rnt = ud * Rn + gp * dn, tht = ud * th + (gm1 * h) * tr, thn = dn * th;
   const double At0 = m0 * rt + beta * Rnt + Y0 * tht, At1 = m1 * rt + m0 * Rnt + Y1 * tht,
                At2 = m2 * rt + X2 * Rnt + m0 * tht, At3 = m3 * rt + X3 * Rnt + Y3 * tht;
+  const double a0 = -(U * Y0 + Y1), a1 = -(U * Y1), a3 = 3.0 * hm0, b0 = h * Y0, b1 = 0.5 * hb, b3 = 3.0 * hm1;
+  const double sig = 2.0 * Rnn - gm1 * tr, dvs = (1.0 - gm1 * k2) * tr - Rnn;
   double F0, F1, F4, FT[3], W0, W1, W4, WT[3], I0 = 0.0, I4 = 0.0;
   const bool heat = ph.viscous && ph.prandtl != 1.0;
   {
     const GksTime<double>& t = c.t;
-    const double z0 = t.q5 * al0 - t.tq4 * At0, z1 = t.q5 * al1 - t.tq4 * At1, z2 = t.q5 * al2 - t.tq4 * At2,
-                 z3 = t.q5 * al3 - t.tq4 * At3;
-    const double hn = t.q5 * thn, hb = t.q5 * thS - t.tq4 * tht, dv = t.q5 * Dv;
-    const double y0 = t.etd * al0 - t.etau * At0, y1 = t.etd * al1 - t.etau * At1, y2 = t.etd * al2 - t.etau * At2;
-    const double wn = t.etd * thn, wb = t.etd * thS - t.etau * tht, wv = t.etd * Dv;
+    const double hn = t.q5 * thn, hs = t.q5 * sig, hd = t.q5 * dvs, ht = t.q54 * tht;
+    const double wn = t.etd * thn, ws = t.etd * sig, wd = t.etd * dvs, wt = t.edd * tht;
+    const double z0 = t.q54 * At0 + a0 * hn + b0 * hs, z1 = t.q54 * At1 + a1 * hn + b1 * hs,
+                 z2 = t.q54 * At2 + hb * hn + hm0 * hs, z3 = t.q54 * At3 + a3 * hn + b3 * hs;
+    const double y0 = t.edd * At0 + a0 * wn + b0 * ws, y1 = t.edd * At1 + a1 * wn + b1 * ws,
+                 y2 = t.edd * At2 + hb * wn + hm0 * ws;
     F0 = -z1;
     F1 = -z2;
-    F4 = hd2 * F0 - (0.5 * z3 + kap * z1 + (k2 * m2) * hn + k2m1 * hb + hm1 * dv);
+    F4 = hd2 * F0 - (0.5 * z3 + kap * z1 + k2m1 * ht + (kap * m0) * hn + hm1 * hd);
     W0 = -y0;
     W1 = -y1;
-    W4 = hd2 * W0 - (0.5 * y2 + kap * y0 + k2m1 * wn + k2m0 * wb + hm0 * wv);
+    W4 = hd2 * W0 - (0.5 * y2 + kap * y0 + k2m0 * wt + (k2 * hb) * wn + hm0 * wd);
     if (heat) {
       I0 = -z0;
-      I4 = hd2 * I0 - (0.5 * z2 + kap * z0 + k2m1 * hn + k2m0 * hb + hm0 * dv);
+      I4 = hd2 * I0 - (0.5 * z2 + kap * z0 + k2m0 * ht + (k2 * hb) * hn + hm0 * hd);
     }
-    const double a0 = m1 * dn + m0 * ds, a1 = m2 * dn + m1 * ds, b0 = m0 * th + h * D0, b1 = m1 * th + h * D1;
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
-      const double Ta0 = a0 * R[i] + b0 * d[i], Ta1 = a1 * R[i] + b1 * d[i], Rt = ud * R[i] + gp * d[i];
-      const double v = t.q5 * Ta1 - (t.tq4 * m1) * Rt, y = t.etd * Ta0 - (t.etau * m0) * Rt;
+      const double Rt = ud * R[i] + gp * d[i], Sh = dn * R[i] + Rn * d[i], thi = th * d[i];
+      const double v = (t.q54 * m1) * Rt + (t.q5 * hm0) * Sh + (t.q5 * b1) * thi;
+      const double y = (t.edd * m0) * Rt + (t.etd * hb) * Sh + (t.etd * b0) * thi;
       F4 -= del[i] * v;
       FT[i] = del[i] * F0 - v;
       W4 -= del[i] * y;
       WT[i] = del[i] * W0 - y;
-      if (heat) I4 -= del[i] * (t.q5 * Ta0 - (t.tq4 * m0) * Rt);
+      if (heat) I4 -= del[i] * ((t.q54 * m0) * Rt + (t.q5 * hb) * Sh + (t.q5 * b0) * thi);
     }
   }
   // the interface equilibrium's gradient (amplitudes along d) and its terms
@@ -553,32 +534,26 @@ HD void gks_gradient_column(const GksSide<double>& g, const GksCentre<double>& c
       e += (del[i] * m0) * R[i];
     }
     const double Rc = D1 - Uc * D0, pc = gm1 * (e - Uc * D1 + (0.5 * Uc * Uc) * D0), tc = pc - hc * D0;
-    const double dc = c.ut[0] * d[0] + c.ut[1] * d[1] + c.ut[2] * d[2];
-    const double nT = n[0] * T[0] + n[1] * T[1] + n[2] * T[2];
-    const double Dc = (T[0] * d[0] + T[1] * d[1] + T[2] * d[2]) - dn * nT;
-    const double n2 = Uc * Uc + hc, n3 = Uc * n2 + 2.0 * hc * Uc, n4 = Uc * n3 + 3.0 * hc * n2;
-    const double E2 = n2 * D0 + 2.0 * Uc * Rc + tc, E3 = n3 * D0 + 3.0 * n2 * Rc + 3.0 * Uc * tc,
-                 E4 = n4 * D0 + 4.0 * n3 * Rc + 6.0 * n2 * tc;
-    const double c0 = dn * D1 + dc * D0 + Dc, c1 = dn * E2 + dc * D1 + Uc * Dc, c2 = dn * E3 + dc * E2 + n2 * Dc,
-                 c3 = dn * E4 + dc * E3 + n3 * Dc;
-    const double tn = dn * tc, tS = dc * tc;
-    const double e0 = 0.5 * c2 + kc * c0 + k2 * (Uc * tn + tS) + hc * Dc;
-    const double e1 = 0.5 * c3 + kc * c1 + (k2 * n2) * tn + (k2 * Uc) * tS + (hc * Uc) * Dc;
-    const double Rt = c1 - Uc * c0, tt = gm1 * (e0 - Uc * c1 + (0.5 * Uc * Uc) * c0) - hc * c0;
+    const double dc = c.ut[0] * d[0] + c.ut[1] * d[1] + c.ut[2] * d[2], uc = Uc * dn + dc;
+    const double nT = n[0] * T[0] + n[1] * T[1] + n[2] * T[2], rc = dn * Rc;
+    const double t2 = (T[0] * d[0] + T[1] * d[1] + T[2] * d[2]) - dn * nT + rc;
+    const double n2 = Uc * Uc + hc, n3 = Uc * n2 + 2.0 * hc * Uc;
+    const double c0 = uc * D0 + t2, Rt = uc * Rc + pc * dn, c1 = Uc * c0 + Rt, tt = uc * tc + (gm1 * hc) * t2, tn = dn * tc;
+    const double sc = 2.0 * rc - gm1 * t2, dv = (1.0 - gm1 * k2) * t2 - rc;
     const double A2 = n2 * c0 + 2.0 * Uc * Rt + tt, A3 = n3 * c0 + 3.0 * n2 * Rt + 3.0 * Uc * tt;
-    const double eA = 0.5 * A3 + kc * c1 + (k2 * Uc) * tt;
-    const double q23 = c.q2 - c.q3, od = c.om * c.dt;
+    const double eA = 0.5 * A3 + kc * c1 + (k2 * Uc) * tt, e1 = (k2 + 1.5) * tn + (1.5 * Uc) * sc + Uc * dv;
+    const double e0 = 0.5 * A2 + kc * c0 + k2 * tt + hc * (dv + 0.5 * sc);
+    const double q23 = c.q2 - c.q3, od = c.om * c.dt, q2h = c.q2 * hc;
     F0 += q23 * c1;
-    F1 += c.q2 * c2 - c.q3 * A2;
-    F4 += c.q2 * e1 - c.q3 * eA;
+    F1 += q23 * A2 + q2h * sc;
+    F4 += q23 * eA + q2h * e1;
     W0 -= od * c0;
     W1 -= od * c1;
     W4 -= od * e0;
-    const double s0 = Uc * dn + dc, s1 = n2 * dn + Uc * dc, v1 = hc * D1 + Uc * tc;
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
-      const double T0 = s0 * T[i] + pc * d[i], T1 = s1 * T[i] + v1 * d[i];
-      FT[i] += c.q2 * T1 - (c.q3 * Uc) * T0;
+      const double T0 = uc * T[i] + pc * d[i];
+      FT[i] += (q23 * Uc) * T0 + q2h * (dn * T[i] + Rc * d[i]);
       WT[i] -= od * T0;
     }
     if (heat) {
