@@ -348,7 +348,8 @@ cgks_status cgks_create(const cgks_params* params, void* cuda_stream, cgks_ctx**
   if ((s = dalloc(ctx, ctx->ctx_allocs, &ctx->derr, 1)) != CGKS_OK ||
       (s = dalloc(ctx, ctx->ctx_allocs, &ctx->d_count, 1)) != CGKS_OK ||
       (s = dalloc(ctx, ctx->ctx_allocs, &ctx->d_skipped, 1)) != CGKS_OK ||
-      (s = dalloc(ctx, ctx->ctx_allocs, &ctx->nrm_part, 1024)) != CGKS_OK ||
+      (s = dalloc(ctx, ctx->ctx_allocs, &ctx->nrm_part, CGKS_NORM_PARTS)) != CGKS_OK ||
+      (s = dalloc(ctx, ctx->ctx_allocs, &ctx->nrm_done, 1)) != CGKS_OK ||
       (s = dalloc(ctx, ctx->ctx_allocs, &ctx->nrm, 1)) != CGKS_OK ||
       (s = upload_tables(ctx)) != CGKS_OK) {
     g_create_error = ctx->err;
@@ -552,7 +553,7 @@ cgks_status cgks_residual(cgks_ctx* ctx, int order, double* res, double* gradW_n
   cudaStream_t st = ctx->stream;
   if (order == 3) {
     CKS(fine_fluxes(ctx, ctx->W, ctx->G, ctx->alpha));
-    CKS(fine_gather(ctx, ctx->W, nullptr, ctx->res, gradW_new, alpha_new, 0));
+    CKS(fine_gather(ctx, ctx->W, nullptr, ctx->res, gradW_new, alpha_new, 0, norm ? ctx->nrm : nullptr));
     if (dt) CK(cudaMemcpyAsync(dt, ctx->dt, sizeof(double) * F.nc, cudaMemcpyDefault, st));
   } else if (order == 1) {
     CKS(kfvs_residual(ctx, 0, ctx->W, ctx->res));
@@ -563,7 +564,7 @@ cgks_status cgks_residual(cgks_ctx* ctx, int order, double* res, double* gradW_n
   }
   if (res) CK(cudaMemcpyAsync(res, ctx->res, sizeof(double) * 5 * F.nc, cudaMemcpyDefault, st));
   if (norm) {
-    CKS(density_norm(ctx, ctx->res, F.vol, F.nc, ctx->nrm));
+    if (order == 1) CKS(density_norm(ctx, ctx->res, F.vol, F.nc, ctx->nrm));
     CKS(read_norm(ctx, ctx->nrm, norm, 1));
   }
   return check_device_error(ctx, "cgks_residual");

@@ -557,9 +557,7 @@ static cgks_status coarse_cycle(cgks_ctx* ctx, int l) {
 cgks_status step_once(cgks_ctx* ctx, double* norm_dev) {
   CKS(fine_fluxes(ctx, ctx->W, ctx->G, ctx->alpha));
   // the gather reads only the Gauss-point records, so W, gradW and alpha are updated in place
-  CKS(fine_gather(ctx, ctx->W, ctx->W, ctx->res, ctx->G, ctx->alpha, 1));
-  if (norm_dev) CKS(density_norm(ctx, ctx->res, ctx->F.vol, ctx->F.nc, norm_dev));
-  return CGKS_OK;
+  return fine_gather(ctx, ctx->W, ctx->W, ctx->res, ctx->G, ctx->alpha, 1, norm_dev);
 }
 
 // one V-cycle (Sec. 4.2)

@@ -15,6 +15,7 @@
 #define CGKS_RC 50            // reconstruction coefficients per cell: 5 variables x 10
 #define CGKS_GPR 14           // Gauss-point record: flux x weight (5), interface state (5), area vector (3), alpha
 #define CGKS_AUX 8            // per-cell constants of the smoothness indicators
+#define CGKS_NORM_PARTS 1024  // per-block parts of a reduction (nrm_part)
 #define CGKS_AGG_CAP 256      // records per coarse cell while building coarse faces
 #define HD __host__ __device__ __forceinline__
 
@@ -135,6 +136,7 @@ struct cgks_ctx {
   double *ffl = nullptr;            // first-order face fluxes of level 0
   float* ffl32 = nullptr;           // their FP32 directional derivatives
   double *nrm_part = nullptr, *nrm = nullptr, *h_nrm = nullptr;
+  unsigned* nrm_done = nullptr;     // blocks of k_gather_vars that have written their part of the norm
   double* tab = nullptr;            // table of half_gauss (fastmath.cuh), built with the context
   DevErr* derr = nullptr;
   DevErr* h_err = nullptr;
@@ -235,8 +237,9 @@ cgks_status check_device_error(cgks_ctx* ctx, const char* where);
 // state false: the Gauss-point fluxes alone (no interface state, area or compression factor in the
 // records), for a residual-only gather
 cgks_status fine_fluxes(cgks_ctx* ctx, const double* W, const double* G, const double* alpha, bool state = true);
+// norm_dev: the norm of the density residual (null: not formed)
 cgks_status fine_gather(cgks_ctx* ctx, const double* W_in, double* W_out, double* res, double* G_out,
-                        double* alpha_out, int update);
+                        double* alpha_out, int update, double* norm_dev = nullptr);
 cgks_status density_norm(cgks_ctx* ctx, const double* res, const double* vol, int64_t n, double* out_dev);
 
 // first-order (KFVS) residual of a level; res may equal nullptr when only the face fluxes are needed
