@@ -6,9 +6,9 @@
 //   skewness  virtual centre C_c = (V_l C_l + V_r C_r)/(V_l + V_r); every face of L or R not between
 //             them must satisfy (d . S n)^2 >= skew_min^2 |d|^2 |S n|^2, d = face centre - C_c,
 //             evaluated with explicitly rounded IEEE operations (no FMA contraction);
-//   merging   greedy pairwise matching in ascending face order, computed by locally-dominant rounds
-//             (a confirmed face whose two cells are unmatched merges when it is the smallest such
-//             face at both cells), which selects exactly the faces of the sequential greedy pass;
+//   merging   greedy pairwise matching in ascending face order: a confirmed face merges its two cells when
+//             both are unmatched and it is the smallest such face of both (k_match), which selects exactly
+//             the faces of the sequential greedy pass;
 //   numbering coarse cells in the order of their smallest member; coarse faces one per
 //             (coarse L < coarse R, periodic side tag) ordered lexicographically, boundary faces one
 //             per (coarse cell, tag) after them; area vectors summed in ascending fine-face order.
@@ -92,66 +92,69 @@ __device__ bool skew_confirmed(const Level& P, const double* __restrict__ fx, in
   return true;
 }
 
-// confirmed faces into `list` (in any order; *n counts them): the winners of their hash buckets that pass the
-// skewness test
+// confirmed faces: the winners of their hash buckets that pass the skewness test
 __global__ void k_select_confirm(Level P, uint64_t seed, uint64_t nfc, const int32_t* bucket, const double* fx,
-                                 double kmin2, int32_t* list, int32_t* n) {
+                                 double kmin2, int8_t* conf) {
   const int64_t f = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (f >= P.nf) return;
-  if (is_candidate(P.fR, P.ftag, f) && bucket[face_hash(P.fL, P.fR, f, seed, nfc)] == (int32_t)f &&
-      skew_confirmed(P, fx, P.fL[f], P.fR[f], kmin2))
-    list[atomicAdd(n, 1)] = (int32_t)f;
+  int8_t ok = 0;
+  if (is_candidate(P.fR, P.ftag, f) && bucket[face_hash(P.fL, P.fR, f, seed, nfc)] == (int32_t)f)
+    ok = skew_confirmed(P, fx, P.fL[f], P.fR[f], kmin2) ? 1 : 0;
+  conf[f] = ok;
 }
 
-// Rounds of the greedy matching: in each, a live face (confirmed, both cells unmatched) that is the smallest
-// live face of both its cells merges them.  best[c] holds (rounds to go, face), so that a later round's
-// entries undercut an earlier one's and nothing is reset.  A round is two passes over the live faces,
-// propose and match; match drops the dead ones into the next round's list.  On meshes numbered along grid
-// lines a face waits for a chain of smaller ones, 20 to 150 rounds for a pass, so a round has to be cheap
-// and the host reads the count of live faces once for MATCH_ROUNDS of them.  (Per round 10 us against 15
-// over all cells and faces with a host read each, 64,000-cell box; finishing the long tail in one block
-// took 50 us per round.)
-#define MATCH_ROUNDS 16
+// Greedy matching in ascending face order, a thread per cell.  Every cell points at its smallest confirmed
+// face that is not known to be dead (its other cell merged elsewhere); a face at which both its cells point
+// merges them, and a cell whose face's other cell has merged elsewhere moves on.  A face is passed only
+// when dead and merged only when no smaller live one remains at either cell: the sequential pass's result,
+// whatever the order of the threads (each writes its own cell's entries; the other cell's only move
+// forward).  On meshes numbered along grid lines a decision waits for a chain of up to 150 others, so the
+// chain runs inside the kernel: a thread looks at its neighbour again, MATCH_POLLS times at most, and what
+// is undecided then goes on in the next launch.  (In rounds of two launches each step of the chain took 10
+// us; 211 of them on the 40x40x40 box.)
+#define MATCH_POLLS 512
 
-__device__ __forceinline__ unsigned long long match_key(int32_t round, int32_t f) {
-  return ((unsigned long long)(unsigned)(INT32_MAX - round) << 32) | (unsigned)f;
+__global__ void k_match_begin(Level P, const int8_t* __restrict__ conf, int32_t* __restrict__ pos,
+                              int32_t* __restrict__ cur) {
+  const int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (c >= P.nc) return;
+  int32_t k = P.c2f_ptr[c];
+  const int32_t e = P.c2f_ptr[c + 1];
+  while (k < e && !conf[P.c2f[k]]) ++k;
+  pos[c] = k;
+  cur[c] = k < e ? P.c2f[k] : -1;
 }
 
-__device__ __forceinline__ void match_propose(const Level& P, int32_t f, int32_t round, const int32_t* partner,
-                                              unsigned long long* best) {
-  const int32_t a = P.fL[f], b = P.fR[f];
-  if (partner[a] >= 0 || partner[b] >= 0) return;
-  const unsigned long long key = match_key(round, f);
-  atomicMin(&best[a], key);
-  atomicMin(&best[b], key);
-}
-
-// whether the face stays live
-__device__ __forceinline__ bool match_merge(const Level& P, int32_t f, int32_t round, int32_t* partner,
-                                            const unsigned long long* best) {
-  const int32_t a = P.fL[f], b = P.fR[f];
-  const unsigned long long key = match_key(round, f), ba = best[a], bb = best[b];
-  if (ba == key && bb == key) {
-    partner[a] = b;
-    partner[b] = a;
-    return false;
+__global__ void k_match(Level P, const int8_t* __restrict__ conf, int32_t* __restrict__ pos, int32_t* cur,
+                        int32_t* partner, unsigned long long* undecided) {
+  const int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (c >= P.nc) return;
+  volatile int32_t* const vcur = cur;
+  volatile int32_t* const vpartner = partner;
+  int32_t f = vcur[c];
+  if (f < 0 || vpartner[c] >= 0) return;
+  int32_t k = pos[c];
+  const int32_t e = P.c2f_ptr[c + 1];
+  int32_t o = P.fL[f] == c ? P.fR[f] : P.fL[f];
+  for (int poll = 0; poll < MATCH_POLLS; ++poll) {
+    const int32_t po = vpartner[o];
+    if (po == c || (po < 0 && vcur[o] == f)) {
+      vpartner[c] = o;
+      return;
+    }
+    if (po < 0) continue;  // the other cell still has a smaller face to decide
+    do ++k;
+    while (k < e && !conf[P.c2f[k]]);
+    if (k == e) {
+      vcur[c] = -1;
+      return;
+    }
+    f = P.c2f[k];
+    o = P.fL[f] == c ? P.fR[f] : P.fL[f];
+    vcur[c] = f;
   }
-  // dead: a cell was matched before this round's proposals (its entry is not of this round)
-  return (ba >> 32) == (key >> 32) && (bb >> 32) == (key >> 32);
-}
-
-__global__ void k_match_propose(Level P, const int32_t* list, const int32_t* n, int32_t round, const int32_t* partner,
-                                unsigned long long* best) {
-  for (int32_t k = blockIdx.x * blockDim.x + threadIdx.x; k < *n; k += gridDim.x * blockDim.x)
-    match_propose(P, list[k], round, partner, best);
-}
-
-__global__ void k_match_merge(Level P, const int32_t* list, const int32_t* n, int32_t round, int32_t* partner,
-                              const unsigned long long* best, int32_t* next, int32_t* nnext) {
-  for (int32_t k = blockIdx.x * blockDim.x + threadIdx.x; k < *n; k += gridDim.x * blockDim.x) {
-    const int32_t f = list[k];
-    if (match_merge(P, f, round, partner, best)) next[atomicAdd(nnext, 1)] = f;
-  }
+  pos[c] = k;
+  atomicAdd(undecided, 1ULL);
 }
 
 __global__ void k_rep_flag(int64_t nc, const int32_t* partner, int32_t* rep) {
@@ -401,39 +404,28 @@ static cgks_status coarsen_pass(cgks_ctx* ctx, const Level& P, Level& Q, int32_t
   CKS(dalloc(ctx, tmp, &cid, P.nc));
   CK(cudaMemsetAsync(partner, 0xFF, sizeof(int32_t) * P.nc, st));
   if (nfc > 0) {
-    int32_t *bucket, *list[2], *n;
-    unsigned long long* best;
+    int32_t *bucket, *pos, *cur;
+    int8_t* conf;
     double* fx;
     CKS(dalloc(ctx, tmp, &bucket, nfc));
-    CKS(dalloc(ctx, tmp, &list[0], nfc));
-    CKS(dalloc(ctx, tmp, &list[1], nfc));
-    CKS(dalloc(ctx, tmp, &n, MATCH_ROUNDS + 1));
-    CKS(dalloc(ctx, tmp, &best, P.nc));
+    CKS(dalloc(ctx, tmp, &pos, P.nc));
+    CKS(dalloc(ctx, tmp, &cur, P.nc));
+    CKS(dalloc(ctx, tmp, &conf, P.nf));
     CKS(dalloc(ctx, tmp, &fx, 3 * P.nf));
     CK(cudaMemsetAsync(bucket, 0x7F, sizeof(int32_t) * nfc, st));
-    CK(cudaMemsetAsync(best, 0xFF, sizeof(unsigned long long) * P.nc, st));
     k_bucket_min<<<grid_for(P.nf, B), B, 0, st>>>(P.nf, P.fL, P.fR, P.ftag, seed, (uint64_t)nfc, bucket);
     k_face_centres<<<grid_for(P.nf, B), B, 0, st>>>(P.nf, P.amom, P.area, fx);
     const double kmin2 = ctx->P.skew_min * ctx->P.skew_min;
-    k_select_confirm<<<grid_for(P.nf, 128), 128, 0, st>>>(P, seed, (uint64_t)nfc, bucket, fx, kmin2, list[0], n);
-    const unsigned gb = grid_for(nfc, B) < 2u * ctx->n_sm ? grid_for(nfc, B) : 2u * ctx->n_sm;
-    // every round with a live face merges at least the smallest one, so nfc rounds bound the loop
-    for (int64_t round = 0; round <= nfc; round += MATCH_ROUNDS) {
-      if (round > 0) {
-        int32_t live = 0;
-        CK(cudaMemcpyAsync(ctx->h_count, n + MATCH_ROUNDS, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
-        CK(cudaStreamSynchronize(st));
-        live = *reinterpret_cast<int32_t*>(ctx->h_count);
-        if (live == 0) break;
-        CK(cudaMemcpyAsync(n, n + MATCH_ROUNDS, sizeof(int32_t), cudaMemcpyDeviceToDevice, st));
-        CK(cudaMemsetAsync(n + 1, 0, sizeof(int32_t) * MATCH_ROUNDS, st));
-      }
-      for (int r = 0; r < MATCH_ROUNDS; ++r) {
-        const int32_t k = (int32_t)round + r;
-        k_match_propose<<<gb, B, 0, st>>>(P, list[r & 1], n + r, k, partner, best);
-        k_match_merge<<<gb, B, 0, st>>>(P, list[r & 1], n + r, k, partner, best, list[1 - (r & 1)], n + r + 1);
-      }
+    k_select_confirm<<<grid_for(P.nf, 128), 128, 0, st>>>(P, seed, (uint64_t)nfc, bucket, fx, kmin2, conf);
+    k_match_begin<<<grid_for(P.nc, B), B, 0, st>>>(P, conf, pos, cur);
+    // a launch decides at least the smallest live face or moves a cell on, so this bounds the loop
+    int64_t left = 1;
+    for (int64_t round = 0; left > 0 && round <= P.nf; ++round) {
+      CK(cudaMemsetAsync(ctx->d_count, 0, sizeof(int64_t), st));
+      k_match<<<grid_for(P.nc, 128), 128, 0, st>>>(P, conf, pos, cur, partner, (unsigned long long*)ctx->d_count);
+      CKS(read_count(ctx, &left));
     }
+    if (left > 0) return cgks_fail(ctx, CGKS_EMESH, "coarsening: the matching did not finish");
     CK(cudaGetLastError());
   }
   k_rep_flag<<<grid_for(P.nc, B), B, 0, st>>>(P.nc, partner, rep);

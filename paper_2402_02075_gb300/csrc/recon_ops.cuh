@@ -179,18 +179,21 @@ __host__ __device__ inline void recon_ops_body(int64_t i, const ROArgs& A_) {
     set_err(err, CGKS_EMESH, (int)i, 51);
     return;
   }
-  // P2 = (BQ2)^+ = Rb^{-1} Qb^T (nz x mb), column by column of the identity
-  double P2[5 * 18];
-  for (int col = 0; col < mb; ++col) {
-    double y[18];
+  // P2 = (BQ2)^+ = Rb^{-1} Qb^T (nz x mb): the first nz columns of Qb, then back substitution per row of
+  // Qb (forming all of Qb^T from the identity would take three times the operations)
+  double Qb[5 * 18];
+  for (int col = 0; col < nz; ++col) {
+    double* y = Qb + col * 18;
     for (int r = 0; r < mb; ++r) y[r] = r == col ? 1.0 : 0.0;
-    house_apply(mb, nz, BQ2, tb, y, true);
+    house_apply(mb, nz, BQ2, tb, y, false);
+  }
+  double P2[5 * 18];
+  for (int col = 0; col < mb; ++col)
     for (int r = nz - 1; r >= 0; --r) {
-      double s = y[r];
+      double s = Qb[r * 18 + col];
       for (int j = r + 1; j < nz; ++j) s -= BQ2[j * mb + r] * P2[col * 5 + j];
       P2[col * 5 + r] = s / BQ2[r * mb + r];
     }
-  }
   // Kg = Q2 P2 (9 x mb); KdQ = A1 - Kg (B A1) (9 x nt)
   double Kg[9 * 18];
   for (int col = 0; col < mb; ++col)
