@@ -56,7 +56,8 @@ __global__ void k_face_centres(int64_t nf, const double* __restrict__ amom, cons
   for (int e = 0; e < 3; ++e) fx[e * nf + f] = __ddiv_rn(amom[e * nf + f], area[f]);
 }
 
-__device__ bool skew_confirmed(const Level& P, const double* __restrict__ fx, int32_t a, int32_t b, double kmin2) {
+// whether the faces of cell x (one of the candidate's cells a, b) outside the pair pass the skewness limit
+__device__ bool skew_side(const Level& P, const double* __restrict__ fx, int32_t a, int32_t b, int32_t x, double kmin2) {
   const int64_t nc = P.nc, nf = P.nf;
   const double Va = P.vol[a], Vb = P.vol[b];
   const double Vs = __dadd_rn(Va, Vb);
@@ -64,43 +65,48 @@ __device__ bool skew_confirmed(const Level& P, const double* __restrict__ fx, in
 #pragma unroll
   for (int e = 0; e < 3; ++e)
     Cc[e] = __ddiv_rn(__dadd_rn(__dmul_rn(Va, P.ctr[e * nc + a]), __dmul_rn(Vb, P.ctr[e * nc + b])), Vs);
-  const int32_t cells[2] = {a, b};
-  for (int side = 0; side < 2; ++side) {
-    const int32_t x = cells[side];
-    for (int32_t k = P.c2f_ptr[x]; k < P.c2f_ptr[x + 1]; ++k) {
-      const int64_t g = P.c2f[k];
-      const int32_t gl = P.fL[g], gr = P.fR[g];
-      const bool inL = gl == a || gl == b, inR = gr == a || gr == b;
-      if (inL && inR) continue;
-      const bool asR = gr == x && gl != x;
-      double d[3], S[3];
+  for (int32_t k = P.c2f_ptr[x]; k < P.c2f_ptr[x + 1]; ++k) {
+    const int64_t g = P.c2f[k];
+    const int32_t gl = P.fL[g], gr = P.fR[g];
+    const bool inL = gl == a || gl == b, inR = gr == a || gr == b;
+    if (inL && inR) continue;
+    const bool asR = gr == x && gl != x;
+    double d[3], S[3];
 #pragma unroll
-      for (int e = 0; e < 3; ++e) {
-        double xg = fx[e * nf + g];
-        if (asR) xg = __dsub_rn(xg, P.shift[e * nf + g]);
-        d[e] = __dsub_rn(xg, Cc[e]);
-        S[e] = P.Sn[e * nf + g];
-      }
-      const double dn = __dadd_rn(__dadd_rn(__dmul_rn(d[0], S[0]), __dmul_rn(d[1], S[1])), __dmul_rn(d[2], S[2]));
-      const double dd = __dadd_rn(__dadd_rn(__dmul_rn(d[0], d[0]), __dmul_rn(d[1], d[1])), __dmul_rn(d[2], d[2]));
-      const double ss = __dadd_rn(__dadd_rn(__dmul_rn(S[0], S[0]), __dmul_rn(S[1], S[1])), __dmul_rn(S[2], S[2]));
-      const double lhs = __dmul_rn(dn, dn);
-      const double rhs = __dmul_rn(__dmul_rn(kmin2, dd), ss);
-      if (!(lhs >= rhs)) return false;
+    for (int e = 0; e < 3; ++e) {
+      double xg = fx[e * nf + g];
+      if (asR) xg = __dsub_rn(xg, P.shift[e * nf + g]);
+      d[e] = __dsub_rn(xg, Cc[e]);
+      S[e] = P.Sn[e * nf + g];
     }
+    const double dn = __dadd_rn(__dadd_rn(__dmul_rn(d[0], S[0]), __dmul_rn(d[1], S[1])), __dmul_rn(d[2], S[2]));
+    const double dd = __dadd_rn(__dadd_rn(__dmul_rn(d[0], d[0]), __dmul_rn(d[1], d[1])), __dmul_rn(d[2], d[2]));
+    const double ss = __dadd_rn(__dadd_rn(__dmul_rn(S[0], S[0]), __dmul_rn(S[1], S[1])), __dmul_rn(S[2], S[2]));
+    const double lhs = __dmul_rn(dn, dn);
+    const double rhs = __dmul_rn(__dmul_rn(kmin2, dd), ss);
+    if (!(lhs >= rhs)) return false;
   }
   return true;
 }
 
-// confirmed faces: the winners of their hash buckets that pass the skewness test
-__global__ void k_select_confirm(Level P, uint64_t seed, uint64_t nfc, const int32_t* bucket, const double* fx,
-                                 double kmin2, int8_t* conf) {
+// winners of the hash buckets into `list` (in any order; *n counts them), so that the skewness test runs on
+// full warps
+__global__ void k_winners(Level P, uint64_t seed, uint64_t nfc, const int32_t* bucket, int32_t* list, int32_t* n) {
   const int64_t f = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (f >= P.nf) return;
-  int8_t ok = 0;
-  if (is_candidate(P.fR, P.ftag, f) && bucket[face_hash(P.fL, P.fR, f, seed, nfc)] == (int32_t)f)
-    ok = skew_confirmed(P, fx, P.fL[f], P.fR[f], kmin2) ? 1 : 0;
-  conf[f] = ok;
+  if (f < P.nf && is_candidate(P.fR, P.ftag, f) && bucket[face_hash(P.fL, P.fR, f, seed, nfc)] == (int32_t)f)
+    list[atomicAdd(n, 1)] = (int32_t)f;
+}
+
+// confirmed faces: the winners that pass the skewness test, two threads per face (its two cells)
+__global__ void k_confirm(Level P, const int32_t* __restrict__ list, const int32_t* n, const double* fx, double kmin2,
+                          int8_t* conf) {
+  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  const bool live = t < 2 * (int64_t)*n;
+  const int32_t f = live ? list[t >> 1] : 0;
+  const int32_t a = P.fL[f], b = P.fR[f];
+  const int ok = live && skew_side(P, fx, a, b, t & 1 ? b : a, kmin2);
+  const int both = ok & __shfl_xor_sync(0xffffffffu, ok, 1);
+  if (live && both && !(t & 1)) conf[f] = 1;
 }
 
 // Greedy matching in ascending face order, a thread per cell.  Every cell points at its smallest confirmed
@@ -404,19 +410,22 @@ static cgks_status coarsen_pass(cgks_ctx* ctx, const Level& P, Level& Q, int32_t
   CKS(dalloc(ctx, tmp, &cid, P.nc));
   CK(cudaMemsetAsync(partner, 0xFF, sizeof(int32_t) * P.nc, st));
   if (nfc > 0) {
-    int32_t *bucket, *pos, *cur;
+    int32_t *bucket, *pos, *cur, *list, *n;
     int8_t* conf;
     double* fx;
     CKS(dalloc(ctx, tmp, &bucket, nfc));
     CKS(dalloc(ctx, tmp, &pos, P.nc));
     CKS(dalloc(ctx, tmp, &cur, P.nc));
     CKS(dalloc(ctx, tmp, &conf, P.nf));
+    CKS(dalloc(ctx, tmp, &list, nfc));
+    CKS(dalloc(ctx, tmp, &n, 1));
     CKS(dalloc(ctx, tmp, &fx, 3 * P.nf));
     CK(cudaMemsetAsync(bucket, 0x7F, sizeof(int32_t) * nfc, st));
     k_bucket_min<<<grid_for(P.nf, B), B, 0, st>>>(P.nf, P.fL, P.fR, P.ftag, seed, (uint64_t)nfc, bucket);
     k_face_centres<<<grid_for(P.nf, B), B, 0, st>>>(P.nf, P.amom, P.area, fx);
     const double kmin2 = ctx->P.skew_min * ctx->P.skew_min;
-    k_select_confirm<<<grid_for(P.nf, 128), 128, 0, st>>>(P, seed, (uint64_t)nfc, bucket, fx, kmin2, conf);
+    k_winners<<<grid_for(P.nf, B), B, 0, st>>>(P, seed, (uint64_t)nfc, bucket, list, n);
+    k_confirm<<<grid_for(2 * nfc, 128), 128, 0, st>>>(P, list, n, fx, kmin2, conf);
     k_match_begin<<<grid_for(P.nc, B), B, 0, st>>>(P, conf, pos, cur);
     // a launch decides at least the smallest live face or moves a cell on, so this bounds the loop
     int64_t left = 1;
