@@ -42,17 +42,21 @@ HD void vjp_point_body(int64_t g, const VjpArgs& a) {
   const double A[3] = {a.gp_A[g], a.gp_A[ngp + g], a.gp_A[2 * ngp + g]};
   // the left cell takes -flux and +A x state / |Omega|; the right cell the opposite
   double ub[10];
-  const double rvL = 1.0 / a.vol[L], rvR = R >= 0 ? 1.0 / a.vol[R] : 0.0;
+  // (the FP64 pipe bounds this kernel: 410 multiply-adds per point, and 60 here instead of 75)
+  const double rvL = fast_rcp(a.vol[L]), rvR = R >= 0 ? fast_rcp(a.vol[R]) : 0.0;
 #pragma unroll
   for (int q = 0; q < 5; ++q) {
-    ub[q] = -a.rbar[q * nc + L] + (R >= 0 ? a.rbar[q * nc + R] : 0.0);
-    double s = 0.0;
-#pragma unroll
-    for (int d = 0; d < 3; ++d)
-      s += A[d] * (a.gbar[(3 * q + d) * nc + L] * rvL - (R >= 0 ? a.gbar[(3 * q + d) * nc + R] * rvR : 0.0));
+    double u = -a.rbar[q * nc + L];
+    double s = rvL * (A[0] * a.gbar[(3 * q) * nc + L] + A[1] * a.gbar[(3 * q + 1) * nc + L] + A[2] * a.gbar[(3 * q + 2) * nc + L]);
+    if (R >= 0) {
+      u += a.rbar[q * nc + R];
+      s -= rvR * (A[0] * a.gbar[(3 * q) * nc + R] + A[1] * a.gbar[(3 * q + 1) * nc + R] + A[2] * a.gbar[(3 * q + 2) * nc + R]);
+    }
+    ub[q] = u;
     ub[5 + q] = s;
   }
   for (int k = 0; k < CGKS_PJ_IN; ++k) {
+    if (R < 0 && k >= 20 && k < 40) continue;  // no right side (and no reader of its cotangents)
     const double* J = a.Jp + (int64_t)(CGKS_PJ_OUT * k) * ngp + g;
     double s = 0.0;
 #pragma unroll
