@@ -244,29 +244,38 @@ __global__ void k_fe_update(int64_t nc, const double* __restrict__ dt, const dou
 
 // coarse state = sum V_i W_i / V_c (and its copy W^0) and coarse defect = sum (R_i [+ F_i]) over the
 // finer cells of each coarse cell, in ascending finer-cell order
+// (a thread per coarse cell and variable: an agglomerate has a handful of members, so the time of a small
+// launch is that of the dependent loads of one thread; four members are in flight at once)
 __global__ void k_restrict(int64_t ncc, int64_t ncf, const int32_t* __restrict__ aptr, const int32_t* __restrict__ agg,
                            const double* __restrict__ vf, const double* __restrict__ vc, const double* __restrict__ Wf,
                            const double* __restrict__ Rf, const double* __restrict__ Ff, double* __restrict__ Wc,
                            double* __restrict__ Wc0, double* __restrict__ Rc) {
   const int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  const int q = blockIdx.y;
   if (c >= ncc) return;
-  double w[5] = {0, 0, 0, 0, 0}, r[5] = {0, 0, 0, 0, 0};
-  for (int32_t k = aptr[c]; k < aptr[c + 1]; ++k) {
-    const int64_t i = agg[k];
-    const double v = vf[i];
+  double w = 0.0, r = 0.0;
+  const int32_t e = aptr[c + 1];
+  for (int32_t k = aptr[c]; k < e; k += 4) {
+    double v[4], x[4], y[4], z[4];
 #pragma unroll
-    for (int q = 0; q < 5; ++q) {
-      w[q] += v * Wf[q * ncf + i];
-      r[q] += Ff ? Rf[q * ncf + i] + Ff[q * ncf + i] : Rf[q * ncf + i];
+    for (int j = 0; j < 4; ++j) {
+      const int64_t i = agg[k + j < e ? k + j : e - 1];
+      v[j] = vf[i];
+      x[j] = Wf[q * ncf + i];
+      y[j] = Rf[q * ncf + i];
+      z[j] = Ff ? Ff[q * ncf + i] : 0.0;
     }
-  }
-  const double rv = 1.0 / vc[c];
 #pragma unroll
-  for (int q = 0; q < 5; ++q) {
-    Wc[q * ncc + c] = w[q] *= rv;
-    Wc0[q * ncc + c] = w[q];
-    Rc[q * ncc + c] = r[q];
+    for (int j = 0; j < 4; ++j)
+      if (k + j < e) {
+        w += v[j] * x[j];
+        r += Ff ? y[j] + z[j] : y[j];
+      }
   }
+  w *= 1.0 / vc[c];
+  Wc[q * ncc + c] = w;
+  Wc0[q * ncc + c] = w;
+  Rc[q * ncc + c] = r;
 }
 
 // W_f += r (W_c - W_c^0) (injection, r = correction_relax); a correction that would make rho or p
@@ -542,7 +551,7 @@ static cgks_status coarse_cycle(cgks_ctx* ctx, int l) {
     CKS(coarse_residual(ctx, l));
     {
       ProfScope ps(ctx, PK_RESTRICT, (double)L.nc, L.nc * 132.0 + Cn.nc * 132.0);
-      k_restrict<<<grid_for(Cn.nc, 256), 256, 0, st>>>(Cn.nc, L.nc, Cn.agg_ptr, Cn.agg, L.vol, Cn.vol, B.W, B.R,
+      k_restrict<<<dim3(grid_for(Cn.nc, 128), 5), 128, 0, st>>>(Cn.nc, L.nc, Cn.agg_ptr, Cn.agg, L.vol, Cn.vol, B.W, B.R,
                                                        forcing(ctx, B), N.W, N.W0, N.Rs);
     }
     CKS(coarse_cycle(ctx, l + 1));
@@ -575,7 +584,7 @@ cgks_status vcycle_once(cgks_ctx* ctx, double* norm_dev) {
   CKS(fine_gather(ctx, ctx->W, nullptr, ctx->res, nullptr, nullptr, 0));
   {
     ProfScope ps(ctx, PK_RESTRICT, (double)F.nc, F.nc * 92.0 + C1.nc * 132.0);
-    k_restrict<<<grid_for(C1.nc, 256), 256, 0, st>>>(C1.nc, F.nc, C1.agg_ptr, C1.agg, ctx->L0c.vol, C1.vol, ctx->W,
+    k_restrict<<<dim3(grid_for(C1.nc, 128), 5), 128, 0, st>>>(C1.nc, F.nc, C1.agg_ptr, C1.agg, ctx->L0c.vol, C1.vol, ctx->W,
                                                      ctx->res, nullptr, B1.W, B1.W0, B1.Rs);
   }
   CKS(coarse_cycle(ctx, 1));
