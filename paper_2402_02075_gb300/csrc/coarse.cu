@@ -8,25 +8,27 @@
 // KFVS face fluxes x area (FP64)
 __global__ void k_kfvs_faces(int64_t nf, const int32_t* __restrict__ fL, const int32_t* __restrict__ fR,
                              const int32_t* __restrict__ ftag, const double* __restrict__ nS, int64_t nc,
-                             const double* __restrict__ W, double* __restrict__ ff, Phys ph, DevErr* err,
-                             const double* __restrict__ tab) {
+                             const double* W, double* ff, Phys ph, DevErr* err, const double* __restrict__ tab) {
   const int64_t f = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (f >= nf) return;
-  const double s = nS[3 * nf + f];
+  const bool live = f < nf;
+  const double s = live ? nS[3 * nf + f] : 0.0;
+  const double n[3] = {live ? nS[f] : 0.0, live ? nS[nf + f] : 0.0, live ? nS[2 * nf + f] : 0.0};
+  const int64_t L = live ? fL[f] : 0, R = live ? fR[f] : 0;
+  const int32_t tag = live && R < 0 ? ftag[f] : 0;
+  wait_prior();
+  if (!live) return;
   if (s == 0.0) {  // a coarse face whose summed area vectors cancel carries no flux
 #pragma unroll
     for (int q = 0; q < 5; ++q) ff[q * nf + f] = 0.0;
     return;
   }
-  const double n[3] = {nS[f], nS[nf + f], nS[2 * nf + f]};
-  const int64_t L = fL[f], R = fR[f];
   double WL[5], WR[5], F[5];
 #pragma unroll
   for (int q = 0; q < 5; ++q) WL[q] = W[q * nc + L];
   if (R >= 0) {
 #pragma unroll
     for (int q = 0; q < 5; ++q) WR[q] = W[q * nc + R];
-  } else if (!bc_ghost<double>(ftag[f], n, WL, nullptr, WR, nullptr, ph.gamma, ph.Winf)) {
+  } else if (!bc_ghost<double>(tag, n, WL, nullptr, WR, nullptr, ph.gamma, ph.Winf)) {
     set_err(err, CGKS_ENAN, (int)L, 20);
   }
   if (!kfvs_flux<double>(WL, WR, n, ph.K, ph.gamma - 1.0, F, tab)) set_err(err, CGKS_ENAN, (int)L, 21);
@@ -39,9 +41,9 @@ __global__ void k_kfvs_faces(int64_t nf, const int32_t* __restrict__ fL, const i
 // differentiated with the cell state it is built from.
 __global__ void k_kfvs_jvp_faces(int64_t nf, const int32_t* __restrict__ fL, const int32_t* __restrict__ fR,
                                  const int32_t* __restrict__ ftag, const double* __restrict__ Sn, int64_t nc,
-                                 const double* __restrict__ W0, const double* __restrict__ X, int x_is_state,
-                                 float* __restrict__ ff, Phys ph, DevErr* err) {
+                                 const double* W0, const double* X, int x_is_state, float* ff, Phys ph, DevErr* err) {
   using D = Dual<float>;
+  wait_prior();
   const int64_t f = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (f >= nf) return;
   const float S[3] = {float(Sn[f]), float(Sn[nf + f]), float(Sn[2 * nf + f])};
@@ -93,14 +95,16 @@ __device__ __forceinline__ double lane_sum(double v) {
 // res = -(sum of outward face fluxes) in FP64
 template <typename T, int LANES>
 __global__ void k_kfvs_gather(int64_t nc, int64_t nf, const int32_t* __restrict__ ptr, const int32_t* __restrict__ c2f,
-                              const int32_t* __restrict__ fL, const int32_t* __restrict__ fR,
-                              const T* __restrict__ ff, double* __restrict__ res) {
+                              const int32_t* __restrict__ fL, const int32_t* __restrict__ fR, const T* ff,
+                              double* res) {
   const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, c = t / LANES;
   const int sub = (int)(t % LANES);
   const bool live = c < nc;
   double r[5] = {0, 0, 0, 0, 0};
   const int32_t e = live ? ptr[c + 1] : 0;
-  for (int32_t k = live ? ptr[c] + sub : 0; k < e; k += LANES) {
+  int32_t k = live ? ptr[c] + sub : 0;
+  wait_prior();
+  for (; k < e; k += LANES) {
     const int64_t f = c2f[k];
     const int32_t a = fL[f], b = fR[f];
     if (a == b) continue;  // a cell's periodic image of itself: the two sides cancel
@@ -130,8 +134,8 @@ __device__ __forceinline__ double coarse_sound(const double w[5], double gamma, 
 template <int LANES>
 __global__ void k_coarse_dt(int64_t nc, int64_t nf, const int32_t* __restrict__ ptr, const int32_t* __restrict__ c2f,
                             const double* __restrict__ nS, const double* __restrict__ area,
-                            const double* __restrict__ vol, const double* __restrict__ W,
-                            double* __restrict__ dt, double gamma, double cfl) {
+                            const double* __restrict__ vol, const double* W, double* dt, double gamma, double cfl) {
+  wait_prior();
   const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, c = t / LANES;
   const int sub = (int)(t % LANES);
   const bool live = c < nc;
@@ -168,28 +172,49 @@ struct CoarseStep {
   DevErr* err;
 };
 
+// what the step needs of face entry k of cell c from the mesh alone
+struct StepFace {
+  int64_t f;
+  int32_t l, r;
+  double n[3], area;
+};
+
+template <bool GATHER>
+__device__ __forceinline__ StepFace step_face(const CoarseStep& a, int32_t k, int32_t e) {
+  StepFace F{};
+  if (k >= e) return F;
+  F.f = a.c2f[k];
+#pragma unroll
+  for (int d = 0; d < 3; ++d) F.n[d] = a.nS[d * a.nf + F.f];
+  F.area = a.area[F.f];
+  if (GATHER) F.l = a.fL[F.f], F.r = a.fR[F.f];
+  return F;
+}
+
 template <typename T, int LANES, bool GATHER>
-__global__ void k_coarse_step(CoarseStep a, const T* __restrict__ ff) {
+__global__ void k_coarse_step(CoarseStep a, const T* ff) {
   const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, c = t / LANES;
   const int64_t nc = a.nc, nf = a.nf;
   const int sub = (int)(t % LANES);
   const bool live = c < nc;
   double w[5], u[3], s = 0.0, r[5] = {0, 0, 0, 0, 0};
+  const int32_t e = live ? a.ptr[c + 1] : 0;
+  int32_t k = live ? a.ptr[c] + sub : 0;
+  StepFace F = step_face<GATHER>(a, k, e);
+  wait_prior();
 #pragma unroll
   for (int q = 0; q < 5; ++q) w[q] = live ? a.W[q * nc + c] : 1.0;
   const double snd = coarse_sound(w, a.gamma, u);
-  const int32_t e = live ? a.ptr[c + 1] : 0;
-  for (int32_t k = live ? a.ptr[c] + sub : 0; k < e; k += LANES) {
-    const int64_t f = a.c2f[k];
-    const double un = fabs(u[0] * a.nS[f] + u[1] * a.nS[nf + f] + u[2] * a.nS[2 * nf + f]);
-    s += a.area[f] * (un + snd);
-    if (GATHER) {
-      const int32_t l = a.fL[f];
-      if (l == a.fR[f]) continue;  // a cell's periodic image of itself
-      const double sg = l == c ? 1.0 : -1.0;
+  while (k < e) {
+    k += LANES;
+    const StepFace next = step_face<GATHER>(a, k, e);
+    s += F.area * (fabs(u[0] * F.n[0] + u[1] * F.n[1] + u[2] * F.n[2]) + snd);
+    if (GATHER && F.l != F.r) {  // not a cell's periodic image of itself
+      const double sg = F.l == c ? 1.0 : -1.0;
 #pragma unroll
-      for (int q = 0; q < 5; ++q) r[q] -= sg * (double)ff[q * nf + f];
+      for (int q = 0; q < 5; ++q) r[q] -= sg * (double)ff[q * nf + F.f];
     }
+    F = next;
   }
   s = lane_sum<LANES>(s);
   if (GATHER)
@@ -215,7 +240,8 @@ __global__ void k_coarse_step(CoarseStep a, const T* __restrict__ ff) {
 }
 
 // F = Rs - R  (FAS forcing term)
-__global__ void k_forcing(int64_t n5, const double* __restrict__ Rs, const double* __restrict__ R, double* __restrict__ F) {
+__global__ void k_forcing(int64_t n5, const double* Rs, const double* R, double* F) {
+  wait_prior();
   const int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (j < n5) F[j] = Rs[j] - R[j];
 }
@@ -247,15 +273,17 @@ __global__ void k_fe_update(int64_t nc, const double* __restrict__ dt, const dou
 // (a thread per coarse cell and variable: an agglomerate has a handful of members, so the time of a small
 // launch is that of the dependent loads of one thread; four members are in flight at once)
 __global__ void k_restrict(int64_t ncc, int64_t ncf, const int32_t* __restrict__ aptr, const int32_t* __restrict__ agg,
-                           const double* __restrict__ vf, const double* __restrict__ vc, const double* __restrict__ Wf,
-                           const double* __restrict__ Rf, const double* __restrict__ Ff, double* __restrict__ Wc,
-                           double* __restrict__ Wc0, double* __restrict__ Rc) {
+                           const double* __restrict__ vf, const double* __restrict__ vc, const double* Wf,
+                           const double* Rf, const double* Ff, double* Wc, double* Wc0, double* Rc) {
   const int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   const int q = blockIdx.y;
-  if (c >= ncc) return;
+  const bool live = c < ncc;
   double w = 0.0, r = 0.0;
-  const int32_t e = aptr[c + 1];
-  for (int32_t k = aptr[c]; k < e; k += 4) {
+  const int32_t e = live ? aptr[c + 1] : 0, k0 = live ? aptr[c] : 0;
+  const double rv = live ? 1.0 / vc[c] : 0.0;
+  wait_prior();
+  if (!live) return;
+  for (int32_t k = k0; k < e; k += 4) {
     double v[4], x[4], y[4], z[4];
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
@@ -272,7 +300,7 @@ __global__ void k_restrict(int64_t ncc, int64_t ncf, const int32_t* __restrict__
         r += Ff ? y[j] + z[j] : y[j];
       }
   }
-  w *= 1.0 / vc[c];
+  w *= rv;
   Wc[q * ncc + c] = w;
   Wc0[q * ncc + c] = w;
   Rc[q * ncc + c] = r;
@@ -280,12 +308,12 @@ __global__ void k_restrict(int64_t ncc, int64_t ncf, const int32_t* __restrict__
 
 // W_f += r (W_c - W_c^0) (injection, r = correction_relax); a correction that would make rho or p
 // non-positive is skipped
-__global__ void k_prolong(int64_t ncf, int64_t ncc, const int32_t* __restrict__ f2c, const double* __restrict__ Wc,
-                          const double* __restrict__ Wc0, double* __restrict__ Wf, double gamma, double relax,
-                          unsigned long long* skipped) {
+__global__ void k_prolong(int64_t ncf, int64_t ncc, const int32_t* __restrict__ f2c, const double* Wc,
+                          const double* Wc0, double* Wf, double gamma, double relax, unsigned long long* skipped) {
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  const int64_t c = i < ncf ? f2c[i] : 0;
+  wait_prior();
   if (i >= ncf) return;
-  const int64_t c = f2c[i];
   double w[5];
 #pragma unroll
   for (int q = 0; q < 5; ++q) w[q] = Wf[q * ncf + i] + relax * (Wc[q * ncc + c] - Wc0[q * ncc + c]);
@@ -337,7 +365,7 @@ __global__ void k_prolong_smooth(int64_t ncf, int64_t ncc, const int32_t* __rest
   }
 }
 
-static void prolong(cgks_ctx* ctx, int lev_fine, const int32_t* f2c, int64_t ncc, const double* Wc,
+static cgks_status prolong(cgks_ctx* ctx, int lev_fine, const int32_t* f2c, int64_t ncc, const double* Wc,
                     const double* Wc0, double* Wf) {
   const Level& L = ctx->L[lev_fine];
   cudaStream_t st = ctx->stream;
@@ -349,15 +377,16 @@ static void prolong(cgks_ctx* ctx, int lev_fine, const int32_t* f2c, int64_t ncc
                                                            Wf, ctx->P.gamma, ctx->P.correction_relax,
                                                            (unsigned long long*)ctx->d_skipped);
   else
-    k_prolong<<<grid_for(L.nc, 256), 256, 0, st>>>(L.nc, ncc, f2c, Wc, Wc0, Wf, ctx->P.gamma, ctx->P.correction_relax,
-                                                   (unsigned long long*)ctx->d_skipped);
+    CK(launch_overlapped(k_prolong, grid_for(L.nc, 256), 256, st, L.nc, ncc, f2c, Wc, Wc0, Wf,
+                         ctx->P.gamma, ctx->P.correction_relax, (unsigned long long*)ctx->d_skipped));
+  return CGKS_OK;
 }
 
 // sqrt(mean (res_rho / V)^2): per-block partial sums, then one warp adds them in a fixed order (lane l the
 // partials l, l + 32, ..., then a tree): 2 us where one thread's chain of 304 loads and additions took 22
-__global__ void k_norm_partial(int64_t n, const double* __restrict__ res, const double* __restrict__ vol,
-                               double* __restrict__ part) {
+__global__ void k_norm_partial(int64_t n, const double* res, const double* __restrict__ vol, double* part) {
   __shared__ double s[256];
+  wait_prior();
   double acc = 0.0;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
     const double x = res[i] / vol[i];
@@ -372,8 +401,8 @@ __global__ void k_norm_partial(int64_t n, const double* __restrict__ res, const 
   if (threadIdx.x == 0) part[blockIdx.x] = s[0];
 }
 
-__global__ void __launch_bounds__(32) k_norm_final(int nparts, int64_t n, const double* __restrict__ part,
-                                                   double* __restrict__ out) {
+__global__ void __launch_bounds__(32) k_norm_final(int nparts, int64_t n, const double* part, double* out) {
+  wait_prior();
   double s = 0.0;
   for (int k = threadIdx.x; k < nparts; k += 32) s += part[k];
 #pragma unroll
@@ -384,8 +413,8 @@ __global__ void __launch_bounds__(32) k_norm_final(int nparts, int64_t n, const 
 cgks_status density_norm(cgks_ctx* ctx, const double* res, const double* vol, int64_t n, double* out_dev) {
   const int parts = 304;
   ProfScope ps(ctx, PK_NORM, (double)n, n * 16.0);
-  k_norm_partial<<<parts, 256, 0, ctx->stream>>>(n, res, vol, ctx->nrm_part);
-  k_norm_final<<<1, 32, 0, ctx->stream>>>(parts, n, ctx->nrm_part, out_dev);
+  CK(launch_overlapped(k_norm_partial, parts, 256, ctx->stream, n, res, vol, ctx->nrm_part));
+  CK(launch_overlapped(k_norm_final, 1, 32, ctx->stream, parts, n, ctx->nrm_part, out_dev));
   CK(cudaGetLastError());
   return CGKS_OK;
 }
@@ -393,46 +422,52 @@ cgks_status density_norm(cgks_ctx* ctx, const double* res, const double* vol, in
 cgks_status global_min_dt(cgks_ctx* ctx, double* dt, int64_t n);
 
 // KFVS face fluxes of level `lev` (FP64)
-static void kfvs_fluxes(cgks_ctx* ctx, int lev, const double* W) {
+static cgks_status kfvs_fluxes(cgks_ctx* ctx, int lev, const double* W) {
   const Level& L = ctx->L[lev];
   double* ff = lev == 0 ? ctx->ffl : ctx->C[lev].ff;
   ProfScope ps(ctx, PK_KFVS_FACES, (double)L.nf, L.nf * 84.0 + L.nc * 40.0);
   const int b = spread_block(L.nf, 256, ctx->n_sm);
-  k_kfvs_faces<<<grid_for(L.nf, b), b, 0, ctx->stream>>>(L.nf, L.fL, L.fR, L.ftag, L.nS, L.nc, W, ff,
-                                                         make_phys(ctx->P), ctx->derr, ctx->tab);
+  CK(launch_overlapped(k_kfvs_faces, grid_for(L.nf, b), b, ctx->stream, L.nf, L.fL, L.fR, L.ftag, L.nS, L.nc, W, ff,
+                       make_phys(ctx->P), ctx->derr, ctx->tab));
+  return CGKS_OK;
 }
 
 // their FP32 directional derivatives at W0
-static void kfvs_jvp_fluxes(cgks_ctx* ctx, int lev, const double* W0, const double* X, int x_is_state) {
+static cgks_status kfvs_jvp_fluxes(cgks_ctx* ctx, int lev, const double* W0, const double* X, int x_is_state) {
   const Level& L = ctx->L[lev];
   float* ff = lev == 0 ? ctx->ffl32 : ctx->C[lev].ff32;
   ProfScope ps(ctx, PK_KFVS_JVP, (double)L.nf, L.nf * 56.0 + L.nc * 80.0);
-  k_kfvs_jvp_faces<<<grid_for(L.nf, 256), 256, 0, ctx->stream>>>(L.nf, L.fL, L.fR, L.ftag, L.Sn, L.nc, W0, X, x_is_state,
-                                                                 ff, make_phys(ctx->P), ctx->derr);
+  CK(launch_overlapped(k_kfvs_jvp_faces, grid_for(L.nf, 256), 256,
+                       ctx->stream, L.nf, L.fL, L.fR, L.ftag, L.Sn, L.nc, W0, X, x_is_state, ff,
+                       make_phys(ctx->P), ctx->derr));
+  return CGKS_OK;
 }
 
 template <typename T>
-static void kfvs_gather(cgks_ctx* ctx, int lev, const T* ff, double* res) {
+static cgks_status kfvs_gather(cgks_ctx* ctx, int lev, const T* ff, double* res) {
   const Level& L = ctx->L[lev];
   ProfScope ps(ctx, PK_KFVS_GATHER, (double)L.nc,
                L.nc * 44.0 + (L.nf + L.n_int + L.n_per) * 4.0 + L.nf * (8.0 + 5.0 * sizeof(T)));
   if (cell_lanes(L.nc, ctx->n_sm) == 8)
-    k_kfvs_gather<T, 8><<<grid_for(8 * L.nc, 64), 64, 0, ctx->stream>>>(L.nc, L.nf, L.c2f_ptr, L.c2f, L.fL, L.fR, ff, res);
+    CK(launch_overlapped(k_kfvs_gather<T, 8>, grid_for(8 * L.nc, 64), 64,
+                         ctx->stream, L.nc, L.nf, L.c2f_ptr, L.c2f, L.fL, L.fR, ff, res));
   else
-    k_kfvs_gather<T, 1><<<grid_for(L.nc, 256), 256, 0, ctx->stream>>>(L.nc, L.nf, L.c2f_ptr, L.c2f, L.fL, L.fR, ff, res);
+    CK(launch_overlapped(k_kfvs_gather<T, 1>, grid_for(L.nc, 256), 256,
+                         ctx->stream, L.nc, L.nf, L.c2f_ptr, L.c2f, L.fL, L.fR, ff, res));
+  return CGKS_OK;
 }
 
 // KFVS residual of level `lev` (FP64)
 cgks_status kfvs_residual(cgks_ctx* ctx, int lev, const double* W, double* res) {
-  kfvs_fluxes(ctx, lev, W);
-  kfvs_gather<double>(ctx, lev, lev == 0 ? ctx->ffl : ctx->C[lev].ff, res);
+  CKS(kfvs_fluxes(ctx, lev, W));
+  CKS(kfvs_gather<double>(ctx, lev, lev == 0 ? ctx->ffl : ctx->C[lev].ff, res));
   CK(cudaGetLastError());
   return CGKS_OK;
 }
 
 cgks_status kfvs_jvp(cgks_ctx* ctx, int lev, const double* W0, const double* X, int x_is_state, double* res) {
-  kfvs_jvp_fluxes(ctx, lev, W0, X, x_is_state);
-  kfvs_gather<float>(ctx, lev, lev == 0 ? ctx->ffl32 : ctx->C[lev].ff32, res);
+  CKS(kfvs_jvp_fluxes(ctx, lev, W0, X, x_is_state));
+  CKS(kfvs_gather<float>(ctx, lev, lev == 0 ? ctx->ffl32 : ctx->C[lev].ff32, res));
   CK(cudaGetLastError());
   return CGKS_OK;
 }
@@ -442,11 +477,13 @@ cgks_status coarse_dt(cgks_ctx* ctx, int lev, const double* W, double* dt) {
   {
     ProfScope ps(ctx, PK_COARSE_DT, (double)L.nc, L.nc * 60.0 + (L.nf + L.n_int + L.n_per) * 4.0 + L.nf * 32.0);
     if (cell_lanes(L.nc, ctx->n_sm) == 8)
-      k_coarse_dt<8><<<grid_for(8 * L.nc, 64), 64, 0, ctx->stream>>>(L.nc, L.nf, L.c2f_ptr, L.c2f, L.nS, L.area, L.vol, W,
-                                                                     dt, ctx->P.gamma, ctx->P.cfl_coarse);
+      CK(launch_overlapped(k_coarse_dt<8>, grid_for(8 * L.nc, 64), 64,
+                           ctx->stream, L.nc, L.nf, L.c2f_ptr, L.c2f, L.nS, L.area, L.vol, W, dt, ctx->P.gamma,
+                           ctx->P.cfl_coarse));
     else
-      k_coarse_dt<1><<<grid_for(L.nc, 256), 256, 0, ctx->stream>>>(L.nc, L.nf, L.c2f_ptr, L.c2f, L.nS, L.area, L.vol, W,
-                                                                   dt, ctx->P.gamma, ctx->P.cfl_coarse);
+      CK(launch_overlapped(k_coarse_dt<1>, grid_for(L.nc, 256), 256,
+                           ctx->stream, L.nc, L.nf, L.c2f_ptr, L.c2f, L.nS, L.area, L.vol, W, dt, ctx->P.gamma,
+                           ctx->P.cfl_coarse));
   }
   if (ctx->P.dt_mode == 1) CKS(global_min_dt(ctx, dt, L.nc));
   CK(cudaGetLastError());
@@ -468,7 +505,7 @@ static cgks_status coarse_forcing(cgks_ctx* ctx, int l) {
   CoarseBuf& B = ctx->C[l];
   const int64_t n5 = 5 * ctx->L[l].nc;
   ProfScope ps(ctx, PK_FORCING, (double)ctx->L[l].nc, n5 * 24.0);
-  k_forcing<<<grid_for(n5, 256), 256, 0, ctx->stream>>>(n5, B.Rs, B.R, B.F);
+  CK(launch_overlapped(k_forcing, grid_for(n5, 256), 256, ctx->stream, n5, B.Rs, B.R, B.F));
   CK(cudaGetLastError());
   return CGKS_OK;
 }
@@ -492,7 +529,7 @@ static cgks_status smooth_from_residual(cgks_ctx* ctx, int l) {
 }
 
 template <typename T, bool GATHER>
-static void coarse_step(cgks_ctx* ctx, int l, const T* ff, bool first) {
+static cgks_status coarse_step(cgks_ctx* ctx, int l, const T* ff, bool first) {
   const Level& L = ctx->L[l];
   CoarseBuf& B = ctx->C[l];
   const CoarseStep a{L.nc, L.nf, L.c2f_ptr, L.c2f, L.fL, L.fR, L.nS, L.area, B.Rs, forcing(ctx, B), B.W, ctx->P.gamma,
@@ -501,9 +538,10 @@ static void coarse_step(cgks_ctx* ctx, int l, const T* ff, bool first) {
                L.nc * (first && GATHER ? 164.0 : 124.0) + (L.nf + L.n_int + L.n_per) * 4.0 +
                    L.nf * (32.0 + (GATHER ? 8.0 + 5.0 * sizeof(T) : 0.0)));
   if (cell_lanes(L.nc, ctx->n_sm) == 8)
-    k_coarse_step<T, 8, GATHER><<<grid_for(8 * L.nc, 64), 64, 0, ctx->stream>>>(a, ff);
+    CK(launch_overlapped(k_coarse_step<T, 8, GATHER>, grid_for(8 * L.nc, 64), 64, ctx->stream, a, ff));
   else
-    k_coarse_step<T, 1, GATHER><<<grid_for(L.nc, 128), 128, 0, ctx->stream>>>(a, ff);
+    CK(launch_overlapped(k_coarse_step<T, 1, GATHER>, grid_for(L.nc, 128), 128, ctx->stream, a, ff));
+  return CGKS_OK;
 }
 
 // one smoothing step of level l.  first: at W = W^0 with the restricted defect in B.Rs, which also fixes
@@ -514,13 +552,13 @@ static cgks_status coarse_smooth(cgks_ctx* ctx, int l, bool first) {
   const bool mixed = ctx->P.precision == 1;
   if (ctx->P.coarse_smoother == 0 && ctx->P.dt_mode == 0) {
     if (mixed && first) {
-      coarse_step<float, false>(ctx, l, nullptr, true);
+      CKS((coarse_step<float, false>(ctx, l, nullptr, true)));
     } else if (mixed) {
-      kfvs_jvp_fluxes(ctx, l, B.W0, B.W, 1);
-      coarse_step<float, true>(ctx, l, B.ff32, false);
+      CKS(kfvs_jvp_fluxes(ctx, l, B.W0, B.W, 1));
+      CKS((coarse_step<float, true>(ctx, l, B.ff32, false)));
     } else {
-      kfvs_fluxes(ctx, l, B.W);
-      coarse_step<double, true>(ctx, l, B.ff, first);
+      CKS(kfvs_fluxes(ctx, l, B.W));
+      CKS((coarse_step<double, true>(ctx, l, B.ff, first)));
     }
     CK(cudaGetLastError());
     return CGKS_OK;
@@ -551,11 +589,11 @@ static cgks_status coarse_cycle(cgks_ctx* ctx, int l) {
     CKS(coarse_residual(ctx, l));
     {
       ProfScope ps(ctx, PK_RESTRICT, (double)L.nc, L.nc * 132.0 + Cn.nc * 132.0);
-      k_restrict<<<dim3(grid_for(Cn.nc, 128), 5), 128, 0, st>>>(Cn.nc, L.nc, Cn.agg_ptr, Cn.agg, L.vol, Cn.vol, B.W, B.R,
-                                                       forcing(ctx, B), N.W, N.W0, N.Rs);
+      CK(launch_overlapped(k_restrict, dim3(grid_for(Cn.nc, 128), 5), 128, st, Cn.nc, L.nc, Cn.agg_ptr, Cn.agg, L.vol,
+                           Cn.vol, B.W, B.R, forcing(ctx, B), N.W, N.W0, N.Rs));
     }
     CKS(coarse_cycle(ctx, l + 1));
-    prolong(ctx, l, Cn.f2c, Cn.nc, N.W, N.W0, B.W);
+    CKS(prolong(ctx, l, Cn.f2c, Cn.nc, N.W, N.W0, B.W));
     for (int s = 0; s < ctx->P.post; ++s) CKS(coarse_smooth(ctx, l, false));
   }
   CK(cudaGetLastError());
@@ -584,11 +622,11 @@ cgks_status vcycle_once(cgks_ctx* ctx, double* norm_dev) {
   CKS(fine_gather(ctx, ctx->W, nullptr, ctx->res, nullptr, nullptr, 0));
   {
     ProfScope ps(ctx, PK_RESTRICT, (double)F.nc, F.nc * 92.0 + C1.nc * 132.0);
-    k_restrict<<<dim3(grid_for(C1.nc, 128), 5), 128, 0, st>>>(C1.nc, F.nc, C1.agg_ptr, C1.agg, ctx->L0c.vol, C1.vol, ctx->W,
-                                                     ctx->res, nullptr, B1.W, B1.W0, B1.Rs);
+    CK(launch_overlapped(k_restrict, dim3(grid_for(C1.nc, 128), 5), 128, st, C1.nc, F.nc, C1.agg_ptr, C1.agg,
+                         ctx->L0c.vol, C1.vol, ctx->W, ctx->res, nullptr, B1.W, B1.W0, B1.Rs));
   }
   CKS(coarse_cycle(ctx, 1));
-  prolong(ctx, 0, C1.f2c, C1.nc, B1.W, B1.W0, ctx->W);
+  CKS(prolong(ctx, 0, C1.f2c, C1.nc, B1.W, B1.W0, ctx->W));
   for (int s = 0; s < ctx->P.post; ++s) CKS(step_once(ctx, nullptr));
   CK(cudaGetLastError());
   return CGKS_OK;

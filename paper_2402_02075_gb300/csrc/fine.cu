@@ -18,7 +18,9 @@ __global__ void __launch_bounds__(RECON_GROUP) k_reconstruct(ReconArgs a) {
   __shared__ double gs[20 * RECON_GROUP];  // ghost (W_c, gradient of W_c) of slot m: [4 c ..][32 m + lane]
   const int lane = threadIdx.x & 31, q = threadIdx.x >> 5;
   const int64_t nc = a.nc, i = blockIdx.x * (int64_t)32 + lane;
-  if (i < nc && q < (a.ctype[i] == 7 ? 5 : a.ctype[i]) && recon_neighbour(i, q, a) < 0) {  // slot q of cell i
+  const bool ghost = i < nc && q < (a.ctype[i] == 7 ? 5 : a.ctype[i]) && recon_neighbour(i, q, a) < 0;
+  wait_prior();
+  if (ghost) {  // slot q of cell i
     double Wg[5], Gg[15];
     recon_ghost(i, q, a, Wg, Gg);
 #pragma unroll
@@ -49,6 +51,7 @@ __global__ void __launch_bounds__(RECON_GROUP) k_reconstruct(ReconArgs a) {
 
 template <bool STATE>
 __global__ void __launch_bounds__(128) k_gks_points(PointArgs a) {
+  wait_prior();
   const int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (g < a.ngp) gks_point_body<STATE>(g, a);
 }
@@ -172,6 +175,7 @@ __global__ void __launch_bounds__(GATHER_VARS) k_gather_vars(GatherArgs a, Gathe
     ng[m] = m < nt ? a.gp_ptr[f + 1] - (int)g0[m] : 0;
     sg[m] = m < nt && a.cside[(int64_t)m * nc + i] ? 0x8000000000000000ull : 0ull;
   }
+  wait_prior();
 #pragma unroll
   for (int m = 0; m < 6; ++m) {
     double v[4][6];  // flux, state, area vector, factor of the face's points
@@ -285,7 +289,7 @@ cgks_status fine_fluxes(cgks_ctx* ctx, const double* W, const double* G, const d
   const double slots = (double)(F.nf + F.n_int + F.n_per);
   {
     ProfScope ps(ctx, PK_RECON, (double)F.nc, F.nc * (306.0 * 8 + 1 + 51.0 * 8) + slots * 5 + F.nf * 36.0);
-    k_reconstruct<<<grid_for(F.nc, 32), RECON_GROUP, 0, ctx->stream>>>(ra);
+    CK(launch_overlapped(k_reconstruct, grid_for(F.nc, 32), RECON_GROUP, ctx->stream, ra));
   }
   if (ctx->P.dt_mode == 1) CKS(global_min_dt(ctx, ctx->dt, F.nc));
   PointArgs pa{F.ngp, F.nf, F.nc, F.gp_face, F.fL, F.fR, F.ftag, F.gp_x, F.gp_A, F.fshift, F.ctr, ctx->rc,
@@ -295,9 +299,9 @@ cgks_status fine_fluxes(cgks_ctx* ctx, const double* W, const double* G, const d
                  F.ngp * (52.0 + (state ? 8.0 * CGKS_GPR : 40.0)) + F.nf * 36.0 + F.nc * 432.0);
     const int b = spread_block(F.ngp, 128, ctx->n_sm);
     if (state)
-      k_gks_points<true><<<grid_for(F.ngp, b), b, 0, ctx->stream>>>(pa);
+      CK(launch_overlapped(k_gks_points<true>, grid_for(F.ngp, b), b, ctx->stream, pa));
     else
-      k_gks_points<false><<<grid_for(F.ngp, b), b, 0, ctx->stream>>>(pa);
+      CK(launch_overlapped(k_gks_points<false>, grid_for(F.ngp, b), b, ctx->stream, pa));
   }
   CK(cudaGetLastError());
   return CGKS_OK;
@@ -320,9 +324,9 @@ cgks_status fine_gather(cgks_ctx* ctx, const double* W_in, double* W_out, double
     if (small) {
       const GatherNorm norm{ctx->nrm_part, norm_dev, ctx->nrm_done};
       if (grad)
-        k_gather_vars<true><<<vars_blocks, GATHER_VARS, 0, ctx->stream>>>(ga, norm);
+        CK(launch_overlapped(k_gather_vars<true>, vars_blocks, GATHER_VARS, ctx->stream, ga, norm));
       else
-        k_gather_vars<false><<<vars_blocks, GATHER_VARS, 0, ctx->stream>>>(ga, norm);
+        CK(launch_overlapped(k_gather_vars<false>, vars_blocks, GATHER_VARS, ctx->stream, ga, norm));
     } else {
       static bool smem_set = false;  // the kernel's dynamic shared memory exceeds the 48 KiB default
       if (!smem_set) {

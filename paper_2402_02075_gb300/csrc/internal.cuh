@@ -208,6 +208,35 @@ void free_list(cgks_ctx* ctx, std::vector<void*>& list);
 
 inline unsigned grid_for(int64_t n, int block) { return (unsigned)((n + block - 1) / block); }
 
+// Chains of short kernels: a kernel launched by launch_overlapped may be set up while the kernel before it
+// on the stream ends, and waits for that one, its writes included, in wait_prior().  Rules:
+// - such a kernel calls wait_prior() in every thread, before any return and before the first access to
+//   anything another kernel writes; above it only the mesh is read (finished before its upload
+//   returned).  So when it has ended, every kernel before it has ended too, and a copy, an event or
+//   an ordinary launch behind it is ordered as ever.
+// - what it reads behind the wait is not declared const __restrict__ (a read-only load may be moved
+//   above the wait, or be served from a line cached before it).
+// It saves 1.5 to 3 us of a launch of 6 to 45: ten steps of the 1,152-cell ramp 936 to 836 us (30
+// launches), a V-cycle of 576 cells 388 to 338 us (20), 50 V-cycles of 7,296 cells 24.7 to 23.4 ms.
+// No kernel lets the next one in before it ends (griddepcontrol.launch_dependents): blocks that come early
+// are placed around those still running, and the FP64 kernels then share sub-partitions while others
+// idle (the same ten steps took 1,268 us).
+__device__ __forceinline__ void wait_prior() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+template <class... P, class... A>
+cudaError_t launch_overlapped(void (*kernel)(P...), dim3 grid, dim3 block, cudaStream_t st, A&&... args) {
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.stream = st;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 // block size of a launch of n long FP64-bound threads: `max_block` when the launch fills every SM,
 // else smaller blocks (a multiple of the warp, at least one) so that the threads spread over all the
 // SMs: an SM issues 2 FP64 operations per clock, so a few blocks queued on a few SMs of a small
