@@ -81,10 +81,10 @@ struct CoarseBuf {  // per coarse level work arrays
   double *W = nullptr, *W0 = nullptr, *Rs = nullptr, *F = nullptr, *R = nullptr, *dt = nullptr, *ff = nullptr;
   float* ff32 = nullptr;  // FP32 directional derivatives of the face fluxes (precision 1)
   // LU-SGS smoother (coarse_smoother 1): colours, colour-major cell order and its offsets,
-  // per-face lambda, diagonal, increments
+  // per-face lambda, diagonal, sweep records (states and increments)
   int32_t *color = nullptr, *order = nullptr;
   std::vector<int64_t> coff;
-  double *lam = nullptr, *Dg = nullptr, *dU = nullptr;
+  double *lam = nullptr, *Dg = nullptr, *sweep = nullptr;
 };
 
 // kernel kinds timed by cgks_profile (ids of cgks_kernel_stats)

@@ -74,15 +74,23 @@ __global__ void k_jpl_assign(int64_t nc, const int32_t* __restrict__ ptr, const 
   }
 }
 
-__device__ __forceinline__ void euler_flux_n(const double W[5], const double n[3], double g, double F[5]) {
-  const double rho = W[0], r = fast_rcp(rho);
-  const double u[3] = {W[1] * r, W[2] * r, W[3] * r};
-  const double p = (g - 1.0) * (W[4] - 0.5 * rho * (u[0] * u[0] + u[1] * u[1] + u[2] * u[2]));
-  const double un = u[0] * n[0] + u[1] * n[1] + u[2] * n[2];
-  F[0] = rho * un;
+// What a sweep reads of a neighbour, one 128-byte line: its state (density, velocity, total enthalpy per
+// mass), the same of U + dU, p(U + dU) - p(U) and dU.  With it F_n(U + dU) - F_n(U) is 20 FP64
+// instructions per face; formed from the conservative states at each of a cell's 10 to 40 faces it was 60.
+// With that and lane_scatter a V-cycle of the 64x32x8 ramp takes 1.77 ms instead of 2.07.
+struct SweepRecord {
+  double rho, u[3], h, rho1, u1[3], h1, dp, dU[5];
+};
+static_assert(sizeof(SweepRecord) == 128, "one line per cell");
+
+// velocity, pressure and enthalpy of a conservative state
+__device__ __forceinline__ double sweep_state(const double w[5], double g, double u[3], double& h) {
+  const double r = fast_rcp(w[0]);
 #pragma unroll
-  for (int d = 0; d < 3; ++d) F[1 + d] = W[1 + d] * un + p * n[d];
-  F[4] = (W[4] + p) * un;
+  for (int d = 0; d < 3; ++d) u[d] = w[1 + d] * r;
+  const double p = (g - 1.0) * (w[4] - 0.5 * w[0] * (u[0] * u[0] + u[1] * u[1] + u[2] * u[2]));
+  h = (w[4] + p) * r;
+  return p;
 }
 
 __device__ __forceinline__ double wave_speed(const double* W, int64_t nc, int64_t i, const double n[3], double g) {
@@ -95,8 +103,8 @@ __device__ __forceinline__ double wave_speed(const double* W, int64_t nc, int64_
 // lambda of every face: max over its cells of |U.n| + c (the cell's own on boundary faces); nS: unit
 // normal and length of the face's summed area vector
 __global__ void k_lusgs_lambda(int64_t nf, const int32_t* __restrict__ fL, const int32_t* __restrict__ fR,
-                               const double* __restrict__ nS, int64_t nc, const double* __restrict__ W, double g,
-                               double* __restrict__ lam) {
+                               const double* __restrict__ nS, int64_t nc, const double* W, double g, double* lam) {
+  wait_prior();
   const int64_t f = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (f >= nf) return;
   if (nS[3 * nf + f] == 0.0) {
@@ -115,7 +123,8 @@ __global__ void k_lusgs_lambda(int64_t nf, const int32_t* __restrict__ fL, const
 // clocks of its sub-partition, about 100 of them per face, and the loads are dependent).  LANES threads
 // share the faces and add their parts in a fixed tree: a quarter warp, or a whole warp where the
 // colour has so few cells that every sub-partition still gets at most two.  V-cycle of the 64x32x8 ramp
-// (8.4 k and 4 k coarse cells, 38 sweeps per step and level): 2.3 ms against 9.7.
+// (8.4 k and 4 k coarse cells, 38 sweeps per step and level): 2.3 ms against 9.7.  The five sums of a
+// cell end in five of its lanes, each of which then does one variable's division.
 template <int LANES>
 __device__ __forceinline__ double lane_sum(double v) {
 #pragma unroll
@@ -123,12 +132,45 @@ __device__ __forceinline__ double lane_sum(double v) {
   return v;
 }
 
-// D_i = |Omega_i| / dt_i + 1/2 sum_p lambda_p S_p
+// the sums over the LANES threads of v[0..4], added pairwise as lane_sum adds them, each left in the lanes
+// whose sweep_variable says so: 6 additions for 8 lanes where five lane_sums take 15
+template <int LANES>
+__device__ __forceinline__ double lane_scatter(const double v[5], int sub) {
+  constexpr unsigned ALL = 0xffffffffu;
+  constexpr int d1 = LANES / 2, d2 = LANES / 4, d3 = LANES / 8;
+  const bool h1 = sub & d1, h2 = sub & d2, h3 = sub & d3;
+  double a = (h1 ? v[3] : v[0]) + __shfl_xor_sync(ALL, h1 ? v[0] : v[3], d1);
+  double b = (h1 ? v[4] : v[1]) + __shfl_xor_sync(ALL, h1 ? v[1] : v[4], d1);
+  double c = (h1 ? 0.0 : v[2]) + __shfl_xor_sync(ALL, h1 ? v[2] : 0.0, d1);
+  a = (h2 ? b : a) + __shfl_xor_sync(ALL, h2 ? a : b, d2);
+  c = (h2 ? 0.0 : c) + __shfl_xor_sync(ALL, h2 ? c : 0.0, d2);
+  a = (h3 ? c : a) + __shfl_xor_sync(ALL, h3 ? a : c, d3);
+#pragma unroll
+  for (int d = d3 / 2; d > 0; d >>= 1) a += __shfl_xor_sync(ALL, a, d);
+  return a;
+}
+
+// the variable whose sum lane_scatter leaves in lane sub (-1: none)
+template <int LANES>
+__device__ __forceinline__ int sweep_variable(int sub) {
+  constexpr int d1 = LANES / 2, d2 = LANES / 4, d3 = LANES / 8;
+  if (sub & d3) return sub & (d1 | d2) ? -1 : 2;
+  return (sub & d1 ? 3 : 0) + (sub & d2 ? 1 : 0);
+}
+
+// the lane that holds variable q
+template <int LANES>
+__device__ __forceinline__ int sweep_lane(int q) {
+  return q == 2 ? LANES / 8 : (q >= 3 ? LANES / 2 : 0) + (q == 1 || q == 4 ? LANES / 4 : 0);
+}
+
+// D_i = |Omega_i| / dt_i + 1/2 sum_p lambda_p S_p, and the cell's state in its sweep record
 template <int LANES>
 __global__ void k_lusgs_diag(int64_t nc, int64_t nf, const int32_t* __restrict__ ptr, const int32_t* __restrict__ c2f,
                              const int32_t* __restrict__ fL, const int32_t* __restrict__ fR,
-                             const double* __restrict__ nS, const double* __restrict__ lam,
-                             const double* __restrict__ vol, const double* __restrict__ dt, double* __restrict__ D) {
+                             const double* __restrict__ nS, const double* lam, const double* __restrict__ vol,
+                             const double* dt, const double* W, double g, double* D, SweepRecord* rec) {
+  wait_prior();
   const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, i = t / LANES;
   const bool live = i < nc;
   double s = 0.0;
@@ -139,76 +181,131 @@ __global__ void k_lusgs_diag(int64_t nc, int64_t nf, const int32_t* __restrict__
     s += lam[f] * nS[3 * nf + f];
   }
   s = lane_sum<LANES>(s);
-  if (live && t % LANES == 0) D[i] = vol[i] / dt[i] + 0.5 * s;
+  if (!live || t % LANES != 0) return;
+  D[i] = vol[i] / dt[i] + 0.5 * s;
+  double w[5], u[3], h;
+#pragma unroll
+  for (int q = 0; q < 5; ++q) w[q] = W[q * nc + i];
+  sweep_state(w, g, u, h);
+  rec[i].rho = w[0];
+#pragma unroll
+  for (int d = 0; d < 3; ++d) rec[i].u[d] = u[d];
+  rec[i].h = h;
 }
 
 struct SweepArgs {
   int64_t nc, nf;
   const int32_t *ptr, *c2f, *fL, *fR, *color, *cells;
   const double *nS, *lam, *W, *R, *F, *D;
-  double* dU;
+  SweepRecord* rec;
   double gamma;
 };
+
+// what a sweep needs of face entry e of cell i from the mesh alone: the neighbour (-1: nothing to add),
+// the unit normal out of the cell and the summed area
+struct SweepFace {
+  int64_t f, j;
+  double n[3], s;
+};
+
+template <bool FWD>
+__device__ __forceinline__ SweepFace sweep_face(const SweepArgs& a, int64_t i, int32_t e, int32_t end, int32_t k) {
+  SweepFace F;
+  F.j = -1;
+  if (e >= end) return F;
+  F.f = a.c2f[e];
+  const int64_t l = a.fL[F.f], r = a.fR[F.f], j = l == i ? r : l;
+  if (r < 0 || l == r || (FWD ? a.color[j] >= k : a.color[j] <= k)) return F;
+  F.s = a.nS[3 * a.nf + F.f];
+  if (F.s == 0.0) return F;
+  F.j = j;
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    const double v = a.nS[d * a.nf + F.f];
+    F.n[d] = l == i ? v : -v;
+  }
+  return F;
+}
 
 // forward (FWD) or backward sweep over the cells of colour k: neighbours of a lower (forward) or
 // higher (backward) colour contribute 1/2 [F_n(U_j + dU_j) - F_n(U_j) - lambda dU_j] S
 template <bool FWD, int LANES>
 __global__ void k_lusgs_sweep(SweepArgs a, int64_t count, int32_t k) {
   const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, pos = t / LANES;
-  const int64_t nc = a.nc, nf = a.nf;
+  const int64_t nc = a.nc;
   const bool live = pos < count;
   const int64_t i = live ? a.cells[pos] : 0;
-  double acc[5] = {0, 0, 0, 0, 0};
+  const int sub = (int)(t % LANES), var = sweep_variable<LANES>(sub), q = var < 0 ? 0 : var;
   const int32_t end = live ? a.ptr[i + 1] : 0;
-  for (int32_t e = live ? a.ptr[i] + (int)(t % LANES) : 0; e < end; e += LANES) {
-    const int64_t f = a.c2f[e];
-    const int64_t j = other_cell(a.fL, a.fR, f, i);
-    if (j < 0) continue;
-    if (FWD ? a.color[j] >= k : a.color[j] <= k) continue;
-    const double s = a.nS[3 * nf + f];
-    if (s == 0.0) continue;
-    const double sg = a.fL[f] == i ? 1.0 : -1.0;
-    const double n[3] = {sg * a.nS[f], sg * a.nS[nf + f], sg * a.nS[2 * nf + f]};
-    double Wj[5], Wp[5], dUj[5], Fp[5], F0[5];
+  int32_t e = live ? a.ptr[i] + sub : 0;
+  SweepFace F = sweep_face<FWD>(a, i, e, end, k);
+  wait_prior();  // everything above is the mesh and its colours; all below may come from the kernel before
+  const double w = a.W[q * nc + i], Di = a.D[i];
+  const double rhs = !live ? 0.0 : FWD ? a.R[q * nc + i] + a.F[q * nc + i] : a.rec[i].dU[q];
+  double acc[5] = {0, 0, 0, 0, 0};
+  while (e < end) {
+    e += LANES;
+    const SweepFace next = sweep_face<FWD>(a, i, e, end, k);
+    if (F.j >= 0) {
+      double2 v[8];
+      const double2* src = reinterpret_cast<const double2*>(a.rec + F.j);
 #pragma unroll
-    for (int q = 0; q < 5; ++q) {
-      Wj[q] = a.W[q * nc + j];
-      dUj[q] = a.dU[q * nc + j];
-      Wp[q] = Wj[q] + dUj[q];
+      for (int m = 0; m < 8; ++m) v[m] = src[m];
+      const double lam = a.lam[F.f], hs = 0.5 * F.s;
+      const double u[3] = {v[0].y, v[1].x, v[1].y}, u1[3] = {v[3].x, v[3].y, v[4].x};
+      const double dU[5] = {v[5].y, v[6].x, v[6].y, v[7].x, v[7].y}, dp = v[5].x;
+      const double m0 = v[0].x * (u[0] * F.n[0] + u[1] * F.n[1] + u[2] * F.n[2]);
+      const double m1 = v[2].y * (u1[0] * F.n[0] + u1[1] * F.n[1] + u1[2] * F.n[2]);
+      acc[0] += (m1 - m0 - lam * dU[0]) * hs;
+#pragma unroll
+      for (int d = 0; d < 3; ++d) acc[1 + d] += (u1[d] * m1 - u[d] * m0 + dp * F.n[d] - lam * dU[1 + d]) * hs;
+      acc[4] += (v[4].y * m1 - v[2].x * m0 - lam * dU[4]) * hs;
     }
-    euler_flux_n(Wp, n, a.gamma, Fp);
-    euler_flux_n(Wj, n, a.gamma, F0);
-    const double lam = a.lam[f], hs = 0.5 * s;
-#pragma unroll
-    for (int q = 0; q < 5; ++q) acc[q] += ((Fp[q] - F0[q]) - lam * dUj[q]) * hs;
+    F = next;
   }
+  const double sum = lane_scatter<LANES>(acc, sub);
+  const double x = FWD ? (rhs - sum) / Di : rhs - sum / Di;  // this lane's variable of dU
+  // the cell's lanes meet for the record of U + dU
+  double w0[5], w1[5], dU[5], u[3], h;
+  const int base = (threadIdx.x & 31) & ~(LANES - 1);
 #pragma unroll
-  for (int q = 0; q < 5; ++q) acc[q] = lane_sum<LANES>(acc[q]);
-  if (!live || t % LANES != 0) return;
-  const double Di = a.D[i];
+  for (int m = 0; m < 5; ++m) {
+    dU[m] = __shfl_sync(0xffffffffu, x, base + sweep_lane<LANES>(m));
+    w0[m] = __shfl_sync(0xffffffffu, w, base + sweep_lane<LANES>(m));
+    w1[m] = w0[m] + dU[m];
+  }
+  const double p1 = sweep_state(w1, a.gamma, u, h);
+  if (!live || sub != 0) return;
+  SweepRecord& r = a.rec[i];
+  const double p0 =
+      (a.gamma - 1.0) * (w0[4] - 0.5 * w0[0] * (r.u[0] * r.u[0] + r.u[1] * r.u[1] + r.u[2] * r.u[2]));
+  r.rho1 = w1[0];
 #pragma unroll
-  for (int q = 0; q < 5; ++q)
-    a.dU[q * nc + i] = FWD ? (a.R[q * nc + i] + a.F[q * nc + i] - acc[q]) / Di : a.dU[q * nc + i] - acc[q] / Di;
+  for (int d = 0; d < 3; ++d) r.u1[d] = u[d];
+  r.h1 = h;
+  r.dp = p1 - p0;
+#pragma unroll
+  for (int m = 0; m < 5; ++m) r.dU[m] = dU[m];
 }
 
 template <bool FWD>
-void sweep(const SweepArgs& a, int64_t cnt, int32_t k, int n_sm, cudaStream_t st) {
+cudaError_t sweep(const SweepArgs& a, int64_t cnt, int32_t k, int n_sm, cudaStream_t st) {
   if (cnt <= (int64_t)n_sm * 4 * 2)
-    k_lusgs_sweep<FWD, 32><<<grid_for(32 * cnt, 32), 32, 0, st>>>(a, cnt, k);
-  else
-    k_lusgs_sweep<FWD, 8><<<grid_for(8 * cnt, 64), 64, 0, st>>>(a, cnt, k);
+    return launch_overlapped(k_lusgs_sweep<FWD, 32>, grid_for(32 * cnt, 32), 32, st, a, cnt, k);
+  return launch_overlapped(k_lusgs_sweep<FWD, 8>, grid_for(8 * cnt, 64), 64, st, a, cnt, k);
 }
 
 // W += dU, skipping (and counting) cells whose rho or p would not stay positive
-__global__ void k_lusgs_apply(int64_t nc, const double* __restrict__ dU, double* __restrict__ W, double g,
-                              unsigned long long* skipped, DevErr* err) {
+__global__ void k_lusgs_apply(int64_t nc, const SweepRecord* rec, double* W, double g, unsigned long long* skipped,
+                              DevErr* err) {
+  wait_prior();
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i >= nc) return;
   double w[5];
   bool fin = true;
 #pragma unroll
   for (int q = 0; q < 5; ++q) {
-    w[q] = W[q * nc + i] + dU[q * nc + i];
+    w[q] = W[q * nc + i] + rec[i].dU[q];
     fin = fin && isfinite(w[q]);
   }
   if (!fin) {
@@ -238,7 +335,7 @@ cgks_status lusgs_colors(cgks_ctx* ctx, int l) {
   CKS(dalloc(ctx, M, &B.order, L.nc));
   CKS(dalloc(ctx, M, &B.lam, L.nf));
   CKS(dalloc(ctx, M, &B.Dg, L.nc));
-  CKS(dalloc(ctx, M, &B.dU, 5 * L.nc));
+  CKS(dalloc(ctx, M, &B.sweep, sizeof(SweepRecord) / sizeof(double) * L.nc));
   std::vector<void*> tmp;
   cgks_status s = dalloc(ctx, tmp, &sel, L.nc);
   if (s != CGKS_OK) {
@@ -285,21 +382,22 @@ cgks_status lusgs_step(cgks_ctx* ctx, int l, const double* F) {
   CoarseBuf& B = ctx->C[l];
   cudaStream_t st = ctx->stream;
   const double g = ctx->P.gamma;
-  k_lusgs_lambda<<<grid_for(L.nf, 128), 128, 0, st>>>(L.nf, L.fL, L.fR, L.nS, L.nc, B.W, g, B.lam);
-  k_lusgs_diag<8><<<grid_for(8 * L.nc, 128), 128, 0, st>>>(L.nc, L.nf, L.c2f_ptr, L.c2f, L.fL, L.fR, L.nS, B.lam, L.vol,
-                                                           B.dt, B.Dg);
-  SweepArgs a{L.nc, L.nf, L.c2f_ptr, L.c2f, L.fL, L.fR, B.color, B.order, L.nS, B.lam, B.W, B.R, F, B.Dg, B.dU, g};
+  SweepRecord* rec = reinterpret_cast<SweepRecord*>(B.sweep);
+  CK(launch_overlapped(k_lusgs_lambda, grid_for(L.nf, 128), 128, st, L.nf, L.fL, L.fR, L.nS, L.nc, B.W, g, B.lam));
+  CK(launch_overlapped(k_lusgs_diag<8>, grid_for(8 * L.nc, 128), 128, st, L.nc, L.nf, L.c2f_ptr, L.c2f, L.fL, L.fR,
+                       L.nS, B.lam, L.vol, B.dt, B.W, g, B.Dg, rec));
+  SweepArgs a{L.nc, L.nf, L.c2f_ptr, L.c2f, L.fL, L.fR, B.color, B.order, L.nS, B.lam, B.W, B.R, F, B.Dg, rec, g};
   const int32_t ncol = (int32_t)B.coff.size() - 1;
   for (int32_t k = 0; k < ncol; ++k) {
     a.cells = B.order + B.coff[k];
-    sweep<true>(a, B.coff[k + 1] - B.coff[k], k, ctx->n_sm, st);
+    CK(sweep<true>(a, B.coff[k + 1] - B.coff[k], k, ctx->n_sm, st));
   }
   for (int32_t k = ncol - 1; k >= 0; --k) {
     a.cells = B.order + B.coff[k];
-    sweep<false>(a, B.coff[k + 1] - B.coff[k], k, ctx->n_sm, st);
+    CK(sweep<false>(a, B.coff[k + 1] - B.coff[k], k, ctx->n_sm, st));
   }
-  k_lusgs_apply<<<grid_for(L.nc, 256), 256, 0, st>>>(L.nc, B.dU, B.W, g, (unsigned long long*)ctx->d_skipped,
-                                                      ctx->derr);
+  CK(launch_overlapped(k_lusgs_apply, grid_for(L.nc, 256), 256, st, L.nc, rec, B.W, g,
+                       (unsigned long long*)ctx->d_skipped, ctx->derr));
   CK(cudaGetLastError());
   return CGKS_OK;
 }
