@@ -47,21 +47,23 @@ SAMPLE = dict(nx=96, ny=4, nz=69, outflow=5)
 # FP64 floating-point operations per Gauss point of the gas-kinetic flux kernel (2 per DFMA, 1 per
 # DADD/DMUL), from the ncu instruction counts of a full capture of the kernel on the 48x32x32 box;
 # the kernel's own arithmetic, all of which the method needs
-FLOP_PER_GP = 3249.5
+FLOP_PER_GP = 2026.4
 # DRAM bytes (read + write) per Gauss point of the same kernel from the same capture (None when the
 # kernel has changed since)
-DRAM_BYTES_PER_GP = 172.3
+DRAM_BYTES_PER_GP = 173.5
 # FP64 operations per unit of the other kernels bound by the FP64 pipe, from ncu instruction counts
 # on the same box (2 per DFMA, 1 per DMUL or DADD; averages over the launches of a V-cycle):
-# reconstruction per cell (DFMA 1,464.3, DMUL 318.1, DADD 155.6), gather with the gradient update per
-# Gauss point seen from a cell (DFMA 16.06, DMUL 2.17, DADD 5.11), the flux alone of the V-cycle's
-# defect per Gauss point (DFMA 1,179.1, DMUL 490.4, DADD 230.0), coarse KFVS face flux per face (DFMA
-# 183.8, DMUL 66.5, DADD 30.9: the launches of a V-cycle weighted by their faces).  The residual-only gather of the defect (5.6 FLOP per point seen), the
-# coarse time step and the KFVS gather are latency-bound gathers, reported against HBM.
-FLOP_PER_CELL_RECON = 3402.2
+# reconstruction per cell (DFMA 1,177.1, DMUL 199.3, DADD 108.3, on the 96x4x69 slab, whose mix of prisms
+# and tetrahedra is the bench box's; a prism of the 48x32x32 box takes 2,956.4), gather with the
+# gradient update per Gauss point seen from a cell (DFMA 16.06, DMUL 2.17, DADD 5.11), the flux alone of the V-cycle's
+# defect per Gauss point (DFMA 682.5, DMUL 293.6, DADD 154.8), coarse KFVS face flux per face (DFMA
+# 83.8, DMUL 59.1, DADD 23.2: the launches of a V-cycle weighted by their faces).  The residual-only
+# gather of the defect (5.6 FLOP per point seen) and the coarse levels' gathers and steps (k_kfvs_gather)
+# are latency-bound, reported against HBM.
+FLOP_PER_CELL_RECON = 2661.8
 FLOP_PER_GP_SIDE_GATHER = 39.39
-FLOP_PER_GP_FLUX = 3078.6
-FLOP_PER_FACE_KFVS = 464.8
+FLOP_PER_GP_FLUX = 1813.4
+FLOP_PER_FACE_KFVS = 249.8
 ALU_KERNELS = {"k_gks_points": FLOP_PER_GP, "k_reconstruct": FLOP_PER_CELL_RECON,
                "k_gather": FLOP_PER_GP_SIDE_GATHER, "k_kfvs_faces": FLOP_PER_FACE_KFVS,
                "k_gks_points_flux": FLOP_PER_GP_FLUX}
@@ -77,23 +79,32 @@ def workload_name(w):
 
 
 def launches_per_vcycle(P, history=False):
-    """Kernels launched by one V-cycle (fine step, defect, restriction, coarse levels, corrections).
-    FP64 (FAS): a coarse level evaluates its KFVS residual at W^0 for the forcing and the first step
-    (faces + gather) plus the forcing kernel; mixed (defect correction): the first step needs no
-    residual (the defect is the restricted one) and later residuals are FP32 directional derivatives
-    (faces + gather)."""
+    """Kernels launched by one V-cycle (fine step, defect, restriction, coarse levels, corrections) on a
+    mesh above 64 cells per SM (below, the gather forms the norm itself).  A coarse forward-Euler step
+    with local time steps is two launches, the KFVS face fluxes (FP64) or their FP32 directional
+    derivatives (mixed) and the step, which also forms the forcing on a level's first step; the mixed
+    cycle's first step needs no residual (the defect is the restricted one).  With one global time step
+    (dt_mode 1) the gather, the forcing, the time step, its minimum and the update are launches of
+    their own."""
     dtm = 2 if P["dt_mode"] == 1 else 0
+    mixed = P["precision"] == 1
     fine_step = 3 + dtm + (2 if history else 0)
     n = fine_step * max(P["pre"], 1)
     nl = P["n_levels"]
     C = P["coarse_steps"]
+
+    def step(first):
+        if dtm:
+            return (0 if mixed and first else 2) + (1 if first and not mixed else 0) + 1 + dtm + 1
+        return 1 if mixed and first else 2
+
     if nl > 1:
         n += 3 + dtm + 1  # defect (reconstruct, points, gather) + restriction
 
         def coarse(l):
-            k = (0 if P["precision"] == 1 else 3) + C * (1 + dtm + 1) + (C - 1) * 2
+            k = sum(step(i == 0) for i in range(C)) + (3 if C == 0 and not mixed else 0)
             if l + 1 < nl:
-                k += 2 + 1 + coarse(l + 1) + 1 + P["post"] * (2 + 1 + dtm + 1)
+                k += 2 + 1 + coarse(l + 1) + 1 + P["post"] * step(False)
             return k
         n += coarse(1) + 1 + P["post"] * fine_step
     return n

@@ -206,9 +206,9 @@ cgks_status cgks_skipped_updates(cgks_ctx* ctx, int64_t* count);
  * (CGKS_EUNSUPPORTED otherwise).  Vectors of 20 rows are [20][N]: the 5 rows of W then the 15 of
  * grad W, in the layouts of cgks_state_init. */
 
-/* Forms and stores the linearisation of (Res, Gnew) at the current state by forward-mode duals
- * (41 x 10 doubles per Gauss point, 2,220 per cell; device memory owned by the context, freed with
- * the mesh).  Errors: CGKS_EINVAL (no state), CGKS_ENOMEM, CGKS_EUNSUPPORTED. */
+/* Forms and stores the linearisation of (Res, Gnew) at the current state (exact derivatives, formed
+ * column by column; 41 x 10 doubles per Gauss point, 2,220 per cell; device memory owned by the
+ * context, freed with the mesh).  Errors: CGKS_EINVAL (no state), CGKS_ENOMEM, CGKS_EUNSUPPORTED. */
 cgks_status cgks_linearize(cgks_ctx* ctx);
 
 /* Transposed product with the stored linearisation: (W_bar, G_bar) = (d(Res, Gnew)/d(W, G))^T
@@ -266,6 +266,9 @@ cgks_status cgks_fp64_peak(double* tflops);
  *  10 FP32 KFVS directional derivative (faces)            11 residual norm (cells)
  *  12 Gauss-point flux alone, for the V-cycle's defect     13 fine gather of the residual alone
  *     (Gauss points)                                          (Gauss points seen from cells)
+ * A coarse forward-Euler step with local time steps is one launch (gather, forcing, time step and
+ * update), counted under 4, or under 5 where it gathers nothing (the mixed cycle's first step of a
+ * level); on meshes of up to 64 cells per SM kernel 2 forms the residual norm as well.
  * cgks_kernel_stats synchronises the stream and returns (host outputs, each nullable) the summed
  * device time in milliseconds, the number of launches, the summed units and the summed algorithmic
  * bytes of kernel `which` recorded since profiling was enabled; an id outside 0..13 is CGKS_EINVAL. */

@@ -6,8 +6,9 @@
 // Res the residual of the explicit update and Gnew the Gauss-Green gradient (compression factor
 // off).  The chain of one evaluation is  (W, G) -> reconstruction (coefficients rc, time step dt)
 // per cell -> gas-kinetic flux per Gauss point (inputs: W and grad W of both sides at the point, dt
-// of the face) -> fixed-order sums per cell.  cgks_linearize forms the Jacobian of each link by
-// forward-mode duals (the residual's own code on Dual<double>, exact to round-off) and keeps it:
+// of the face) -> fixed-order sums per cell.  cgks_linearize forms the Jacobian of each link (exact to
+// round-off; the passive part of a point or of a cell's variable is evaluated once, its columns share
+// it) and keeps it:
 //   Jp [41 x 10][ngp]   per Gauss point
 //   Jr [2,220][nc]      per cell: own slot 20 inputs x (50 coefficients, dt); each of up to 6
 //                       neighbour slots 5 variables x 4 inputs x 10 coefficients (block diagonal)
