@@ -8,44 +8,69 @@
 __host__ __device__ __forceinline__ int cell_nfaces(int t) { return t == 7 ? 5 : t; }
 
 // ---- dense helpers of the reconstruction-operator precompute (per thread, column-major) --------
+//
+// The number of faces is a template parameter, so that every loop is unrolled and every index known: the
+// matrices then live in registers and in spill slots that are read once or twice.  With run-time sizes
+// all of them (5.5 KB per thread) were local memory read at every multiply-add: 17.0 ms for the
+// 1.51 M cells of the 96x64x69 boundary layer against 12.0 now, the FP64 pipe 91 % busy.
 
-// Householder QR of A (m x n, m >= n, column-major, leading dimension m): R in the upper triangle,
-// reflector k stored in A[k+1:, k] with an implicit unit leading entry, scale in tau[k].
-__host__ __device__ inline bool house_qr(int m, int n, double* A, double* tau) {
-  for (int k = 0; k < n; ++k) {
-    double* a = A + k * m;
-    double s = 0.0;
-    for (int i = k + 1; i < m; ++i) s += a[i] * a[i];
-    const double x0 = a[k];
-    const double nrm = sqrt(x0 * x0 + s);
-    if (nrm == 0.0) return false;
-    const double beta = x0 >= 0.0 ? -nrm : nrm;
-    const double v0 = x0 - beta;
-    for (int i = k + 1; i < m; ++i) a[i] /= v0;
-    tau[k] = (beta - x0) / beta;
-    a[k] = beta;
-    for (int j = k + 1; j < n; ++j) {
-      double* b = A + j * m;
-      double d = b[k];
-      for (int i = k + 1; i < m; ++i) d += a[i] * b[i];
-      d *= tau[k];
-      b[k] -= d;
-      for (int i = k + 1; i < m; ++i) b[i] -= d * a[i];
-    }
-  }
-  return true;
+// s / d from r = 1/d: the product and one correction by its residual (P. W. Markstein, IBM J. Res. Dev. 34,
+// 1990), as accurate as a division (within an ulp) and 3 FP64 instructions against 9; the operators take
+// about 190 quotients by 25 divisors per cell.
+__host__ __device__ __forceinline__ double quotient(double s, double d, double r) {
+  const double q = s * r;
+  return fma(fma(-q, d, s), r, q);
 }
 
-// y <- Q y (Q = H_0 H_1 ... H_{n-1}) or y <- Q^T y
-__host__ __device__ inline void house_apply(int m, int n, const double* A, const double* tau, double* y, bool transpose) {
-  for (int kk = 0; kk < n; ++kk) {
-    const int k = transpose ? kk : n - 1 - kk;
-    const double* a = A + k * m;
+// Householder QR of A (M x N, M >= N, column-major, leading dimension M): R in the upper triangle,
+// reflector k stored in A[k+1:, k] with an implicit unit leading entry, scale in tau[k].
+template <int M, int N>
+__host__ __device__ __forceinline__ bool house_qr(double* A, double* tau) {
+  bool ok = true;
+#pragma unroll
+  for (int k = 0; k < N; ++k) {
+    double* a = A + k * M;
+    double s = 0.0;
+#pragma unroll
+    for (int i = k + 1; i < M; ++i) s += a[i] * a[i];
+    const double x0 = a[k];
+    const double nrm = sqrt(x0 * x0 + s);
+    ok = ok && nrm != 0.0;
+    const double beta = x0 >= 0.0 ? -nrm : nrm;
+    const double v0 = x0 - beta, rv = 1.0 / v0;
+#pragma unroll
+    for (int i = k + 1; i < M; ++i) a[i] = quotient(a[i], v0, rv);
+    tau[k] = (beta - x0) / beta;
+    a[k] = beta;
+#pragma unroll
+    for (int j = k + 1; j < N; ++j) {
+      double* b = A + j * M;
+      double d = b[k];
+#pragma unroll
+      for (int i = k + 1; i < M; ++i) d += a[i] * b[i];
+      d *= tau[k];
+      b[k] -= d;
+#pragma unroll
+      for (int i = k + 1; i < M; ++i) b[i] -= d * a[i];
+    }
+  }
+  return ok;
+}
+
+// y <- Q y (Q = H_0 H_1 ... H_{N-1}) or y <- Q^T y
+template <int M, int N, bool TRANSPOSE>
+__host__ __device__ __forceinline__ void house_apply(const double* A, const double* tau, double* y) {
+#pragma unroll
+  for (int kk = 0; kk < N; ++kk) {
+    const int k = TRANSPOSE ? kk : N - 1 - kk;
+    const double* a = A + k * M;
     double d = y[k];
-    for (int i = k + 1; i < m; ++i) d += a[i] * y[i];
+#pragma unroll
+    for (int i = k + 1; i < M; ++i) d += a[i] * y[i];
     d *= tau[k];
     y[k] -= d;
-    for (int i = k + 1; i < m; ++i) y[i] -= d * a[i];
+#pragma unroll
+    for (int i = k + 1; i < M; ++i) y[i] -= d * a[i];
   }
 }
 
@@ -63,9 +88,9 @@ struct ROArgs {
   DevErr* err;
 };
 
-__host__ __device__ inline void recon_ops_body(int64_t i, const ROArgs& A_) {
+template <int nt>
+__host__ __device__ __forceinline__ void recon_ops_cell(int64_t i, const ROArgs& A_) {
   const int64_t nc = A_.nc, nf = A_.nf;
-  const int8_t* ctype = A_.ctype;
   const int32_t* cf = A_.cf;
   const int8_t* cside = A_.cside;
   const int32_t *fL = A_.fL, *fR = A_.fR;
@@ -73,12 +98,12 @@ __host__ __device__ inline void recon_ops_body(int64_t i, const ROArgs& A_) {
                *fctr = A_.fctr, *fnrm = A_.fnrm;
   double *Kop = A_.Kop, *ggw = A_.ggw, *lsw = A_.lsw, *aux = A_.aux, *dtw = A_.dtw;
   DevErr* err = A_.err;
-  const int nt = cell_nfaces(ctype[i]);
   const double V = vol[i];
   double c0[3], M0[6];
   for (int d = 0; d < 3; ++d) c0[d] = ctr[d * nc + i];
   for (int j = 0; j < 6; ++j) M0[j] = m2[j * nc + i];
-  double dl[6][3], Mn[6][6];
+  double dl[nt][3], Mn[nt][6];
+#pragma unroll
   for (int m = 0; m < nt; ++m) {
     const int64_t f = cf[(int64_t)m * nc + i];
     const bool side = cside[(int64_t)m * nc + i] != 0;
@@ -124,121 +149,145 @@ __host__ __device__ inline void recon_ops_body(int64_t i, const ROArgs& A_) {
     for (int d = 0; d < 3; ++d) ggw[(3 * m + d) * nc + i] = 0.0;
     for (int d = 0; d < 4; ++d) dtw[(4 * m + d) * nc + i] = 0.0;
   }
-  // C (nt x 9): averages of the basis X,Y,Z,X^2,Y^2,Z^2,XY,YZ,XZ over the neighbour minus over the cell;
-  // B (3nt x 9): averages of their derivatives over the neighbour
-  double Ct[9 * 6];   // C^T, column-major 9 x nt
-  double Bm[18 * 9];  // B, column-major (3nt) x 9
-  const int mb = 3 * nt;
+  // C (nt x 9): averages of the basis X,Y,Z,X^2,Y^2,Z^2,XY,YZ,XZ over the neighbour minus over the cell
+  constexpr int mb = 3 * nt, nz = 9 - nt;
+  double Ct[9 * nt];  // C^T, column-major 9 x nt
+#pragma unroll
   for (int m = 0; m < nt; ++m) {
     const double* x = dl[m];
     const double* M = Mn[m];
     const double row[9] = {x[0], x[1], x[2], M[0] + x[0] * x[0] - M0[0], M[1] + x[1] * x[1] - M0[1],
                            M[2] + x[2] * x[2] - M0[2], M[3] + x[0] * x[1] - M0[3], M[4] + x[1] * x[2] - M0[4],
                            M[5] + x[0] * x[2] - M0[5]};
+#pragma unroll
     for (int j = 0; j < 9; ++j) Ct[m * 9 + j] = row[j];
-    const double dx[9] = {1, 0, 0, 2 * x[0], 0, 0, x[1], 0, x[2]};
-    const double dy[9] = {0, 1, 0, 0, 2 * x[1], 0, x[0], x[2], 0};
-    const double dz[9] = {0, 0, 1, 0, 0, 2 * x[2], 0, x[1], x[0]};
-    for (int j = 0; j < 9; ++j) {
-      Bm[j * mb + 3 * m + 0] = dx[j];
-      Bm[j * mb + 3 * m + 1] = dy[j];
-      Bm[j * mb + 3 * m + 2] = dz[j];
-    }
   }
-  double tc[6];
-  if (!house_qr(9, nt, Ct, tc)) {
+  // product of row 3 m + d of B (3nt x 9) with y: averages of the derivatives of the basis over neighbour
+  // m, 4 of the 9 not zero
+  const auto B_row = [&dl](int m, int d, const double* y) {
+    const double* x = dl[m];
+    double s = y[d];
+    s += 2 * x[d] * y[3 + d];
+    s += d == 0 ? x[1] * y[6] : d == 1 ? x[0] * y[6] : x[1] * y[7];
+    s += d == 0 ? x[2] * y[8] : d == 1 ? x[2] * y[7] : x[0] * y[8];
+    return s;
+  };
+  double tc[nt];
+  if (!house_qr<9, nt>(Ct, tc)) {
     set_err(err, CGKS_EMESH, (int)i, 50);
     return;
   }
-  // Q (9 x 9) explicit
-  double Q[81];
-  for (int col = 0; col < 9; ++col) {
-    double* y = Q + col * 9;
+  // A1 = Q1 R^{-T} (9 x nt), Q1 the first nt columns of Q: each row x of A1 solves R x^T = (row of Q1)^T,
+  // back substitution; R[k][j] is stored at Ct[j*9 + k]
+  double A1[9 * nt];
+#pragma unroll
+  for (int col = 0; col < nt; ++col) {
+    double* y = A1 + col * 9;
+#pragma unroll
     for (int r = 0; r < 9; ++r) y[r] = r == col ? 1.0 : 0.0;
-    house_apply(9, nt, Ct, tc, y, false);
+    house_apply<9, nt, false>(Ct, tc, y);
   }
-  // A1 = Q1 R^{-T} (9 x nt): each row x of A1 solves R x^T = (row of Q1)^T, back substitution;
-  // R[k][j] is stored at Ct[j*9 + k]
-  double A1[9 * 6];
+  double rc[nt];
+#pragma unroll
+  for (int k = 0; k < nt; ++k) rc[k] = 1.0 / Ct[k * 9 + k];
+#pragma unroll
   for (int r = 0; r < 9; ++r)
+#pragma unroll
     for (int k = nt - 1; k >= 0; --k) {
-      double s = Q[k * 9 + r];
+      double s = A1[k * 9 + r];
+#pragma unroll
       for (int j = k + 1; j < nt; ++j) s -= Ct[j * 9 + k] * A1[j * 9 + r];
-      A1[k * 9 + r] = s / Ct[k * 9 + k];
+      A1[k * 9 + r] = quotient(s, Ct[k * 9 + k], rc[k]);
     }
-  // BQ2 (mb x nz)
-  const int nz = 9 - nt;
-  double BQ2[18 * 5], tb[5];
-  for (int c = 0; c < nz; ++c)
-    for (int r = 0; r < mb; ++r) {
-      double s = 0.0;
-      for (int j = 0; j < 9; ++j) s += Bm[j * mb + r] * Q[(nt + c) * 9 + j];
-      BQ2[c * mb + r] = s;
-    }
-  if (!house_qr(mb, nz, BQ2, tb)) {
+  double BA[nt * mb];  // B A1 (mb x nt)
+#pragma unroll
+  for (int k = 0; k < nt; ++k)
+#pragma unroll
+    for (int r = 0; r < mb; ++r) BA[k * mb + r] = B_row(r / 3, r % 3, A1 + k * 9);
+  // Q2 (9 x nz), the other columns of Q, and B Q2 (mb x nz)
+  double Q2[9 * nz], BQ2[mb * nz], tb[nz];
+#pragma unroll
+  for (int c = 0; c < nz; ++c) {
+    double* y = Q2 + c * 9;
+#pragma unroll
+    for (int r = 0; r < 9; ++r) y[r] = r == nt + c ? 1.0 : 0.0;
+    house_apply<9, nt, false>(Ct, tc, y);
+#pragma unroll
+    for (int r = 0; r < mb; ++r) BQ2[c * mb + r] = B_row(r / 3, r % 3, y);
+  }
+  if (!house_qr<mb, nz>(BQ2, tb)) {
     set_err(err, CGKS_EMESH, (int)i, 51);
     return;
   }
   // P2 = (BQ2)^+ = Rb^{-1} Qb^T (nz x mb): the first nz columns of Qb, then back substitution per row of
   // Qb (forming all of Qb^T from the identity would take three times the operations)
-  double Qb[5 * 18];
+  double P2[nz * mb];
+#pragma unroll
   for (int col = 0; col < nz; ++col) {
-    double* y = Qb + col * 18;
+    double* y = P2 + col * mb;
+#pragma unroll
     for (int r = 0; r < mb; ++r) y[r] = r == col ? 1.0 : 0.0;
-    house_apply(mb, nz, BQ2, tb, y, false);
+    house_apply<mb, nz, false>(BQ2, tb, y);
   }
-  double P2[5 * 18];
+  double rb[nz];
+#pragma unroll
+  for (int r = 0; r < nz; ++r) rb[r] = 1.0 / BQ2[r * mb + r];
+#pragma unroll
   for (int col = 0; col < mb; ++col)
+#pragma unroll
     for (int r = nz - 1; r >= 0; --r) {
-      double s = Qb[r * 18 + col];
-      for (int j = r + 1; j < nz; ++j) s -= BQ2[j * mb + r] * P2[col * 5 + j];
-      P2[col * 5 + r] = s / BQ2[r * mb + r];
+      double s = P2[r * mb + col];
+#pragma unroll
+      for (int j = r + 1; j < nz; ++j) s -= BQ2[j * mb + r] * P2[j * mb + col];
+      P2[r * mb + col] = quotient(s, BQ2[r * mb + r], rb[r]);
     }
-  // Kg = Q2 P2 (9 x mb); KdQ = A1 - Kg (B A1) (9 x nt)
-  double Kg[9 * 18];
-  for (int col = 0; col < mb; ++col)
-    for (int r = 0; r < 9; ++r) {
-      double s = 0.0;
-      for (int j = 0; j < nz; ++j) s += Q[(nt + j) * 9 + r] * P2[col * 5 + j];
-      Kg[col * 9 + r] = s;
-    }
-  for (int k = 0; k < nt; ++k) {
-    double BA[18];
-    for (int r = 0; r < mb; ++r) {
-      double s = 0.0;
-      for (int j = 0; j < 9; ++j) s += Bm[j * mb + r] * A1[k * 9 + j];
-      BA[r] = s;
-    }
-    for (int r = 0; r < 9; ++r) {
-      double s = A1[k * 9 + r];
-      for (int j = 0; j < mb; ++j) s -= Kg[j * 9 + r] * BA[j];
-      Kop[(r * 24 + k) * nc + i] = s;
-    }
-  }
+  // row by row: Kg = Q2 P2 (9 x mb), KdQ = A1 - Kg (B A1) (9 x nt)
+#pragma unroll
   for (int r = 0; r < 9; ++r) {
-    for (int k = nt; k < 6; ++k) Kop[(r * 24 + k) * nc + i] = 0.0;
-    for (int col = 0; col < 18; ++col) Kop[(r * 24 + 6 + col) * nc + i] = col < mb ? Kg[col * 9 + r] : 0.0;
+    double dq[nt];
+#pragma unroll
+    for (int k = 0; k < nt; ++k) dq[k] = A1[k * 9 + r];
+#pragma unroll
+    for (int col = 0; col < mb; ++col) {
+      double s = 0.0;
+#pragma unroll
+      for (int j = 0; j < nz; ++j) s += Q2[j * 9 + r] * P2[j * mb + col];
+      Kop[(r * 24 + 6 + col) * nc + i] = s;
+#pragma unroll
+      for (int k = 0; k < nt; ++k) dq[k] -= s * BA[k * mb + col];
+    }
+#pragma unroll
+    for (int k = 0; k < 6; ++k) Kop[(r * 24 + k) * nc + i] = k < nt ? dq[k < nt ? k : 0] : 0.0;
+#pragma unroll
+    for (int col = mb; col < 18; ++col) Kop[(r * 24 + 6 + col) * nc + i] = 0.0;
   }
   // least-squares gradient weights: D^+ with D = [dl_m] (nt x 3)
-  double D[6 * 3], td[3];
+  double D[nt * 3], td[3];
+#pragma unroll
   for (int d = 0; d < 3; ++d)
+#pragma unroll
     for (int m = 0; m < nt; ++m) D[d * nt + m] = dl[m][d];
-  if (!house_qr(nt, 3, D, td)) {
+  if (!house_qr<nt, 3>(D, td)) {
     set_err(err, CGKS_EMESH, (int)i, 52);
     return;
   }
+  double rd[3];
+#pragma unroll
+  for (int r = 0; r < 3; ++r) rd[r] = 1.0 / D[r * nt + r];
+#pragma unroll
   for (int m = 0; m < 6; ++m) {
-    double y[6] = {0, 0, 0, 0, 0, 0}, g[3];
+    double y[nt], g[3] = {0.0, 0.0, 0.0};
     if (m < nt) {
-      y[m] = 1.0;
-      house_apply(nt, 3, D, td, y, true);
+#pragma unroll
+      for (int r = 0; r < nt; ++r) y[r] = r == m ? 1.0 : 0.0;
+      house_apply<nt, 3, true>(D, td, y);
+#pragma unroll
       for (int r = 2; r >= 0; --r) {
         double s = y[r];
+#pragma unroll
         for (int j = r + 1; j < 3; ++j) s -= D[j * nt + r] * g[j];
-        g[r] = s / D[r * nt + r];
+        g[r] = quotient(s, D[r * nt + r], rd[r]);
       }
-    } else {
-      g[0] = g[1] = g[2] = 0.0;
     }
     for (int d = 0; d < 3; ++d) lsw[(3 * m + d) * nc + i] = g[d];
   }
@@ -248,3 +297,10 @@ __host__ __device__ inline void recon_ops_body(int64_t i, const ROArgs& A_) {
   for (int j = 0; j < 6; ++j) aux[(2 + j) * nc + i] = M0[j];
 }
 
+__host__ __device__ inline void recon_ops_body(int64_t i, const ROArgs& a) {
+  switch (cell_nfaces(a.ctype[i])) {
+    case 4: recon_ops_cell<4>(i, a); break;
+    case 5: recon_ops_cell<5>(i, a); break;
+    default: recon_ops_cell<6>(i, a); break;
+  }
+}
