@@ -221,8 +221,8 @@ static constexpr int kGmresM = 30;  // Krylov vectors per restart
 // the functional's per-cell shares and the reduction partials (small: the wall force needs no more)
 static cgks_status small_buffers(cgks_ctx* ctx) {
   if (ctx->ajc) return CGKS_OK;
-  CKS(dalloc(ctx, ctx->mesh_allocs, &ctx->apart, kSumParts + 1));
-  CKS(dalloc(ctx, ctx->mesh_allocs, &ctx->ajc, ctx->F.nc));
+  CKS(dalloc(ctx, ctx->adj_allocs, &ctx->apart, kSumParts + 1));
+  CKS(dalloc(ctx, ctx->adj_allocs, &ctx->ajc, ctx->F.nc));
   return CGKS_OK;
 }
 
@@ -230,7 +230,7 @@ static cgks_status adjoint_buffers(cgks_ctx* ctx) {
   CKS(small_buffers(ctx));
   if (ctx->pbar) return CGKS_OK;
   const Fine& F = ctx->F;
-  auto& M = ctx->mesh_allocs;
+  auto& M = ctx->adj_allocs;
   CKS(dalloc(ctx, M, &ctx->Jp, (size_t)CGKS_PJ_IN * CGKS_PJ_OUT * F.ngp));
   CKS(dalloc(ctx, M, &ctx->adt, F.nc));
   CKS(dalloc(ctx, M, &ctx->pbar, (size_t)CGKS_PB * F.ngp));
@@ -290,12 +290,12 @@ cgks_status cgks_linearize(cgks_ctx* ctx) {
   ctx->lin_recompute = ctx->P.adjoint_recompute != 0;
   if (ctx->lin_recompute) {
     // keep the state; the reconstruction's transposed product is recomputed from it in every product
-    if (!ctx->aWG) CKS(dalloc(ctx, ctx->mesh_allocs, &ctx->aWG, (size_t)21 * F.nc));
+    if (!ctx->aWG) CKS(dalloc(ctx, ctx->adj_allocs, &ctx->aWG, (size_t)21 * F.nc));
     CK(cudaMemcpyAsync(ctx->aWG, ctx->W, sizeof(double) * 5 * F.nc, cudaMemcpyDeviceToDevice, ctx->stream));
     CK(cudaMemcpyAsync(ctx->aWG + 5 * F.nc, ctx->G, sizeof(double) * 15 * F.nc, cudaMemcpyDeviceToDevice, ctx->stream));
     CK(cudaMemcpyAsync(ctx->aWG + 20 * F.nc, ctx->alpha, sizeof(double) * F.nc, cudaMemcpyDeviceToDevice, ctx->stream));
   } else {
-    if (!ctx->Jr) CKS(dalloc(ctx, ctx->mesh_allocs, &ctx->Jr, (size_t)CGKS_RJ_ROWS * F.nc));
+    if (!ctx->Jr) CKS(dalloc(ctx, ctx->adj_allocs, &ctx->Jr, (size_t)CGKS_RJ_ROWS * F.nc));
     k_recon_jac<<<grid_for(F.nc, 32), 192, 0, ctx->stream>>>(ra, ctx->Jr);
   }
   PointArgs pa{F.ngp, F.nf, F.nc, F.gp_face, F.fL, F.fR, F.ftag, F.gp_x, F.gp_A, F.fshift, F.ctr, ctx->rc,
@@ -454,7 +454,7 @@ cgks_status cgks_adjoint_solve(cgks_ctx* ctx, const double* dJ_du, int method, i
   if (!(gn > 0.0)) {
     rel = 0.0;
   } else if (method == 1) {
-    if (!ctx->akry) CKS(dalloc(ctx, ctx->mesh_allocs, &ctx->akry, (size_t)(kGmresM + 1) * 20 * nc));
+    if (!ctx->akry) CKS(dalloc(ctx, ctx->adj_allocs, &ctx->akry, (size_t)(kGmresM + 1) * 20 * nc));
     CKS(gmres(ctx, mu, g, gn, max_iters, tol, &it, &rel));
   } else {
     const int check = 25;

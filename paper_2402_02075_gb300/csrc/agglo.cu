@@ -391,11 +391,7 @@ static cgks_status build_c2f(cgks_ctx* ctx, std::vector<void*>& M, std::vector<v
 // one coarsening pass P -> Q with map[P.nc]
 static cgks_status coarsen_pass(cgks_ctx* ctx, const Level& P, Level& Q, int32_t* map) {
   std::vector<void*> tmp;
-  struct Guard {
-    cgks_ctx* ctx;
-    std::vector<void*>& t;
-    ~Guard() { free_list(ctx, t); }
-  } guard{ctx, tmp};
+  const FreeList guard{ctx, tmp};
   auto& M = ctx->mesh_allocs;
   cudaStream_t st = ctx->stream;
   const int B = 256;
@@ -507,6 +503,7 @@ cgks_status build_levels(cgks_ctx* ctx) {
     cur.f2c = comp;
     cur.nc_finer = prev.nc;
     std::vector<void*> tmp;
+    const FreeList guard{ctx, tmp};
     int32_t *cnt, *cursor;
     CKS(dalloc(ctx, tmp, &cnt, cur.nc));
     CKS(dalloc(ctx, tmp, &cursor, cur.nc));
@@ -516,7 +513,6 @@ cgks_status build_levels(cgks_ctx* ctx) {
     CKS(dalloc(ctx, M, &cur.agg, tot));
     k_member_fill<<<grid_for(prev.nc, 256), 256, 0, st>>>(prev.nc, comp, cur.agg_ptr, cursor, cur.agg);
     k_sort_segments<<<grid_for(cur.nc, 128), 128, 0, st>>>(cur.nc, cur.agg_ptr, cur.agg);
-    free_list(ctx, tmp);
     ctx->L.push_back(cur);
   }
   for (Level& L : ctx->L) {

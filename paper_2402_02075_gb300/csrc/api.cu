@@ -20,60 +20,28 @@ cgks_status cgks_fail(cgks_ctx* c, cgks_status s, const std::string& msg) {
   return s;
 }
 
-// Device memory of a context.  Freed blocks stay with the context and serve its later allocations: a mesh
-// upload takes about 150 arrays, most of them temporary, and cudaMalloc and cudaFree (which waits for the
-// device) cost more than its kernels on small meshes; a step with a norm history took two of them.
-// Every use is on the context's stream, so a block is reused in stream order.  An upload gives back what
-// is above kPoolKeep at its end, and an allocation that fails gives back everything and tries again.
-static constexpr size_t kPoolKeep = (size_t)256 << 20;
-
-static void pool_trim(cgks_ctx* ctx, size_t keep) {
-  auto& pool = ctx->pool;
-  size_t total = 0;
-  for (const PoolBlock& b : pool) total += b.bytes;
-  std::sort(pool.begin(), pool.end(), [](const PoolBlock& x, const PoolBlock& y) { return x.bytes < y.bytes; });
-  while (!pool.empty() && total > keep) {
-    total -= pool.back().bytes;
-    ctx->block_bytes.erase(pool.back().p);
-    cudaFree(pool.back().p);
-    pool.pop_back();
-  }
-}
-
+// Device memory of a context (device_pool.h): a mesh upload takes about 150 arrays, most of them temporary, and
+// cudaMalloc and cudaFree (which waits for the device) cost more than its kernels on small meshes; a step
+// with a norm history took two of them.
 cgks_status dev_alloc(cgks_ctx* ctx, std::vector<void*>& list, void** p, size_t bytes) {
-  *p = nullptr;
-  const size_t want = (bytes + 511) / 512 * 512;
-  auto& pool = ctx->pool;
-  size_t best = pool.size();
-  for (size_t k = 0; k < pool.size(); ++k)  // the smallest block that fits without wasting more than half of it
-    if (pool[k].bytes >= want && pool[k].bytes <= 2 * want && (best == pool.size() || pool[k].bytes < pool[best].bytes)) best = k;
-  if (best < pool.size()) {
-    *p = pool[best].p;
-    pool[best] = pool.back();
-    pool.pop_back();
-  } else {
-    cudaError_t e = cudaMalloc(p, want);
-    if (e != cudaSuccess) {
-      cudaGetLastError();
-      pool_trim(ctx, 0);
-      e = cudaMalloc(p, want);
-    }
-    if (e != cudaSuccess) {
-      cudaGetLastError();
-      *p = nullptr;
-      return cgks_fail(ctx, CGKS_ENOMEM, std::string("cudaMalloc of ") + std::to_string(bytes) + " bytes: " +
-                                             cudaGetErrorString(e));
-    }
-    ctx->block_bytes[*p] = want;
+  const cudaError_t e = ctx->pool.take(p, bytes);
+  if (e != cudaSuccess)
+    return cgks_fail(ctx, CGKS_ENOMEM, std::string("cudaMalloc of ") + std::to_string(bytes) + " bytes: " +
+                                           cudaGetErrorString(e));
+  try {
+    list.push_back(*p);
+  } catch (const std::bad_alloc&) {
+    ctx->pool.give(*p);
+    *p = nullptr;
+    return cgks_fail(ctx, CGKS_ENOMEM, "host allocation");
   }
-  list.push_back(*p);
-  const cudaError_t e = cudaMemsetAsync(*p, 0, bytes, ctx->stream);
-  if (e != cudaSuccess) return cgks_fail(ctx, CGKS_ECUDA, cudaGetErrorString(e));
+  const cudaError_t z = cudaMemsetAsync(*p, 0, bytes, ctx->stream);
+  if (z != cudaSuccess) return cgks_fail(ctx, CGKS_ECUDA, cudaGetErrorString(z));
   return CGKS_OK;
 }
 
-void free_list(cgks_ctx* ctx, std::vector<void*>& list) {
-  for (void* p : list) ctx->pool.push_back({p, ctx->block_bytes[p]});
+void free_list(cgks_ctx* ctx, std::vector<void*>& list) noexcept {
+  for (void* p : list) ctx->pool.give(p);
   list.clear();
 }
 
@@ -182,6 +150,7 @@ cgks_status scan_exclusive(cgks_ctx* ctx, const int32_t* in, int32_t* out, int64
   }
   const int64_t ntiles = (n + SCAN_TILE - 1) / SCAN_TILE;
   std::vector<void*> tmp;
+  const FreeList guard{ctx, tmp};
   int32_t* ts;
   int64_t* dtot;
   CKS(dalloc(ctx, tmp, &ts, ntiles));
@@ -195,7 +164,6 @@ cgks_status scan_exclusive(cgks_ctx* ctx, const int32_t* in, int32_t* out, int64
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     *total = *ctx->h_count;
   }
-  free_list(ctx, tmp);
   if (e != cudaSuccess) return cgks_fail(ctx, CGKS_ECUDA, std::string("scan: ") + cudaGetErrorString(e));
   return CGKS_OK;
 }
@@ -371,9 +339,9 @@ cgks_status cgks_destroy(cgks_ctx* ctx) {
   }
   for (cudaEvent_t e : ctx->gev)
     if (e) cudaEventDestroy(e);
+  free_list(ctx, ctx->adj_allocs);
   free_list(ctx, ctx->mesh_allocs);
   free_list(ctx, ctx->ctx_allocs);
-  pool_trim(ctx, 0);
   if (ctx->h_err) cudaFreeHost(ctx->h_err);
   if (ctx->h_count) cudaFreeHost(ctx->h_count);
   if (ctx->h_nrm) cudaFreeHost(ctx->h_nrm);
@@ -406,8 +374,25 @@ cgks_status cgks_mesh_upload(cgks_ctx* ctx, int64_t n_nodes, const double* xyz, 
       if (bface_ptr[b + 1] < bface_ptr[b]) return cgks_fail(ctx, CGKS_EMESH, "bface_ptr not monotone");
   }
   CK(cudaStreamSynchronize(ctx->stream));
+  // A mesh of the same sizes (the same one with displaced nodes: a design point, a shape derivative) asks for
+  // the same arrays, so the present mesh's stay for it; else they are given back before the new mesh is
+  // built.  What the upload leaves over, or all it built where it fails, goes back on every way out.
+  // Second uploads with and without: 377,856 cells 11.7 ms and 16.1, 1.51 M cells 38.4 and 50.1.
+  struct Scope {
+    cgks_ctx* ctx;
+    ~Scope() {
+      cudaStreamSynchronize(ctx->stream);
+      if (!ctx->has_mesh) free_list(ctx, ctx->mesh_allocs);
+      ctx->pool.hold(false);
+    }
+  };
+  const bool same = ctx->has_mesh && (int64_t)ctx->h_xyz.size() == 3 * n_nodes && (int64_t)ctx->h_ctype.size() == n_cells &&
+                    (int64_t)ctx->h_cnodes.size() == cell_ptr[n_cells] && (int64_t)ctx->h_btag.size() == n_bfaces &&
+                    (int64_t)ctx->h_pairs.size() == 2 * n_periodic;
+  free_list(ctx, ctx->adj_allocs);
+  ctx->pool.hold(same);
+  const Scope scope{ctx};
   free_list(ctx, ctx->mesh_allocs);
-  // the adjoint's arrays were in mesh_allocs
   ctx->Jp = ctx->Jr = ctx->adt = ctx->pbar = ctx->aself = ctx->arec = ctx->avec = ctx->apart = ctx->akry = nullptr;
   ctx->ajc = ctx->acb = ctx->aWG = nullptr;
   ctx->lin_recompute = false;
@@ -448,7 +433,6 @@ cgks_status cgks_mesh_upload(cgks_ctx* ctx, int64_t n_nodes, const double* xyz, 
   CKS(dalloc(ctx, M, &ctx->ffl, 5 * F.nf));
   CKS(dalloc(ctx, M, &ctx->ffl32, 5 * F.nf));
   CK(cudaStreamSynchronize(ctx->stream));
-  pool_trim(ctx, kPoolKeep);
   ctx->has_mesh = true;
   return CGKS_OK;
 }
@@ -590,13 +574,13 @@ static cgks_status run_iterations(cgks_ctx* ctx, int n, double* norm_hist, bool 
   NEED_STATE();
   if (n < 0) return cgks_fail(ctx, CGKS_EINVAL, "negative iteration count");
   std::vector<void*> tmp;
+  const FreeList guard{ctx, tmp};
   double* hist = nullptr;
   if (norm_hist && n > 0) CKS(dalloc(ctx, tmp, &hist, n));
   cgks_status s = CGKS_OK;
   for (int k = 0; k < n && s == CGKS_OK; ++k) s = multigrid ? vcycle_once(ctx, hist ? hist + k : nullptr)
                                                             : step_once(ctx, hist ? hist + k : nullptr);
   if (s == CGKS_OK && hist) s = read_norm(ctx, hist, norm_hist, n);
-  free_list(ctx, tmp);
   CKS(s);
   ctx->iters += n;
   return check_device_error(ctx, name);
@@ -672,6 +656,7 @@ cgks_status cgks_steady_solve(cgks_ctx* ctx, int multigrid, double drop, int64_t
   if (!(drop > 0.0) || max_iters < 1) return cgks_fail(ctx, CGKS_EINVAL, "drop must be > 0 and max_iters >= 1");
   const int check_every = 10;
   std::vector<void*> tmp;
+  const FreeList guard{ctx, tmp};
   double* hist;
   CKS(dalloc(ctx, tmp, &hist, check_every));
   std::vector<double> h(check_every);
@@ -703,7 +688,6 @@ cgks_status cgks_steady_solve(cgks_ctx* ctx, int multigrid, double drop, int64_t
   }
   if (exec) cudaGraphExecDestroy(exec);
   const double sec = std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();
-  free_list(ctx, tmp);
   CKS(s);
   ctx->iters += it;
   if (iters_done) *iters_done = it;

@@ -5,10 +5,10 @@
 
 #include <cstdint>
 #include <string>
-#include <unordered_map>
 #include <vector>
 
 #include "cgks.h"
+#include "device_pool.h"
 
 #define CGKS_MAXNF 6          // faces of a hexahedron
 #define CGKS_KOP 216          // reconstruction operator entries per cell: 9 x (4 * 6)
@@ -16,6 +16,7 @@
 #define CGKS_GPR 14           // Gauss-point record: flux x weight (5), interface state (5), area vector (3), alpha
 #define CGKS_AUX 8            // per-cell constants of the smoothness indicators
 #define CGKS_NORM_PARTS 1024  // per-block parts of a reduction (nrm_part)
+#define CGKS_POOL_KEEP ((size_t)256 << 20)  // device memory a context holds beyond its arrays, at most
 #define CGKS_AGG_CAP 256      // records per coarse cell while building coarse faces
 #define HD __host__ __device__ __forceinline__
 
@@ -111,10 +112,19 @@ struct ProfRec {
   double units, bytes;
 };
 
-// a freed device block that the context keeps
-struct PoolBlock {
-  void* p;
-  size_t bytes;
+struct DeviceMemory {  // the device, for DevicePool
+  using Error = cudaError_t;
+  static constexpr Error ok = cudaSuccess, out_of_memory = cudaErrorMemoryAllocation;
+  const cudaStream_t* stream;
+  Error alloc(void** p, size_t bytes) {
+    const Error e = cudaMalloc(p, bytes);
+    if (e != ok) cudaGetLastError();
+    return e;
+  }
+  void release(void* p) {
+    cudaStreamSynchronize(*stream);  // work that still uses the block
+    cudaFree(p);
+  }
 };
 
 struct cgks_ctx {
@@ -146,7 +156,7 @@ struct cgks_ctx {
   double r1 = 0.0;
   int64_t iters = 0;
   // adjoint: the stored linearisation at the state of the last cgks_linearize, its time steps,
-  // and the work arrays of the transposed products (in mesh_allocs)
+  // and the work arrays of the transposed products (in adj_allocs)
   double *Jp = nullptr, *Jr = nullptr, *adt = nullptr;
   double* aWG = nullptr;       // [21][nc] (W, grad W, alpha) at cgks_linearize (adjoint_recompute 1)
   bool lin_recompute = false;  // the last cgks_linearize stored no reconstruction linearisation
@@ -160,9 +170,9 @@ struct cgks_ctx {
   std::vector<int64_t> h_cptr, h_bptr;
   std::vector<int32_t> h_cnodes, h_bnodes, h_btag, h_pairs;
   std::vector<void*> mesh_allocs;   // freed on re-upload / destroy
+  std::vector<void*> adj_allocs;    // the adjoint's, freed with the mesh
   std::vector<void*> ctx_allocs;    // freed on destroy
-  std::vector<PoolBlock> pool;      // freed blocks, and the size of every block the context holds
-  std::unordered_map<void*, size_t> block_bytes;
+  DevicePool<DeviceMemory> pool{DeviceMemory{&stream}, CGKS_POOL_KEEP};
   // kernel timing (cgks_profile): event pairs per kernel kind, with the units and the algorithmic
   // bytes of each recorded launch
   bool prof = false;
@@ -204,7 +214,12 @@ cgks_status dalloc(cgks_ctx* ctx, std::vector<void*>& list, T** p, size_t count)
   return dev_alloc(ctx, list, reinterpret_cast<void**>(p), sizeof(T) * (count ? count : 1));
 }
 // the blocks of `list` back to the context
-void free_list(cgks_ctx* ctx, std::vector<void*>& list);
+void free_list(cgks_ctx* ctx, std::vector<void*>& list) noexcept;
+struct FreeList {  // on every way out of a scope
+  cgks_ctx* ctx;
+  std::vector<void*>& list;
+  ~FreeList() { free_list(ctx, list); }
+};
 
 inline unsigned grid_for(int64_t n, int block) { return (unsigned)((n + block - 1) / block); }
 

@@ -337,11 +337,8 @@ cgks_status lusgs_colors(cgks_ctx* ctx, int l) {
   CKS(dalloc(ctx, M, &B.Dg, L.nc));
   CKS(dalloc(ctx, M, &B.sweep, sizeof(SweepRecord) / sizeof(double) * L.nc));
   std::vector<void*> tmp;
-  cgks_status s = dalloc(ctx, tmp, &sel, L.nc);
-  if (s != CGKS_OK) {
-    free_list(ctx, tmp);
-    return s;
-  }
+  const FreeList guard{ctx, tmp};
+  CKS(dalloc(ctx, tmp, &sel, L.nc));
   std::vector<int32_t> minus1(L.nc, -1);
   cudaError_t e = cudaMemcpyAsync(B.color, minus1.data(), sizeof(int32_t) * L.nc, cudaMemcpyHostToDevice, st);
   // each round colours at least the uncoloured cell of highest priority, so nc rounds bound it
@@ -356,7 +353,6 @@ cgks_status lusgs_colors(cgks_ctx* ctx, int l) {
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e == cudaSuccess) left = *ctx->h_count;
   }
-  free_list(ctx, tmp);
   CK(e);
   if (left > 0) return cgks_fail(ctx, CGKS_EINVAL, "LU-SGS colouring did not finish");
   // colour-major order, ascending cell id within a colour (counting sort on the host)

@@ -590,11 +590,7 @@ cgks_status build_fine_mesh(cgks_ctx* ctx, int64_t n_nodes, const double* xyz, i
                             const int64_t* bface_ptr, const int32_t* bface_nodes, const int32_t* bface_tag,
                             const int32_t* periodic_pairs, int64_t n_periodic) {
   std::vector<void*> tmp;
-  struct Guard {
-    cgks_ctx* ctx;
-    std::vector<void*>& t;
-    ~Guard() { free_list(ctx, t); }
-  } guard{ctx, tmp};
+  const FreeList guard{ctx, tmp};
   cudaStream_t st = ctx->stream;
   Fine& F = ctx->F;
   auto& M = ctx->mesh_allocs;
