@@ -366,11 +366,7 @@ static cgks_status read_count(cgks_ctx* ctx, int64_t* out) {
 static cgks_status csr_from_counts(cgks_ctx* ctx, std::vector<void*>& M, int32_t* cnt, int64_t n, int32_t** ptr,
                                    int64_t* total) {
   CKS(dalloc(ctx, M, ptr, n + 1));
-  CKS(scan_exclusive(ctx, cnt, *ptr, n, total));
-  const int32_t t32 = (int32_t)*total;
-  // (pageable: copied out of t32 before the call returns)
-  CK(cudaMemcpyAsync(*ptr + n, &t32, sizeof(int32_t), cudaMemcpyHostToDevice, ctx->stream));
-  return CGKS_OK;
+  return scan_exclusive(ctx, cnt, *ptr, n, total, true);
 }
 
 static cgks_status build_c2f(cgks_ctx* ctx, std::vector<void*>& M, std::vector<void*>& tmp, Level& Q) {

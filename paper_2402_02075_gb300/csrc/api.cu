@@ -137,12 +137,14 @@ __global__ void k_scan_tile_sums(int32_t* tile_sum, int64_t ntiles, int64_t* tot
   if (threadIdx.x == 0) *total = tot;
 }
 
-__global__ void k_scan_add(int32_t* out, int64_t n, const int32_t* tile_sum) {
+// end: the total into out[n] as well (the last offset of a CSR)
+__global__ void k_scan_add(int32_t* out, int64_t n, const int32_t* tile_sum, const int64_t* total, int end) {
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i < n) out[i] += tile_sum[i / SCAN_TILE];
+  if (i == 0 && end) out[n] = (int32_t)*total;
 }
 
-cgks_status scan_exclusive(cgks_ctx* ctx, const int32_t* in, int32_t* out, int64_t n, int64_t* total) {
+cgks_status scan_exclusive(cgks_ctx* ctx, const int32_t* in, int32_t* out, int64_t n, int64_t* total, bool end) {
   cudaStream_t st = ctx->stream;
   if (n == 0) {
     if (total) *total = 0;
@@ -157,7 +159,7 @@ cgks_status scan_exclusive(cgks_ctx* ctx, const int32_t* in, int32_t* out, int64
   CKS(dalloc(ctx, tmp, &dtot, 1));
   k_scan_tiles<<<(unsigned)ntiles, SCAN_THREADS, 0, st>>>(in, out, n, ts);
   k_scan_tile_sums<<<1, SCAN_THREADS, 0, st>>>(ts, ntiles, dtot);
-  k_scan_add<<<grid_for(n, 256), 256, 0, st>>>(out, n, ts);
+  k_scan_add<<<grid_for(n, 256), 256, 0, st>>>(out, n, ts, dtot, end);
   cudaError_t e = cudaGetLastError();
   if (e == cudaSuccess && total) {
     e = cudaMemcpyAsync(ctx->h_count, dtot, sizeof(int64_t), cudaMemcpyDeviceToHost, st);

@@ -263,9 +263,10 @@ inline int spread_block(int64_t n, int max_block, int n_sm) {
   return (int)(b < 32 ? 32 : b);
 }
 
-// exclusive prefix sum of n int32 values (device), total returned through *total (host) when
-// non-null (synchronises).  Uses ctx scratch allocated on demand.
-cgks_status scan_exclusive(cgks_ctx* ctx, const int32_t* in, int32_t* out, int64_t n, int64_t* total);
+// exclusive prefix sum of n int32 values (device; end: and the total into out[n]), total returned through
+// *total (host) when non-null (synchronises).  Uses ctx scratch allocated on demand.
+cgks_status scan_exclusive(cgks_ctx* ctx, const int32_t* in, int32_t* out, int64_t n, int64_t* total,
+                           bool end = false);
 
 // entry points between translation units
 cgks_status build_fine_mesh(cgks_ctx* ctx, int64_t n_nodes, const double* xyz, int64_t n_cells, const int8_t* ctype,

@@ -675,9 +675,7 @@ cgks_status build_fine_mesh(cgks_ctx* ctx, int64_t n_nodes, const double* xyz, i
   CKS(dalloc(ctx, M, &F.gp_ptr, nf + 1));
   k_gp_count<<<grid_for(nf, B), B, 0, st>>>(nf, F.fL, F.flf, d_ct, gcnt);
   int64_t ngp = 0;
-  CKS(scan_exclusive(ctx, gcnt, F.gp_ptr, nf, &ngp));
-  int32_t ngp32 = (int32_t)ngp;
-  CK(cudaMemcpyAsync(F.gp_ptr + nf, &ngp32, sizeof(int32_t), cudaMemcpyHostToDevice, st));
+  CKS(scan_exclusive(ctx, gcnt, F.gp_ptr, nf, &ngp, true));
   F.ngp = ngp;
   Level L0;
   L0.nc = nc;
@@ -705,9 +703,7 @@ cgks_status build_fine_mesh(cgks_ctx* ctx, int64_t n_nodes, const double* xyz, i
   CKS(dalloc(ctx, M, &F.c2f_ptr, nc + 1));
   k_types_to_int<<<grid_for(nc, B), B, 0, st>>>(nc, d_ct, tcnt);
   int64_t nlinks = 0;
-  CKS(scan_exclusive(ctx, tcnt, F.c2f_ptr, nc, &nlinks));
-  int32_t nl32 = (int32_t)nlinks;
-  CK(cudaMemcpyAsync(F.c2f_ptr + nc, &nl32, sizeof(int32_t), cudaMemcpyHostToDevice, st));
+  CKS(scan_exclusive(ctx, tcnt, F.c2f_ptr, nc, &nlinks, true));
   CKS(dalloc(ctx, M, &F.c2f, nlinks));
   k_fill_c2f<<<grid_for(nc, B), B, 0, st>>>(nc, d_ct, F.cf, F.c2f_ptr, F.c2f);
   CKS(check_device_error(ctx, "geometry"));
