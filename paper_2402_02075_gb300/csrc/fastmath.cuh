@@ -122,10 +122,11 @@ HD bool positive(double x) {
 #endif
 }
 
-// the smaller of two positive numbers, by an integer comparison (a NaN loses, as with fmin)
+// the smaller of two numbers that are not negative, by an integer comparison (unsigned, so that a NaN of
+// either sign loses, as with fmin)
 HD double min_positive(double a, double b) {
 #ifdef __CUDA_ARCH__
-  return __double_as_longlong(b) < __double_as_longlong(a) ? b : a;
+  return (unsigned long long)__double_as_longlong(b) < (unsigned long long)__double_as_longlong(a) ? b : a;
 #else
   return fmin(a, b);
 #endif
