@@ -4,10 +4,12 @@
 // GB300 issues 2 FP64 operations per clock and SM (conversions between double and the other types
 // count as FP64 operations too), against 64 to 128 integer and FP32 ones, so what these functions cost
 // is their FP64 operations.  Measured on GB300 against a chain of multiply-adds, CUDA's 1/x takes
-// 5.6 of them, rsqrt 5, exp 16 and erfc 60; here the reciprocal takes 3, rsqrt 5 and exp with erfc
-// together 22, the rest of each being integer and FP32 work on the idle pipes:
-//  - reciprocals: the hardware's approximation (about 20 bits) and one cubic (Halley-type) correction
-//    r (1 + e + e^2), e = 1 - x r, whose remainder e^3 is below 2^-56;
+// 5.6 of them, rsqrt 5, exp 16 and erfc 60; here the reciprocal takes 3 and exp with erfc together 22, the
+// rest of each being integer and FP32 work on the idle pipes (rsqrt is CUDA's: a cubic correction of the
+// hardware's approximation takes 5 as well, and the residuals of 576 to 1.51 M cells the same time):
+//  - reciprocal: the hardware's approximation (20 bits) and one cubic step of Householder's method (A. S.
+//    Householder, The Numerical Treatment of a Single Nonlinear Equation, 1970), r (1 + e + e^2) with
+//    e = 1 - x r, whose remainder e^3 is below 2^-55;
 //  - exp(-a^2) table-driven (P. T. P. Tang, ACM TOMS 15, 1989): a^2 = (n ln 2)/64 + r with n found in
 //    FP32, 2^(-n/64) from a table of 64 and the Taylor polynomial of exp(-r), |r| <= ln 2/128; a^2 is
 //    never rounded, the reduction is one fused multiply-add;
@@ -55,10 +57,7 @@ HD double fast_rcp(double x) {
 
 HD double fast_rsqrt(double x) {
 #ifdef __CUDA_ARCH__
-  double y;
-  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-  const double e = fma(-(x * y), y, 1.0);
-  return fma(y * e, fma(0.375, e, 0.5), y);
+  return rsqrt(x);
 #else
   return 1.0 / sqrt(x);
 #endif
