@@ -270,14 +270,19 @@ __global__ void k_fe_update(int64_t nc, const double* __restrict__ dt, const dou
 }
 
 // coarse state = sum V_i W_i / V_c (and its copy W^0) and coarse defect = sum (R_i [+ F_i]) over the
-// finer cells of each coarse cell, in ascending finer-cell order
-// (a thread per coarse cell and variable: an agglomerate has a handful of members, so the time of a small
-// launch is that of the dependent loads of one thread; four members are in flight at once.  With one
-// thread for all five variables 442 cells took 10.6 us against 6.3 now, 5,079 cells 11.6 against 6.9,
-// 1.1 M cells 73 against 86, 0.05 % of that V-cycle)
-__global__ void k_restrict(int64_t ncc, int64_t ncf, const int32_t* __restrict__ aptr, const int32_t* __restrict__ agg,
-                           const double* __restrict__ vf, const double* __restrict__ vc, const double* Wf,
-                           const double* Rf, const double* Ff, double* Wc, double* Wc0, double* Rc) {
+// finer cells of each coarse cell, in ascending finer-cell order, by one of two kernels with the same sums:
+// a thread per coarse cell and variable where the level is small, since an agglomerate has a handful of
+// members and the time of a small launch is that of the dependent loads of one thread (four members
+// are in flight at once); a thread for all five variables above RESTRICT_CELLS coarse cells per SM, since
+// there the member lists and volumes are read from memory once instead of five times.  Per launch (the
+// mean of both levels' restrictions), by variable and by cell: 340 cells 6.6 and 10.8 us, 33,945 cells 11.3
+// and 13.3, 143,000 cells 26.6 and 26.6, 205,000 cells 35.8 and 32.9, 554,000 cells 83.9 and 71.7.
+#define RESTRICT_CELLS 1024
+
+__global__ void k_restrict_vars(int64_t ncc, int64_t ncf, const int32_t* __restrict__ aptr,
+                                const int32_t* __restrict__ agg, const double* __restrict__ vf,
+                                const double* __restrict__ vc, const double* Wf, const double* Rf, const double* Ff,
+                                double* Wc, double* Wc0, double* Rc) {
   const int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   const int q = blockIdx.y;
   const bool live = c < ncc;
@@ -307,6 +312,50 @@ __global__ void k_restrict(int64_t ncc, int64_t ncf, const int32_t* __restrict__
   Wc[q * ncc + c] = w;
   Wc0[q * ncc + c] = w;
   Rc[q * ncc + c] = r;
+}
+
+__global__ void k_restrict_cells(int64_t ncc, int64_t ncf, const int32_t* __restrict__ aptr,
+                                 const int32_t* __restrict__ agg, const double* __restrict__ vf,
+                                 const double* __restrict__ vc, const double* Wf, const double* Rf, const double* Ff,
+                                 double* Wc, double* Wc0, double* Rc) {
+  const int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  const bool live = c < ncc;
+  double w[5] = {0, 0, 0, 0, 0}, r[5] = {0, 0, 0, 0, 0};
+  const int32_t e = live ? aptr[c + 1] : 0, k0 = live ? aptr[c] : 0;
+  const double rv = live ? 1.0 / vc[c] : 0.0;
+  wait_prior();
+  if (!live) return;
+  for (int32_t k = k0; k < e; ++k) {
+    const int64_t i = agg[k];
+    const double v = vf[i];
+#pragma unroll
+    for (int q = 0; q < 5; ++q) {
+      w[q] += v * Wf[q * ncf + i];
+      r[q] += Ff ? Rf[q * ncf + i] + Ff[q * ncf + i] : Rf[q * ncf + i];
+    }
+  }
+#pragma unroll
+  for (int q = 0; q < 5; ++q) {
+    w[q] *= rv;
+    Wc[q * ncc + c] = w[q];
+    Wc0[q * ncc + c] = w[q];
+    Rc[q * ncc + c] = r[q];
+  }
+}
+
+// restriction from a finer level of n cells (volumes vf, state W, residual R and forcing F or null) to level l
+static cgks_status restrict_to(cgks_ctx* ctx, int l, int64_t n, const double* vf, const double* W, const double* R,
+                               const double* F) {
+  const Level& L = ctx->L[l];
+  CoarseBuf& B = ctx->C[l];
+  ProfScope ps(ctx, PK_RESTRICT, (double)n, n * (F ? 132.0 : 92.0) + L.nc * 132.0);
+  if (L.nc <= (int64_t)ctx->n_sm * RESTRICT_CELLS)
+    CK(launch_overlapped(k_restrict_vars, dim3(grid_for(L.nc, 128), 5), 128, ctx->stream, L.nc, n, L.agg_ptr, L.agg, vf,
+                         L.vol, W, R, F, B.W, B.W0, B.Rs));
+  else
+    CK(launch_overlapped(k_restrict_cells, grid_for(L.nc, 256), 256, ctx->stream, L.nc, n, L.agg_ptr, L.agg, vf, L.vol, W,
+                         R, F, B.W, B.W0, B.Rs));
+  return CGKS_OK;
 }
 
 // W_f += r (W_c - W_c^0) (injection, r = correction_relax); a correction that would make rho or p
@@ -580,7 +629,6 @@ static cgks_status coarse_smooth(cgks_ctx* ctx, int l, bool first) {
 static cgks_status coarse_cycle(cgks_ctx* ctx, int l) {
   const Level& L = ctx->L[l];
   CoarseBuf& B = ctx->C[l];
-  cudaStream_t st = ctx->stream;
   if (ctx->P.coarse_steps == 0 && ctx->P.precision == 0) {  // the forcing alone
     CKS(coarse_residual(ctx, l));
     CKS(coarse_forcing(ctx, l));
@@ -590,11 +638,7 @@ static cgks_status coarse_cycle(cgks_ctx* ctx, int l) {
     const Level& Cn = ctx->L[l + 1];
     CoarseBuf& N = ctx->C[l + 1];
     CKS(coarse_residual(ctx, l));
-    {
-      ProfScope ps(ctx, PK_RESTRICT, (double)L.nc, L.nc * 132.0 + Cn.nc * 132.0);
-      CK(launch_overlapped(k_restrict, dim3(grid_for(Cn.nc, 128), 5), 128, st, Cn.nc, L.nc, Cn.agg_ptr, Cn.agg, L.vol,
-                           Cn.vol, B.W, B.R, forcing(ctx, B), N.W, N.W0, N.Rs));
-    }
+    CKS(restrict_to(ctx, l + 1, L.nc, L.vol, B.W, B.R, forcing(ctx, B)));
     CKS(coarse_cycle(ctx, l + 1));
     CKS(prolong(ctx, l, Cn.f2c, Cn.nc, N.W, N.W0, B.W));
     for (int s = 0; s < ctx->P.post; ++s) CKS(coarse_smooth(ctx, l, false));
@@ -612,7 +656,6 @@ cgks_status step_once(cgks_ctx* ctx, double* norm_dev) {
 
 // one V-cycle (Sec. 4.2)
 cgks_status vcycle_once(cgks_ctx* ctx, double* norm_dev) {
-  cudaStream_t st = ctx->stream;
   const int pre = ctx->P.pre > 0 ? ctx->P.pre : 1;
   for (int s = 0; s < pre; ++s) CKS(step_once(ctx, s == 0 ? norm_dev : nullptr));
   if (ctx->L.size() <= 1) return CGKS_OK;
@@ -623,11 +666,7 @@ cgks_status vcycle_once(cgks_ctx* ctx, double* norm_dev) {
   // factor is formed)
   CKS(fine_fluxes(ctx, ctx->W, ctx->G, ctx->alpha, false));
   CKS(fine_gather(ctx, ctx->W, nullptr, ctx->res, nullptr, nullptr, 0));
-  {
-    ProfScope ps(ctx, PK_RESTRICT, (double)F.nc, F.nc * 92.0 + C1.nc * 132.0);
-    CK(launch_overlapped(k_restrict, dim3(grid_for(C1.nc, 128), 5), 128, st, C1.nc, F.nc, C1.agg_ptr, C1.agg,
-                         ctx->L0c.vol, C1.vol, ctx->W, ctx->res, nullptr, B1.W, B1.W0, B1.Rs));
-  }
+  CKS(restrict_to(ctx, 1, F.nc, ctx->L0c.vol, ctx->W, ctx->res, nullptr));
   CKS(coarse_cycle(ctx, 1));
   CKS(prolong(ctx, 0, C1.f2c, C1.nc, B1.W, B1.W0, ctx->W));
   for (int s = 0; s < ctx->P.post; ++s) CKS(step_once(ctx, nullptr));

@@ -98,7 +98,7 @@ enum ProfKind {
   PK_COARSE_DT,    // k_coarse_dt: cells
   PK_FORCING,      // k_forcing: cells
   PK_FE_UPDATE,    // k_fe_update: cells
-  PK_RESTRICT,     // k_restrict: cells of the finer level
+  PK_RESTRICT,     // k_restrict_vars, k_restrict_cells: cells of the finer level
   PK_PROLONG,      // k_prolong / k_prolong_smooth: cells of the finer level
   PK_KFVS_JVP,     // k_kfvs_jvp_faces: faces
   PK_NORM,         // k_norm_partial + k_norm_final: cells
