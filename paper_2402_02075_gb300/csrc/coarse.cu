@@ -78,12 +78,19 @@ __global__ void k_kfvs_jvp_faces(int64_t nf, const int32_t* __restrict__ fL, con
 // ---- sums over a coarse cell's faces -------------------------------------------------------------
 //
 // A coarse cell has 10 to 40 faces, read through its face list: a thread that walks them alone takes
-// as many dependent trips to L2.  Where the level has less than one warp of cells per sub-partition,
-// eight threads share a cell's faces and add their partial sums in a fixed tree; above that one thread
-// per cell is faster, since a warp's FP64 addition takes as long for a few active lanes as for 32.
-// Measured per launch of k_coarse_step with one thread and with eight: 2,357 cells 21.8 and 12.0 us,
-// 5,982 cells 22.0 and 11.3, 37,331 cells 34 and 55, 0.58 M cells 232 and 782.
-inline int cell_lanes(int64_t nc, int n_sm) { return nc < (int64_t)n_sm * 4 * 32 ? 8 : 1; }
+// as many dependent trips to L2.  Where a level is small, eight threads share a cell's faces and add their
+// partial sums in a fixed tree; above that one thread per cell is faster, since a warp's FP64 addition takes
+// as long for a few active lanes as for 32.  Per launch, with one thread and with eight, in us (the mean
+// over the launches of two levels, whose mean number of cells is given):
+//   step       9,500 cells 23.5 and 21.8,  11,200 23.7 and 24.6,  14,700 23.9 and 30.4,  21,300 26.0 and 40.3
+//   time step 11,200 cells 16.3 and 13.4,  14,700 15.8 and 15.7,  17,100 16.8 and 18.2,  21,300 15.8 and 19.9
+//   gather    11,400 cells 21.9 and 14.9,  18,500 22.2 and 20.7,  21,300 20.1 and 19.3,  26,200 20.5 and 20.9
+// The step's line depends on the faces per cell: 10,500 cells on a first coarse level (about 12 faces), 13,700
+// on a second (about 22); it is put where one thread is the faster on both.
+#define STEP_LANE_CELLS 96  // cells per SM below which eight threads share a cell
+#define DT_LANE_CELLS 96
+#define GATHER_LANE_CELLS 128
+inline bool share_cells(int64_t nc, int n_sm, int cells) { return nc < (int64_t)n_sm * cells; }
 
 template <int LANES>
 __device__ __forceinline__ double lane_sum(double v) {
@@ -500,7 +507,7 @@ static cgks_status kfvs_gather(cgks_ctx* ctx, int lev, const T* ff, double* res)
   const Level& L = ctx->L[lev];
   ProfScope ps(ctx, PK_KFVS_GATHER, (double)L.nc,
                L.nc * 44.0 + (L.nf + L.n_int + L.n_per) * 4.0 + L.nf * (8.0 + 5.0 * sizeof(T)));
-  if (cell_lanes(L.nc, ctx->n_sm) == 8)
+  if (share_cells(L.nc, ctx->n_sm, GATHER_LANE_CELLS))
     CK(launch_overlapped(k_kfvs_gather<T, 8>, grid_for(8 * L.nc, 64), 64,
                          ctx->stream, L.nc, L.nf, L.c2f_ptr, L.c2f, L.fL, L.fR, ff, res));
   else
@@ -528,7 +535,7 @@ cgks_status coarse_dt(cgks_ctx* ctx, int lev, const double* W, double* dt) {
   const Level& L = ctx->L[lev];
   {
     ProfScope ps(ctx, PK_COARSE_DT, (double)L.nc, L.nc * 60.0 + (L.nf + L.n_int + L.n_per) * 4.0 + L.nf * 32.0);
-    if (cell_lanes(L.nc, ctx->n_sm) == 8)
+    if (share_cells(L.nc, ctx->n_sm, DT_LANE_CELLS))
       CK(launch_overlapped(k_coarse_dt<8>, grid_for(8 * L.nc, 64), 64,
                            ctx->stream, L.nc, L.nf, L.c2f_ptr, L.c2f, L.nS, L.area, L.vol, W, dt, ctx->P.gamma,
                            ctx->P.cfl_coarse));
@@ -589,7 +596,7 @@ static cgks_status coarse_step(cgks_ctx* ctx, int l, const T* ff, bool first) {
   ProfScope ps(ctx, GATHER ? PK_KFVS_GATHER : PK_COARSE_DT, (double)L.nc,
                L.nc * (first && GATHER ? 164.0 : 124.0) + (L.nf + L.n_int + L.n_per) * 4.0 +
                    L.nf * (32.0 + (GATHER ? 8.0 + 5.0 * sizeof(T) : 0.0)));
-  if (cell_lanes(L.nc, ctx->n_sm) == 8)
+  if (share_cells(L.nc, ctx->n_sm, STEP_LANE_CELLS))
     CK(launch_overlapped(k_coarse_step<T, 8, GATHER>, grid_for(8 * L.nc, 64), 64, ctx->stream, a, ff));
   else
     CK(launch_overlapped(k_coarse_step<T, 1, GATHER>, grid_for(L.nc, 128), 128, ctx->stream, a, ff));

@@ -123,8 +123,11 @@ __global__ void k_lusgs_lambda(int64_t nf, const int32_t* __restrict__ fL, const
 // clocks of its sub-partition, about 100 of them per face, and the loads are dependent).  LANES threads
 // share the faces and add their parts in a fixed tree: a quarter warp, or a whole warp where the
 // colour has so few cells that every sub-partition still gets at most two.  V-cycle of the 64x32x8 ramp
-// (8.4 k and 4 k coarse cells, 38 sweeps per step and level): 2.3 ms against 9.7.  The five sums of a
-// cell end in five of its lanes, each of which then does one variable's division.
+// (7,235 and 4,102 coarse cells, 18 and 20 sweeps per step): 2.3 ms against 9.7.  Two V-cycles by that rule,
+// with a quarter warp always and with a whole one always, since their records and scattered sums: 64x32x8 ramp
+// (colours of up to 1,613 cells) 3.50, 3.88 and 3.53 ms, 64x32x16 ramp (3,300) 5.82, 6.11 and 6.03, 96x4x69
+// boundary layer (12,284) 9.68, 9.80 and 11.25.  The five sums of a cell end in five of its lanes, each of
+// which then does one variable's division.
 template <int LANES>
 __device__ __forceinline__ double lane_sum(double v) {
 #pragma unroll
