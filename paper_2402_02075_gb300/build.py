@@ -16,7 +16,7 @@ OUT = os.path.join(HERE, "libcgks.so")
 BUILD = os.path.join(HERE, "_build")
 SOURCES = ["api.cu", "mesh.cu", "agglo.cu", "fine.cu", "coarse.cu", "lusgs.cu", "noalloc.cu", "adjoint.cu"]
 GENCODE = ["-gencode", "arch=compute_103a,code=sm_103a"]
-FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "--expt-relaxed-constexpr",
+FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-DCGKS_LIBRARY", "-Xcompiler", "-fPIC", "--expt-relaxed-constexpr",
          "-I" + os.path.join(ROOT, "include"), "-I" + CSRC]
 
 

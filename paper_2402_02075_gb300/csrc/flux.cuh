@@ -1,7 +1,7 @@
 // The time-dependent gas-kinetic flux of a Gauss point (Eq. 2nd-flux of the paper, Sec. 2.3-2.4) in FP64.
 //
 // The FP64 pipe bounds it, so the form is the one with the fewest FP64 instructions found so far.  It
-// evaluates the same integrals as point_flux (fine.cuh), which serves the other scalar types:
+// evaluates the same integrals as point_flux (flux_generic.cuh), the form that the tests compare it with:
 //  - gradients are primitive: for every direction k of the global frame (d rho, R_i = rho d u_i, d p).
 //    The micro-slope of a Maxwellian is diagonal in them: with the peculiar velocity u - U,
 //    h = p/rho and th = d p - h d rho,
@@ -33,6 +33,7 @@
 // The state dependence can be differentiated by dual numbers: S is the scalar of a side's state, T of
 // what both sides and the time step enter (double for the flux itself; one of the sides or both DualD
 // for a column of the linearisation); gradients stay double.
+
 // one side of the interface: state, half-space seeds
 template <typename S>
 struct GksSide {
@@ -265,11 +266,6 @@ HD void gks_to_global(T F0, T F1, T F4, const T Ft[3], const double n[3], const 
 template <typename T>
 HD T viscosity(const Phys& ph, T t);
 
-// flux of one Gauss point: n the unit normal, weight the length of its area vector; WL, GL, WR, GR the
-// states and gradients of both sides (global frame; on a boundary face the ghost's), dt the face's time
-// step.  F: flux x weight averaged over dt; Wg (STATE): the interface state at dt; alpha (STATE): the
-// compression factor (1 on boundary faces and with the factor off).  Returns 0, or the number of the
-// check that failed (4 a side, 5 the interface state).  gks_flux is the flux itself, gks_flux_t its dual form
 // what the equilibrium part of a flux and of a column of its linearisation share
 template <typename T>
 struct GksCentre {
@@ -332,7 +328,12 @@ HD bool gks_centre(const GksSide<SL>& gl, const GksSide<SR>& gr, D dt, const Phy
   return positive(c.rho) && positive(c.p);
 }
 
-// T: the wider of the scalars of the sides and the time step.  n, weight and the gradients are double
+// flux of one Gauss point: n the unit normal, weight the length of its area vector; WL, GL, WR, GR the
+// states and gradients of both sides (global frame; on a boundary face the ghost's), dt the face's time
+// step.  F: flux x weight averaged over dt; Wg (STATE): the interface state at dt; alpha (STATE): the
+// compression factor (1 on boundary faces and with the factor off).  Returns 0, or the number of the
+// check that failed (4 a side, 5 the interface state).  T: the wider of the scalars of the sides and the time
+// step; n, weight and the gradients are double.  gks_flux is the flux itself, gks_flux_t its dual form
 template <bool STATE, typename SL, typename SR, typename T, typename D>
 HD int gks_flux_t(const double n[3], double weight, bool bnd, const SL WL[5], const double GL[15], const SR WR[5],
                   const double GR[15], D dt, const Phys& ph, const double* tab, T F[5], T Wg[5], T& alpha) {

@@ -191,41 +191,6 @@ HD DualD trsqrt<DualD>(DualD x) {
   return {r, -0.5 * r * r * r * x.d};
 }
 
-// branchless orthonormal basis (t1, t2) completing the unit normal n (Duff et al., JCGT 6(1), 2017)
-template <typename T>
-HD void face_frame(const T n[3], T t1[3], T t2[3]) {
-  const T sign = n[2] >= T(0) ? T(1) : T(-1);
-  const T a = T(-1) / (sign + n[2]);
-  const T b = n[0] * n[1] * a;
-  t1[0] = T(1) + sign * n[0] * n[0] * a;
-  t1[1] = sign * b;
-  t1[2] = -sign * n[0];
-  t2[0] = b;
-  t2[1] = sign + n[1] * n[1] * a;
-  t2[2] = -n[1];
-}
-
-// conservative state in the face frame -> primitive; false when rho <= 0 or p <= 0
-
-template <typename T>
-HD void rotate_in(const T W[5], const T n[3], const T t1[3], const T t2[3], T w[5]) {
-  w[0] = W[0];
-  w[1] = W[1] * n[0] + W[2] * n[1] + W[3] * n[2];
-  w[2] = W[1] * t1[0] + W[2] * t1[1] + W[3] * t1[2];
-  w[3] = W[1] * t2[0] + W[2] * t2[1] + W[3] * t2[2];
-  w[4] = W[4];
-}
-
-template <typename T>
-HD void rotate_out(const T f[5], const T n[3], const T t1[3], const T t2[3], T F[5]) {
-  F[0] = f[0];
-  F[1] = f[1] * n[0] + f[2] * t1[0] + f[3] * t2[0];
-  F[2] = f[1] * n[1] + f[2] * t1[1] + f[3] * t2[1];
-  F[3] = f[1] * n[2] + f[2] * t1[2] + f[3] * t2[2];
-  F[4] = f[4];
-}
-
-
 // x^(1/(gamma - 1)); the exponent of a diatomic gas is 5/2 (a power costs about 150 FP64 instructions)
 template <typename T>
 HD T tpow_igm1(T x, T igm1) {
