@@ -27,20 +27,20 @@ class DevicePool {
   DevicePool(const DevicePool&) = delete;
   DevicePool& operator=(const DevicePool&) = delete;
 
-  // what a request takes of the device: from 1 MiB on, whole pages of 2 MiB
-  static size_t rounded(size_t bytes) {
-    const size_t grain = bytes < ((size_t)1 << 20) ? 512 : (size_t)2 << 20;
-    return (bytes + grain - 1) / grain * grain;
+  // what an allocation takes of the device, which the bound counts: from 1 MiB on, whole pages of 2 MiB
+  static size_t device_bytes(size_t bytes) {
+    const size_t n = round_up(bytes, 512);
+    return n < ((size_t)1 << 20) ? n : round_up(n, (size_t)2 << 20);
   }
 
   // a block of at least `bytes`; the smallest free one that fits without wasting more than half of it
   Error take(void** p, size_t bytes) noexcept {
     *p = nullptr;
-    const size_t want = rounded(bytes);
-    if (want < bytes) return Api::out_of_memory;
+    const size_t want = round_up(bytes, 512), cost = device_bytes(bytes);
+    if (cost < bytes) return Api::out_of_memory;
     Block* best = nullptr;
     for (Block& b : blocks_)
-      if (!b.live && b.bytes >= want && b.bytes / 2 <= want && slack_ + (b.bytes - want) <= limit_ &&
+      if (!b.live && b.bytes >= want && b.bytes / 2 <= want && slack_ + (b.cost - cost) <= limit_ &&
           (!best || b.bytes < best->bytes))
         best = &b;
     if (!best) {
@@ -53,14 +53,14 @@ class DevicePool {
       Error e = api_.alloc(&q, want);
       if (e != Api::ok && drop(0)) e = api_.alloc(&q, want);
       if (e != Api::ok) return e;
-      blocks_.push_back({q, want, 0, false});  // within the capacity
+      blocks_.push_back({q, want, cost, 0, false});  // within the capacity
       best = &blocks_.back();
-      free_ += want;
+      free_ += cost;
     }
     best->live = true;
-    best->used = want;
-    free_ -= best->bytes;
-    slack_ += best->bytes - want;
+    best->used = cost;
+    free_ -= best->cost;
+    slack_ += best->cost - cost;
     *p = best->p;
     return Api::ok;
   }
@@ -70,8 +70,8 @@ class DevicePool {
     for (Block& b : blocks_)
       if (b.p == p && b.live) {
         b.live = false;
-        free_ += b.bytes;
-        slack_ -= b.bytes - b.used;
+        free_ += b.cost;
+        slack_ -= b.cost - b.used;
         break;
       }
     if (!hold_) drop(limit_);
@@ -86,9 +86,11 @@ class DevicePool {
   size_t slack() const { return slack_; }
 
  private:
+  static size_t round_up(size_t bytes, size_t grain) { return (bytes + grain - 1) / grain * grain; }
+
   struct Block {
     void* p;
-    size_t bytes, used;  // of the block, of the live request
+    size_t bytes, cost, used;  // of the block, on the device, of that the live request's
     bool live;
   };
 
@@ -101,7 +103,7 @@ class DevicePool {
         if (!blocks_[k].live && (big == blocks_.size() || blocks_[k].bytes > blocks_[big].bytes)) big = k;
       if (big == blocks_.size()) break;
       api_.release(blocks_[big].p);
-      free_ -= blocks_[big].bytes;
+      free_ -= blocks_[big].cost;
       blocks_[big] = blocks_.back();
       blocks_.pop_back();
       any = true;

@@ -19,27 +19,28 @@ struct Device {
   size_t used = 0, capacity = 0;
   long allocs = 0, failed = 0;
 };
+static size_t up(size_t n);
 struct Fake {
   using Error = int;
   static constexpr int ok = 0, out_of_memory = 2;
   Device* d;
   int alloc(void** p, size_t n) {
-    if (d->used + n > d->capacity) { ++d->failed; return out_of_memory; }
+    if (d->used + up(n) > d->capacity) { ++d->failed; return out_of_memory; }
     *p = std::malloc(1);
     d->blocks[*p] = n;
-    d->used += n;
+    d->used += up(n);
     ++d->allocs;
     return 0;
   }
   void release(void* p) {
     if (!d->blocks.count(p)) { std::puts("released twice or unknown"); std::exit(1); }
-    d->used -= d->blocks[p];
+    d->used -= up(d->blocks[p]);
     d->blocks.erase(p);
     std::free(p);
   }
 };
+static size_t up(size_t n) { return DevicePool<Fake>::device_bytes(n); }  // whole pages
 #define REQUIRE(c) do { if (!(c)) { std::printf("line %d: %s\n", __LINE__, #c); std::exit(1); } } while (0)
-static size_t up(size_t n) { return DevicePool<Fake>::rounded(n); }
 int main() {
   for (unsigned seed = 0; seed < 200; ++seed) {
     std::mt19937 rng(seed);
@@ -61,7 +62,7 @@ int main() {
             REQUIRE(!p && pool.held() == pool.slack() && dev.used + up(bytes) > dev.capacity);  // no free block left
             continue;
           }
-          REQUIRE(p && !live.count(p) && dev.blocks.at(p) >= up(bytes));
+          REQUIRE(p && !live.count(p) && dev.blocks.at(p) >= bytes);
           live[p] = up(bytes);
           total += up(bytes);
         } else {
