@@ -47,7 +47,7 @@ SAMPLE = dict(nx=96, ny=4, nz=69, outflow=5)
 # FP64 floating-point operations per Gauss point of the gas-kinetic flux kernel (2 per DFMA, 1 per
 # DADD/DMUL), from the ncu instruction counts of a full capture of the kernel on the 48x32x32 box;
 # the kernel's own arithmetic, all of which the method needs
-FLOP_PER_GP = 2026.4
+FLOP_PER_GP = 2027.4
 # DRAM bytes (read + write) per Gauss point of the same kernel from the same capture (None when the
 # kernel has changed since)
 DRAM_BYTES_PER_GP = 173.5
@@ -56,14 +56,14 @@ DRAM_BYTES_PER_GP = 173.5
 # reconstruction per cell (DFMA 1,177.1, DMUL 199.3, DADD 108.3, on the 96x4x69 slab, whose mix of prisms
 # and tetrahedra is the bench box's; a prism of the 48x32x32 box takes 2,956.4), gather with the
 # gradient update per Gauss point seen from a cell (DFMA 16.06, DMUL 2.17, DADD 5.11), the flux alone of the V-cycle's
-# defect per Gauss point (DFMA 682.5, DMUL 293.6, DADD 154.8), coarse KFVS face flux per face (DFMA
-# 83.8, DMUL 59.1, DADD 23.2: the launches of a V-cycle weighted by their faces).  The residual-only
+# defect per Gauss point (DFMA 688.5, DMUL 297.6, DADD 148.8), coarse KFVS face flux per face (DFMA
+# 77.8, DMUL 56.1, DADD 22.2: the launches of a V-cycle weighted by their faces).  The residual-only
 # gather of the defect (5.6 FLOP per point seen) and the coarse levels' gathers and steps (k_kfvs_gather)
 # are latency-bound, reported against HBM.
 FLOP_PER_CELL_RECON = 2661.8
 FLOP_PER_GP_SIDE_GATHER = 39.39
-FLOP_PER_GP_FLUX = 1813.4
-FLOP_PER_FACE_KFVS = 249.8
+FLOP_PER_GP_FLUX = 1823.4
+FLOP_PER_FACE_KFVS = 233.8
 ALU_KERNELS = {"k_gks_points": FLOP_PER_GP, "k_reconstruct": FLOP_PER_CELL_RECON,
                "k_gather": FLOP_PER_GP_SIDE_GATHER, "k_kfvs_faces": FLOP_PER_FACE_KFVS,
                "k_gks_points_flux": FLOP_PER_GP_FLUX}

@@ -165,10 +165,11 @@ __global__ void k_coarse_dt(int64_t nc, int64_t nf, const int32_t* __restrict__ 
 // F = Res* - R (stored), and W += dt / |Omega| (R + F).  GATHER false (first step of the mixed cycle):
 // R = 0 and F = Res*.  An update that would make rho or p non-positive is skipped for that cell
 // (counted), a non-finite one is an error.  The faces' fluxes are those of W before the step, so W is
-// updated in place.  Bound by its FP64 additions, with lanes idle where a warp's cells differ in faces (48-byte
-// face and flux records instead of component arrays changed nothing).  One launch instead of four (gather, forcing, time step, update), and the cell's
-// face list is read once: 0.23 ms per step of the 96x64x69 boundary layer (0.58 M cells on average)
-// against 0.31, 12 us against 45 on the 24x4x24 one (2,231 cells).
+// updated in place.  Bound by its FP64 additions, with lanes idle where a warp's cells differ in faces
+// (48-byte face and flux records instead of component arrays changed nothing).  One launch instead of four
+// (gather, forcing, time step, update), and the cell's face list is read once: 0.23 ms per step of the
+// 96x64x69 boundary layer (0.58 M cells on average) against 0.31, 12 us against 45 on the 24x4x24 one
+// (2,231 cells).
 struct CoarseStep {
   int64_t nc, nf;
   const int32_t *ptr, *c2f, *fL, *fR;

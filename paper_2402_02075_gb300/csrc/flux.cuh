@@ -22,8 +22,8 @@
 //    the final projection removes;
 //  - both sides' moments are summed in the frame moving with the interface's tangential velocity, where
 //    the heat flux of the Prandtl correction needs three of the time-integrated moments only.
-// Measured on the 96x64x69 boundary layer (10.67 M points), CUDA events: 23.4 ms with the interface
-// state, 21.2 ms the flux alone (1,255 and 1,131 FP64 instructions per point), against 37.6 and 35.6 ms
+// Measured on the 96x64x69 boundary layer (10.67 M points), CUDA events: 23.5 ms with the interface
+// state, 21.2 ms the flux alone (1,256 and 1,135 FP64 instructions per point), against 37.6 and 35.6 ms
 // (2,007 and 1,900) by point_flux<double>.  Blocks of 32, 64 and 128 threads take the same time; three or
 // four blocks of 128 per SM (168 or 128 registers, with spills) 2 to 3 % more.
 #pragma once
